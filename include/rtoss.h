@@ -384,6 +384,12 @@ rtoss_status rtoss_chain_deps_spans(const uint64_t* spans, int n, uint32_t* afte
  * per-kernel patterns on ordinary weights; 9 - k of every 9 with rtoss_select_patterns_shared); inside a block the
  * pruned taps are multiplied as zeros.  Results agree with the FMA path to fp32 summation order.
  *
+ * RTOSS_PATH_AUTO also brings 16-bit calls there whose x it cannot read in place (NCHW; channels last with Cin no multiple
+ * of 8): x is first written once as channels last, into stream-ordered memory of the context (at most 1 GiB of it is kept
+ * between calls; rtoss_destroy gives it back; a call for which there is no memory runs on the FMA path), and y is written
+ * in the layout asked for.  Such calls take no residual operand; RTOSS_PATH_TENSOR refuses them, RTOSS_PATH_FMA does
+ * without the copy.
+ *
  * Device-side waits of that path are bounded.  If one runs out, the kernel records a non-zero code in
  * the context and returns; rtoss_device_status synchronises the device, reports the code
  * (RTOSS_ERR_TIMEOUT when non-zero) and clears it. */

@@ -112,13 +112,13 @@ __global__ void __launch_bounds__(kChunk) batch_select_pack_kernel(const BatchLa
             const unsigned m = s_masks[best];
             if (L.v_dtype == RTOSS_F32)
                 rtoss_dev::pack_one<float>(v, m, i, L.k, (float*)L.val, (float*)L.wtc, L.ksize, L.Cin, L.lay.rows, L.lay.rep_rows,
-                                           L.lay.copies);
+                                           L.lay.copies, L.lay.cin_p);
             else if (L.v_dtype == RTOSS_BF16)
                 rtoss_dev::pack_one<__nv_bfloat16>(v, m, i, L.k, (__nv_bfloat16*)L.val, (__nv_bfloat16*)L.wtc, L.ksize, L.Cin,
-                                                   L.lay.rows, L.lay.rep_rows, L.lay.copies);
+                                                   L.lay.rows, L.lay.rep_rows, L.lay.copies, L.lay.cin_p);
             else
                 rtoss_dev::pack_one<__half>(v, m, i, L.k, (__half*)L.val, (__half*)L.wtc, L.ksize, L.Cin, L.lay.rows, L.lay.rep_rows,
-                                            L.lay.copies);
+                                            L.lay.copies, L.lay.cin_p);
         }
     }
 }
@@ -221,7 +221,7 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
         B.issue = p->issue;
         B.issue_n = p->issue_n;
         B.n_kernels = p->n_kernels;
-        B.lay = rtoss_wtc_layout_of(it.Cout, it.ksize);
+        B.lay = rtoss_wtc_layout_of(it.Cout, it.Cin, it.ksize, p->dtype);
         B.Cout = it.Cout;
         B.Cin = it.Cin;
         B.ksize = it.ksize;

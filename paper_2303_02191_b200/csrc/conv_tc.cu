@@ -111,7 +111,11 @@ struct TcArgs {
     int tap_sub[9], tap_shift[9];  // which sub-tile tap t reads, and from which start row
     int G;                                     // taps per weight stage (one barrier round trip per G taps)
     unsigned a_tx_bytes, b_tx_bytes;
+    // Output element (n, oy, ox, co) lies at n * y_img + (oy * Wo + ox) * y_c_stride + (y_c_off + co) * y_co:
+    // channels last y_co = 1; NCHW (nchw = 1) y_co = the plane, y_c_stride = 1.
     int act, y_c_off, y_c_stride, is_bf16;
+    int nchw, y_co;
+    long long y_img;
     unsigned idesc;
     int w_rows;           // filter rows per staged weight tile (128; fewer with positions as the M operand)
     int rep_rows, R;      // filters as M, narrow layer: the tile holds R copies of rep_rows filter rows (else 128, 1)
@@ -357,6 +361,11 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&r)[16]) {
         : "memory");
 }
 
+// Internal activation code: SiLU in the exponential form of the FMA path for 16-bit outputs too (calls that path used
+// to take keep its precision: the tanh form's 2^-11 is as coarse as half a unit in the last place of fp16).
+constexpr int kActSiluX = 3;
+__device__ __forceinline__ float silu_exp(float v) { return __fdividef(v, 1.f + __expf(-v)); }
+
 // Sixteen consecutive filters of one position (positions as the M operand): bias, activation, rounding, packed
 // two to a register in memory order.
 template <typename T, int ACT>
@@ -373,6 +382,7 @@ __device__ __forceinline__ void act_pack16(const unsigned (&r)[16], const float*
                 asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(0.5f * v[e]));
                 v[e] = v[e] * fmaf(0.5f, th, 0.5f);
             }
+            if (ACT == kActSiluX) v[e] = silu_exp(v[e]);
         }
         o[j >> 1] = pack2<T>(v[0], v[1]);
     }
@@ -420,6 +430,7 @@ __device__ __forceinline__ float bias_act(unsigned acc_bits, float bs) {
         asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(h));
         return fmaf(h, th, h);
     }
+    if (ACT == kActSiluX) return silu_exp(acc + bs);   // (bs is the plain bias)
     return acc + bs;
 }
 
@@ -608,6 +619,62 @@ __device__ __forceinline__ void epilogue_chunks_res(unsigned d_base, int c0, int
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// NCHW outputs: sixteen positions of 32 filters (a half chunk).  NCHW wants the positions of one filter side by side,
+// which is what a lane holds, but a store wants its 32 lanes to be neighbours: the half chunk goes through the warp's
+// patch (32 rows of eight words, word j of filter f at column j ^ (f / 4): both the stores, all filters of one position
+// pair, and the loads, eight pairs of four filters, touch 32 different banks) and leaves as 32-byte runs, one word of
+// two positions per lane where the pair is one aligned word, else one element at a time.  pair_ok: planes of an even
+// number of elements, so that one look at the offsets holds for every filter.
+template <typename T, int ACT>
+__device__ __forceinline__ void epilogue_half_nchw(const unsigned (&r)[16], float bs, unsigned patch, unsigned tab_at, T* yb,
+                                                   unsigned ry, unsigned rx, int lane, int n_co, int plane, bool pair_ok) {
+    const unsigned wr = patch + (unsigned)lane * 32u;
+    const unsigned sw = (unsigned)(lane >> 2) & 7u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const unsigned w = round_pack<T, ACT == RTOSS_ACT_RELU>(bias_act<ACT>(r[2 * j], bs), bias_act<ACT>(r[2 * j + 1], bs));
+        asm volatile("st.shared.u32 [%0], %1;" ::"r"(wr + ((j ^ sw) << 2)), "r"(w) : "memory");
+    }
+    __syncwarp();
+    const int jj = lane & 7, f0 = lane >> 3;
+    unsigned e[4];   // table entries of positions 2 jj and 2 jj + 1
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3]) : "r"(tab_at + (unsigned)jj * 16u));
+    const bool ok0 = (e[1] >> 16) < ry && (e[1] & 0xFFFFu) < rx, ok1 = (e[3] >> 16) < ry && (e[3] & 0xFFFFu) < rx;
+    const bool pair = pair_ok && ok0 && ok1 && e[2] == e[0] + 1 && !(reinterpret_cast<uintptr_t>(yb + e[0]) & 3);
+    T* d = yb + (size_t)f0 * plane;
+#pragma unroll
+    for (int i = 0; i < 8; ++i, d += (size_t)4 * plane) {
+        const int f = 4 * i + f0;
+        unsigned w;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w) : "r"(patch + (unsigned)f * 32u + ((jj ^ i) << 2)));   // (f / 4 = i)
+        if (f < n_co) {
+            if (pair) {
+                *reinterpret_cast<unsigned*>(d + e[0]) = w;
+            } else {
+                const T* h = reinterpret_cast<const T*>(&w);
+                if (ok0) d[e[0]] = h[0];
+                if (ok1) d[e[2]] = h[1];
+            }
+        }
+    }
+    __syncwarp();
+}
+template <typename T, int ACT>
+__device__ __forceinline__ void epilogue_chunks_nchw(unsigned d_base, int c0, int c_step, int n_px, float bs, unsigned patch, unsigned tab,
+                                                     T* yb, unsigned ry, unsigned rx, int lane, int n_co, int plane, bool pair_ok) {
+    if (c0 >= n_px) return;
+    unsigned ra[16], rb[16];
+    tmem_ld16(d_base + (unsigned)c0, ra);
+    for (; c0 < n_px; c0 += c_step) {
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_ld16(d_base + (unsigned)(c0 + kPatchRows), rb);
+        epilogue_half_nchw<T, ACT>(ra, bs, patch, tab + (unsigned)c0 * 8, yb, ry, rx, lane, n_co, plane, pair_ok);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (c0 + c_step < n_px) tmem_ld16(d_base + (unsigned)(c0 + c_step), ra);
+        epilogue_half_nchw<T, ACT>(rb, bs, patch, tab + (unsigned)(c0 + kPatchRows) * 8, yb, ry, rx, lane, n_co, plane, pair_ok);
+    }
+}
+
 // Split K, second half.  Every CTA of the cluster owns the 32-column chunks c of the tile with c % KS == its rank
 // (its local chunk lc = c / KS) and holds, in its own shared memory at `buf`, what each of the KS shares summed
 // for them: share i, local chunk lc, column col, accumulator lane row at ((i * n_lc + lc) * 32 + col) * 128 + row
@@ -615,7 +682,8 @@ __device__ __forceinline__ void epilogue_chunks_res(unsigned d_base, int c0, int
 template <typename T, int ACT>
 __device__ __forceinline__ void epilogue_from_shares(unsigned buf, int KS, int rank, int n_lc, int sub, int row, int n_px, float bs,
                                                      bool vec_ok, bool co_ok, unsigned patch, unsigned tab, const uint2* pos_tab,
-                                                     T* yb, unsigned ry, unsigned rx, int lane, const T* rb, bool post) {
+                                                     T* yb, unsigned ry, unsigned rx, int lane, const T* rb, bool post, bool nchw,
+                                                     int n_co, int y_co) {
     const unsigned wr = patch + lane * 4;
     const unsigned rd = patch + (lane >> 2) * kPairPitch + (lane & 3) * 32;
     const unsigned tab_l = tab + (unsigned)(2 * (lane >> 2)) * 8;
@@ -643,6 +711,9 @@ __device__ __forceinline__ void epilogue_from_shares(unsigned buf, int KS, int r
         if constexpr (sizeof(T) == 2) {
             if (vec_ok) {
                 epilogue_half<T, ACT>(r, bs, wr, rd, tab_l + (unsigned)c0 * 8, ybv, ry, rx, rbv, post);
+                done = true;
+            } else if (nchw) {
+                epilogue_half_nchw<T, ACT>(r, bs, patch, tab + (unsigned)c0 * 8, yb, ry, rx, lane, n_co, y_co, (y_co & 1) == 0);
                 done = true;
             }
         }
@@ -762,7 +833,9 @@ __device__ __forceinline__ bool wait_deps(const G& g, unsigned dep_mask) {
     return true;
 }
 
-template <typename T, typename G>
+// kRep: the launch follows a layout pass (rtoss_launch_conv_tc_repacked): 16-bit outputs may be NCHW and SiLU takes its
+// exponential form.  An instantiation of its own: carried as run-time branches the two cost every other launch 0.5-1 %.
+template <typename T, typename G, bool kRep = false>
 __global__ void __launch_bounds__(kTcThreads, 1)
 conv_tc_kernel(const __grid_constant__ G g) {
     constexpr bool kMulti = sizeof(G) > sizeof(TcLaunch1);
@@ -1220,7 +1293,8 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const unsigned d_base = tmem_base + (unsigned)(as * g.acc_stride) + ((unsigned)(quarter * 32) << 16);
-                T* yb = yg + (((size_t)n * a.Ho + y0) * a.Wo + x0) * a.y_c_stride + a.y_c_off;
+                T* yb = kRep ? yg + (size_t)n * a.y_img + ((size_t)y0 * a.Wo + x0) * a.y_c_stride + (size_t)a.y_c_off * a.y_co
+                             : yg + (((size_t)n * a.Ho + y0) * a.Wo + x0) * a.y_c_stride + a.y_c_off;
                 const unsigned ry = (unsigned)min(a.TH, a.Ho - y0), rx = (unsigned)min(a.TW, a.Wo - x0);
                 for (int item = sub; item < items; item += 4) {
                     const int h = item / n_chunks, c = item - h * n_chunks;
@@ -1233,18 +1307,19 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     unsigned o[8];
                     if (a.act == RTOSS_ACT_SILU) act_pack16<T, RTOSS_ACT_SILU>(r, b16, o);
                     else if (a.act == RTOSS_ACT_RELU) act_pack16<T, RTOSS_ACT_RELU>(r, b16, o);
+                    else if (kRep && a.act == kActSiluX) act_pack16<T, kActSiluX>(r, b16, o);
                     else act_pack16<T, RTOSS_ACT_NONE>(r, b16, o);
                     if (px_ok) {
-                        T* dst = yb + e.x + c * 16;
+                        T* dst = yb + e.x + (kRep ? (size_t)(c * 16) * a.y_co : (size_t)(c * 16));   // (NCHW: a store covers 32 neighbouring positions of a filter)
                         if (vec_ok && c * 16 + 16 <= a.Cout) {
                             reinterpret_cast<uint4*>(dst)[0] = make_uint4(o[0], o[1], o[2], o[3]);
                             reinterpret_cast<uint4*>(dst)[1] = make_uint4(o[4], o[5], o[6], o[7]);
                         } else {
-                            // ragged filter count or unaligned channel slice: element stores
+                            // NCHW, ragged filter count or unaligned channel slice: element stores
                             const T* ov = reinterpret_cast<const T*>(o);
 #pragma unroll
                             for (int j = 0; j < 16; ++j)
-                                if (c * 16 + j < a.Cout) dst[j] = ov[j];
+                                if (c * 16 + j < a.Cout) dst[kRep ? (size_t)j * a.y_co : (size_t)j] = ov[j];
                         }
                     }
                 }
@@ -1277,7 +1352,9 @@ conv_tc_kernel(const __grid_constant__ G g) {
             const unsigned patch = s_tmem_ptr + 16 + (unsigned)(warp - 2) * kPatchBytes;  // shared address
             // (fp32 outputs leave through the element stores below: a warp's 32 filters of one position are 128 contiguous bytes)
             const bool vec_ok = !kF32 && (a.y_c_stride % 8 == 0) && ((a.y_c_off + co0) % 8 == 0) && (co0 + row0 + 32 <= a.Cout);
-            T* yb = yg + (((size_t)n * a.Ho + y0) * a.Wo + x0) * a.y_c_stride + a.y_c_off + co0 + row0;
+            T* yb = kRep ? yg + (size_t)n * a.y_img + ((size_t)y0 * a.Wo + x0) * a.y_c_stride + (size_t)(a.y_c_off + co0 + row0) * a.y_co
+                         : yg + (((size_t)n * a.Ho + y0) * a.Wo + x0) * a.y_c_stride + a.y_c_off + co0 + row0;
+            const int n_co = a.Cout - co0 - row0;   // this quarter's filters inside the layer (at most 32 count)
             const unsigned ry = (unsigned)min(a.TH, a.Ho - y0), rx = (unsigned)min(a.TW, a.Wo - x0);  // rows / columns inside the image
             const int c_first = (sub + 4 * copy) * 32, c_step = 128 * a.R;
             const T* rb = a.resid ? reinterpret_cast<const T*>(a.resid) + (yb - yg) : nullptr;   // laid out like y
@@ -1312,11 +1389,13 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 if (ok) {
                     const int row = quarter * 32 + lane;
                     if (a.act == RTOSS_ACT_SILU)
-                        epilogue_from_shares<T, RTOSS_ACT_SILU>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post);
+                        epilogue_from_shares<T, RTOSS_ACT_SILU>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post, kRep && a.nchw, n_co, a.y_co);
                     else if (a.act == RTOSS_ACT_RELU)
-                        epilogue_from_shares<T, RTOSS_ACT_RELU>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post);
+                        epilogue_from_shares<T, RTOSS_ACT_RELU>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post, kRep && a.nchw, n_co, a.y_co);
+                    else if (kRep && a.act == kActSiluX)
+                        epilogue_from_shares<T, kActSiluX>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post, kRep && a.nchw, n_co, a.y_co);
                     else
-                        epilogue_from_shares<T, RTOSS_ACT_NONE>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post);
+                        epilogue_from_shares<T, RTOSS_ACT_NONE>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post, kRep && a.nchw, n_co, a.y_co);
                 }
                 continue;
             }
@@ -1342,8 +1421,19 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         epilogue_chunks<T, RTOSS_ACT_SILU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
                     else if (a.act == RTOSS_ACT_RELU)
                         epilogue_chunks<T, RTOSS_ACT_RELU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
+                    else if (kRep && a.act == kActSiluX)
+                        epilogue_chunks<T, kActSiluX>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
                     else
                         epilogue_chunks<T, RTOSS_ACT_NONE>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
+                } else if (kRep && a.nchw) {
+                    stored = true;
+                    const bool pair_ok = (a.y_co & 1) == 0;
+                    if (a.act == kActSiluX)
+                        epilogue_chunks_nchw<T, kActSiluX>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, n_co, a.y_co, pair_ok);
+                    else if (a.act == RTOSS_ACT_RELU)
+                        epilogue_chunks_nchw<T, RTOSS_ACT_RELU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, n_co, a.y_co, pair_ok);
+                    else
+                        epilogue_chunks_nchw<T, RTOSS_ACT_NONE>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, n_co, a.y_co, pair_ok);
                 }
             }
             if (!stored) {
@@ -1368,6 +1458,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                 v = v * fmaf(0.5f, th, 0.5f);
                             }
                         }
+                        if (kRep && a.act == kActSiluX) v = silu_exp(v);
                         if (rb && in_img && post) v = to_f32<T>(from_f32<T>(v)) + to_f32<T>(__ldcg(rb + e.x + lane));   // behind the activation
                         if (co_ok && (e.y >> 16) < ry && (e.y & 0xFFFFu) < rx) yb[e.x + lane] = from_f32<T>(v);
                     }
@@ -1608,7 +1699,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     pp->a_stage_bytes = plan.n_sub * plan.sub_rows * row_bytes * (f32 ? 2 : 1);
     a.w_rows = w_rows;
     // narrow 3x3 layers keep the filters on M and repeat them down the 128 rows of the tile
-    const rtoss_wtc_layout lay = rtoss_wtc_layout_of(p->Cout, p->ksize);  // how rtoss_pack laid the weights out
+    const rtoss_wtc_layout lay = rtoss_wtc_layout_of(p->Cout, p->Cin, p->ksize, p->dtype);  // how rtoss_pack laid the weights out
     a.rep_rows = lay.copies > 1 ? lay.rep_rows : 128;
     a.R = lay.copies;
     a.rep_shift = a.rep_rows == 32 ? 5 : a.rep_rows == 64 ? 6 : 7;
@@ -1619,7 +1710,11 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     a.b_tx_bytes = (unsigned)(row_bytes * w_rows);
     a.act = (int)d->act;
     a.y_c_off = d->y_channel_offset;
-    a.y_c_stride = d->y_channel_stride ? d->y_channel_stride : p->Cout;
+    const int cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;   // channels of the output tensor
+    a.nchw = d->layout == RTOSS_NCHW ? 1 : 0;   // (of the output: x is channels last here, see rtoss_launch_conv_tc_repacked)
+    a.y_c_stride = a.nchw ? 1 : cs;
+    a.y_co = a.nchw ? Ho * Wo : 1;
+    a.y_img = (long long)cs * Ho * Wo;
     a.is_bf16 = p->dtype == RTOSS_BF16;
     // instruction descriptor: fp32 accumulate, A and B of the io type (f16 0, bf16 1; kind::tf32: tf32 2), both K-major,
     // N/8 and M/16
@@ -1650,8 +1745,9 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     if (!ea) {
         ea = &ctx->tmap_cache[ctx->tmap_next];
         ctx->tmap_next = (ctx->tmap_next + 1) % 32;
-        cuuint64_t dims[4] = {(cuuint64_t)p->Cin, (cuuint64_t)d->W, (cuuint64_t)d->H, (cuuint64_t)d->N};
-        cuuint64_t strides[3] = {(cuuint64_t)p->Cin * esize, (cuuint64_t)d->W * p->Cin * esize, (cuuint64_t)d->H * d->W * p->Cin * esize};
+        const cuuint64_t cp = (cuuint64_t)lay.cin_p;   // pixels are cin_p channels apart (the caller's tensor: cin_p == Cin)
+        cuuint64_t dims[4] = {cp, (cuuint64_t)d->W, (cuuint64_t)d->H, (cuuint64_t)d->N};
+        cuuint64_t strides[3] = {cp * esize, (cuuint64_t)d->W * cp * esize, (cuuint64_t)d->H * d->W * cp * esize};
         // with element strides the box is counted in traversed elements: S*n covers n fetched pixels
         cuuint32_t box[4] = {(cuuint32_t)a.cb_ch, (cuuint32_t)(plan.Wq * S), (cuuint32_t)(plan.rows_staged * S), 1};
         cuuint32_t es[4] = {1, (cuuint32_t)S, (cuuint32_t)S, 1};
@@ -1667,8 +1763,8 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     // weights: one descriptor per handle
     rtoss_tmap_entry* eb = &p->wtc_map;
     if (!eb->valid || eb->base != p->wtc || eb->dims[0] != w_rows || eb->dims[1] != plan.G) {
-        cuuint64_t dims[3] = {(cuuint64_t)p->Cin, (cuuint64_t)lay.rows, (cuuint64_t)a.taps};
-        cuuint64_t strides[2] = {(cuuint64_t)p->Cin * esize, (cuuint64_t)lay.rows * p->Cin * esize};
+        cuuint64_t dims[3] = {(cuuint64_t)lay.cin_p, (cuuint64_t)lay.rows, (cuuint64_t)a.taps};
+        cuuint64_t strides[2] = {(cuuint64_t)lay.cin_p * esize, (cuuint64_t)lay.rows * lay.cin_p * esize};
         cuuint32_t box[3] = {(cuuint32_t)a.cb_ch, (cuuint32_t)w_rows, (cuuint32_t)plan.G};  // a weight stage is one copy
         cuuint32_t es[3] = {1, 1, 1};
         eb->valid = 0;
@@ -1731,6 +1827,10 @@ int ensure_smem_attr(const rtoss_ctx* ctx) {
             e = cudaFuncSetAttribute(conv_tc_kernel<float, TcLaunch1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(conv_tc_kernel<float, TcLaunchN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(conv_tc_kernel<__nv_bfloat16, TcLaunch1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(conv_tc_kernel<__half, TcLaunch1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return (int)e;
         if (dev_slot >= 0) attr_set[dev_slot].store(true, std::memory_order_release);
     }
@@ -1750,13 +1850,15 @@ void launch_common(const rtoss_ctx* ctx, G* g) {
 
 }  // namespace
 
-bool rtoss_tc_weights_eligible(const rtoss_packed* p) {
-    return ((p->dtype == RTOSS_BF16 || p->dtype == RTOSS_F16) && p->Cin % 8 == 0) || (p->dtype == RTOSS_F32 && p->Cin % 4 == 0);  // 16-byte rows for TMA
-}
+// Handles that get weights for the tensor path: 16-bit ones (rows padded to 16 bytes), fp32 ones whose rows are multiples
+// of 16 bytes as they are.
+bool rtoss_tc_weights_eligible(const rtoss_packed* p) { return p->dtype != RTOSS_F32 || p->Cin % 4 == 0; }
+// Layers whose channels-last activations TMA can read where they lie.
+static bool rows_fit_tma(const rtoss_packed* p) { return p->Cin % (p->dtype == RTOSS_F32 ? 4 : 8) == 0; }
 
 // Can this call run on the tensor path?
 bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y) {
-    if (!p->wtc || !rtoss_tc_weights_eligible(p)) return false;
+    if (!p->wtc || !rows_fit_tma(p)) return false;
     if (d->layout != RTOSS_NHWC || (int)d->io_dtype != (int)p->dtype) return false;
     if ((reinterpret_cast<uintptr_t>(x) & 15) || (reinterpret_cast<uintptr_t>(y) & 15)) return false;
     if (!encode_fn()) return false;
@@ -1791,7 +1893,7 @@ bool rtoss_tc_prefers_split(const rtoss_ctx* ctx, const rtoss_packed* p, const r
     const long tiles = (long)d->N * ((Ho + plan.TH - 1) / plan.TH) * plan.tiles_x * co_tiles;
     if (tiles_out) *tiles_out = tiles;
     int ks = 1, cb_per = 0;
-    pick_split(p->ksize, pxm, rtoss_wtc_layout_of(p->Cout, p->ksize).copies, tiles, (p->Cin + cb_ch - 1) / cb_ch, plan.N_px,
+    pick_split(p->ksize, pxm, rtoss_wtc_layout_of(p->Cout, p->Cin, p->ksize, p->dtype).copies, tiles, (p->Cin + cb_ch - 1) / cb_ch, plan.N_px,
                plan.NA * a_stage + plan.NB * b_stage, sms, &ks, &cb_per);
     return ks > 1;
 }
@@ -1806,7 +1908,7 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     memset(&fake, 0, sizeof(fake));
     fake.Cin = Cin, fake.Cout = Cout, fake.ksize = ksize, fake.dtype = dtype;
     const rtoss_packed* p = &fake;
-    if (!rtoss_tc_weights_eligible(p) || d->layout != RTOSS_NHWC) return RTOSS_OK;   // (eligible stays 0)
+    if (!rows_fit_tma(p) || d->layout != RTOSS_NHWC) return RTOSS_OK;   // (eligible stays 0)
     const int sms = sm_count > 0 ? sm_count : 148;
     const int Ho = (d->H - 1) / d->stride + 1, Wo = (d->W - 1) / d->stride + 1;
     const bool pxm = use_pxm(p), f32 = dtype == RTOSS_F32;
@@ -1828,13 +1930,21 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     const long tiles = (long)d->N * ((Ho + plan.TH - 1) / plan.TH) * plan.tiles_x * (pxm ? 1 : co_tiles);
     out->tiles = (int)(tiles > 0x7FFFFFFF ? 0x7FFFFFFF : tiles);
     int ks = 1, cb_per = 0;
-    pick_split(ksize, pxm, rtoss_wtc_layout_of(Cout, ksize).copies, tiles, ncb, plan.N_px,
+    pick_split(ksize, pxm, rtoss_wtc_layout_of(Cout, Cin, ksize, dtype).copies, tiles, ncb, plan.N_px,
                plan.NA * out->act_stage_bytes + plan.NB * out->weight_stage_bytes, sms, &ks, &cb_per);
     out->split_k = ks;
     return RTOSS_OK;
 }
 
-int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d,
+// The instantiation a launch of one convolution runs.
+static void (*single_kernel(bool f32, bool bf16, bool repacked))(const TcLaunch1) {
+    if (f32) return conv_tc_kernel<float, TcLaunch1>;
+    if (repacked) return bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1, true> : conv_tc_kernel<__half, TcLaunch1, true>;
+    return bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1> : conv_tc_kernel<__half, TcLaunch1>;
+}
+
+// One convolution, channels last in x.  repacked: x is the copy of rtoss_launch_conv_tc_repacked.
+static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, bool repacked,
                          void* stream) {
     const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
     static thread_local TcLaunch1 g;   // several KB: kept off the stack
@@ -1843,6 +1953,7 @@ int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     int e = build_problem(ctx, p, x, y, d, 1, sms, &g.prob[0], &pp, &g.tmA[0], &g.tmB[0]);
     if (e) return e;
     TcArgs& a = g.prob[0];
+    if (repacked && a.act == RTOSS_ACT_SILU) a.act = kActSiluX;
     const TcPlan& plan = pp.plan;
     const bool f32 = p->dtype == RTOSS_F32;
     a.NA = plan.NA;
@@ -1878,9 +1989,7 @@ int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     cudaError_t le;
     if (a.KS > 1) {
         // one cluster per tile; if the device cannot place the clusters the layer runs uncut
-        le = f32 ? rtoss_dev::launch_pdl(conv_tc_kernel<float, TcLaunch1>, grid, kTcThreads, smem, (cudaStream_t)stream, a.KS, g)
-             : a.is_bf16 ? rtoss_dev::launch_pdl(conv_tc_kernel<__nv_bfloat16, TcLaunch1>, grid, kTcThreads, smem, (cudaStream_t)stream, a.KS, g)
-                         : rtoss_dev::launch_pdl(conv_tc_kernel<__half, TcLaunch1>, grid, kTcThreads, smem, (cudaStream_t)stream, a.KS, g);
+        le = rtoss_dev::launch_pdl(single_kernel(f32, a.is_bf16, repacked), grid, kTcThreads, smem, (cudaStream_t)stream, a.KS, g);
         if (le == cudaSuccess) return 0;
         cudaGetLastError();
         a.KS = 1;
@@ -1890,10 +1999,62 @@ int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void
         g.unit_end[0] = (int)n_units;
         grid = dim3((unsigned)(n_units < (size_t)sms ? n_units : (size_t)sms));
     }
-    le = f32 ? rtoss_dev::launch_pdl(conv_tc_kernel<float, TcLaunch1>, grid, kTcThreads, smem, (cudaStream_t)stream, 1, g)
-         : a.is_bf16 ? rtoss_dev::launch_pdl(conv_tc_kernel<__nv_bfloat16, TcLaunch1>, grid, kTcThreads, smem, (cudaStream_t)stream, 1, g)
-                     : rtoss_dev::launch_pdl(conv_tc_kernel<__half, TcLaunch1>, grid, kTcThreads, smem, (cudaStream_t)stream, 1, g);
+    le = rtoss_dev::launch_pdl(single_kernel(f32, a.is_bf16, repacked), grid, kTcThreads, smem, (cudaStream_t)stream, 1, g);
     return (int)le;
+}
+
+int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d,
+                         void* stream) {
+    return launch_single(ctx, p, x, y, d, false, stream);
+}
+
+// The calls the tensor path takes behind a pass that lays x out for it (repack.cu): 16-bit data in NCHW, or channels last
+// with pixels of no multiple of 16 bytes.  What then runs: 1x1 layers of stride 2 keep only the pixels they read and
+// become layers of stride 1.  Three-channel stems stay with their own kernel (conv3x3_small_cin_kernel), which reads the
+// image once and has next to nothing to contract.
+static rtoss_conv_desc repacked_desc(const rtoss_packed* p, const rtoss_conv_desc* d) {
+    rtoss_conv_desc dd = *d;
+    if (p->ksize == 1 && d->stride == 2) {
+        dd.H = (d->H - 1) / 2 + 1;
+        dd.W = (d->W - 1) / 2 + 1;
+        dd.stride = 1;
+    }
+    return dd;
+}
+bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) {
+    if (d->path != RTOSS_PATH_AUTO || d->residual_dev || !p->wtc || p->dtype == RTOSS_F32 || (int)d->io_dtype != (int)p->dtype) return false;
+    if (d->layout == RTOSS_NHWC && rows_fit_tma(p)) return false;   // (native, or declined for another reason)
+    if (p->ksize == 3 && p->Cin <= 4) return false;
+    if (!encode_fn()) return false;
+    const rtoss_conv_desc dd = repacked_desc(p, d);
+    const int Ho = (dd.H - 1) / dd.stride + 1, Wo = (dd.W - 1) / dd.stride + 1;
+    // Small 3x3 layers of few channels: two launches cost more than the FMA kernel's few rounds (16->32 @42x10, batch 8:
+    // 27.9 us here, 10.3 us there; 16->30 @23x20: 21 / 10; from about 2^17 outputs on the FMA kernel needs more than one
+    // wave: 16->32 @100x101, batch 2: 19 us here, 46 us there).
+    if (p->ksize == 3 && p->Cin <= 16 && (long long)dd.N * Ho * Wo * p->Cout <= (1 << 17)) return false;
+    const bool pxm = use_pxm(p);
+    TcPlan plan;
+    return plan_tc(dd.N, Ho, Wo, p->ksize, dd.stride, (p->Cout + kMTile - 1) / kMTile, 148, pxm, pxm ? round_up(p->Cout, 16) : kMTile, false,
+                   &plan, 1, false, 0, 1, row_bytes_of(p), ncb_of(p));
+}
+// Returns a cudaError_t, or -1 when there was no memory for the channels-last copy (nothing was launched).  The copy
+// lives from here to the end of the convolution in the stream's order, in the context's pool: any number of streams and
+// threads may be in such a call, and inside a stream capture the copy belongs to the graph.
+int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d,
+                                  void* stream) {
+    const rtoss_conv_desc dd = repacked_desc(p, d);
+    const int cp = rtoss_cin_pitch(p->Cin, p->dtype), S = dd.stride == d->stride ? 1 : 2;
+    void* ws = nullptr;
+    const size_t bytes = (size_t)dd.N * dd.H * dd.W * cp * 2;
+    void* pool = rtoss_ctx_pool(ctx);
+    if (!pool || cudaMallocFromPoolAsync(&ws, bytes, (cudaMemPool_t)pool, (cudaStream_t)stream) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
+    }
+    int e = rtoss_launch_repack16(x, ws, dd.N, p->Cin, cp, d->H, d->W, S, d->layout, stream);
+    if (!e) e = launch_single(ctx, p, ws, y, &dd, true, stream);
+    const cudaError_t fe = cudaFreeAsync(ws, (cudaStream_t)stream);
+    return e ? e : (int)fe;
 }
 
 // Several convolutions in ONE launch: independent ones side by side, dependent ones one behind the other.

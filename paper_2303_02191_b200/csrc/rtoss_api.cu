@@ -4,6 +4,7 @@
 
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <vector>
 #include <new>
 
@@ -98,6 +99,10 @@ int dispatch_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
         return 0;
     }
     if (tc_ok) return rtoss_launch_conv_tc(ctx, p, x, y, d, stream);
+    if (rtoss_tc_repack_eligible(p, d)) {
+        const int e = rtoss_launch_conv_tc_repacked(ctx, p, x, y, d, stream);
+        if (e >= 0) return e;   // (-1: no memory for the copy of x; the FMA path needs none)
+    }
     return p->ksize == 3 ? rtoss_launch_conv3x3(ctx, p, x, y, d, stream) : rtoss_launch_conv1x1(ctx, p, x, y, d, stream);
 }
 
@@ -108,6 +113,26 @@ rtoss_device_guard::rtoss_device_guard(int device) : prev(device), switched(fals
 }
 rtoss_device_guard::~rtoss_device_guard() {
     if (switched) cudaSetDevice(prev);
+}
+
+void* rtoss_ctx_pool(const rtoss_ctx* ctx) {
+    static std::mutex making;   // (two threads may make their first such call on one context at once)
+    std::lock_guard<std::mutex> hold(making);
+    if (!ctx->pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        cudaMemPool_t pool = nullptr;
+        unsigned long long keep = kPoolKeep;
+        if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            ctx->pool = pool;
+        } else {
+            cudaGetLastError();   // (without a pool the calls that want one run on the FMA path)
+        }
+    }
+    return ctx->pool;
 }
 
 extern "C" {
@@ -167,6 +192,7 @@ void rtoss_destroy(rtoss_ctx* ctx) {
     if (ctx->ws_y) cudaFree(ctx->ws_y);
     if (ctx->dev_status) cudaFree(ctx->dev_status);
     if (ctx->chain_done) cudaFree(ctx->chain_done);
+    if (ctx->pool) cudaMemPoolDestroy((cudaMemPool_t)ctx->pool);   // (memory still in use by the stream is released when its free is reached)
     cudaSetDevice(prev);
     delete ctx;
 }
@@ -285,8 +311,9 @@ rtoss_status rtoss_pack(rtoss_ctx* ctx, const void* w_dev, rtoss_dtype w_dtype, 
         }
         if (e == cudaSuccess && rtoss_tc_weights_eligible(p)) {
             // dense-expanded weights of the tensor path; zeroed once: the trailing Cout*Cin mod 9 weights of a 1x1
-            // layer are pruned for good and no later pack writes them
-            const size_t wtc_bytes = (size_t)(ksize == 3 ? 9 : 1) * rtoss_wtc_layout_of(Cout, ksize).rows * Cin *
+            // layer are pruned for good, and neither they nor the padding of the rows are written by a later pack
+            const rtoss_wtc_layout lay = rtoss_wtc_layout_of(Cout, Cin, ksize, compute_dtype);
+            const size_t wtc_bytes = (size_t)(ksize == 3 ? 9 : 1) * lay.rows * lay.cin_p *
                                      rtoss_dtype_size(compute_dtype) * (compute_dtype == RTOSS_F32 ? 2 : 1);   // fp32: heads + remainders
             e = cudaMalloc(&p->wtc, wtc_bytes);
             if (e == cudaSuccess) e = cudaMemsetAsync(p->wtc, 0, wtc_bytes, s);

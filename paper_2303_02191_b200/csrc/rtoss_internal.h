@@ -15,6 +15,7 @@ struct rtoss_tmap_entry {
     alignas(64) unsigned char map[128];
 };
 
+constexpr unsigned long long kPoolKeep = 1ull << 30;  // bytes a context's pool holds on to between calls
 constexpr int kHostChunks = 8;  // the host-buffer path cuts a batch into at most this many chunks
 
 // Launches that carry dependent convolutions count completed problems in device memory: a block of
@@ -42,6 +43,7 @@ struct rtoss_ctx {
     mutable int inject_next;   // failure-detection test hook: the next tensor-path launch withholds its first weight copy
     mutable rtoss_tmap_entry tmap_cache[32];  // activation descriptors of the tensor path, round robin
     mutable int tmap_next;
+    mutable void* pool;        // cudaMemPool_t, made at first use (rtoss_ctx_pool), of the channels-last copies some calls need (stream-ordered; keeps at most kPoolKeep bytes)
     unsigned* chain_done;      // device: RTOSS_CHAIN_SLOTS x RTOSS_CHAIN_SLOT_WORDS completion counters, all zero at rest
     mutable int chain_next;    // the block the next launch with dependent convolutions takes
 };
@@ -56,7 +58,7 @@ struct rtoss_packed {
     uint32_t* perm;        // [Cin*Cout]      (ksize 3)
     uint32_t* bucket_off;  // [Cin*(P+1)]     (ksize 3)
     uint16_t* masks_dev;   // [256]
-    void* wtc;             // tensor path: dense-expanded weights [taps][Cout][Cin] in dtype, or NULL
+    void* wtc;             // tensor path: dense-expanded weights [taps][rows][cin_p] in dtype (rtoss_wtc_layout_of), or NULL
     unsigned long long* issue;  // tensor path, ksize 3: per (tile of 128 filters, block of 64 channels) which (tap, 16-channel
                                 // slab) pairs hold any kept weight (bit 4*tap + slab); [issue_n] words, or NULL
     int issue_n;
@@ -91,9 +93,12 @@ static inline size_t rtoss_dtype_size(rtoss_dtype d) { return d == RTOSS_F32 ? 4
 // epilogue warp has lanes to read.
 struct rtoss_wtc_layout {
     int rows, rep_rows, copies;
+    int cin_p;   // channels per row as stored: rows of 16-bit weights are padded with zeros to a multiple of 16 bytes (TMA strides)
 };
-static inline rtoss_wtc_layout rtoss_wtc_layout_of(int Cout, int ksize) {
+static inline int rtoss_cin_pitch(int Cin, rtoss_dtype d) { return d == RTOSS_F32 ? Cin : (Cin + 7) / 8 * 8; }
+static inline rtoss_wtc_layout rtoss_wtc_layout_of(int Cout, int Cin, int ksize, rtoss_dtype d) {
     rtoss_wtc_layout l;
+    l.cin_p = rtoss_cin_pitch(Cin, d);
     if (ksize == 3 && Cout <= 64) {
         l.rep_rows = Cout <= 32 ? 32 : 64;
         l.rows = 128;
@@ -126,7 +131,7 @@ int rtoss_launch_conv1x1(const rtoss_ctx* ctx, const rtoss_packed* p, const void
 static inline int rtoss_issue_cb_log2(rtoss_dtype d) { return d == RTOSS_F32 ? 5 : 6; }   // channels per 128-byte block
 static inline int rtoss_issue_words(int Cout, int Cin, int ksize, rtoss_dtype d) {
     const int cb = 1 << rtoss_issue_cb_log2(d);
-    return ((rtoss_wtc_layout_of(Cout, ksize).rows + 127) / 128) * ((Cin + cb - 1) / cb);
+    return ((rtoss_wtc_layout_of(Cout, Cin, ksize, d).rows + 127) / 128) * ((Cin + cb - 1) / cb);
 }
 
 // tensor path (conv_tc.cu)
@@ -134,6 +139,12 @@ bool rtoss_tc_weights_eligible(const rtoss_packed* p);
 bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y);
 int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                          const rtoss_conv_desc* d, void* stream);
+// 16-bit calls the tensor path takes after a pass that writes x channels last (repack.cu); -1: no memory for the copy
+bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d);
+int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
+                                  const rtoss_conv_desc* d, void* stream);
+void* rtoss_ctx_pool(const rtoss_ctx* ctx);   // null: none to be had
+int rtoss_launch_repack16(const void* x, void* out, int N, int Cin, int cp, int H, int W, int S, rtoss_layout layout, void* stream);
 bool rtoss_tc_groupable(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y);
 // several independent convolutions in one launch: 0 = launched, -1 = the set cannot share a launch (nothing launched)
 int rtoss_launch_conv_tc_group(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const void* const* xs,

@@ -44,12 +44,12 @@ template <> __device__ __forceinline__ __half narrow_to<__half>(float v) { retur
 
 // Writes of one kernel (3x3) or run of nine (1x1) with mask m: its k kept values, ascending taps, rounded to V, to
 // val[i*k ...]; and, where the handle carries dense-expanded weights for the tensor path (wtc != nullptr), all nine
-// taps, pruned ones as +0:  3x3 -> wtc[t][row][ci] with `rows` rows per tap, filter co = i / Cin at rows
-// c*rep_rows + co for c < copies (one copy at row co in the plain layout);  1x1 -> wtc[9*i + t].  fp32 handles hold
+// taps, pruned ones as +0:  3x3 -> wtc[t][row][ci] with `rows` rows of cin_p channels per tap, filter co = i / Cin at rows
+// c*rep_rows + co for c < copies (one copy at row co in the plain layout);  1x1 -> position 9*i + t of the flat matrix.  fp32 handles hold
 // two such arrays back to back: tf32 heads, then remainders.
 template <typename V>
 __device__ __forceinline__ void pack_one(const float (&w)[9], unsigned m, int64_t i, int k, V* __restrict__ val,
-                                         V* __restrict__ wtc, int ksize, int Cin, int rows, int rep_rows, int copies) {
+                                         V* __restrict__ wtc, int ksize, int Cin, int rows, int rep_rows, int copies, int cin_p) {
     V* out = val + i * k;
     if (k * (int)sizeof(V) == 8) {
         // the k kept values of a kernel are 8 aligned bytes (four 16-bit or two 32-bit values): pushed into a 64-bit word
@@ -81,7 +81,7 @@ __device__ __forceinline__ void pack_one(const float (&w)[9], unsigned m, int64_
         const int64_t co = (int64_t)((unsigned)i / (unsigned)Cin), ci = i - co * Cin;
         // fp32: the tensor path multiplies tf32 operands, so every weight is stored as its tf32 head (the 19 leading bits)
         // and, in a second copy of the array behind the first, the remainder (exact in fp32)
-        const int64_t lo_at = (int64_t)(ksize == 3 ? 9 : 1) * rows * Cin;
+        const int64_t lo_at = (int64_t)(ksize == 3 ? 9 : 1) * rows * cin_p;
 #pragma unroll
         for (int t = 0; t < 9; ++t) {
             V v = (m & (1u << t)) ? narrow_to<V>(w[t]) : narrow_to<V>(0.f);
@@ -93,14 +93,16 @@ __device__ __forceinline__ void pack_one(const float (&w)[9], unsigned m, int64_
                 lo = narrow_to<V>(__fsub_rn(f, head));
             }
             if (ksize == 3) {
-                const int64_t at = ((int64_t)t * rows + co) * Cin + ci;   // copy 0; copy c lies c * rep_rows rows further down
+                const int64_t at = ((int64_t)t * rows + co) * cin_p + ci;   // copy 0; copy c lies c * rep_rows rows further down
                 for (int c = 0; c < copies; ++c) {
-                    wtc[at + (int64_t)c * rep_rows * Cin] = v;
-                    if (sizeof(V) == 4) wtc[lo_at + at + (int64_t)c * rep_rows * Cin] = lo;
+                    wtc[at + (int64_t)c * rep_rows * cin_p] = v;
+                    if (sizeof(V) == 4) wtc[lo_at + at + (int64_t)c * rep_rows * cin_p] = lo;
                 }
             } else {
-                wtc[i * 9 + t] = v;
-                if (sizeof(V) == 4) wtc[lo_at + i * 9 + t] = lo;
+                int64_t at = i * 9 + t;   // flat position; rows are cin_p apart where they are padded
+                if (cin_p != Cin) at += (int64_t)((unsigned)at / (unsigned)Cin) * (cin_p - Cin);
+                wtc[at] = v;
+                if (sizeof(V) == 4) wtc[lo_at + at] = lo;
             }
         }
     }

@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(kSelThreads) pack_values_kernel(const T* __res
             float v[9];
 #pragma unroll
             for (int t = 0; t < 9; ++t) v[t] = widen<T>(sw[threadIdx.x * 9 + t]);
-            rtoss_dev::pack_one<V>(v, table.m[id], i, k, val, wtc, ksize, Cin, lay.rows, lay.rep_rows, lay.copies);
+            rtoss_dev::pack_one<V>(v, table.m[id], i, k, val, wtc, ksize, Cin, lay.rows, lay.rep_rows, lay.copies, lay.cin_p);
         }
     }
 }
@@ -239,7 +239,7 @@ static int launch_pack_values_t(const T* w, int64_t n, const MaskTable& t, const
 int rtoss_launch_pack_values(const void* w, rtoss_dtype wdt, int64_t n_kernels, const MaskTable& t, const uint8_t* pid,
                              int k, void* val, rtoss_dtype vdt, uint8_t* pid_copy, void* wtc, int ksize, int Cout, int Cin,
                              void* stream) {
-    const rtoss_wtc_layout lay = rtoss_wtc_layout_of(Cout, ksize);
+    const rtoss_wtc_layout lay = rtoss_wtc_layout_of(Cout, Cin, ksize, vdt);
     if (n_kernels <= 0) return 0;
     cudaStream_t s = (cudaStream_t)stream;
     switch (wdt) {
