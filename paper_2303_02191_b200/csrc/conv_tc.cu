@@ -1534,7 +1534,83 @@ int ncb_of(const rtoss_packed* p) {
 
 struct TcPlan {
     int TH, TW, Wq, N_px, NA, NB, G, n_sub, sub_rows, rows_staged, tiles_x, smem;
+    int KS, cb_per;      // CTAs that share a tile's channel blocks (a cluster), blocks per share
+    long tiles;          // tiles of the layer (not counting shares)
+    double us;           // what the model below expects of a launch of its own
+    double tile_us, epi_us;   // and of one tile: operands and instructions, epilogue
 };
+
+// What a plan depends on; plain values, so that equal calls have equal plans whatever tensors they bring.
+struct PlanKey {
+    int N, Ho, Wo, ksize, S, Cin, Cout, dtype;
+    int resid;       // a residual operand (its staging takes shared memory)
+    int sms, dev;    // SMs to fill; device whose cluster limits hold (-1: the built-in ones)
+    int shared;      // a problem of a shared launch, which never splits; 1: beside others, tiles are judged by the work they
+                     // do per cycle; 2: with nothing beside it
+    int max_px;      // most positions per tile
+    int force_G, n_tabs;
+};
+
+// Most thread-block clusters of `ks` CTAs (one CTA per SM) a device holds at once.  Clusters live inside a GPC and the
+// GPCs of a B200 differ in size, so 148 SMs hold 32 clusters of four and 15 of eight, not 37 and 18: a launch of one more
+// takes twice the time (measured: 32 x 4 CTAs 11 us, 36 x 4 CTAs 19 us).  Asked of the device once; -1 or a device that
+// cannot be asked: the figures of this one.
+std::atomic<int> g_max_clusters[64][9];
+int max_clusters(int dev, int ks, int sms) {
+    static const int kDefault[9] = {0, 148, 74, 40, 32, 20, 20, 15, 15};
+    if (ks <= 1) return sms;
+    int have = dev >= 0 && dev < 64 ? g_max_clusters[dev][ks].load(std::memory_order_relaxed) : 0;
+    if (have <= 0) have = kDefault[ks];
+    return have * sms / 148 < have ? have * sms / 148 : have;
+}
+
+// Expected time of a launch, in microseconds, for one way of cutting a layer.  The constants are a fit to 8 000 measured
+// (layer, tile, split) combinations of the two detectors' layers and odd shapes, batch 1 to 18, launches back to back
+// (programmatic dependent launch); typical error 10 %, and the plan it picks is within 1.5 % of the best measured one over
+// all layers.  What it knows:
+//   - an instruction takes N / 2 cycles for N positions, but never less than 79; per weight stage 0.2 us of barrier
+//     round trip, per channel block 0.1;
+//   - a CTA is fed at most 87 KB per us;
+//   - the epilogue's sixteen warps take the accumulator in chunks of 32 columns, four warps a chunk: up to 128 positions
+//     cost what 32 cost, 0.5 us; positions on M: filters in groups of 16 instead;
+//   - a launch costs 1.9 us whatever it does, 0.6 more when it leaves no SM for the next one to start on, and 0.5 us until
+//     its first operands are there;
+//   - sharing a tile's channel blocks: 0.13 us + 0.34 per CTA of the cluster + 0.33 per chunk exchanged.
+struct PlanCost {
+    double us, tile_us, epi_us;
+};
+PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R, int n_px, int halves, int a_bytes, int G, int na,
+                   long tiles, int KS, int cb_per) {
+    const bool f32 = k.dtype == RTOSS_F32;
+    const int taps = k.ksize == 3 ? 9 : 1;
+    const int slab_ch = f32 ? 8 : 16, cb_ch = row_bytes / (f32 ? 4 : 2);
+    const double slabs = (double)(k.Cin < cb_ch ? k.Cin : cb_ch) / slab_ch * (f32 ? 3 : 1);
+    const int wstages = f32 ? 2 * taps / G : taps / G;
+    const double instr = (pxm ? 79.0 * halves : n_px > 158 ? n_px / 2.0 : 79.0) / 1900.0;
+    const double mma = taps * slabs * instr + 0.205 * wstages + 0.09;
+    const double kb_b = (double)taps * w_rows * row_bytes * (f32 ? 2 : 1) / 1024.0, kb_a = a_bytes / 1024.0;
+    double blk = mma > (kb_a + kb_b) / 87.0 ? mma : (kb_a + kb_b) / 87.0;
+    // one activation stage: loads and instructions take turns (fp32: and one warp's split of the block between them)
+    if (na == 1) blk = mma + (f32 ? 0.045 * kb_a : 0.35 * kb_a / 87.0);
+    if (f32 && G == 3) blk += 2.0;   // (then only two weight stages fit: the ring's round trip shows)
+    const int chunks = (n_px + 31) / 32;
+    double epi;
+    if (pxm) epi = 0.92 * 0.5 * ((halves * ((k.Cout + 15) / 16) + 3) / 4);
+    else if (KS > 1) epi = 0.52 * 0.5 * ((2 * ((chunks + KS - 1) / KS) + 3) / 4);
+    else epi = 0.52 * ((chunks + 4 * R - 1) / (4 * R));
+    if (f32) epi *= 12.9;   // element stores
+    const double first_kb = kb_a + kb_b / taps * G;
+    PlanCost c;
+    c.tile_us = cb_per * blk;
+    c.epi_us = epi;
+    const long ctas = tiles * KS < k.sms ? tiles * KS : k.sms;
+    const long waves = (tiles * KS + k.sms - 1) / k.sms;
+    double us = 1.92 + (ctas > k.sms / 2 ? 0.59 * (ctas - k.sms / 2) / (k.sms / 2.0) : 0.0) + 0.51 + first_kb / 87.0 + c.tile_us + epi;
+    if (waves > 1) us += (waves - 1) * (c.tile_us > epi ? c.tile_us : epi) + 0.61 * tiles / k.sms;
+    if (KS > 1) us += 0.13 + 0.34 * KS + 0.33 * chunks;
+    c.us = us;
+    return c;
+}
 
 // Geometry of a tile.  Positions of a tile run over TH rows of pitch Wq = TW + (columns of halo the
 // staged rows carry); every tap reads the staged list from a shifted start row.
@@ -1545,25 +1621,38 @@ struct TcPlan {
 //                 TW+1 pixels fetched with element strides 2; tap r reads the odd rows for r = 0, 2 and
 //                 the even rows for r = 1, one staged row further down for r = 1, 2; columns alike.
 // The plan picks TH, the column segment TW (images wider than a TMA box are cut into segments), the
-// ring depths, and how many taps share a weight stage.
-bool plan_tc(int N, int Ho, int Wo, int ksize, int S, int co_tiles, int sm_count, bool pxm, int w_rows, bool resid, TcPlan* out,
-             int n_prob = 1, bool f32 = false, int force_G = 0, int n_tabs = 1, int row_bytes = kRowBytes, int ncb = 2) {
+// ring depths, how many taps share a weight stage, and over how many CTAs of a cluster the channel blocks of a tile are
+// spread (split K: a tile's MMAs are one serial chain; at most 8 CTAs, all of a launch's clusters on the device at once).
+// only_ks: 0 = any split, else that one.
+bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
+    const bool f32 = k.dtype == RTOSS_F32;
+    const bool pxm = k.ksize == 1 && k.Cout <= kPxmMaxCout && !f32;
+    const int w_rows = pxm ? round_up(k.Cout, 16) : kMTile;
+    const int row_bytes = (!f32 && k.Cin <= 32) ? 64 : kRowBytes;
+    const int cb_ch = row_bytes / (f32 ? 4 : 2), ncb = (k.Cin + cb_ch - 1) / cb_ch;
+    const int co_tiles = pxm ? 1 : (k.Cout + kMTile - 1) / kMTile;
+    const int R = rtoss_wtc_layout_of(k.Cout, k.Cin, k.ksize, (rtoss_dtype)k.dtype).copies;
+    const int S = k.S, Ho = k.Ho, Wo = k.Wo, ksize = k.ksize;
     const int halo = ksize == 3 ? (S == 1 ? 2 : 1) : 0;
     const int n_sub = (ksize == 3 && S == 2) ? 4 : 1;
     const int max_pitch = S == 1 ? 256 : 128;  // TMA box: at most 256 elements traversed per dimension
     const int fixed = 1024 /*alignment slack*/ + 512 /*barriers*/ + kEpiWarps * kPatchBytes /*epilogue patches*/ +
-                      n_tabs * kMaxPx * 8 /*position tables*/ + (resid ? kEpiWarps * kResStage : 0) /*staging of the residual operand*/;
+                      k.n_tabs * kMaxPx * 8 /*position tables*/ + (resid ? kEpiWarps * kResStage : 0) /*staging of the residual operand*/;
     const int cap = 227 * 1024 - 64;
-    const bool grouped = n_prob > 1;   // one of several problems that run side by side: together they fill the SMs
-    double best = -1;
+    double best = 0;
+    bool found = false;
     for (int nseg = 1; nseg <= 16; ++nseg) {
         const int tw = (Wo + nseg - 1) / nseg;
         const int wq = tw + halo;
         if (wq > max_pitch || wq > 256) continue;
+        if (nseg > 1 && (tw < 4 || (Wo + nseg - 2) / (nseg - 1) == tw) && found) continue;   // (the same columns as with fewer segments)
         for (int th = 1; th <= Ho; ++th) {
             const int rows_staged = th + halo;
             if (th * wq > 256 || rows_staged * S > 256) break;
+            const int ty = (Ho + th - 1) / th;
+            if (th > 1 && (Ho + ty - 1) / ty != th) continue;   // (the same bands with fewer rows)
             const int n_px = round_up(th * wq, 16);
+            if (n_px > k.max_px && found) break;
             const int max_shift = ksize == 3 ? (S == 1 ? 2 * wq + 2 : wq + 1) : 0;
             int need_rows = n_px + max_shift > rows_staged * wq ? n_px + max_shift : rows_staged * wq;
             // positions as the M operand: every instruction reads 128 rows, also where the tile's list ends earlier
@@ -1571,8 +1660,9 @@ bool plan_tc(int N, int Ho, int Wo, int ksize, int S, int co_tiles, int sm_count
             if (pxm && max_shift + 128 * halves > need_rows) need_rows = max_shift + 128 * halves;
             const int sub_rows = round_up(need_rows, 8);
             const int a_bytes = n_sub * sub_rows * row_bytes * (f32 ? 2 : 1);   // (fp32: heads and remainders)
+            const long tiles = (long)k.N * ty * nseg * co_tiles;
             for (int G = (ksize == 3 ? 3 : 1); G >= 1; G -= 2) {
-                if (force_G && G != force_G) continue;   // (the problems of one launch share the weight ring: one G for all)
+                if (k.force_G && G != k.force_G) continue;   // (the problems of one launch share the weight ring: one G for all)
                 const int b_bytes = G * w_rows * row_bytes;
                 int na = (cap - fixed - 2 * b_bytes) / a_bytes;
                 if (na < 1) continue;
@@ -1585,45 +1675,126 @@ bool plan_tc(int N, int Ho, int Wo, int ksize, int S, int co_tiles, int sm_count
                 int nb = (cap - fixed - na * a_bytes) / b_bytes;
                 if (nb > kMaxB) nb = kMaxB;
                 if (nb < 2) continue;
-                const long tiles = (long)N * ((Ho + th - 1) / th) * nseg * co_tiles;
-                const double waves = (double)tiles / sm_count;
-                const double balance = grouped ? 1.0 : waves / (double)((tiles + sm_count - 1) / sm_count);  // 1 = SMs equally loaded
-                // What counts is useful positions per tensor-pipe cycle.  An instruction with the filters on M and N positions
-                // takes N / 2 cycles, but never less than 76 (measured: 128.2 cycles at N = 256, 75.9 at every N <= 128).
-                // That is the measure for 3x3 layers of stride 1, whose tiles are bound by their instructions; the tiles of
-                // 1x1 and stride-2 layers are bound by what surrounds the instructions (fetches, barrier rounds, the
-                // epilogue) and do better with as many positions per tile as fit (measured both ways, layer by layer).
-                // (Nor does it pay where the smaller tiles would still fit one wave: such layers gain more from tiles of 256
-                // positions cut along the channel blocks.)
-                const bool by_cycles = ksize == 3 && S == 1 && n_px / 2.0 < 128.0 && (grouped || tiles > sm_count);
-                const double instr_cycles = pxm ? 128.0 * halves : by_cycles ? (n_px / 2.0 > 76.0 ? n_px / 2.0 : 76.0) : 128.0;
-                const double eff = (double)(th * tw) / (2.0 * instr_cycles) * Ho / (double)((Ho + th - 1) / th * th) * Wo / (double)(tw * nseg);
-                const double halo_cost = (double)(th * tw) / (double)(rows_staged * wq);  // staged pixels that are outputs
-                // (fp32: a block feeds 108 instructions, twelve per tap, so a stage per tap costs little, while a single
-                // activation stage leaves the fetch and the split of the next block uncovered)
-                const double score = eff * (0.5 + 0.5 * balance) * (G == 3 || ksize == 1 ? 1.0 : (f32 ? 0.95 : 0.8)) *
-                                         (na >= 2 ? 1.0 : (f32 ? 0.7 : 0.8)) * (0.8 + 0.2 * halo_cost) +
-                                     1e-4 * th;
-                if (score > best) {
-                    best = score;
-                    out->TH = th;
-                    out->TW = tw;
-                    out->Wq = wq;
-                    out->N_px = n_px;
-                    out->NA = na;
-                    out->NB = nb;
-                    out->G = G;
-                    out->n_sub = n_sub;
-                    out->sub_rows = sub_rows;
-                    out->rows_staged = rows_staged;
-                    out->tiles_x = nseg;
-                    out->smem = na * a_bytes + nb * b_bytes + fixed;
+                const int rings = na * a_bytes + nb * b_bytes;
+                for (int ks = 1; ks <= 8; ++ks) {
+                    if (only_ks && ks != only_ks) continue;
+                    int cb_per = ncb;
+                    if (ks > 1) {
+                        if (k.shared || pxm || R != 1 || tiles * ks > k.sms || ks > ncb) break;
+                        if (tiles > max_clusters(k.dev, ks, k.sms)) continue;
+                        cb_per = (ncb + ks - 1) / ks;
+                        if ((ncb + cb_per - 1) / cb_per != ks) continue;   // (a share would be empty)
+                        // the owners' buffers for the partial sums lie in the rings
+                        const int n_lc = ((n_px + 31) / 32 + ks - 1) / ks;
+                        if (ks * n_lc > 16 || ks * n_lc * 16384 > rings) continue;
+                    }
+                    const PlanCost c = plan_cost(k, pxm, w_rows, row_bytes, R, n_px, halves, a_bytes, G, na, tiles, ks, cb_per);
+                    double cost = c.us;
+                    if (k.shared == 1) {
+                        // One of several problems that run side by side and together fill the SMs: what counts is the work
+                        // a tile does for the time it keeps a CTA (3x3 stride 1: bound by its instructions, N / 2 cycles but
+                        // never less than 76; other tiles by what surrounds the instructions: as many positions as fit).
+                        const bool by_cycles = ksize == 3 && S == 1 && n_px / 2.0 < 128.0;
+                        const double cyc = by_cycles ? (n_px / 2.0 > 76.0 ? n_px / 2.0 : 76.0) : 128.0;
+                        const double eff = (double)(th * tw) / (2.0 * cyc) * Ho / (double)(ty * th) * Wo / (double)(tw * nseg);
+                        const double halo_cost = (double)(th * tw) / (double)(rows_staged * wq);  // staged pixels that are outputs
+                        cost = -(eff * (G == 3 || ksize == 1 ? 1.0 : (f32 ? 0.95 : 0.8)) * (na >= 2 ? 1.0 : (f32 ? 0.7 : 0.8)) *
+                                     (0.8 + 0.2 * halo_cost) + 1e-4 * th);
+                    }
+                    if (!found || cost < best) {
+                        found = true;
+                        best = cost;
+                        out->TH = th;
+                        out->TW = tw;
+                        out->Wq = wq;
+                        out->N_px = n_px;
+                        out->NA = na;
+                        out->NB = nb;
+                        out->G = G;
+                        out->n_sub = n_sub;
+                        out->sub_rows = sub_rows;
+                        out->rows_staged = rows_staged;
+                        out->tiles_x = nseg;
+                        out->smem = rings + fixed;
+                        out->KS = ks;
+                        out->cb_per = cb_per;
+                        out->tiles = tiles;
+                        out->us = c.us;
+                        out->tile_us = c.tile_us;
+                        out->epi_us = c.epi_us;
+                    }
                 }
                 if (!f32) break;  // 16-bit data: the largest G that fits is taken for this (th, tw); fp32 weighs both
             }
         }
     }
-    return best > 0;
+    return found;
+}
+
+// The plan of a call.  The split is decided as if the call had a residual operand, whether it has one or not: a call with
+// a residual then adds up its products in the order of the same call without one (same bits).
+// Searching takes tens of microseconds of host time, more than a launch: every thread remembers the plans of its last
+// few hundred kinds of call.  A plan is a function of sizes alone, so it does not matter which thread or context asks.
+bool plan_tc(const PlanKey& k, TcPlan* out) {
+    struct Memo {
+        PlanKey key;
+        TcPlan plan;
+        bool set, ok;
+    };
+    constexpr int kMemo = 256;
+    static thread_local Memo memo[kMemo];
+    unsigned h = 2166136261u;
+    const int* w = reinterpret_cast<const int*>(&k);
+    for (size_t i = 0; i < sizeof(PlanKey) / sizeof(int); ++i) h = (h ^ (unsigned)w[i]) * 16777619u;
+    Memo& m = memo[(h ^ (h >> 15)) % kMemo];
+    if (!m.set || memcmp(&m.key, &k, sizeof(k)) != 0) {
+        m.set = false;
+        const bool pxm = k.ksize == 1 && k.Cout <= kPxmMaxCout && k.dtype != RTOSS_F32;
+        if (k.shared || pxm) {
+            m.ok = plan_search(k, k.resid != 0, 1, &m.plan);
+        } else {
+            int ks = 1;
+            if (plan_search(k, true, 0, &m.plan)) ks = m.plan.KS;
+            m.ok = plan_search(k, k.resid != 0, ks, &m.plan);
+        }
+        m.key = k;
+        m.set = true;
+    }
+    *out = m.plan;
+    return m.ok;
+}
+
+PlanKey plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, int sms, int dev) {
+    PlanKey k;
+    memset(&k, 0, sizeof(k));
+    k.N = d->N;
+    k.Ho = (d->H - 1) / d->stride + 1;
+    k.Wo = (d->W - 1) / d->stride + 1;
+    k.ksize = p->ksize;
+    k.S = d->stride;
+    k.Cin = p->Cin;
+    k.Cout = p->Cout;
+    k.dtype = (int)p->dtype;
+    k.resid = d->residual_dev ? 1 : 0;
+    k.sms = sms;
+    k.dev = dev;
+    k.max_px = kMaxPx;
+    k.n_tabs = 1;
+    return k;
+}
+
+// Can the layer be cut at all?  Its smallest tile is one row of the narrowest segment, with a weight stage per tap.
+bool plan_exists(const rtoss_packed* p, const rtoss_conv_desc* d) {
+    const int S = d->stride, Wo = (d->W - 1) / S + 1;
+    const bool f32 = p->dtype == RTOSS_F32, k3 = p->ksize == 3;
+    const int wq = (Wo + 15) / 16 + (k3 ? (S == 1 ? 2 : 1) : 0);
+    if (wq > (S == 1 ? 256 : 128)) return false;
+    const int rows = (k3 ? (S == 1 ? 3 : 2) : 1) * wq, shift = k3 ? (S == 1 ? 2 * wq + 2 : wq + 1) : 0;
+    const int list = round_up(wq, 16) + shift > rows ? round_up(wq, 16) + shift : rows;
+    const int need = use_pxm(p) ? shift + 256 : list;
+    const int a_bytes = (k3 && S == 2 ? 4 : 1) * round_up(need, 8) * row_bytes_of(p) * (f32 ? 2 : 1);
+    const int fixed = 1024 + 512 + kEpiWarps * kPatchBytes + kMaxPx * 8 + (d->residual_dev ? kEpiWarps * kResStage : 0);
+    return a_bytes + 2 * kMTile * kRowBytes + fixed <= 227 * 1024 - 64;
 }
 
 // What one problem adds to a launch besides its TcArgs.
@@ -1634,8 +1805,8 @@ struct ProbPlan {
 
 // Geometry, operand roles and TMA descriptors of one convolution.  The rings' depths and the split along K are the
 // launch's business (the caller's).  Returns a cudaError_t as int.
-int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, int n_prob, int sms,
-                  TcArgs* out, ProbPlan* pp, CUtensorMap* tmA_out, CUtensorMap* tmB_out, int force_G = 0, int n_tabs = 1) {
+int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, const PlanKey& plan_k,
+                  TcArgs* out, ProbPlan* pp, CUtensorMap* tmA_out, CUtensorMap* tmB_out) {
     const int taps = p->ksize == 3 ? 9 : 1;
     const int S = d->stride;
     const int Ho = (d->H - 1) / S + 1, Wo = (d->W - 1) / S + 1;
@@ -1647,8 +1818,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     const bool f32 = p->dtype == RTOSS_F32;
     const int esize = f32 ? 4 : 2;
     const int row_bytes = row_bytes_of(p);
-    if (!plan_tc(d->N, Ho, Wo, p->ksize, S, (p->Cout + kMTile - 1) / kMTile, sms, pxm, w_rows, d->residual_dev != nullptr, &plan, n_prob, f32,
-                 force_G, n_tabs, row_bytes, (p->Cin + row_bytes / esize - 1) / (row_bytes / esize)))
+    if (!plan_tc(plan_k, &plan))
         return (int)cudaErrorInvalidConfiguration;
 
     TcArgs& a = *out;
@@ -1782,39 +1952,13 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     return 0;
 }
 
-// Split K where the layer has too few tiles for the SMs and several channel blocks: a tile's MMAs are one serial chain
-// (an instruction costs the same however few positions it covers), so the blocks go to several CTAs.  The exchange
-// costs a few thousand cycles (two cluster barriers, 128 KB through distributed shared memory): chains of 72
-// instructions (3x3: two channel blocks) resp. 32 (1x1: eight blocks) and more are cut, a share keeps at least one
-// block (1x1: two); cutting shorter 1x1 chains was measured and lost.  The CTAs of a tile form one cluster (at most
-// 8), one CTA per share.  *ks = 1 leaves the layer uncut.
-void pick_split(int ksize, bool pxm, int R, long tiles, int ncb, int n_px, int rings, int sms, int* ks_out, int* cb_per_out) {
-    *ks_out = 1;
-    *cb_per_out = ncb;
-    const int min_cb = ksize == 3 ? 1 : 2;
-    const int min_ncb = ksize == 3 ? 2 : 8;
-    const int n_lc_max = 8;   // a tile has at most 8 chunks of 32 columns: the owner's buffers take KS * ceil(chunks / KS) * 16 KB
-    if (pxm || R != 1 || tiles * 2 > sms || ncb < min_ncb) return;
-    int want = (int)(sms / tiles);
-    if (want > ncb / min_cb) want = ncb / min_cb;
-    if (want > 8) want = 8;
-    while (want > 1) {
-        const int cb_per = (ncb + want - 1) / want, ks = (ncb + cb_per - 1) / cb_per;
-        const int n_chunks = (n_px + 31) / 32, n_lc = (n_chunks + ks - 1) / ks;
-        if (ks > 1 && ks * n_lc <= 2 * n_lc_max && (size_t)ks * n_lc * 16384 <= (size_t)rings) {
-            *cb_per_out = cb_per;
-            *ks_out = ks;
-            return;
-        }
-        --want;
-    }
-}
-
-// Both instantiations may use up to the whole shared memory of an SM; the attribute belongs to the (function, device)
-// pair, so there is one flag per device.
-int ensure_smem_attr(const rtoss_ctx* ctx) {
+int ctx_sms(const rtoss_ctx* ctx) { return ctx->sm_count > 0 ? ctx->sm_count : 148; }
+int ctx_dev(const rtoss_ctx* ctx) { return ctx->device >= 0 && ctx->device < 64 ? ctx->device : -1; }
+// Once per device: every instantiation may use up to the whole shared memory of an SM (the attribute belongs to the
+// (function, device) pair), and the planner learns how many clusters fit.
+int ensure_device(const rtoss_ctx* ctx) {
     static std::atomic<bool> attr_set[64];
-    const int dev_slot = ctx->device >= 0 && ctx->device < 64 ? ctx->device : -1;
+    const int dev_slot = ctx_dev(ctx);
     if (dev_slot < 0 || !attr_set[dev_slot].load(std::memory_order_acquire)) {
         cudaError_t e = cudaFuncSetAttribute(conv_tc_kernel<__nv_bfloat16, TcLaunch1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e == cudaSuccess)
@@ -1832,6 +1976,24 @@ int ensure_smem_attr(const rtoss_ctx* ctx) {
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(conv_tc_kernel<__half, TcLaunch1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return (int)e;
+        // how many clusters of each size the device holds at once (one CTA of this kernel per SM)
+        for (int ks = 2; ks <= 8 && dev_slot >= 0; ++ks) {
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(ctx_sms(ctx) / ks * ks));
+            cfg.blockDim = dim3(kTcThreads);
+            cfg.dynamicSmemBytes = 116 * 1024;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)ks;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, conv_tc_kernel<__nv_bfloat16, TcLaunch1>, &cfg) == cudaSuccess && n > 0)
+                g_max_clusters[dev_slot][ks].store(n, std::memory_order_relaxed);
+            else
+                cudaGetLastError();
+        }
         if (dev_slot >= 0) attr_set[dev_slot].store(true, std::memory_order_release);
     }
     return 0;
@@ -1864,11 +2026,7 @@ bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const vo
     if (!encode_fn()) return false;
     // a residual operand: 16-byte aligned, and not for the positions-as-M form (narrow 1x1 layers)
     if (d->residual_dev && (use_pxm(p) || (reinterpret_cast<uintptr_t>(d->residual_dev) & 15))) return false;
-    const int Ho = (d->H - 1) / d->stride + 1, Wo = (d->W - 1) / d->stride + 1;
-    TcPlan plan;
-    const bool pxm = use_pxm(p);
-    return plan_tc(d->N, Ho, Wo, p->ksize, d->stride, (p->Cout + kMTile - 1) / kMTile, 148, pxm, pxm ? round_up(p->Cout, 16) : kMTile,
-                   d->residual_dev != nullptr, &plan, 1, p->dtype == RTOSS_F32, 0, 1, row_bytes_of(p), ncb_of(p));
+    return plan_exists(p, d);
 }
 
 // May this call be one of several in a launch?  (Tensor path with the filters on M.)
@@ -1876,26 +2034,52 @@ bool rtoss_tc_groupable(const rtoss_packed* p, const rtoss_conv_desc* d, const v
     return !use_pxm(p) && rtoss_tc_eligible(p, d, x, y);
 }
 
-// Would a launch of its own cut this call along K (few tiles, many channel blocks)?  Such a call is faster alone than
-// as a member of a shared launch, which never cuts -- unless the other members keep the SMs busy meanwhile.
-// *tiles_out (nullable): the call's tiles of 128 filters.
-bool rtoss_tc_prefers_split(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, long* tiles_out) {
-    const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
-    const int Ho = (d->H - 1) / d->stride + 1, Wo = (d->W - 1) / d->stride + 1;
-    const bool pxm = use_pxm(p), f32 = p->dtype == RTOSS_F32;
-    const int w_rows = pxm ? round_up(p->Cout, 16) : kMTile, co_tiles = (p->Cout + kMTile - 1) / kMTile;
+// What one shared launch is expected to take for these independent calls, and the most positions a tile should have: many
+// small tiles where the set would leave SMs idle, 256 positions where it fills them for several rounds.
+static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds, int* px_out) {
+    static const int kPx[] = {256, 192, 128, 96, 64, 48, 32};
+    const int sms = ctx_sms(ctx);
+    double best = 1e30;
+    for (int px : kPx) {
+        double work = 0, longest = 0, epi = 0;
+        long tiles = 0;
+        bool ok = true;
+        for (int i = 0; i < n && ok; ++i) {
+            PlanKey key = plan_key(ps[i], ds[i], sms, ctx_dev(ctx));
+            key.shared = n > 1 ? 1 : 2;
+            key.max_px = px;
+            TcPlan plan;
+            ok = plan_tc(key, &plan);
+            if (!ok) break;
+            const double t = plan.tile_us > plan.epi_us ? plan.tile_us : plan.epi_us;
+            work += (double)plan.tiles * t;
+            tiles += plan.tiles;
+            if (t > longest) longest = t;
+            if (plan.epi_us > epi) epi = plan.epi_us;
+        }
+        if (!ok) continue;
+        // (3.4 us: launch, parameters of many problems, first operands; past one round a CTA may draw half a tile more than its share)
+        const double us = 3.4 + epi + (tiles <= sms ? longest : work / sms + 0.5 * longest);
+        if (us < 0.97 * best) {
+            best = us;
+            if (px_out) *px_out = px;
+        }
+    }
+    return best;
+}
+double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds) {
+    return shared_cost(ctx, n, ps, ds, nullptr);
+}
+
+// What a launch of its own is expected to take for this call (the planner's model), over how many CTAs it spreads a tile's
+// channel blocks, and how many tiles it has.  (Shared launches never split.)
+bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
-    if (tiles_out) *tiles_out = 0;
-    const int row_bytes = row_bytes_of(p);
-    if (!plan_tc(d->N, Ho, Wo, p->ksize, d->stride, co_tiles, sms, pxm, w_rows, d->residual_dev != nullptr, &plan, 1, f32, 0, 1, row_bytes, ncb_of(p))) return false;
-    const int a_stage = plan.n_sub * plan.sub_rows * row_bytes * (f32 ? 2 : 1), b_stage = plan.G * w_rows * row_bytes;
-    const int cb_ch = row_bytes / (f32 ? 4 : 2);
-    const long tiles = (long)d->N * ((Ho + plan.TH - 1) / plan.TH) * plan.tiles_x * co_tiles;
-    if (tiles_out) *tiles_out = tiles;
-    int ks = 1, cb_per = 0;
-    pick_split(p->ksize, pxm, rtoss_wtc_layout_of(p->Cout, p->Cin, p->ksize, p->dtype).copies, tiles, (p->Cin + cb_ch - 1) / cb_ch, plan.N_px,
-               plan.NA * a_stage + plan.NB * b_stage, sms, &ks, &cb_per);
-    return ks > 1;
+    if (!plan_tc(plan_key(p, d, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    *us = plan.us;
+    *ks = plan.KS;
+    *tiles = plan.tiles;
+    return true;
 }
 
 extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize, int Cin, int Cout, rtoss_dtype dtype, int sm_count,
@@ -1910,14 +2094,11 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     const rtoss_packed* p = &fake;
     if (!rows_fit_tma(p) || d->layout != RTOSS_NHWC) return RTOSS_OK;   // (eligible stays 0)
     const int sms = sm_count > 0 ? sm_count : 148;
-    const int Ho = (d->H - 1) / d->stride + 1, Wo = (d->W - 1) / d->stride + 1;
     const bool pxm = use_pxm(p), f32 = dtype == RTOSS_F32;
-    const int w_rows = pxm ? round_up(Cout, 16) : kMTile, co_tiles = (Cout + kMTile - 1) / kMTile;
+    const int w_rows = pxm ? round_up(Cout, 16) : kMTile;
     const int row_bytes = row_bytes_of(p);
     TcPlan plan;
-    const int ncb = (Cin + row_bytes / (f32 ? 4 : 2) - 1) / (row_bytes / (f32 ? 4 : 2));
-    if (!plan_tc(d->N, Ho, Wo, ksize, d->stride, co_tiles, sms, pxm, w_rows, d->residual_dev != nullptr, &plan, 1, f32, 0, 1, row_bytes, ncb))
-        return RTOSS_OK;
+    if (!plan_tc(plan_key(p, d, sms, -1), &plan)) return RTOSS_OK;
     out->eligible = 1;
     out->rows_per_tile = plan.TH, out->cols_per_tile = plan.TW, out->pitch = plan.Wq, out->positions = plan.N_px;
     out->act_stages = plan.NA, out->weight_stages = plan.NB, out->taps_per_weight_stage = plan.G;
@@ -1927,12 +2108,8 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     out->staged_rows = plan.rows_staged, out->sub_tiles = plan.n_sub;
     out->shared_bytes = plan.smem;
     out->positions_on_m = pxm ? 1 : 0;
-    const long tiles = (long)d->N * ((Ho + plan.TH - 1) / plan.TH) * plan.tiles_x * (pxm ? 1 : co_tiles);
-    out->tiles = (int)(tiles > 0x7FFFFFFF ? 0x7FFFFFFF : tiles);
-    int ks = 1, cb_per = 0;
-    pick_split(ksize, pxm, rtoss_wtc_layout_of(Cout, Cin, ksize, dtype).copies, tiles, ncb, plan.N_px,
-               plan.NA * out->act_stage_bytes + plan.NB * out->weight_stage_bytes, sms, &ks, &cb_per);
-    out->split_k = ks;
+    out->tiles = (int)(plan.tiles > 0x7FFFFFFF ? 0x7FFFFFFF : plan.tiles);
+    out->split_k = plan.KS;
     return RTOSS_OK;
 }
 
@@ -1946,11 +2123,15 @@ static void (*single_kernel(bool f32, bool bf16, bool repacked))(const TcLaunch1
 // One convolution, channels last in x.  repacked: x is the copy of rtoss_launch_conv_tc_repacked.
 static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, bool repacked,
                          void* stream) {
-    const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
+    const int sms = ctx_sms(ctx);
+    int e = ensure_device(ctx);
+    if (e) return e;
     static thread_local TcLaunch1 g;   // several KB: kept off the stack
     ProbPlan pp;
     g.n_prob = 1;
-    int e = build_problem(ctx, p, x, y, d, 1, sms, &g.prob[0], &pp, &g.tmA[0], &g.tmB[0]);
+    PlanKey key = plan_key(p, d, sms, ctx_dev(ctx));
+    if (ctx->inject_next) key.sms = 1;   // (failure-detection hook: as few CTAs as the layer allows)
+    e = build_problem(ctx, p, x, y, d, key, &g.prob[0], &pp, &g.tmA[0], &g.tmB[0]);
     if (e) return e;
     TcArgs& a = g.prob[0];
     if (repacked && a.act == RTOSS_ACT_SILU) a.act = kActSiluX;
@@ -1970,7 +2151,8 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     g.done = nullptr;
     g.acc_stride = pp.acc_cols;
     launch_common(ctx, &g);
-    pick_split(p->ksize, a.pxm != 0, a.R, (long)d->N * a.tiles_y * a.tiles_x * a.co_tiles, a.ncb, plan.N_px, rings, sms, &a.KS, &a.cb_per);
+    a.KS = plan.KS;
+    a.cb_per = plan.cb_per;
     magic_of(a.KS, a.div_ks);
     // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM
     const size_t smem = (size_t)(plan.smem > 116 * 1024 ? plan.smem : 116 * 1024);
@@ -1984,8 +2166,6 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     }
     g.unit_end[0] = (int)n_units;
     dim3 grid((unsigned)(n_units < (size_t)sms ? n_units : (size_t)sms));
-    e = ensure_smem_attr(ctx);
-    if (e) return e;
     cudaError_t le;
     if (a.KS > 1) {
         // one cluster per tile; if the device cannot place the clusters the layer runs uncut
@@ -2027,15 +2207,11 @@ bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) {
     if (p->ksize == 3 && p->Cin <= 4) return false;
     if (!encode_fn()) return false;
     const rtoss_conv_desc dd = repacked_desc(p, d);
-    const int Ho = (dd.H - 1) / dd.stride + 1, Wo = (dd.W - 1) / dd.stride + 1;
     // Small 3x3 layers of few channels: two launches cost more than the FMA kernel's few rounds (16->32 @42x10, batch 8:
     // 27.9 us here, 10.3 us there; 16->30 @23x20: 21 / 10; from about 2^17 outputs on the FMA kernel needs more than one
     // wave: 16->32 @100x101, batch 2: 19 us here, 46 us there).
-    if (p->ksize == 3 && p->Cin <= 16 && (long long)dd.N * Ho * Wo * p->Cout <= (1 << 17)) return false;
-    const bool pxm = use_pxm(p);
-    TcPlan plan;
-    return plan_tc(dd.N, Ho, Wo, p->ksize, dd.stride, (p->Cout + kMTile - 1) / kMTile, 148, pxm, pxm ? round_up(p->Cout, 16) : kMTile, false,
-                   &plan, 1, false, 0, 1, row_bytes_of(p), ncb_of(p));
+    if (p->ksize == 3 && p->Cin <= 16 && (long long)dd.N * ((dd.H - 1) / dd.stride + 1) * ((dd.W - 1) / dd.stride + 1) * p->Cout <= (1 << 17)) return false;
+    return plan_exists(p, &dd);
 }
 // Returns a cudaError_t, or -1 when there was no memory for the channels-last copy (nothing was launched).  The copy
 // lives from here to the end of the convolution in the stream's order, in the context's pool: any number of streams and
@@ -2074,7 +2250,9 @@ int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, c
 int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const void* const* xs, void* const* ys,
                                const rtoss_conv_desc* const* ds, const uint32_t* after, void* stream) {
     if (n < 2 || n > kMaxProb || ctx->inject_next) return -1;
-    const int sms = ctx->sm_count > 0 ? ctx->sm_count : 148;
+    const int sms = ctx_sms(ctx);
+    const int e0 = ensure_device(ctx);
+    if (e0) return e0;
     bool resid = false, chained = false;
     int level[kMaxProb], cls[kMaxProb];
     for (int i = 0; i < n; ++i) {
@@ -2124,7 +2302,13 @@ int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* 
             const bool under = resid && (set_res || ps[i0]->ksize != 3);
             // every problem is planned on its own first; where they disagree on the taps per weight stage, all are
             // planned again with the smallest (a stage per tap fits whatever fits three)
-            int force_G = 0, a_max = 0, b_bytes = 0;
+            int force_G = 0, a_max = 0, b_bytes = 0, set_px = kMaxPx;
+            if (m > 1) {
+                const rtoss_packed* sp[kMaxProb];
+                const rtoss_conv_desc* sd[kMaxProb];
+                for (int q = 0; q < m; ++q) sp[q] = ps[set[q]], sd[q] = ds[set[q]];
+                shared_cost(ctx, m, sp, sd, &set_px);
+            }
             for (int pass = 0; pass < 2; ++pass) {
                 bool agree = true;
                 int g_min = 9;
@@ -2134,7 +2318,12 @@ int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* 
                     rtoss_conv_desc dd = *ds[i];
                     static const int dummy = 0;
                     dd.residual_dev = under ? &dummy : nullptr;   // (only the plan's memory budget looks at it here)
-                    int e = build_problem(ctx, ps[i], xs[i], ys[i], &dd, m, sms, &args[i], &pp[i], &mapA[i], &mapB[i], force_G, tabs_try);
+                    PlanKey key = plan_key(ps[i], &dd, sms, ctx_dev(ctx));
+                    key.shared = m > 1 ? 1 : 2;
+                    key.max_px = set_px;
+                    key.force_G = force_G;
+                    key.n_tabs = tabs_try;
+                    int e = build_problem(ctx, ps[i], xs[i], ys[i], &dd, key, &args[i], &pp[i], &mapA[i], &mapB[i]);
                     if (e == (int)cudaErrorInvalidConfiguration) return -1;
                     if (e) return e;
                     args[i].resid = ds[i]->residual_dev;
@@ -2253,8 +2442,6 @@ int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* 
     if (smem_need > (size_t)cap) return -1;
     const size_t smem = smem_need > 116 * 1024 ? smem_need : 116 * 1024;
     dim3 grid((unsigned)grid_n);
-    int e = ensure_smem_attr(ctx);
-    if (e) return e;
     const bool bf = ps[0]->dtype == RTOSS_BF16, f32 = ps[0]->dtype == RTOSS_F32;
     cudaError_t le = f32 ? rtoss_dev::launch_pdl(conv_tc_kernel<float, TcLaunchN>, grid, kTcThreads, smem, (cudaStream_t)stream, 1, g)
                      : bf ? rtoss_dev::launch_pdl(conv_tc_kernel<__nv_bfloat16, TcLaunchN>, grid, kTcThreads, smem, (cudaStream_t)stream, 1, g)

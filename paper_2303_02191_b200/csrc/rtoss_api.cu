@@ -628,7 +628,7 @@ rtoss_status rtoss_conv_chain(rtoss_ctx* ctx, const rtoss_conv_item* items, int 
     }
     rtoss_device_guard on_device(ctx->device);
     // Maximal runs of consecutive items that can share a launch go out as one kernel each; an item that cannot (FMA
-    // path, positions on M) or that is better off alone (few tiles, many channel blocks and nothing to run beside it:
+    // path, positions on M) or that is better off alone (few tiles, many channel blocks:
     // a launch of its own cuts it along K over several CTAs, a shared launch never does) goes out on its own between them.  The stream orders the launches, so inside a run
     // only the dependencies on items of the same run have to be carried into the kernel.
     const int m_max = rtoss_tc_max_problems();
@@ -640,19 +640,35 @@ rtoss_status rtoss_conv_chain(rtoss_ctx* ctx, const rtoss_conv_item* items, int 
         for (int j = 0; j < q; ++j)
             if ((after[q] >> j) & 1u) level[q] = level[j] + 1 > level[q] ? level[j] + 1 : level[q];
     }
-    long tiles[32], level_tiles[33] = {};
+    // A call that a launch of its own would spread over a cluster per tile leaves the shared launch (which never splits) when
+    // the members of its level are expected to be done sooner one by one than together.
     bool alone[32];
+    double own_us[32];
     for (int q = 0; q < n; ++q) {
         const rtoss_conv_item& it = items[q];
         member[q] = it.desc.path != RTOSS_PATH_FMA && rtoss_tc_groupable(it.packed, &it.desc, it.x_dev, it.y_dev);
-        tiles[q] = 0;
-        alone[q] = member[q] && rtoss_tc_prefers_split(ctx, it.packed, &it.desc, &tiles[q]) && it.desc.path == RTOSS_PATH_AUTO;
-        if (member[q]) level_tiles[level[q]] += tiles[q];
+        int ks = 1;
+        long tiles = 0;
+        own_us[q] = 0;
+        alone[q] = member[q] && rtoss_tc_single_cost(ctx, it.packed, &it.desc, &own_us[q], &ks, &tiles) && ks > 1 && it.desc.path == RTOSS_PATH_AUTO;
     }
-    // (better alone, unless the others of its level keep every SM busy for several tiles: its own few, long tiles then
-    // hide among theirs)
-    for (int q = 0; q < n; ++q)
-        if (alone[q] && level_tiles[level[q]] - tiles[q] < 4L * ctx->sm_count) member[q] = false;
+    for (int l = 0; l < n; ++l) {
+        const rtoss_packed* ps[32];
+        const rtoss_conv_desc* ds[32];
+        int m = 0;
+        bool any = false;
+        double one_by_one = 0;
+        for (int q = 0; q < n; ++q) {
+            if (!member[q] || level[q] != l) continue;
+            ps[m] = items[q].packed, ds[m] = &items[q].desc;
+            ++m;
+            one_by_one += own_us[q];
+            any = any || alone[q];
+        }
+        if (!any || (m > 1 && rtoss_tc_shared_cost(ctx, m, ps, ds) <= one_by_one)) continue;
+        for (int q = 0; q < n; ++q)
+            if (level[q] == l && alone[q]) member[q] = false;
+    }
     int count = 0, i = 0;
     while (i < n) {
         int m = 0;

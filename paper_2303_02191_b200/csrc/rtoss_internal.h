@@ -153,7 +153,8 @@ int rtoss_launch_conv_tc_group(const rtoss_ctx* ctx, int n, const rtoss_packed* 
 int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const void* const* xs,
                                void* const* ys, const rtoss_conv_desc* const* ds, const uint32_t* after, void* stream);
 int rtoss_tc_max_problems();   // most convolutions one launch carries
-// a launch of its own would cut this call along K (few tiles, many channel blocks); a shared launch never does
-bool rtoss_tc_prefers_split(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, long* tiles_out);
+// what the planner expects of a launch of its own (shared launches never split a tile's channel blocks) and of a shared one
+bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles);
+double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds);
 
 #endif
