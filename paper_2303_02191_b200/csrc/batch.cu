@@ -2,12 +2,12 @@
 // of a model in two launches instead of three per layer.  The per-kernel arithmetic is the one of the single-layer
 // calls (select_core.cuh), so the results are the same bits.
 //
-//   batch_select_pack_kernel : one thread per kernel / run of nine, 256 per block step; a block step ("chunk")
-//                              belongs to one layer, found through a chunk -> layer table built at plan time.
+//   batch_select_pack_kernel : two kernels / runs of nine per thread, 512 per block step; a block step ("chunk")
+//                              belongs to one layer and is described by a table built at plan time.
 //                              Writes the pattern id (caller's array and the handle's), the k kept values and the
 //                              tensor path's dense-expanded weights.
-//   batch_order_kernel       : per (3x3 layer, input channel) the stable order of filters by pattern id, one warp
-//                              each, through a task -> layer table.
+//   batch_order_kernel       : per (3x3 layer, input channel) the stable order of filters by pattern id, sixteen
+//                              channels to a block, through a task -> layer table.
 //
 // A layer that inherits its parent's patterns (Section IV.A: children of a group share the parent's kernel
 // patterns) evaluates the selection on the PARENT's weights and packs its own with the result; it reads no other
@@ -19,6 +19,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "conv_common.cuh"
@@ -27,12 +28,13 @@
 
 namespace {
 
-constexpr int kChunk = 256;     // kernels per block step
-constexpr int kOrderWarps = 4;  // channels per block of the ordering kernel
+constexpr int kBatchThreads = 256;
+constexpr int kChunk = kBatchThreads * rtoss_dev::kPair;   // kernels per block step
 
-struct BatchLayer {
+struct alignas(16) BatchLayer {
     const void* w;      // weights to pack
     const void* w_sel;  // weights the selection reads: w, or the group parent's
+    int pid_out_vec;    // the caller's id array takes 2-byte stores
     uint8_t* pid_out;   // caller's id array (nullable)
     uint8_t* pid;       // the handle's arrays
     void* val;
@@ -44,17 +46,18 @@ struct BatchLayer {
     long long n_kernels;
     rtoss_wtc_layout lay;  // layout of wtc
     int Cout, Cin, ksize, P, k;
+    unsigned k_magic;   // ceil(2^16 / k): o / k = o * k_magic >> 16 for o below 2^13
     int w_dtype, sel_dtype, v_dtype;
     unsigned chunk0;  // first chunk of this layer
     unsigned task0;   // first ordering task (3x3 layers)
     uint16_t masks[256];
 };
 
-__device__ __forceinline__ float load_any(const unsigned char* raw, int idx, int dtype) {
-    if (dtype == RTOSS_F32) return reinterpret_cast<const float*>(raw)[idx];
-    if (dtype == RTOSS_BF16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(raw)[idx]);
-    return __half2float(reinterpret_cast<const __half*>(raw)[idx]);
-}
+// A block step: where its weights (those the selection reads) lie, how many bytes, whose they are.
+struct BatchChunk {
+    const unsigned char* src;
+    unsigned bytes, layer;
+};
 
 // 9*count weights of `count` consecutive kernels starting at kernel `first`, as raw bytes, coalesced; 16 bytes per
 // thread where the chunk is whole (a whole chunk is a multiple of 16 bytes and the base is 16-byte aligned).
@@ -64,77 +67,312 @@ __device__ __forceinline__ void stage_raw(const void* w, long long first, int co
     if (count == kChunk) {
         const uint4* s4 = reinterpret_cast<const uint4*>(src);
         uint4* d4 = reinterpret_cast<uint4*>(smem);
-        for (int i = threadIdx.x; i < bytes / 16; i += kChunk) d4[i] = __ldg(s4 + i);
+        for (int i = threadIdx.x; i < bytes / 16; i += kBatchThreads) d4[i] = __ldg(s4 + i);
     } else if (esize == 4) {
         const uint32_t* s1 = reinterpret_cast<const uint32_t*>(src);
         uint32_t* d1 = reinterpret_cast<uint32_t*>(smem);
-        for (int i = threadIdx.x; i < bytes / 4; i += kChunk) d1[i] = s1[i];
+        for (int i = threadIdx.x; i < bytes / 4; i += kBatchThreads) d1[i] = s1[i];
     } else {
         const uint16_t* s1 = reinterpret_cast<const uint16_t*>(src);
         uint16_t* d1 = reinterpret_cast<uint16_t*>(smem);
-        for (int i = threadIdx.x; i < bytes / 2; i += kChunk) d1[i] = s1[i];
+        for (int i = threadIdx.x; i < bytes / 2; i += kBatchThreads) d1[i] = s1[i];
     }
 }
 
-__global__ void __launch_bounds__(kChunk) batch_select_pack_kernel(const BatchLayer* __restrict__ layers,
-                                                                   const uint32_t* __restrict__ chunk_layer,
-                                                                   unsigned n_chunks) {
-    rtoss_dev::pdl_enter_handle_writer();
-    __shared__ __align__(16) unsigned char s_sel[kChunk * 9 * 4];
-    __shared__ __align__(16) unsigned char s_own[kChunk * 9 * 4];
-    __shared__ uint16_t s_masks[256];
-    for (unsigned chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-        const BatchLayer& L = layers[chunk_layer[chunk]];
-        const long long first = (long long)(chunk - L.chunk0) * kChunk;
-        const long long left = L.n_kernels - first;
-        const int count = (int)(left < kChunk ? left : kChunk);
-        const bool inherits = L.w_sel != L.w;
-        // the layer's first chunk clears its issue words: the ordering kernel (next launch) ORs the bits in
-        if (chunk == L.chunk0 && L.issue)
-            for (int i = threadIdx.x; i < L.issue_n; i += kChunk) L.issue[i] = 0ull;
-        __syncthreads();  // the previous step's readers are done
-        stage_raw(L.w_sel, first, count, L.sel_dtype == RTOSS_F32 ? 4 : 2, s_sel);
-        if (inherits) stage_raw(L.w, first, count, L.w_dtype == RTOSS_F32 ? 4 : 2, s_own);
-        if ((int)threadIdx.x < L.P) s_masks[threadIdx.x] = L.masks[threadIdx.x];
-        __syncthreads();
-        if ((int)threadIdx.x < count) {
-            const long long i = first + threadIdx.x;
-            float v[9];
-#pragma unroll
-            for (int t = 0; t < 9; ++t) v[t] = load_any(s_sel, threadIdx.x * 9 + t, L.sel_dtype);
-            const int best = rtoss_dev::select_best(v, s_masks, L.P);
-            if (L.pid_out) L.pid_out[i] = (uint8_t)best;
-            L.pid[i] = (uint8_t)best;
-            if (inherits) {
-#pragma unroll
-                for (int t = 0; t < 9; ++t) v[t] = load_any(s_own, threadIdx.x * 9 + t, L.w_dtype);
+__device__ __forceinline__ void cp_async16(void* smem, const void* g) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(g) : "memory");
+}
+
+// Starts fetching a chunk: the layer's record (unless it is there already) and the weights its selection reads.  A ragged chunk's last bytes are plain
+// loads (16-bit weights: 2-byte pieces).
+__device__ __forceinline__ void fetch_chunk(const BatchLayer* layers, const BatchChunk& c, BatchLayer* s_layer, unsigned char* raw) {
+    const unsigned char* rec = reinterpret_cast<const unsigned char*>(layers + c.layer);
+    if (s_layer)
+        for (int o = (int)threadIdx.x * 16; o < (int)sizeof(BatchLayer); o += kBatchThreads * 16) 
+            cp_async16(reinterpret_cast<unsigned char*>(s_layer) + o, rec + o);
+    const int whole = (int)(c.bytes & ~15u);
+    for (int o = (int)threadIdx.x * 16; o < whole; o += kBatchThreads * 16) cp_async16(raw + o, c.src + o);
+    const int o = whole + (int)threadIdx.x * 2;
+    if (o < (int)c.bytes) *reinterpret_cast<uint16_t*>(raw + o) = *reinterpret_cast<const uint16_t*>(c.src + o);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// ---- one chunk ----------------------------------------------------------------------------------------------------
+// The chunk's weights lie in shared memory as they are in memory.  Phase 1: a thread selects for two neighbouring kernels
+// and leaves their pattern ids and masks in shared memory.  Phase 2: the outputs are written the way memory wants them,
+// whatever kernel an element belongs to: kept values and the flat 1x1 expansion as consecutive words, the 3x3 expansion tap
+// by tap (consecutive kernels are consecutive channels).  Nothing per kernel is held in registers between the phases.
+
+template <typename T> __device__ __forceinline__ float raw_at(const unsigned char* raw, int e) {
+    if constexpr (sizeof(T) == 4) return reinterpret_cast<const float*>(raw)[e];
+    else return rtoss_dev::to_f32<T>(reinterpret_cast<const T*>(raw)[e]);
+}
+
+template <typename T>
+__device__ __forceinline__ void select_chunk(const BatchLayer& L, long long first, int count, const unsigned char* raw, const rtoss_dev::PatternFactors* factors,
+                                             uint8_t* s_pid, uint16_t* s_mask) {
+    using namespace rtoss_dev;
+    const int base = (int)threadIdx.x * kPair;
+    if (base >= count) return;
+    f32x2 q[9];
+    int best[kPair];
+    load_pair<T>(raw, (int)threadIdx.x, q);
+    select_best2(q, L.masks, factors, L.P, best);
+    const long long i = first + base;
+    const unsigned ids = (unsigned)best[0] | (unsigned)best[1] << 8;
+    *reinterpret_cast<uint16_t*>(s_pid + base) = (uint16_t)ids;
+    *reinterpret_cast<unsigned*>(s_mask + base) = (unsigned)L.masks[best[0]] | (unsigned)L.masks[best[1]] << 16;
+    if (base + 1 < count) {
+        *reinterpret_cast<uint16_t*>(L.pid + i) = (uint16_t)ids;
+        if (L.pid_out && L.pid_out_vec) {
+            *reinterpret_cast<uint16_t*>(L.pid_out + i) = (uint16_t)ids;
+        } else if (L.pid_out) {
+            L.pid_out[i] = (uint8_t)best[0];
+            L.pid_out[i + 1] = (uint8_t)best[1];
+        }
+    } else {
+        L.pid[i] = (uint8_t)best[0];
+        if (L.pid_out) L.pid_out[i] = (uint8_t)best[0];
+    }
+}
+
+template <typename V> __device__ __forceinline__ unsigned round2(float a, float b) {
+    if constexpr (std::is_same<V, __half>::value) {
+        const __half2 u = __floats2half2_rn(a, b);
+        return *reinterpret_cast<const unsigned*>(&u);
+    } else {
+        const __nv_bfloat162 u = __floats2bfloat162_rn(a, b);
+        return *reinterpret_cast<const unsigned*>(&u);
+    }
+}
+// Two neighbouring positions as one aligned word; fp32: tf32 heads, and the remainders lo_at further on (see expand_one).
+template <typename V> __device__ __forceinline__ void put_pair(V* at, int64_t lo_at, float a, float b) {
+    using namespace rtoss_dev;
+    if constexpr (sizeof(V) == 4) {
+        *reinterpret_cast<float2*>(at) = make_float2(tf32_head(a), tf32_head(b));
+        *reinterpret_cast<float2*>(at + lo_at) = make_float2(__fsub_rn(a, tf32_head(a)), __fsub_rn(b, tf32_head(b)));
+    } else {
+        *reinterpret_cast<unsigned*>(at) = round2<V>(a, b);
+    }
+}
+template <typename V> __device__ __forceinline__ void put_one(V* at, int64_t lo_at, float a) {
+    using namespace rtoss_dev;
+    if constexpr (sizeof(V) == 4) {
+        *at = tf32_head(a);
+        at[lo_at] = __fsub_rn(a, tf32_head(a));
+    } else {
+        *at = narrow_to<V>(a);
+    }
+}
+
+template <typename T, typename V>
+__device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first, int count, const unsigned char* raw, const uint8_t* s_pid,
+                                           const uint16_t* s_mask, const unsigned long long* s_taps) {
+    using namespace rtoss_dev;
+    V* val = reinterpret_cast<V*>(L.val) + first * L.k;   // (a chunk's first value is at a multiple of 512 k)
+    if (sizeof(V) == 2 && L.k == 4) {
+        // the usual case: a kernel's four values are one aligned 8-byte word
+        for (int g = (int)threadIdx.x; g < count; g += kBatchThreads) {
+            const unsigned taps = (unsigned)s_taps[s_pid[g]];
+            const unsigned char* w = raw + (size_t)g * 9 * sizeof(T);
+            uint2 u;
+            u.x = round2<V>(raw_at<T>(w, taps & 15), raw_at<T>(w, (taps >> 4) & 15));
+            u.y = round2<V>(raw_at<T>(w, (taps >> 8) & 15), raw_at<T>(w, (taps >> 12) & 15));
+            *reinterpret_cast<uint2*>(val + 4 * g) = u;
+        }
+    } else {
+        // value o of the chunk is the (o mod k)-th kept tap of kernel o / k; two to a thread
+        const int n = count * L.k, k = L.k;
+        auto value = [&](int o) {
+            const int g = (int)(((unsigned)o * L.k_magic) >> 16);   // o / k
+            const int tap = (int)(s_taps[s_pid[g]] >> (4 * (o - g * k))) & 15;
+            return raw_at<T>(raw, g * 9 + tap);
+        };
+        for (int o = 2 * (int)threadIdx.x; o < n; o += 2 * kBatchThreads) {
+            const float a = value(o);
+            if (o + 1 < n) {
+                const float b = value(o + 1);
+                if constexpr (sizeof(V) == 4) *reinterpret_cast<float2*>(val + o) = make_float2(a, b);
+                else *reinterpret_cast<unsigned*>(val + o) = round2<V>(a, b);
+            } else {
+                val[o] = narrow_to<V>(a);
             }
-            const unsigned m = s_masks[best];
-            if (L.v_dtype == RTOSS_F32)
-                rtoss_dev::pack_one<float>(v, m, i, L.k, (float*)L.val, (float*)L.wtc, L.ksize, L.Cin, L.lay.rows, L.lay.rep_rows,
-                                           L.lay.copies, L.lay.cin_p);
-            else if (L.v_dtype == RTOSS_BF16)
-                rtoss_dev::pack_one<__nv_bfloat16>(v, m, i, L.k, (__nv_bfloat16*)L.val, (__nv_bfloat16*)L.wtc, L.ksize, L.Cin,
-                                                   L.lay.rows, L.lay.rep_rows, L.lay.copies, L.lay.cin_p);
-            else
-                rtoss_dev::pack_one<__half>(v, m, i, L.k, (__half*)L.val, (__half*)L.wtc, L.ksize, L.Cin, L.lay.rows, L.lay.rep_rows,
-                                            L.lay.copies, L.lay.cin_p);
+        }
+    }
+    if (!L.wtc) return;
+    V* wtc = reinterpret_cast<V*>(L.wtc);
+    const int Cin = L.Cin, cin_p = L.lay.cin_p;
+    const int64_t tap_step = (int64_t)L.lay.rows * cin_p;
+    if (L.ksize == 3) {
+        const int64_t lo_at = 9 * tap_step, copy_step = (int64_t)L.lay.rep_rows * cin_p;
+        const int base = (int)threadIdx.x * kPair;
+        if (base >= count) return;
+        const unsigned mm = *reinterpret_cast<const unsigned*>(s_mask + base);
+        const bool two = base + 1 < count;
+        // kernel i lies at flat position i of a tap's matrix; where the stored rows are longer than the layer's, further on
+        int64_t p0 = first + base, p1 = p0 + 1;
+        if (cin_p != Cin) {
+            p0 += (int64_t)((unsigned)p0 / (unsigned)Cin) * (cin_p - Cin);
+            p1 += (int64_t)((unsigned)p1 / (unsigned)Cin) * (cin_p - Cin);
+        }
+        const bool word = two && p1 == p0 + 1 && (p0 & 1) == 0 && (tap_step & 1) == 0 && (copy_step & 1) == 0;
+        V* at = wtc + p0;
+        const int64_t d1 = p1 - p0;
+        if (word && L.lay.copies == 1) {
+#pragma unroll
+            for (int t = 0; t < 9; ++t, at += tap_step) {
+                const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
+                const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
+                put_pair<V>(at, lo_at, a, b);
+            }
+            return;
+        }
+#pragma unroll 1
+        for (int t = 0; t < 9; ++t, at += tap_step) {
+            const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
+            const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
+            V* to = at;
+            for (int c = 0; c < L.lay.copies; ++c, to += copy_step) {
+                if (word) {
+                    put_pair<V>(to, lo_at, a, b);
+                } else {
+                    put_one<V>(to, lo_at, a);
+                    if (two) put_one<V>(to + d1, lo_at, b);
+                }
+            }
+        }
+    } else {
+        // the flat matrix: four positions to a thread (a multiple of four: at most two kernels, one aligned word)
+        const int n = count * 9;
+        const bool words = cin_p == Cin && (tap_step & 3) == 0;   // (rows as long as the layer's; fp32 remainders aligned alike)
+        for (int e = 4 * (int)threadIdx.x; e < n; e += 4 * kBatchThreads) {
+            const int g = (int)(((unsigned)e * 7282u) >> 16);   // e / 9 (e is below 2^13)
+            const unsigned mm = ((unsigned)s_mask[g] | (unsigned)s_mask[min(g + 1, kChunk - 1)] << 9) >> (e - 9 * g);   // bit j: position e + j is kept
+            const int64_t f = first * 9 + e;
+            float v[4];
+            if constexpr (sizeof(T) == 4) {
+                const float4 x = *reinterpret_cast<const float4*>(raw + (size_t)e * 4);
+                v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+            } else {
+                const uint2 x = *reinterpret_cast<const uint2*>(raw + (size_t)e * 2);
+                const T* h = reinterpret_cast<const T*>(&x);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[j] = to_f32<T>(h[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = (mm >> j) & 1u ? v[j] : 0.f;
+            if (words && e + 4 <= n) {
+                if constexpr (sizeof(V) == 4) {
+                    *reinterpret_cast<float4*>(wtc + f) = make_float4(tf32_head(v[0]), tf32_head(v[1]), tf32_head(v[2]), tf32_head(v[3]));
+                    *reinterpret_cast<float4*>(wtc + f + tap_step) =
+                        make_float4(__fsub_rn(v[0], tf32_head(v[0])), __fsub_rn(v[1], tf32_head(v[1])), __fsub_rn(v[2], tf32_head(v[2])), __fsub_rn(v[3], tf32_head(v[3])));
+                } else {
+                    *reinterpret_cast<uint2*>(wtc + f) = make_uint2(round2<V>(v[0], v[1]), round2<V>(v[2], v[3]));
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (e + j < n) put_one<V>(wtc + f + j + (cin_p != Cin ? (int64_t)((unsigned)(f + j) / (unsigned)Cin) * (cin_p - Cin) : 0), tap_step, v[j]);
+            }
         }
     }
 }
 
-__global__ void __launch_bounds__(kOrderWarps * 32) batch_order_kernel(const BatchLayer* __restrict__ layers,
-                                                                       const uint32_t* __restrict__ task_layer,
-                                                                       unsigned n_tasks) {
+// Bound by instructions (0.75 a cycle and scheduler; 35 % of the copy rate).  32 M weights, 8 patterns of four taps: 131 us
+// with one kernel per thread that held its weights in registers through all outputs, 65 us in this form; 20 us instead of
+// 31 for 7 M.  (Prefetching the next chunk with a second buffer cost occupancy and was slower: 142 us on the older form.)
+__global__ void __launch_bounds__(kBatchThreads, 6) batch_select_pack_kernel(const BatchLayer* __restrict__ layers,
+                                                                          const BatchChunk* __restrict__ chunks,
+                                                                          unsigned n_chunks) {
     rtoss_dev::pdl_enter_handle_writer();
-    __shared__ uint32_t fill_all[kOrderWarps][256];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (unsigned task = blockIdx.x * kOrderWarps + warp; task < n_tasks; task += gridDim.x * kOrderWarps) {
-        const BatchLayer& L = layers[task_layer[task]];
-        rtoss_dev::order_channel(L.pid, L.Cout, L.Cin, L.P, (int)(task - L.task0), L.perm, L.bucket_off, fill_all[warp],
-                                 lane, L.masks, L.issue, L.v_dtype == RTOSS_F32 ? 5 : 6);
-        __syncwarp();
+    __shared__ __align__(16) unsigned char raw[kChunk * 9 * 4];
+    __shared__ BatchLayer s_layer;
+    __shared__ __align__(16) uint16_t s_mask[kChunk];
+    __shared__ __align__(16) uint8_t s_pid[kChunk];
+    __shared__ rtoss_dev::PatternFactors s_factors[rtoss_dev::kFactorPatterns];
+    __shared__ unsigned long long s_taps[256];   // a pattern's taps in ascending order, four bits each
+    const unsigned per = n_chunks / gridDim.x, extra = n_chunks % gridDim.x;
+    const unsigned begin = blockIdx.x * per + min(blockIdx.x, extra), end = begin + per + (blockIdx.x < extra ? 1u : 0u);
+    if (begin >= end) return;
+    BatchChunk c = chunks[begin];
+    uint32_t have = 0xFFFFFFFFu;   // which layer s_layer is
+    for (unsigned chunk = begin; chunk < end; ++chunk) {
+        const bool fresh = c.layer != have;
+        fetch_chunk(layers, c, fresh ? &s_layer : nullptr, raw);
+        have = c.layer;
+        c = chunks[min(chunk + 1, end - 1)];
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const BatchLayer& L = s_layer;
+        const long long first = (long long)(chunk - L.chunk0) * kChunk;
+        const int count = (int)(L.n_kernels - first < kChunk ? L.n_kernels - first : kChunk);
+        // the layer's first chunk clears its issue words: the ordering kernel (next launch) ORs the bits in
+        if (chunk == L.chunk0 && L.issue)
+            for (int i = threadIdx.x; i < L.issue_n; i += kBatchThreads) L.issue[i] = 0ull;
+        if (fresh && (int)threadIdx.x < L.P) {
+            const unsigned m = L.masks[threadIdx.x];
+            unsigned long long taps = 0;
+            int j = 0;
+#pragma unroll
+            for (int t = 0; t < 9; ++t)
+                if (m & (1u << t)) taps |= (unsigned long long)t << (4 * j++);
+            s_taps[threadIdx.x] = taps;
+            if (threadIdx.x < rtoss_dev::kFactorPatterns) {
+#pragma unroll
+                for (int t = 0; t < 10; ++t) {
+                    const float f = (m >> t) & 1u ? 1.f : 0.f;   // (bit 9 is never set)
+                    s_factors[threadIdx.x].f[t] = rtoss_dev::pack_f32x2(f, f);
+                }
+            }
+        }
+        if (fresh) __syncthreads();
+        if (L.sel_dtype == RTOSS_F32) select_chunk<float>(L, first, count, raw, s_factors, s_pid, s_mask);
+        else if (L.sel_dtype == RTOSS_BF16) select_chunk<__nv_bfloat16>(L, first, count, raw, s_factors, s_pid, s_mask);
+        else select_chunk<__half>(L, first, count, raw, s_factors, s_pid, s_mask);
+        __syncthreads();
+        if (L.w_sel != L.w) {   // the patterns are inherited: this layer's own weights take the buffer
+            stage_raw(L.w, first, count, L.w_dtype == RTOSS_F32 ? 4 : 2, raw);
+            __syncthreads();
+        }
+#define RTOSS_PACK(T_, V_) pack_chunk<T_, V_>(L, first, count, raw, s_pid, s_mask, s_taps)
+#define RTOSS_PACK_TO(V_)                                       \
+    if (L.w_dtype == RTOSS_F32) RTOSS_PACK(float, V_);          \
+    else if (L.w_dtype == RTOSS_BF16) RTOSS_PACK(__nv_bfloat16, V_); \
+    else RTOSS_PACK(__half, V_)
+        if (L.v_dtype == RTOSS_F32) { RTOSS_PACK_TO(float); }
+        else if (L.v_dtype == RTOSS_BF16) { RTOSS_PACK_TO(__nv_bfloat16); }
+        else { RTOSS_PACK_TO(__half); }
+#undef RTOSS_PACK_TO
+#undef RTOSS_PACK
+        __syncthreads();   // the buffer and the record are free
     }
+    rtoss_dev::handle_writer_done();
+}
+
+__global__ void __launch_bounds__(rtoss_dev::kOrderThreads, 4) batch_order_kernel(const BatchLayer* __restrict__ layers,
+                                                                             const uint32_t* __restrict__ task_layer, unsigned n_tasks) {
+    using namespace rtoss_dev;
+    pdl_enter_handle_writer();
+    __shared__ union {
+        struct {
+            uint32_t fill[kOrderThreads / 32][256];
+            uint16_t mask[kOrderThreads / 32][256];
+        } many;
+        OrderFew few;
+    } sh;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (unsigned task = blockIdx.x; task < n_tasks; task += gridDim.x) {
+        const BatchLayer& L = layers[task_layer[task]];
+        const int ci0 = (int)(task - L.task0) * kOrderChannels, cb_log2 = L.v_dtype == RTOSS_F32 ? 5 : 6;
+        if (order_few(L.Cout, L.P)) {
+            order_channels_few(L.pid, L.Cout, L.Cin, L.P, ci0, L.perm, L.bucket_off, sh.few, L.masks, L.issue, cb_log2);
+        } else {
+            for (int ci = ci0 + warp; ci < min(ci0 + kOrderChannels, L.Cin); ci += kOrderThreads / 32)
+                order_channel(L.pid, L.Cout, L.Cin, L.P, ci, L.perm, L.bucket_off, sh.many.fill[warp], sh.many.mask[warp], lane, L.masks, L.issue, cb_log2);
+        }
+        __syncthreads();   // the shared arrays are free
+    }
+    handle_writer_done();
 }
 
 void set_err(rtoss_ctx* ctx, const char* what) {
@@ -148,7 +386,7 @@ struct rtoss_batch {
     int device;
     int L;
     BatchLayer* layers_dev;
-    uint32_t* chunk_layer_dev;
+    BatchChunk* chunks_dev;
     uint32_t* task_layer_dev;
     unsigned n_chunks, n_tasks;
 };
@@ -163,7 +401,8 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
     }
     *out = nullptr;
     std::vector<BatchLayer> layers((size_t)L);
-    std::vector<uint32_t> chunk_layer, task_layer;
+    std::vector<BatchChunk> chunks;
+    std::vector<uint32_t> task_layer;
     for (int i = 0; i < L; ++i) {
         const rtoss_batch_item& it = items[i];
         rtoss_packed* p = it.packed;
@@ -213,6 +452,7 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
             return RTOSS_ERR_INVALID_ARG;
         }
         B.pid_out = it.pid_dev;
+        B.pid_out_vec = (reinterpret_cast<uintptr_t>(it.pid_dev) & 1) == 0;
         B.pid = p->pid;
         B.val = p->val;
         B.wtc = p->wtc;
@@ -227,34 +467,40 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
         B.ksize = it.ksize;
         B.P = it.P;
         B.k = it.k;
+        B.k_magic = (65536u + (unsigned)it.k - 1u) / (unsigned)it.k;
         B.v_dtype = (int)p->dtype;
         memcpy(B.masks, it.masks_host, sizeof(uint16_t) * (size_t)it.P);
-        B.chunk0 = (unsigned)chunk_layer.size();
+        B.chunk0 = (unsigned)chunks.size();
         const long long nc = (p->n_kernels + kChunk - 1) / kChunk;
-        if ((long long)chunk_layer.size() + nc > 0x7FFFFFFFLL) {
+        if ((long long)chunks.size() + nc > 0x7FFFFFFFLL) {
             set_err(ctx, "model too large for one batch");
             return RTOSS_ERR_UNSUPPORTED;
         }
-        chunk_layer.insert(chunk_layer.end(), (size_t)nc, (uint32_t)i);
+        const size_t kernel_bytes = 9 * (B.sel_dtype == RTOSS_F32 ? 4 : 2);
+        for (long long c = 0; c < nc; ++c) {
+            const long long left = p->n_kernels - c * kChunk;
+            chunks.push_back(BatchChunk{static_cast<const unsigned char*>(B.w_sel) + (size_t)c * kChunk * kernel_bytes,
+                                        (unsigned)((left < kChunk ? left : kChunk) * (long long)kernel_bytes), (unsigned)i});
+        }
         B.task0 = (unsigned)task_layer.size();
-        if (it.ksize == 3) task_layer.insert(task_layer.end(), (size_t)it.Cin, (uint32_t)i);
+        if (it.ksize == 3) task_layer.insert(task_layer.end(), (size_t)((it.Cin + rtoss_dev::kOrderChannels - 1) / rtoss_dev::kOrderChannels), (uint32_t)i);
     }
     rtoss_batch* b = new (std::nothrow) rtoss_batch();
     if (!b) return RTOSS_ERR_ALLOC;
     memset(b, 0, sizeof(*b));
     b->device = ctx->device;
     b->L = L;
-    b->n_chunks = (unsigned)chunk_layer.size();
+    b->n_chunks = (unsigned)chunks.size();
     b->n_tasks = (unsigned)task_layer.size();
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(ctx->device);
     cudaError_t e = cudaMalloc((void**)&b->layers_dev, sizeof(BatchLayer) * (size_t)L);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&b->chunk_layer_dev, sizeof(uint32_t) * (chunk_layer.size() + 1));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&b->chunks_dev, sizeof(BatchChunk) * (chunks.size() + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->task_layer_dev, sizeof(uint32_t) * (task_layer.size() + 1));
     if (e == cudaSuccess) e = cudaMemcpy(b->layers_dev, layers.data(), sizeof(BatchLayer) * (size_t)L, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !chunk_layer.empty())
-        e = cudaMemcpy(b->chunk_layer_dev, chunk_layer.data(), sizeof(uint32_t) * chunk_layer.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && !chunks.empty())
+        e = cudaMemcpy(b->chunks_dev, chunks.data(), sizeof(BatchChunk) * chunks.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !task_layer.empty())
         e = cudaMemcpy(b->task_layer_dev, task_layer.data(), sizeof(uint32_t) * task_layer.size(), cudaMemcpyHostToDevice);
     // the handles take the batch's tables (a convolution reads the handle's device copy of the masks)
@@ -288,14 +534,14 @@ rtoss_status rtoss_batch_select_pack(rtoss_ctx* ctx, const rtoss_batch* b, void*
     cudaError_t e = cudaSuccess;
     const unsigned cap = (unsigned)ctx->sm_count * 8u;
     if (b->n_chunks) {
-        const unsigned grid = b->n_chunks < cap ? b->n_chunks : cap;
-        e = rtoss_dev::launch_pdl(batch_select_pack_kernel, grid, kChunk, 0, s, (const BatchLayer*)b->layers_dev,
-                                  (const uint32_t*)b->chunk_layer_dev, b->n_chunks);
+        const unsigned resident = (unsigned)ctx->sm_count * 6u;   // (what the kernel's launch bounds allow)
+        const unsigned grid = b->n_chunks < resident ? b->n_chunks : resident;
+        e = rtoss_dev::launch_pdl(batch_select_pack_kernel, grid, kBatchThreads, 0, s, (const BatchLayer*)b->layers_dev,
+                                  (const BatchChunk*)b->chunks_dev, b->n_chunks);
     }
     if (e == cudaSuccess && b->n_tasks) {
-        unsigned grid = (b->n_tasks + kOrderWarps - 1) / kOrderWarps;
-        if (grid > cap) grid = cap;
-        e = rtoss_dev::launch_pdl(batch_order_kernel, grid, kOrderWarps * 32, 0, s, (const BatchLayer*)b->layers_dev,
+        const unsigned grid = b->n_tasks < cap ? b->n_tasks : cap;
+        e = rtoss_dev::launch_pdl(batch_order_kernel, grid, rtoss_dev::kOrderThreads, 0, s, (const BatchLayer*)b->layers_dev,
                                   (const uint32_t*)b->task_layer_dev, b->n_tasks);
     }
     if (e != cudaSuccess) {
@@ -312,7 +558,7 @@ void rtoss_batch_destroy(rtoss_batch* b) {
     cudaGetDevice(&prev);
     cudaSetDevice(b->device);
     if (b->layers_dev) cudaFree(b->layers_dev);
-    if (b->chunk_layer_dev) cudaFree(b->chunk_layer_dev);
+    if (b->chunks_dev) cudaFree(b->chunks_dev);
     if (b->task_layer_dev) cudaFree(b->task_layer_dev);
     cudaSetDevice(prev);
     delete b;

@@ -48,7 +48,10 @@ __device__ __forceinline__ void pdl_enter() {
 // with this instead: they wait like every other kernel but never let the next kernel start early.  The tensor-path
 // convolution relies on it: it fetches its weights before its own wait (they are constant while a network runs), which is
 // safe because whatever may still be writing them -- one of these kernels -- has completed before the convolution starts.
+// They end with handle_writer_done(): whatever they wrote is performed before the block leaves, so that a kernel which
+// starts behind them sees it without a wait of its own.
 __device__ __forceinline__ void pdl_enter_handle_writer() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void handle_writer_done() { __threadfence(); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
