@@ -461,7 +461,10 @@ __device__ __forceinline__ uint4 add_residual8(uint4 o, const uint4 rv) {
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
-// Sixteen positions of one filter (a half chunk): round, transpose through the patch, store.  See epilogue_chunks.
+// Sixteen positions of one filter per lane (a half chunk of split K, whose sums come from shared memory that way): round,
+// transpose through the patch, store.  A lane rounds two neighbouring positions of its filter into one word and stores it
+// to row (position pair), column (filter); lane (pair lane / 4, filter group lane % 4) reads its group's eight words, splits
+// low and high halves and writes each as one 16-byte store.
 // With a residual operand (rbv, laid out like the output) the activation moves behind the residual add.
 template <typename T, int ACT>
 __device__ __forceinline__ void epilogue_half(const unsigned (&r)[16], float bs, unsigned wr, unsigned rd, unsigned tab_at,
@@ -500,89 +503,130 @@ __device__ __forceinline__ void epilogue_half(const unsigned (&r)[16], float bs,
     __syncwarp();
 }
 
-// One tile of the filters-as-M epilogue for one warp: its lane quarter of the accumulator stage at d_base, the
-// 32-column chunks c0, c0 + c_step, ...  A warp holds 32 filters (lanes) x 16 positions (registers) at a time;
-// NHWC wants the filters of one position side by side.  The shared-memory pipe (one 128-byte wavefront a cycle,
-// which the tensor cores' operand reads also use) is what bounds the transpose, so it moves full wavefronts:
-//   * a lane rounds two neighbouring positions of its filter into one 32-bit word and stores it to row
-//     (position pair), column (filter) of the warp's patch: eight conflict-free 128-byte stores per 16 positions;
-//   * lane (pair jp = lane / 4, filter group v = lane % 4) reads the eight words of its group (two 16-byte
-//     loads; rows are 36 words apart, so the two rows a quarter warp touches fall on disjoint banks), splits
-//     them into the low halves (position 2 jp) and the high halves (position 2 jp + 1) and writes each as one
-//     16-byte store: four lanes cover the 64 contiguous bytes of a position.
-// The accumulator is read sixteen columns at a time into two register sets: the load of the next sixteen is in
-// flight while the current ones are processed (a load takes a few hundred cycles when all warps read at once).
-// Where a position goes comes from the table built in the prologue (no division here): tab[p] = {element offset
-// inside the tile, row << 16 | column}.  patch and tab are shared-memory addresses (32 bits: the accesses are
-// spelled out so that none is compiled as a generic one).
+// ---- the filters-as-M epilogue of 16-bit layers ------------------------------------------------------------------
+// A warp owns 32 filters (its TMEM lane quarter) and takes the positions sixteen at a time (a half chunk); NHWC wants the
+// filters of one position side by side.  The accumulator is read as matrix fragments (tcgen05.ld 16x256b: a thread gets
+// two neighbouring positions of one filter per register pair, four filters in all), so that after bias, activation and
+// rounding a packed register is exactly what stmatrix takes, and two transposing stmatrix.x4 lay the half chunk down as
+// sixteen rows of 64 bytes, one per position.  The 16-byte piece g of row p sits at piece g ^ ((p / 2) mod 4): the eight
+// rows stmatrix writes at once and the two rows eight lanes read at once both fall on 32 different banks.  A lane then
+// reads the piece (position lane / 4 resp. + 8, filters 8 (lane mod 4) ...) and stores its 16 bytes: four lanes cover the
+// 64 contiguous bytes of a position.
+// Where a position goes comes from the table built in the prologue: tab[p] = {element offset inside the tile, row << 16 |
+// column}.  Two register sets: the next half chunk's loads are in flight while the current one is worked on.
+// (The form before this read a filter per lane, stored eight words, read three vectors and split them with eight byte
+// permutes per half chunk: 171 warp instructions all told, a third of its shared-memory wavefronts bank conflicts.)
+__device__ __forceinline__ void tmem_ld_frag(unsigned taddr, unsigned (&lo)[8], unsigned (&hi)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(lo[0]), "=r"(lo[1]), "=r"(lo[2]), "=r"(lo[3]), "=r"(lo[4]), "=r"(lo[5]), "=r"(lo[6]), "=r"(lo[7])
+                 : "r"(taddr)
+                 : "memory");
+    asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(hi[0]), "=r"(hi[1]), "=r"(hi[2]), "=r"(hi[3]), "=r"(hi[4]), "=r"(hi[5]), "=r"(hi[6]), "=r"(hi[7])
+                 : "r"(taddr + (16u << 16))
+                 : "memory");
+}
+
+// What a lane needs for every half chunk of a tile.
+struct FragLane {
+    float b[4];      // bias of filters lane / 4 + 0, 8, 16, 24 (as bias_act expects it)
+    unsigned st;     // stmatrix row address of this lane (position lane mod 8, piece lane / 8)
+    unsigned rd;     // this lane's piece of position lane / 4
+    unsigned tab;    // table entry of position lane / 4 of the tile
+};
+__device__ __forceinline__ FragLane frag_lane(float bs, unsigned patch, unsigned tab, int lane) {
+    FragLane f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) f.b[q] = __shfl_sync(0xFFFFFFFFu, bs, 8 * q + (lane >> 2));
+    const unsigned p = (unsigned)lane & 7u, g = (unsigned)lane >> 3;
+    f.st = patch + p * 64u + ((g ^ ((p >> 1) & 3u)) << 4);
+    const unsigned q = (unsigned)lane >> 2, h = (unsigned)lane & 3u;
+    f.rd = patch + q * 64u + ((h ^ ((q >> 1) & 3u)) << 4);
+    f.tab = tab + q * 8u;
+    return f;
+}
+
+// Half chunk -> patch.  ACT = none and RELU false: the plain rounded sum.
+template <typename T, int ACT>
+__device__ __forceinline__ void frag_to_patch(const unsigned (&lo)[8], const unsigned (&hi)[8], const FragLane& f) {
+    constexpr bool kRelu = ACT == RTOSS_ACT_RELU;
+#pragma unroll
+    for (int po = 0; po < 2; ++po) {   // positions 8 po ... 8 po + 7
+        const unsigned w0 = round_pack<T, kRelu>(bias_act<ACT>(lo[4 * po], f.b[0]), bias_act<ACT>(lo[4 * po + 1], f.b[0]));
+        const unsigned w1 = round_pack<T, kRelu>(bias_act<ACT>(lo[4 * po + 2], f.b[1]), bias_act<ACT>(lo[4 * po + 3], f.b[1]));
+        const unsigned w2 = round_pack<T, kRelu>(bias_act<ACT>(hi[4 * po], f.b[2]), bias_act<ACT>(hi[4 * po + 1], f.b[2]));
+        const unsigned w3 = round_pack<T, kRelu>(bias_act<ACT>(hi[4 * po + 2], f.b[3]), bias_act<ACT>(hi[4 * po + 3], f.b[3]));
+        asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(f.st + 512u * po), "r"(w0), "r"(w1),
+                     "r"(w2), "r"(w3)
+                     : "memory");
+    }
+    __syncwarp();
+}
+__device__ __forceinline__ uint4 lds128(unsigned at) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(at));
+    return v;
+}
+__device__ __forceinline__ uint2 lds64(unsigned at) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(at));
+    return v;
+}
+__device__ __forceinline__ bool inside(const uint2& e, unsigned ry, unsigned rx) { return (e.y >> 16) < ry && (e.y & 0xFFFFu) < rx; }
+
+template <typename T, int ACT>
+__device__ __forceinline__ void frag_half(const unsigned (&lo)[8], const unsigned (&hi)[8], const FragLane& f, unsigned c0, T* ybv, unsigned ry,
+                                          unsigned rx) {
+    const uint2 e0 = lds64(f.tab + c0 * 8u), e1 = lds64(f.tab + c0 * 8u + 64u);
+    frag_to_patch<T, ACT>(lo, hi, f);
+    const uint4 o0 = lds128(f.rd), o1 = lds128(f.rd + 512u);
+    if (inside(e0, ry, rx)) *reinterpret_cast<uint4*>(ybv + e0.x) = o0;
+    if (inside(e1, ry, rx)) *reinterpret_cast<uint4*>(ybv + e1.x) = o1;
+    __syncwarp();
+}
+
+// One tile for one warp: its lane quarter of the accumulator stage at d_base, the 32-column chunks c0, c0 + c_step, ...
 template <typename T, int ACT>
 __device__ __forceinline__ void epilogue_chunks(unsigned d_base, int c0, int c_step, int n_px, float bs,
-                                                unsigned patch, unsigned tab, T* yb, unsigned ry, unsigned rx,
-                                                int lane, const T* rb) {
-    const unsigned wr = patch + lane * 4;                                       // this lane's column of the patch
-    const unsigned rd = patch + (lane >> 2) * kPairPitch + (lane & 3) * 32;   // row lane / 4, filter group lane % 4
-    const unsigned tab_l = tab + (unsigned)(2 * (lane >> 2)) * 8;
+                                                unsigned patch, unsigned tab, T* yb, unsigned ry, unsigned rx, int lane) {
+    const FragLane f = frag_lane(bs, patch, tab, lane);
     T* ybv = yb + (lane & 3) * 8;
-    const T* rbv = rb ? rb + (lane & 3) * 8 : nullptr;
     if (c0 >= n_px) return;
-    unsigned ra[16], rb2[16];
-    tmem_ld16(d_base + (unsigned)c0, ra);
+    unsigned la[8], ha[8], lb[8], hb[8];
+    tmem_ld_frag(d_base + (unsigned)c0, la, ha);
     for (; c0 < n_px; c0 += c_step) {
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        tmem_ld16(d_base + (unsigned)(c0 + kPatchRows), rb2);
-        epilogue_half<T, ACT>(ra, bs, wr, rd, tab_l + (unsigned)c0 * 8, ybv, ry, rx, rbv);
+        tmem_ld_frag(d_base + (unsigned)(c0 + kPatchRows), lb, hb);
+        frag_half<T, ACT>(la, ha, f, (unsigned)c0, ybv, ry, rx);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (c0 + c_step < n_px) tmem_ld16(d_base + (unsigned)(c0 + c_step), ra);
-        epilogue_half<T, ACT>(rb2, bs, wr, rd, tab_l + (unsigned)(c0 + kPatchRows) * 8, ybv, ry, rx, rbv);
+        if (c0 + c_step < n_px) tmem_ld_frag(d_base + (unsigned)(c0 + c_step), la, ha);
+        frag_half<T, ACT>(lb, hb, f, (unsigned)(c0 + kPatchRows), ybv, ry, rx);
     }
 }
 
 // The same with a residual operand.  Its values arrive by asynchronous 16-byte copies (global -> shared, no
-// registers held while they fly): every lane fetches the two pieces it will add (positions 2 jp and 2 jp + 1, its
+// registers held while they fly): every lane fetches the two pieces it will add (positions lane / 4 and + 8, its
 // eight filters) into its own slots of the warp's staging area, one half chunk ahead of the one being finished, so a
 // load from memory has a whole half chunk of work to hide behind.  A lane reads back only what it fetched itself:
 // cp.async.wait_group is all the ordering needed.  stage: shared address of the warp's kResStage bytes, two buffers
 // of [2 pieces][32 lanes] x 16 bytes.
 template <typename T>
 __device__ __forceinline__ void fetch_residual(unsigned tab_at, const T* rbv, unsigned ry, unsigned rx, unsigned slot) {
-    unsigned e[4];
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3]) : "r"(tab_at));
-    if ((e[1] >> 16) < ry && (e[1] & 0xFFFFu) < rx)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot), "l"(rbv + e[0]) : "memory");
-    if ((e[3] >> 16) < ry && (e[3] & 0xFFFFu) < rx)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + 512u), "l"(rbv + e[2]) : "memory");
+    const uint2 e0 = lds64(tab_at), e1 = lds64(tab_at + 64u);
+    if (inside(e0, ry, rx)) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot), "l"(rbv + e0.x) : "memory");
+    if (inside(e1, ry, rx)) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + 512u), "l"(rbv + e1.x) : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
+// POST: activated and rounded as without a residual (the bias is then what bias_act expects); else the plain sum first.
 template <typename T, int ACT, bool POST>
-__device__ __forceinline__ void epilogue_half_res(const unsigned (&r)[16], float bias, unsigned wr, unsigned rd, unsigned tab_at,
-                                                  T* ybv, unsigned ry, unsigned rx, unsigned slot) {
-#pragma unroll
-    for (int jp = 0; jp < kPatchRows / 2; ++jp) {
-        // POST: activated and rounded as without a residual (bias is then what bias_act expects); else the plain sum
-        const unsigned w = POST ? round_pack<T, ACT == RTOSS_ACT_RELU>(bias_act<ACT>(r[2 * jp], bias), bias_act<ACT>(r[2 * jp + 1], bias))
-                                : round_pack<T, false>(__uint_as_float(r[2 * jp]) + bias, __uint_as_float(r[2 * jp + 1]) + bias);
-        asm volatile("st.shared.u32 [%0], %1;" ::"r"(wr + jp * kPairPitch), "r"(w) : "memory");
-    }
-    __syncwarp();
-    unsigned w[8], e[4];
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(rd));
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]) : "r"(rd + 16));
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3]) : "r"(tab_at));
-    if ((e[1] >> 16) < ry && (e[1] & 0xFFFFu) < rx) {
-        uint4 rv;
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(rv.x), "=r"(rv.y), "=r"(rv.z), "=r"(rv.w) : "r"(slot));
-        const uint4 o = make_uint4(__byte_perm(w[0], w[1], 0x5410), __byte_perm(w[2], w[3], 0x5410),
-                                   __byte_perm(w[4], w[5], 0x5410), __byte_perm(w[6], w[7], 0x5410));
-        *reinterpret_cast<uint4*>(ybv + e[0]) = add_residual8<T, POST ? RTOSS_ACT_NONE : ACT>(o, rv);
-    }
-    if ((e[3] >> 16) < ry && (e[3] & 0xFFFFu) < rx) {
-        uint4 rv;
-        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(rv.x), "=r"(rv.y), "=r"(rv.z), "=r"(rv.w) : "r"(slot + 512u));
-        const uint4 o = make_uint4(__byte_perm(w[0], w[1], 0x7632), __byte_perm(w[2], w[3], 0x7632),
-                                   __byte_perm(w[4], w[5], 0x7632), __byte_perm(w[6], w[7], 0x7632));
-        *reinterpret_cast<uint4*>(ybv + e[2]) = add_residual8<T, POST ? RTOSS_ACT_NONE : ACT>(o, rv);
-    }
+__device__ __forceinline__ void frag_half_res(const unsigned (&lo)[8], const unsigned (&hi)[8], const FragLane& f, unsigned c0, T* ybv,
+                                              unsigned ry, unsigned rx, unsigned slot) {
+    const uint2 e0 = lds64(f.tab + c0 * 8u), e1 = lds64(f.tab + c0 * 8u + 64u);
+    frag_to_patch<T, POST ? ACT : RTOSS_ACT_NONE>(lo, hi, f);
+    const uint4 o0 = lds128(f.rd), o1 = lds128(f.rd + 512u);
+    if (inside(e0, ry, rx)) *reinterpret_cast<uint4*>(ybv + e0.x) = add_residual8<T, POST ? RTOSS_ACT_NONE : ACT>(o0, lds128(slot));
+    if (inside(e1, ry, rx)) *reinterpret_cast<uint4*>(ybv + e1.x) = add_residual8<T, POST ? RTOSS_ACT_NONE : ACT>(o1, lds128(slot + 512u));
     __syncwarp();
 }
 
@@ -590,31 +634,29 @@ template <typename T, int ACT, bool POST>
 __device__ __forceinline__ void epilogue_chunks_res(unsigned d_base, int c0, int c_step, int n_px, float bias,
                                                     unsigned patch, unsigned tab, T* yb, unsigned ry, unsigned rx,
                                                     int lane, const T* rb, unsigned stage) {
-    const unsigned wr = patch + lane * 4;
-    const unsigned rd = patch + (lane >> 2) * kPairPitch + (lane & 3) * 32;
-    const unsigned tab_l = tab + (unsigned)(2 * (lane >> 2)) * 8;
+    const FragLane f = frag_lane(bias, patch, tab, lane);
     T* ybv = yb + (lane & 3) * 8;
     const T* rbv = rb + (lane & 3) * 8;
     if (c0 >= n_px) return;
     const unsigned slot0 = stage + (unsigned)lane * 16, slot1 = slot0 + 1024u;
-    unsigned ra[16], rb2[16];
-    fetch_residual<T>(tab_l + (unsigned)c0 * 8, rbv, ry, rx, slot0);
-    tmem_ld16(d_base + (unsigned)c0, ra);
+    unsigned la[8], ha[8], lb[8], hb[8];
+    fetch_residual<T>(f.tab + (unsigned)c0 * 8, rbv, ry, rx, slot0);
+    tmem_ld_frag(d_base + (unsigned)c0, la, ha);
     for (; c0 < n_px; c0 += c_step) {
-        fetch_residual<T>(tab_l + (unsigned)(c0 + kPatchRows) * 8, rbv, ry, rx, slot1);
+        fetch_residual<T>(f.tab + (unsigned)(c0 + kPatchRows) * 8, rbv, ry, rx, slot1);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        tmem_ld16(d_base + (unsigned)(c0 + kPatchRows), rb2);
+        tmem_ld_frag(d_base + (unsigned)(c0 + kPatchRows), lb, hb);
         asm volatile("cp.async.wait_group 1;" ::: "memory");   // the pieces of this half are in
-        epilogue_half_res<T, ACT, POST>(ra, bias, wr, rd, tab_l + (unsigned)c0 * 8, ybv, ry, rx, slot0);
+        frag_half_res<T, ACT, POST>(la, ha, f, (unsigned)c0, ybv, ry, rx, slot0);
         const bool more = c0 + c_step < n_px;
         if (more)
-            fetch_residual<T>(tab_l + (unsigned)(c0 + c_step) * 8, rbv, ry, rx, slot0);
+            fetch_residual<T>(f.tab + (unsigned)(c0 + c_step) * 8, rbv, ry, rx, slot0);
         else
             asm volatile("cp.async.commit_group;" ::: "memory");   // keeps the group count in step
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (more) tmem_ld16(d_base + (unsigned)(c0 + c_step), ra);
+        if (more) tmem_ld_frag(d_base + (unsigned)(c0 + c_step), la, ha);
         asm volatile("cp.async.wait_group 1;" ::: "memory");
-        epilogue_half_res<T, ACT, POST>(rb2, bias, wr, rd, tab_l + (unsigned)(c0 + kPatchRows) * 8, ybv, ry, rx, slot1);
+        frag_half_res<T, ACT, POST>(lb, hb, f, (unsigned)(c0 + kPatchRows), ybv, ry, rx, slot1);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
@@ -1418,13 +1460,13 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         }
 #undef RTOSS_RES_CALL
                     } else if (a.act == RTOSS_ACT_SILU)
-                        epilogue_chunks<T, RTOSS_ACT_SILU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
+                        epilogue_chunks<T, RTOSS_ACT_SILU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane);
                     else if (a.act == RTOSS_ACT_RELU)
-                        epilogue_chunks<T, RTOSS_ACT_RELU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
+                        epilogue_chunks<T, RTOSS_ACT_RELU>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane);
                     else if (kRep && a.act == kActSiluX)
-                        epilogue_chunks<T, kActSiluX>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
+                        epilogue_chunks<T, kActSiluX>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane);
                     else
-                        epilogue_chunks<T, RTOSS_ACT_NONE>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane, rb);
+                        epilogue_chunks<T, RTOSS_ACT_NONE>(d_base, c_first, c_step, a.N_px, bs, patch, s_tab, yb, ry, rx, lane);
                 } else if (kRep && a.nchw) {
                     stored = true;
                     const bool pair_ok = (a.y_co & 1) == 0;
