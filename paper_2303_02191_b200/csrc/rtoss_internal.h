@@ -152,6 +152,11 @@ int rtoss_launch_conv_tc_group(const rtoss_ctx* ctx, int n, const rtoss_packed* 
 // the same with dependencies: bit j of after[i] = convolution i waits (inside the launch) for convolution j < i
 int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const void* const* xs,
                                void* const* ys, const rtoss_conv_desc* const* ds, const uint32_t* after, void* stream);
+// kernels compiled for one kind of launch (conv_tc_forms.cuh), or null; prepare: per device, before the first launch
+void* rtoss_tc_form_bf16(int form, bool shared);
+void* rtoss_tc_form_f16(int form, bool shared);
+int rtoss_tc_prepare_forms_bf16();
+int rtoss_tc_prepare_forms_f16();
 int rtoss_tc_max_problems();   // most convolutions one launch carries
 // what the planner expects of a launch of its own (shared launches never split a tile's channel blocks) and of a shared one
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles);
