@@ -254,22 +254,34 @@ __host__ __device__ __forceinline__ unsigned long long make_sw_desc(unsigned add
     return d;
 }
 
+// The MMA warp runs its loop as one, every value in it the same for all lanes, and only the elected lane (leader != 0)
+// issues: descriptors and addresses then live in uniform registers, which is where tcgen05.mma takes them from.  (With the
+// loop inside "if (lane == 0)" a 1x1 layer's thread took 870 cycles for the four instructions of a channel block, 660 in
+// this form: 1x1 128->128 @40x40 3.3 -> 2.9 us, 256->1024 @50x68 batch 4 13.3 -> 11.8, 3x3 32->32 @160x160 batch 16 31.3 ->
+// 24.7.  The producers' loops, which issue few copies, were 1 to 3 % slower this way and stay with one lane.)
+__device__ __forceinline__ unsigned elect_one() {
+    unsigned e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e;
+}
 template <bool TF32>
-__device__ __forceinline__ void umma_f16(unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc,
+__device__ __forceinline__ void umma_f16(unsigned leader, unsigned d_tmem, unsigned long long adesc, unsigned long long bdesc,
                                          unsigned idesc, unsigned accumulate) {
     if (TF32)
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, pe;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            "setp.ne.b32 pe, %5, 0;\n\t"
+            "@pe tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
             : "memory");
     else
         asm volatile(
-            "{\n\t.reg .pred p;\n\t"
+            "{\n\t.reg .pred p, pe;\n\t"
             "setp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+            "setp.ne.b32 pe, %5, 0;\n\t"
+            "@pe tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(leader)
             : "memory");
 }
 // The MMAs of one tap of one channel block (filters on M) for the 16-channel slabs named by the mask m4 (bit s = slab
@@ -322,8 +334,11 @@ __device__ __forceinline__ unsigned umma_block_peek(unsigned d_tmem, unsigned lo
                 : umma_block_peek_f16(d_tmem, adesc, bdesc, idesc, accumulate, m4, barA, parA, barB, parB);
 }
 // Arrive on an mbarrier once all tcgen05.mma issued so far by this thread have completed.
-__device__ __forceinline__ void umma_commit(unsigned bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+__device__ __forceinline__ void umma_commit(unsigned leader, unsigned bar) {
+    asm volatile(
+        "{\n\t.reg .pred pe;\n\tsetp.ne.b32 pe, %1, 0;\n\t"
+        "@pe tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar), "r"(leader)
+        : "memory");
 }
 
 __device__ __forceinline__ void tmem_ld32(unsigned taddr, unsigned (&r)[32]) {
@@ -1110,8 +1125,9 @@ conv_tc_kernel(const __grid_constant__ G g) {
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
+        // ---------------- MMA issuer (the whole warp, see umma_f16)
+        {
+            const unsigned leader = elect_one();
             // One thread issues every tcgen05.mma, so the instructions between two of them are the budget: with one or
             // two instructions per tap (few channels, or few filters with the positions as M) the tensor pipe waits
             // for this thread.  Hence: ring positions and phases are carried as counters (no division), a descriptor
@@ -1139,8 +1155,8 @@ conv_tc_kernel(const __grid_constant__ G g) {
 #pragma unroll
                     for (int k4 = 0; k4 < kKBlock / 16; ++k4) {
                         if (m4 & (1u << k4)) {
-                            umma_f16<kF32>(d_base, mk(xl + 2 * k4), mk(wl + 2 * k4), idesc, acc);
-                            if (two) umma_f16<kF32>(d_base + hi_cols, mk(xl + half16 + 2 * k4), mk(wl + 2 * k4), idesc, acc);
+                            umma_f16<kF32>(leader, d_base, mk(xl + 2 * k4), mk(wl + 2 * k4), idesc, acc);
+                            if (two) umma_f16<kF32>(leader, d_base + hi_cols, mk(xl + half16 + 2 * k4), mk(wl + 2 * k4), idesc, acc);
                             acc = 1;
                         }
                     }
@@ -1148,7 +1164,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
 #pragma unroll
                     for (int k4 = 0; k4 < kKBlock / 16; ++k4) {
                         if (m4 & (1u << k4)) {
-                            umma_f16<kF32>(d_base, mk(wl + 2 * k4), mk(xl + 2 * k4), idesc, acc);
+                            umma_f16<kF32>(leader, d_base, mk(wl + 2 * k4), mk(xl + 2 * k4), idesc, acc);
                             acc = 1;
                         }
                     }
@@ -1176,7 +1192,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                             if (!ok) break;
                         }
                         // rings of another layout: the producers may write them once everything issued so far has read its operands
-                        umma_commit(bar_switch);
+                        umma_commit(leader, bar_switch);
                         ra.s = rb.s = 0;
                         peek = 0;
                     }
@@ -1228,26 +1244,26 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         const unsigned wl0 = desc_lo0 + (sB >> 4) + (unsigned)sb * bstage16;
                         const unsigned xl0 = desc_lo0 + (sA >> 4) + (unsigned)sa * astage16;
                         if (kAny ? !pxm : kKind != 2) {
-                            peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl0), idesc, acc, nkmask, bar_rdyA + 8 * sa_n, pa_n,
+                            peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl0), idesc, acc, leader ? nkmask : 0u, bar_rdyA + 8 * sa_n, pa_n,
                                                    bar_fullB + 8 * sb_n, pb_n);
                         } else {
                             // positions on M: the first 128 positions with the look ahead, then the second 128
-                            peek = umma_block_peek<kF32>(d_base, mk(xl0), mk(wl0), idesc, acc, nkmask, bar_rdyA + 8 * sa_n, pa_n,
+                            peek = umma_block_peek<kF32>(d_base, mk(xl0), mk(wl0), idesc, acc, leader ? nkmask : 0u, bar_rdyA + 8 * sa_n, pa_n,
                                                    bar_fullB + 8 * sb_n, pb_n);
                             if (two) {
                                 unsigned acc2 = acc;
 #pragma unroll
                                 for (int k4 = 0; k4 < kKBlock / 16; ++k4) {
                                     if (k4 < nk4) {
-                                        umma_f16<kF32>(d_base + hi_cols, mk(xl0 + half16 + 2 * k4), mk(wl0 + 2 * k4), idesc, acc2);
+                                        umma_f16<kF32>(leader, d_base + hi_cols, mk(xl0 + half16 + 2 * k4), mk(wl0 + 2 * k4), idesc, acc2);
                                         acc2 = 1;
                                     }
                                 }
                             }
                         }
                         acc = 1;
-                        umma_commit(bar_emptyB + 8 * sb);
-                        umma_commit(bar_emptyA + 8 * sa);
+                        umma_commit(leader, bar_emptyB + 8 * sb);
+                        umma_commit(leader, bar_emptyA + 8 * sa);
                         continue;
                     }
                     const unsigned long long bits_n = (iss && cb + 1 < cb_end) ? __ldg(iss + cb + 1) : ~0ull;
@@ -1270,7 +1286,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                 rb.advance(NB);
                                 if (kAny ? !pxm : true) {
                                     // the first tap of the stage goes out together with a look at the next stages
-                                    peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl0 + tap16[s3 * 3]), idesc, acc, m_first,
+                                    peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl0 + tap16[s3 * 3]), idesc, acc, leader ? m_first : 0u,
                                                            bar_rdyA + 8 * sa_n, pa_n, bar_fullB + 8 * rb.s, rb.parity());
                                     if (m_first) acc = 1;
 #pragma unroll
@@ -1283,7 +1299,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                         issue_tap(d_base, wl0 + i * wtile16, xl0 + tap16[s3 * 3 + i],
                                                   (unsigned)(bits >> (12 * s3 + 4 * i)) & nkmask, acc);
                                 }
-                                umma_commit(bar_emptyB + 8 * sb);  // this weight stage may be refilled once the MMAs have read it
+                                umma_commit(leader, bar_emptyB + 8 * sb);  // this weight stage may be refilled once the MMAs have read it
                             }
                         }
                     } else if constexpr (kAny) {
@@ -1303,14 +1319,14 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                 issue_tap(d_base, wl0 + i * wtile16, xl0 + off, m4, acc);
                                 if (kF32 && v < a.taps_real) issue_tap(d_base, wl0 + i * wtile16, xl0 + off + ((unsigned)a.lo_off >> 4), m4, acc);
                             }
-                            umma_commit(bar_emptyB + 8 * sb);
+                            umma_commit(leader, bar_emptyB + 8 * sb);
                             rb.advance(NB);
                         }
                     }
-                    if (ok) umma_commit(bar_emptyA + 8 * sa);
+                    if (ok) umma_commit(leader, bar_emptyA + 8 * sa);
                     bits = bits_n;
                 }
-                if (ok) umma_commit(bar_accFull + 8 * as);
+                if (ok) umma_commit(leader, bar_accFull + 8 * as);
                 since_res = a.resid ? 0 : since_res + 1;
                 if (++as == g.AS) {
                     as = 0;
@@ -1326,7 +1342,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 }
                 ok = mbar_wait(bar_accEmpty + 8 * as, pacc, g.wait_cycles);
             }
-            if (!ok) atomicExch(g.status, 2);
+            if (!ok && leader) atomicExch(g.status, 2);
         }
         __syncwarp();
     } else {
