@@ -32,6 +32,7 @@
 //     multiple of 8.  Weights: Cin a multiple of 8.  Anything else takes a plain
 //     load-convert-store path inside the same kernel.
 #include <cstring>
+#include <type_traits>
 
 #include "conv_common.cuh"
 
@@ -422,15 +423,9 @@ struct Variant {
 // neighbouring output pixels of one row for 32 filters: its input window (3 rows x ((kStemPx-1)*S+3)
 // columns x CIN) sits in registers, the dense-expanded weights (pruned taps are zeros: with 9*CIN <= 36
 // multiply-adds per output the zeros cost less than skipping them) are read from shared memory once per
-// filter as 16-byte loads and used for all kStemPx pixels.  The layer's bound is its traffic, so loads and
-// stores must be whole segments:
-//   * the detector stem proper (three 16-bit channels, NHWC, stride 2, rows of a multiple of 8 pixels): a
-//     thread's window of 9 pixels x 3 channels is 54 contiguous bytes that start 6 bytes before a 16-byte
-//     boundary, so it comes in as four aligned 16-byte loads per row and every value sits at a position
-//     known at compile time (81 separate 2-byte loads a thread, each lane in its own sector, were what
-//     bounded the kernel before);
-//   * with 16-bit NHWC outputs a block's 512 pixels x 32 filters are gathered in shared memory and written
-//     out with consecutive lanes on consecutive 16 bytes.
+// filter as 16-byte loads and used for all kStemPx pixels.  16-bit NHWC outputs (a block's 512 pixels x 32
+// filters) are gathered in shared memory and written out with consecutive lanes on consecutive 16 bytes.
+// (The detector stem proper has its own kernel, below.)
 // A block walks the pixel groups in steps of the grid, so the weight table is built once per block.
 constexpr int kStemCo = 32;
 constexpr int kStemPx = 4;
@@ -493,7 +488,6 @@ __global__ void __launch_bounds__(kStemThreads) conv3x3_small_cin_kernel(const C
     // 16-bit NHWC outputs whose rows hold whole groups: pixel index = kStemPx * group index + px, the pixels of a
     // round of the block are consecutive, and the stores go through the staging buffer
     const bool staged = sizeof(T) == 2 && vec && a.Wo % kStemPx == 0;
-    const bool fast_in = sizeof(T) == 2 && CIN == 3 && S == 2 && kStemPx == 4 && a.layout == RTOSS_NHWC && a.W % 8 == 0;
     const int groups = (a.Wo + kStemPx - 1) / kStemPx;      // groups of kStemPx output columns per row
     const long long total = (long long)a.N * a.Ho * groups;
     const long long px_total = (long long)a.N * a.Ho * a.Wo;
@@ -506,46 +500,19 @@ __global__ void __launch_bounds__(kStemThreads) conv3x3_small_cin_kernel(const C
         const long long r1 = gi / groups;
         const int oy = (int)(r1 % a.Ho), n = (int)(r1 / a.Ho);
         float xin[CIN][3][WIN];
-        if (fast_in) {
 #pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const int iy = oy * S + r - 1;
-                const bool row_ok = iy >= 0 && iy < a.H;
-                // 16-byte piece 3 * (ox0 / 4) of the row holds input pixel 2 * ox0; the window starts one pixel earlier
-                const uint4* rowp = reinterpret_cast<const uint4*>(xg + ((size_t)n * a.H + (row_ok ? iy : 0)) * a.W * CIN) + (ox0 / kStemPx) * 3;
-                const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
-                uint4 ch[4];
-                ch[0] = (row_ok && ox0 > 0) ? __ldg(rowp - 1) : zero;
+        for (int r = 0; r < 3; ++r) {
+            const int iy = oy * S + r - 1;
+            const bool row_ok = iy >= 0 && iy < a.H;
 #pragma unroll
-                for (int i = 1; i < 4; ++i) ch[i] = row_ok ? __ldg(rowp + i - 1) : zero;
-                const unsigned wds[16] = {ch[0].x, ch[0].y, ch[0].z, ch[0].w, ch[1].x, ch[1].y, ch[1].z, ch[1].w,
-                                          ch[2].x, ch[2].y, ch[2].z, ch[2].w, ch[3].x, ch[3].y, ch[3].z, ch[3].w};
+            for (int c = 0; c < WIN; ++c) {
+                const int ix = ox0 * S + c - 1;
+                const bool ok = row_ok && ix >= 0 && ix < a.W;
 #pragma unroll
-                for (int c = 0; c < WIN; ++c)
-#pragma unroll
-                    for (int ci = 0; ci < CIN; ++ci) {
-                        const int hi = (5 + c * CIN + ci) & 31;   // 16-bit index inside the 64 bytes: the window starts at byte 10
-                        const unsigned short bits = (hi & 1) ? (unsigned short)(wds[hi >> 1] >> 16) : (unsigned short)(wds[hi >> 1] & 0xFFFFu);
-                        T v;
-                        memcpy(&v, &bits, sizeof(bits));
-                        xin[ci][r][c] = to_f32<T>(v);
-                    }
-            }
-        } else {
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                const int iy = oy * S + r - 1;
-                const bool row_ok = iy >= 0 && iy < a.H;
-#pragma unroll
-                for (int c = 0; c < WIN; ++c) {
-                    const int ix = ox0 * S + c - 1;
-                    const bool ok = row_ok && ix >= 0 && ix < a.W;
-#pragma unroll
-                    for (int ci = 0; ci < CIN; ++ci) {
-                        const size_t idx = a.layout == RTOSS_NCHW ? (((size_t)n * CIN + ci) * a.H + iy) * a.W + ix
-                                                                  : (((size_t)n * a.H + iy) * a.W + ix) * CIN + ci;
-                        xin[ci][r][c] = ok ? to_f32<T>(xg[idx]) : 0.f;
-                    }
+                for (int ci = 0; ci < CIN; ++ci) {
+                    const size_t idx = a.layout == RTOSS_NCHW ? (((size_t)n * CIN + ci) * a.H + iy) * a.W + ix
+                                                              : (((size_t)n * a.H + iy) * a.W + ix) * CIN + ci;
+                    xin[ci][r][c] = ok ? to_f32<T>(xg[idx]) : 0.f;
                 }
             }
         }
@@ -616,6 +583,238 @@ __global__ void __launch_bounds__(kStemThreads) conv3x3_small_cin_kernel(const C
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// The detector stem proper: three 16-bit channels, channels last, stride 2, rows of an even number of pixels.  With 27
+// products per output the layer's bound is its traffic (16 frames of 640 x 640: 144 MB, 22 us), which the kernel above is
+// far from: its multiply-adds, the shared-memory loads of their weights and the conversions came to 103 us.  Here they
+// are matrix instructions: 16 neighbouring output pixels of a row are the rows of a fragment, a window's 27 values (padded
+// to 32) its columns.  An output pixel's window is nine consecutive values in each of three input rows, and begins at an
+// odd one: with the value before it (masked, its weight is zero too) that makes five aligned pairs a row, fifteen in all,
+// and pair p is the fragment's columns 2p and 2p + 1 -- so a lane's share of the window is eight 4-byte reads at fixed
+// offsets, without a conversion.  Filters are dealt to the fragment's columns so that a lane ends up with eight
+// neighbouring ones: the outputs leave as 16-byte stores, four lanes to a pixel, without a transpose.
+// A block works on two output rows x up to 320 columns at a time; their five input rows are in shared memory (outside the
+// image zeros), the next band's on their way there: 31 us (one frame: 5.3 instead of 12.5).  Fragments read from global
+// memory, one ahead, took 66 us: too few bytes in flight, and a third of the instructions were addresses and bounds.
+constexpr int kStemMmaThreads = 256;
+
+template <typename T>
+__device__ __forceinline__ void mma_16x8x16(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+    if constexpr (std::is_same<T, __half>::value)
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+    else
+        asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+            : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// SiLU of two sums: v / 2 + v / 2 * tanh(v / 2), see stem_act.
+template <typename T, int ACT>
+__device__ __forceinline__ unsigned stem_pair(float a, float b) {
+    if constexpr (ACT == RTOSS_ACT_SILU) {
+        unsigned long long v, h;
+        float ha, hb, ta, tb;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+        asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(h) : "l"(v), "l"(0x3F0000003F000000ull));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(ha), "=f"(hb) : "l"(h));
+        asm("tanh.approx.f32 %0, %1;" : "=f"(ta) : "f"(ha));
+        asm("tanh.approx.f32 %0, %1;" : "=f"(tb) : "f"(hb));
+        asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(ta), "f"(tb));
+        asm("fma.rn.f32x2 %0, %1, %2, %1;" : "=l"(h) : "l"(h), "l"(v));
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(h));
+    } else {
+        a = activate(a, ACT);
+        b = activate(b, ACT);
+    }
+    if constexpr (std::is_same<T, __half>::value) {
+        const __half2 u = __floats2half2_rn(a, b);
+        return *reinterpret_cast<const unsigned*>(&u);
+    } else {
+        const __nv_bfloat162 u = __floats2bfloat162_rn(a, b);
+        return *reinterpret_cast<const unsigned*>(&u);
+    }
+}
+
+// How a stem call is cut: bands of two output rows and tile_w output columns (a multiple of 16).
+struct StemPlan {
+    int tile_w, tiles_x, bands, pitch;   // pitch: bytes of a staged input row
+    unsigned units;
+};
+
+// VB: bytes of one asynchronous copy (16 where rows are whole 16-byte pieces, else 4).
+template <typename T, int ACT, int VB>
+__global__ void __launch_bounds__(kStemMmaThreads, 3) conv3x3_stem_mma_kernel(const Conv3Args a, const StemPlan pl) {
+    static_assert(sizeof(T) == 2, "16-bit data");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    extern __shared__ __align__(16) unsigned char stem_smem[];   // two bands of five rows
+    __shared__ __align__(16) T sW[kStemCo][40];   // [filter][2 * pair + half]; rows of 80 bytes: a fragment's loads meet different banks
+    const int co0 = blockIdx.y * kStemCo;
+    for (int i = threadIdx.x; i < kStemCo * 40 / 2; i += kStemMmaThreads) reinterpret_cast<unsigned*>(sW)[i] = 0u;
+    __syncthreads();
+    if (threadIdx.x < kStemCo * 3) {   // (a handle's arrays may be read ahead of the wait, see conv_common.cuh)
+        const int col = threadIdx.x / 3, ci = threadIdx.x - col * 3, co = co0 + col;
+        if (co < a.Cout) {
+            const size_t kid = (size_t)co * 3 + ci;
+            const unsigned m = a.masks[a.pid[kid]];
+            const T* v = reinterpret_cast<const T*>(a.val) + kid * a.k;
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const int d = (t % 3) * 3 + ci + 1;   // position in the row's ten values
+                if (m & (1u << t)) sW[col][(t / 3) * 10 + d] = *v++;
+            }
+        }
+    }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
+    // column c of fragment j is filter 8 * (c / 2) + 2 * j + c % 2: a lane's accumulators (columns 2 t4, 2 t4 + 1 of each
+    // fragment) are filters 8 t4 .. 8 t4 + 7
+    unsigned wb[4][2][2];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const T* row = sW[8 * (g >> 1) + 2 * j + (g & 1)] + 16 * s + 2 * t4;
+            wb[j][s][0] = *reinterpret_cast<const unsigned*>(row);
+            wb[j][s][1] = *reinterpret_cast<const unsigned*>(row + 8);
+        }
+    // this lane's pairs: t4, t4 + 4, t4 + 8, t4 + 12 (the last lane's pair 15 is padding: it reads pair 14 and drops it).  A
+    // staged row begins 16 bytes, two pixels and two values, ahead of the first window's second pixel.
+    unsigned at[4], keep[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int p = min(t4 + 4 * i, 14), r = p / 5, j = p - r * 5;
+        at[i] = (unsigned)(r * pl.pitch + 12 * g + 8 + 4 * j);
+        keep[i] = t4 + 4 * i == 15 ? 0u : j == 0 ? 0xFFFF0000u : 0xFFFFFFFFu;
+    }
+    const unsigned char* __restrict__ xg = reinterpret_cast<const unsigned char*>(a.x);
+    T* __restrict__ yg = reinterpret_cast<T*>(a.y);
+    const int row_bytes = a.W * 6, pieces = pl.pitch / VB, frags = pl.tile_w >> 4, stage_bytes = 5 * pl.pitch;
+    const unsigned smem0 = (unsigned)__cvta_generic_to_shared(stem_smem);
+    struct At { int n, band, tx; };
+    auto place = [&](unsigned unit) {
+        At u;
+        const unsigned q = unit / (unsigned)pl.tiles_x;
+        u.tx = (int)(unit - q * (unsigned)pl.tiles_x);
+        u.n = (int)(q / (unsigned)pl.bands);
+        u.band = (int)(q - (unsigned)u.n * (unsigned)pl.bands);
+        return u;
+    };
+    auto fetch = [&](const At& u, int stage) {
+        const int x0 = u.tx * pl.tile_w * 12 - 16;   // byte of the image row at which the staged row begins
+#pragma unroll
+        for (int r = 0; r < 5; ++r) {
+            const int iy = 4 * u.band - 1 + r;
+            const bool row_ok = iy >= 0 && iy < a.H;
+            const unsigned char* src = xg + ((size_t)u.n * a.H + (row_ok ? iy : 0)) * (size_t)row_bytes;
+            const unsigned dst = smem0 + (unsigned)(stage * stage_bytes + r * pl.pitch);
+            for (int c = threadIdx.x; c < pieces; c += kStemMmaThreads) {
+                const int b = x0 + c * VB;
+                const bool ok = row_ok && b >= 0 && b < row_bytes;
+                if constexpr (VB == 16)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + c * 16), "l"(src + (ok ? b : 0)), "r"(ok ? 16 : 0) : "memory");
+                else
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst + c * 4), "l"(src + (ok ? b : 0)), "r"(ok ? 4 : 0) : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    unsigned unit = blockIdx.x;
+    if (unit >= pl.units) return;
+    At cur = place(unit), nxt = cur;
+    fetch(cur, 0);
+    float bias[8];
+#pragma unroll
+    for (int f = 0; f < 8; ++f) bias[f] = (a.bias && co0 + 8 * t4 + f < a.Cout) ? __ldg(a.bias + co0 + 8 * t4 + f) : 0.f;
+    const bool vec = (a.y_c_stride % 8 == 0) && ((a.y_c_off + co0) % 8 == 0) && (reinterpret_cast<uintptr_t>(yg) & 15) == 0 && co0 + 8 * t4 + 8 <= a.Cout;
+    for (int stage = 0; unit < pl.units; unit += gridDim.x, cur = nxt, stage ^= 1) {
+        if (unit + gridDim.x < pl.units) {
+            nxt = place(unit + gridDim.x);
+            fetch(nxt, stage ^ 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const int oy0 = cur.band * 2, ox0 = cur.tx * pl.tile_w, rows = min(2, a.Ho - oy0);
+        T* ytile = yg + (((size_t)cur.n * a.Ho + oy0) * a.Wo + ox0) * a.y_c_stride + a.y_c_off + co0 + 8 * t4;
+        for (int f = warp; f < rows * frags; f += kStemMmaThreads / 32) {
+            const int rr = f >= frags ? 1 : 0, c = f - rr * frags;
+            const unsigned char* sp = stem_smem + stage * stage_bytes + rr * 2 * pl.pitch + c * 192;
+            unsigned xa[2][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                xa[i >> 1][(i & 1) * 2] = *reinterpret_cast<const unsigned*>(sp + at[i]) & keep[i];
+                xa[i >> 1][(i & 1) * 2 + 1] = *reinterpret_cast<const unsigned*>(sp + at[i] + 96) & keep[i];
+            }
+            float acc[4][4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[j][0] = acc[j][2] = bias[2 * j];
+                acc[j][1] = acc[j][3] = bias[2 * j + 1];
+#pragma unroll
+                for (int s = 0; s < 2; ++s) mma_16x8x16<T>(acc[j], xa[s], wb[j][s][0], wb[j][s][1]);
+            }
+            const int px = c * 16 + g;
+            T* dst = ytile + ((size_t)(rr * a.Wo) + px) * a.y_c_stride;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                unsigned o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) o[j] = stem_pair<T, ACT>(acc[j][2 * q], acc[j][2 * q + 1]);
+                if (ox0 + px + 8 * q < a.Wo) {
+                    T* to = dst + (size_t)(8 * q) * a.y_c_stride;
+                    if (vec) {
+                        *reinterpret_cast<uint4*>(to) = make_uint4(o[0], o[1], o[2], o[3]);
+                    } else {
+                        const T* ov = reinterpret_cast<const T*>(o);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            if (co0 + 8 * t4 + e < a.Cout) to[e] = ov[e];
+                    }
+                }
+            }
+        }
+        __syncthreads();   // the stage may be filled again
+    }
+}
+
+// Values of the data's own type, aligned pairs of them (even rows), units and row bytes that 31 bits count.
+template <typename T>
+bool stem_mma_ok(const Conv3Args& a, int stride) {
+    if (sizeof(T) != 2 || a.Cin != 3 || stride != 2 || a.layout != RTOSS_NHWC || a.W % 2 != 0 || a.val_dtype != (std::is_same<T, __half>::value ? RTOSS_F16 : RTOSS_BF16)) return false;
+    return (reinterpret_cast<uintptr_t>(a.x) & 3) == 0 && a.W < (1 << 24) && (long long)a.N * a.Ho * ((a.Wo + 15) / 16) < (1ll << 30);
+}
+
+template <typename T, int ACT>
+void launch_stem_act(const Conv3Args& a, const StemPlan& pl, dim3 grid, cudaStream_t stream) {
+    const size_t smem = 10 * (size_t)pl.pitch;
+    if (a.W % 8 == 0 && (reinterpret_cast<uintptr_t>(a.x) & 15) == 0)
+        rtoss_dev::launch_pdl(conv3x3_stem_mma_kernel<T, ACT, 16>, grid, kStemMmaThreads, smem, stream, a, pl);
+    else
+        rtoss_dev::launch_pdl(conv3x3_stem_mma_kernel<T, ACT, 4>, grid, kStemMmaThreads, smem, stream, a, pl);
+}
+
+template <typename T>
+int launch_stem_mma(const Conv3Args& a, cudaStream_t stream) {
+    StemPlan pl;
+    pl.bands = (a.Ho + 1) / 2;
+    // columns: at most 320 (39 KB staged, three blocks an SM), at least 64 (a fragment per warp), and within that narrow
+    // enough for six bands a SM where the images are small
+    const long long per_x = (long long)a.N * pl.bands, want = (148 * 6 + per_x - 1) / per_x;
+    const int most = (a.Wo + 63) / 64, least = (a.Wo + 319) / 320;
+    const int tiles = want < least ? least : want > most ? most : (int)want;
+    pl.tile_w = ((a.Wo + tiles - 1) / tiles + 15) / 16 * 16;
+    pl.tiles_x = (a.Wo + pl.tile_w - 1) / pl.tile_w;
+    pl.pitch = 12 * pl.tile_w + 16;
+    pl.units = (unsigned)(per_x * pl.tiles_x);
+    const dim3 grid(pl.units < 148u * 3u ? pl.units : 148u * 3u, (unsigned)((a.Cout + kStemCo - 1) / kStemCo));
+    if (a.act == RTOSS_ACT_SILU) launch_stem_act<T, RTOSS_ACT_SILU>(a, pl, grid, stream);
+    else if (a.act == RTOSS_ACT_RELU) launch_stem_act<T, RTOSS_ACT_RELU>(a, pl, grid, stream);
+    else launch_stem_act<T, RTOSS_ACT_NONE>(a, pl, grid, stream);
+    return (int)cudaGetLastError();
+}
+
 template <typename T, int S>
 int launch_small_cin_s(const Conv3Args& a, cudaStream_t stream) {
     const long long total = (long long)a.N * a.Ho * ((a.Wo + kStemPx - 1) / kStemPx);
@@ -633,6 +832,8 @@ int launch_small_cin_s(const Conv3Args& a, cudaStream_t stream) {
 
 template <typename T>
 int launch_small_cin(const Conv3Args& a, int stride, cudaStream_t stream) {
+    if constexpr (sizeof(T) == 2)
+        if (stem_mma_ok<T>(a, stride)) return launch_stem_mma<T>(a, stream);
     return stride == 1 ? launch_small_cin_s<T, 1>(a, stream) : launch_small_cin_s<T, 2>(a, stream);
 }
 
