@@ -227,17 +227,42 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
             }
             return;
         }
+        // Narrow layers (repeated filters) and odd rows: the nine taps in registers, then copy by copy, nine independent
+        // stores at a time.  (Tap by tap with the copies inside, a value was read, rounded and stored 36 times one after the
+        // other: 9 600 cycles for 18 filters, of a launch that holds four blocks; 4 200 now.)
+        if constexpr (sizeof(V) == 2) {
+            unsigned u[9];
+#pragma unroll
+            for (int t = 0; t < 9; ++t)
+                u[t] = round2<V>((mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f, (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f);
 #pragma unroll 1
-        for (int t = 0; t < 9; ++t, at += tap_step) {
-            const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
-            const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
-            V* to = at;
-            for (int c = 0; c < L.lay.copies; ++c, to += copy_step) {
+            for (int c = 0; c < L.lay.copies; ++c, at += copy_step) {
+                V* to = at;
                 if (word) {
-                    put_pair<V>(to, lo_at, a, b);
+#pragma unroll
+                    for (int t = 0; t < 9; ++t, to += tap_step) *reinterpret_cast<unsigned*>(to) = u[t];
                 } else {
-                    put_one<V>(to, lo_at, a);
-                    if (two) put_one<V>(to + d1, lo_at, b);
+#pragma unroll
+                    for (int t = 0; t < 9; ++t, to += tap_step) {
+                        *reinterpret_cast<uint16_t*>(to) = (uint16_t)u[t];
+                        if (two) *reinterpret_cast<uint16_t*>(to + d1) = (uint16_t)(u[t] >> 16);
+                    }
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int c = 0; c < L.lay.copies; ++c, at += copy_step) {
+                V* to = at;
+#pragma unroll
+                for (int t = 0; t < 9; ++t, to += tap_step) {
+                    const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
+                    const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
+                    if (word) {
+                        put_pair<V>(to, lo_at, a, b);
+                    } else {
+                        put_one<V>(to, lo_at, a);
+                        if (two) put_one<V>(to + d1, lo_at, b);
+                    }
                 }
             }
         }
@@ -283,7 +308,10 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
 // 31 for 7 M.  (Prefetching the next chunk with a second buffer cost occupancy and was slower: 142 us on the older form.)
 __global__ void __launch_bounds__(kBatchThreads, 6) batch_select_pack_kernel(const BatchLayer* __restrict__ layers,
                                                                           const BatchChunk* __restrict__ chunks,
-                                                                          unsigned n_chunks) {
+                                                                          unsigned n_chunks, int order_follows) {
+    // The ordering kernel behind this one waits for the end of this grid and does not let its own successors start before
+    // its end, so it may be set up meanwhile; no other kernel may be (a reader of handles does not wait).
+    if (order_follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     rtoss_dev::pdl_enter_handle_writer();
     __shared__ __align__(16) unsigned char raw[kChunk * 9 * 4];
     __shared__ BatchLayer s_layer;
@@ -352,7 +380,6 @@ __global__ void __launch_bounds__(kBatchThreads, 6) batch_select_pack_kernel(con
 __global__ void __launch_bounds__(rtoss_dev::kOrderThreads, 4) batch_order_kernel(const BatchLayer* __restrict__ layers,
                                                                              const uint32_t* __restrict__ task_layer, unsigned n_tasks) {
     using namespace rtoss_dev;
-    pdl_enter_handle_writer();
     __shared__ union {
         struct {
             uint32_t fill[kOrderThreads / 32][256];
@@ -361,6 +388,9 @@ __global__ void __launch_bounds__(rtoss_dev::kOrderThreads, 4) batch_order_kerne
         OrderFew few;
     } sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the first task's record is the plan's, which no kernel writes: it comes in ahead of the wait for the pattern ids
+    if (blockIdx.x < n_tasks) asm volatile("prefetch.global.L2 [%0];" ::"l"(layers + __ldg(task_layer + blockIdx.x)));
+    pdl_enter_handle_writer();
     for (unsigned task = blockIdx.x; task < n_tasks; task += gridDim.x) {
         const BatchLayer& L = layers[task_layer[task]];
         const int ci0 = (int)(task - L.task0) * kOrderChannels, cb_log2 = L.v_dtype == RTOSS_F32 ? 5 : 6;
@@ -537,7 +567,7 @@ rtoss_status rtoss_batch_select_pack(rtoss_ctx* ctx, const rtoss_batch* b, void*
         const unsigned resident = (unsigned)ctx->sm_count * 6u;   // (what the kernel's launch bounds allow)
         const unsigned grid = b->n_chunks < resident ? b->n_chunks : resident;
         e = rtoss_dev::launch_pdl(batch_select_pack_kernel, grid, kBatchThreads, 0, s, (const BatchLayer*)b->layers_dev,
-                                  (const BatchChunk*)b->chunks_dev, b->n_chunks);
+                                  (const BatchChunk*)b->chunks_dev, b->n_chunks, (int)(b->n_tasks != 0));
     }
     if (e == cudaSuccess && b->n_tasks) {
         const unsigned grid = b->n_tasks < cap ? b->n_tasks : cap;

@@ -329,15 +329,15 @@ __device__ __forceinline__ void order_channel(const uint8_t* __restrict__ pid, i
 }
 
 // The same for layers of at most 512 filters and 36 patterns (every layer of the two detectors but the widest, the preset
-// tables of up to four taps), sixteen neighbouring channels to a block of 256 threads.  A thread is (segment of 32 filters,
-// channel): it counts its segment's patterns one filter after the other into a column of its own, a scan over segments and
+// tables of up to four taps), sixteen neighbouring channels to a block of 256 threads.  A thread is (segment of up to 32
+// filters, channel): it counts its segment's patterns one filter after the other into a column of its own, a scan over segments and
 // patterns turns counts into first positions, a second walk places the filters in shared memory, and the lists leave in
 // whole lines.  Sixteen channels ride along in every instruction, where the form above spends 75 instructions on every
 // 32 filters of every channel (33 us for the 7 000 channels of the larger detector; both its id loads, a line per filter,
 // and its instructions were in the way; 15 us now).
 constexpr int kFewFilters = 512, kFewPatterns = 36, kOrderThreads = 256;
 constexpr int kOrderChannels = 16, kOrderSegs = kOrderThreads / kOrderChannels, kIdPitch = kOrderChannels + 4;
-static_assert(kOrderSegs * 32 == kFewFilters, "a segment is 32 filters");
+static_assert(kOrderSegs * 32 == kFewFilters, "a segment is at most 32 filters");
 struct OrderFew {
     uint8_t ids[kFewFilters * kIdPitch];
     uint16_t cnt[kOrderSegs][kFewPatterns][kOrderChannels];
@@ -367,24 +367,59 @@ __device__ __forceinline__ void order_channels_few(const uint8_t* __restrict__ p
             unsigned* to = reinterpret_cast<unsigned*>(sh.ids + co * kIdPitch);
             if (co < Cout) to[0] = v[q].x, to[1] = v[q].y, to[2] = v[q].z, to[3] = v[q].w;
         }
+    } else if ((Cin & 3) == 0) {
+        // aligned words of four ids, eight of a thread's loads in flight (88 channels, 400 filters, byte by byte: 8 000 cycles)
+        constexpr int kQ = 8;
+        for (int i0 = tid; i0 < Cout * (kOrderChannels / 4); i0 += kQ * kOrderThreads) {
+            unsigned v[kQ];
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) {
+                const int i = i0 + q * kOrderThreads, co = i >> 2, c = (i & 3) * 4;
+                v[q] = ~0u;
+                if (co < Cout && ci0 + c < Cin) v[q] = __ldcg(reinterpret_cast<const unsigned*>(pid + (size_t)co * Cin + ci0 + c));
+            }
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) {
+                const int i = i0 + q * kOrderThreads, co = i >> 2;
+                if (co < Cout) *reinterpret_cast<unsigned*>(sh.ids + co * kIdPitch + (i & 3) * 4) = v[q];
+            }
+        }
     } else {
-#pragma unroll 8
-        for (int i = tid; i < Cout * kOrderChannels; i += kOrderThreads) {
-            const int co = i / kOrderChannels, c = i % kOrderChannels;
-            sh.ids[co * kIdPitch + c] = ci0 + c < Cin ? pid[(size_t)co * Cin + ci0 + c] : (uint8_t)255;
+        constexpr int kQ = 8;
+        for (int i0 = tid; i0 < Cout * kOrderChannels; i0 += kQ * kOrderThreads) {
+            uint8_t v[kQ];
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) {
+                const int i = i0 + q * kOrderThreads, co = i / kOrderChannels, c = i % kOrderChannels;
+                v[q] = co < Cout && ci0 + c < Cin ? __ldcg(pid + (size_t)co * Cin + ci0 + c) : (uint8_t)255;
+            }
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) {
+                const int i = i0 + q * kOrderThreads, co = i / kOrderChannels;
+                if (co < Cout) sh.ids[co * kIdPitch + i % kOrderChannels] = v[q];
+            }
         }
     }
-    const int c = tid % kOrderChannels, s = tid / kOrderChannels, co0 = 32 * s, co1 = min(co0 + 32, Cout);
+    // Filters of a segment: as few as the sixteen segments allow, a power of two so that none crosses a tile of 128.  (Always
+    // 32: 3 000 cycles per walk for layers of 64 filters, of which two threads in sixteen did the work; 900 and 2 100 now.)
+    int seg = 32;
+    while (seg > 1 && (seg / 2) * kOrderSegs >= Cout) seg >>= 1;
+    const int c = tid % kOrderChannels, s = tid / kOrderChannels, co0 = min(seg * s, Cout), co1 = min(co0 + seg, Cout);
     const bool real = ci0 + c < Cin;
     for (int p = 0; p < P; ++p) sh.cnt[s][p][c] = 0;
     __syncthreads();
     unsigned used = 0;   // taps kept by any filter of the segment
-#pragma unroll 4
-    for (int co = co0; co < co1; ++co) {
-        const unsigned p = sh.ids[co * kIdPitch + c];
-        if (p < (unsigned)P) {   // (an id outside the table is not placed)
-            sh.cnt[s][p][c] = (uint16_t)(sh.cnt[s][p][c] + 1);
-            used |= sh.masks[p];
+    constexpr int kWalk = 8;   // ids read ahead of the counts, which the compiler takes for the same memory
+    for (int f0 = co0; f0 < co1; f0 += kWalk) {
+        unsigned id[kWalk];
+#pragma unroll
+        for (int j = 0; j < kWalk; ++j) id[j] = sh.ids[min(f0 + j, co1 - 1) * kIdPitch + c];
+#pragma unroll
+        for (int j = 0; j < kWalk; ++j) {
+            if (f0 + j < co1 && id[j] < (unsigned)P) {   // (an id outside the table is not placed)
+                used |= sh.masks[id[j]];
+                sh.cnt[s][id[j]][c] = (uint16_t)(sh.cnt[s][id[j]][c] + 1);
+            }
         }
     }
     if (issue) {
@@ -428,13 +463,19 @@ __device__ __forceinline__ void order_channels_few(const uint8_t* __restrict__ p
         sh.start[P][tid] = (uint16_t)sum;   // filters placed (fewer than Cout only where ids lie outside the table)
     }
     __syncthreads();
-#pragma unroll 4
-    for (int co = co0; co < co1; ++co) {
-        const unsigned p = sh.ids[co * kIdPitch + c];
-        if (p < (unsigned)P) {
-            const unsigned n = sh.cnt[s][p][c];
-            sh.cnt[s][p][c] = (uint16_t)(n + 1);
-            sh.list[c][sh.start[p][c] + n] = (uint16_t)co;
+    for (int f0 = co0; f0 < co1; f0 += kWalk) {
+        unsigned id[kWalk], at[kWalk];
+#pragma unroll
+        for (int j = 0; j < kWalk; ++j) id[j] = sh.ids[min(f0 + j, co1 - 1) * kIdPitch + c];
+#pragma unroll
+        for (int j = 0; j < kWalk; ++j) at[j] = id[j] < (unsigned)P ? sh.start[id[j]][c] : 0u;
+#pragma unroll
+        for (int j = 0; j < kWalk; ++j) {
+            if (f0 + j < co1 && id[j] < (unsigned)P) {
+                const unsigned n = sh.cnt[s][id[j]][c];
+                sh.cnt[s][id[j]][c] = (uint16_t)(n + 1);
+                sh.list[c][at[j] + n] = (uint16_t)(f0 + j);
+            }
         }
     }
     const int off_n = P + 1;

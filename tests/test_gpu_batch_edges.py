@@ -26,6 +26,9 @@ CASES = [
     (64, 73, 1, 2, "conn4", "bf16", "f32"),        # 1x1 to fp32 (no tensor-path weights)
     (40, 68, 1, 4, "centre8", "f32", "f32"),       # 1x1, heads and remainders
     (20, 44, 3, 2, "conn4", "f16", "f32"),
+    (18, 77, 3, 4, "centre8", "f16", "bf16"),      # four copies of every filter, odd rows, segments of two filters
+    (40, 30, 3, 3, "conn4", "f32", "f16"),         # two copies, whole words; ids byte by byte
+    (257, 20, 3, 4, "centre8", "f32", "bf16"),     # words of four ids; segments of 32, the last of one filter
 ]
 PRESET = {"centre8": 2, "conn4": 1, "all": 0}
 
