@@ -301,6 +301,9 @@ typedef struct {
                                * y = round(act(conv + bias)) + residual, rounded once more: bit for bit (every
                                * activation) what the convolution followed by rtoss_add_act with act = none gives
                                * (the shortcut of a bottleneck block whose last convolution carries the activation). */
+    int x_channel_stride;     /* x may be a channel slice too (x_dev points at its first element): channels of the tensor
+                               * it lies in, 0 = Cin.  Other than 0 and Cin: tensor path only (NHWC, the pixel pitch a
+                               * multiple of 16 bytes); other calls return RTOSS_ERR_UNSUPPORTED. */
 } rtoss_conv_desc;
 
 /* y[n,co,oy,ox] = act( bias[co] + sum_ci sum_{t in mask(pid[co,ci])}
@@ -472,6 +475,16 @@ rtoss_status rtoss_maxpool2d(const void* x_dev, void* y_dev, int N, int C, int H
 /* Nearest-neighbour up-sampling by 2: y[n,c,oh,ow] = x[n,c,oh/2,ow/2], output 2H x 2W. */
 rtoss_status rtoss_upsample2x(const void* x_dev, void* y_dev, int N, int C, int H, int W, rtoss_layout layout,
                               rtoss_dtype dtype, int y_channel_offset, int y_channel_stride, void* cuda_stream);
+/* The same from a channel slice: x_dev points at its first element, x_channel_stride (0 = C) are the channels of the
+ * tensor it lies in. */
+rtoss_status rtoss_upsample2x_slice(const void* x_dev, int x_channel_stride, void* y_dev, int N, int C, int H, int W,
+                                    rtoss_layout layout, rtoss_dtype dtype, int y_channel_offset, int y_channel_stride,
+                                    void* cuda_stream);
+/* Three chained k x k max-pools of stride 1 (k odd, padding k/2) inside one tensor: channels [offset, offset + C) are
+ * the input, the pooled maps go to the three C-channel slices behind it (what rtoss_maxpool2d gives, three times).
+ * 16-bit NHWC, C, offset and stride multiples of 8, y_dev 16-byte aligned, H*W <= 6400; else RTOSS_ERR_UNSUPPORTED. */
+rtoss_status rtoss_pool_pyramid(void* y_dev, int N, int C, int H, int W, int k, rtoss_layout layout, rtoss_dtype dtype,
+                                int y_channel_offset, int y_channel_stride, void* cuda_stream);
 /* y = act(a + b) over n_elements contiguous elements (residual connections); the sum is formed in fp32 and
  * rounded once.  y may alias a or b. */
 rtoss_status rtoss_add_act(const void* a_dev, const void* b_dev, void* y_dev, int64_t n_elements, rtoss_dtype dtype,

@@ -28,6 +28,7 @@ SYMBOLS = [
     "rtoss_pattern_table_validate", "rtoss_group_layers", "rtoss_select_patterns", "rtoss_pack",
     "rtoss_packed_info_get", "rtoss_packed_export", "rtoss_packed_to_dense", "rtoss_packed_destroy",
     "rtoss_conv3x3_pattern", "rtoss_conv1x1_pattern", "rtoss_conv_pattern_host", "rtoss_device_status", "rtoss_prune_dense_static", "rtoss_maxpool2d", "rtoss_upsample2x", "rtoss_add_act", "rtoss_pattern_usage",
+    "rtoss_upsample2x_slice", "rtoss_pool_pyramid",
     "rtoss_pattern_rank", "rtoss_pattern_table_derive",
     "rtoss_batch_create", "rtoss_batch_select_pack", "rtoss_batch_destroy",
     "rtoss_select_patterns_shared", "rtoss_conv_group", "rtoss_set_wait_limit", "rtoss_inject_lost_copy",
@@ -62,7 +63,8 @@ class ConvDesc(ctypes.Structure):
     _fields_ = [("N", ctypes.c_int), ("H", ctypes.c_int), ("W", ctypes.c_int), ("stride", ctypes.c_int),
                 ("layout", ctypes.c_int), ("io_dtype", ctypes.c_int), ("act", ctypes.c_int),
                 ("bias_dev", ctypes.c_void_p), ("y_channel_offset", ctypes.c_int), ("y_channel_stride", ctypes.c_int),
-                ("path", ctypes.c_int), ("residual_dev", ctypes.c_void_p), ("residual_after_act", ctypes.c_int)]
+                ("path", ctypes.c_int), ("residual_dev", ctypes.c_void_p), ("residual_after_act", ctypes.c_int),
+                ("x_channel_stride", ctypes.c_int)]
 
 
 class FmaPlan(ctypes.Structure):
@@ -124,6 +126,8 @@ def _load():
     lib.rtoss_prune_dense_static.argtypes = [vp, ci, ci, ci, ci, vp, ci, ci, vp, vp]
     lib.rtoss_maxpool2d.argtypes = [vp, vp, ci, ci, ci, ci, ci, ci, ci, ci, ci, ci, ci, vp]
     lib.rtoss_upsample2x.argtypes = [vp, vp, ci, ci, ci, ci, ci, ci, ci, ci, vp]
+    lib.rtoss_upsample2x_slice.argtypes = [vp, ci, vp, ci, ci, ci, ci, ci, ci, ci, ci, vp]
+    lib.rtoss_pool_pyramid.argtypes = [vp, ci, ci, ci, ci, ci, ci, ci, ci, ci, vp]
     lib.rtoss_add_act.argtypes = [vp, vp, vp, ctypes.c_int64, ci, ci, vp]
     lib.rtoss_pattern_usage.argtypes = [vp, vp, ci, ctypes.c_int64, vp, ci, ci, vp, vp, vp]
     lib.rtoss_batch_create.argtypes = [vp, ctypes.POINTER(BatchItem), ci, ctypes.POINTER(vp)]
@@ -209,6 +213,20 @@ def rtoss_maxpool2d(x, y, N, C, H, W, k, stride, pad, layout=NCHW, y_channel_off
 def rtoss_upsample2x(x, y, N, C, H, W, layout=NCHW, y_channel_offset=0, y_channel_stride=0):
     _glue_check(lib.rtoss_upsample2x(x.data_ptr(), y.data_ptr(), N, C, H, W, layout, _torch_dtype_code(x), y_channel_offset,
                                      y_channel_stride, _stream()))
+    return y
+
+
+def rtoss_upsample2x_slice(x, x_channel_stride, y, N, C, H, W, layout=NCHW, y_channel_offset=0, y_channel_stride=0):
+    """x: a view whose first element is the slice's first, in a tensor of x_channel_stride channels."""
+    _glue_check(lib.rtoss_upsample2x_slice(x.data_ptr(), x_channel_stride, y.data_ptr(), N, C, H, W, layout, _torch_dtype_code(x),
+                                           y_channel_offset, y_channel_stride, _stream()))
+    return y
+
+
+def rtoss_pool_pyramid(y, N, C, H, W, k, layout=NHWC, y_channel_offset=0, y_channel_stride=0):
+    """Channels [offset, offset + C) of y, pooled once, twice and three times, into the three slices behind them."""
+    _glue_check(lib.rtoss_pool_pyramid(y.data_ptr(), N, C, H, W, k, layout, _torch_dtype_code(y), y_channel_offset,
+                                       y_channel_stride, _stream()))
     return y
 
 
@@ -374,11 +392,11 @@ class Context:
         return Batch(self, items)
 
     def _desc(self, x_shape_nchw, stride, layout, io_dtype, act, bias, y_off, y_stride, path=PATH_AUTO, residual=None,
-              residual_after_act=False):
+              residual_after_act=False, x_stride=0):
         N, _, H, W = x_shape_nchw
         return ConvDesc(int(N), int(H), int(W), int(stride), int(layout), int(io_dtype), int(act),
                         bias.data_ptr() if bias is not None else None, int(y_off), int(y_stride), int(path),
-                        residual.data_ptr() if residual is not None else None, 1 if residual_after_act else 0)
+                        residual.data_ptr() if residual is not None else None, 1 if residual_after_act else 0, int(x_stride))
 
     def rtoss_device_status(self):
         """Synchronise the device and return the code a timed-out device wait left (0 = none)."""
@@ -389,24 +407,26 @@ class Context:
         return code.value
 
     def rtoss_conv3x3_pattern(self, packed, x, y, N, H, W, stride=1, layout=NCHW, act=ACT_NONE, bias=None,
-                              y_channel_offset=0, y_channel_stride=0, path=PATH_AUTO, residual=None, residual_after_act=False):
+                              y_channel_offset=0, y_channel_stride=0, path=PATH_AUTO, residual=None, residual_after_act=False,
+                              x_channel_stride=0):
         d = self._desc((N, 0, H, W), stride, layout, _torch_dtype_code(x), act, bias, y_channel_offset, y_channel_stride,
-                       path, residual, residual_after_act)
+                       path, residual, residual_after_act, x_channel_stride)
         self._check(lib.rtoss_conv3x3_pattern(self.h, packed.h, x.data_ptr(), y.data_ptr(), ctypes.byref(d), _stream()))
         return y
 
     def rtoss_conv1x1_pattern(self, packed, x, y, N, H, W, stride=1, layout=NCHW, act=ACT_NONE, bias=None,
-                              y_channel_offset=0, y_channel_stride=0, path=PATH_AUTO, residual=None, residual_after_act=False):
+                              y_channel_offset=0, y_channel_stride=0, path=PATH_AUTO, residual=None, residual_after_act=False,
+                              x_channel_stride=0):
         d = self._desc((N, 0, H, W), stride, layout, _torch_dtype_code(x), act, bias, y_channel_offset, y_channel_stride,
-                       path, residual, residual_after_act)
+                       path, residual, residual_after_act, x_channel_stride)
         self._check(lib.rtoss_conv1x1_pattern(self.h, packed.h, x.data_ptr(), y.data_ptr(), ctypes.byref(d), _stream()))
         return y
 
     def conv_item(self, packed, x, y, N, H, W, stride=1, layout=NCHW, act=ACT_NONE, bias=None, y_channel_offset=0,
-                  y_channel_stride=0, path=PATH_AUTO, residual=None, residual_after_act=False):
+                  y_channel_stride=0, path=PATH_AUTO, residual=None, residual_after_act=False, x_channel_stride=0):
         """One entry for rtoss_conv_group (arguments as rtoss_conv3x3_pattern / rtoss_conv1x1_pattern)."""
         d = self._desc((N, 0, H, W), stride, layout, _torch_dtype_code(x), act, bias, y_channel_offset, y_channel_stride,
-                       path, residual, residual_after_act)
+                       path, residual, residual_after_act, x_channel_stride)
         return ConvItem(packed.h.value, x.data_ptr(), y.data_ptr(), d)
 
     def rtoss_conv_group(self, items):

@@ -418,15 +418,16 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     if (!enc) return (int)cudaErrorNotSupported;
     const CUtensorMapDataType dt = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : a.is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
     // activations: descriptor cached per (pointer, shape, box)
-    const int key[6] = {d->N, d->H, d->W, p->Cin, plan.rows_staged * 8 + S, plan.Wq * 4 + (int)p->dtype};   // (row size: a function of Cin and dtype)
+    const int key[7] = {d->N, d->H, d->W, p->Cin, plan.rows_staged * 8 + S, plan.Wq * 4 + (int)p->dtype, d->x_channel_stride};   // (row size: a function of Cin and dtype)
     rtoss_tmap_entry* ea = nullptr;
     for (rtoss_tmap_entry& e : ctx->tmap_cache)
         if (e.valid && e.base == x && memcmp(e.dims, key, sizeof(key)) == 0) ea = &e;
     if (!ea) {
         ea = &ctx->tmap_cache[ctx->tmap_next];
         ctx->tmap_next = (ctx->tmap_next + 1) % 32;
-        const cuuint64_t cp = (cuuint64_t)lay.cin_p;   // pixels are cin_p channels apart (the caller's tensor: cin_p == Cin)
-        cuuint64_t dims[4] = {cp, (cuuint64_t)d->W, (cuuint64_t)d->H, (cuuint64_t)d->N};
+        const cuuint64_t cin_p = (cuuint64_t)lay.cin_p;   // (the caller's tensor: cin_p == Cin)
+        const cuuint64_t cp = d->x_channel_stride ? (cuuint64_t)d->x_channel_stride : cin_p;   // pixels are cp channels apart
+        cuuint64_t dims[4] = {cin_p, (cuuint64_t)d->W, (cuuint64_t)d->H, (cuuint64_t)d->N};
         cuuint64_t strides[3] = {cp * esize, (cuuint64_t)d->W * cp * esize, (cuuint64_t)d->H * d->W * cp * esize};
         // with element strides the box is counted in traversed elements: S*n covers n fetched pixels
         cuuint32_t box[4] = {(cuuint32_t)a.cb_ch, (cuuint32_t)(plan.Wq * S), (cuuint32_t)(plan.rows_staged * S), 1};
@@ -540,6 +541,7 @@ bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const vo
     if (!p->wtc || !rows_fit_tma(p)) return false;
     if (d->layout != RTOSS_NHWC || (int)d->io_dtype != (int)p->dtype) return false;
     if ((reinterpret_cast<uintptr_t>(x) & 15) || (reinterpret_cast<uintptr_t>(y) & 15)) return false;
+    if (d->x_channel_stride % (p->dtype == RTOSS_F32 ? 4 : 8) != 0) return false;   // a slice: the pitch as TMA wants it
     if (!encode_fn()) return false;
     // a residual operand: 16-byte aligned, and not for the positions-as-M form (narrow 1x1 layers)
     if (d->residual_dev && (use_pxm(p) || (reinterpret_cast<uintptr_t>(d->residual_dev) & 15))) return false;
@@ -738,6 +740,7 @@ int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void
 // image once and has next to nothing to contract.
 static rtoss_conv_desc repacked_desc(const rtoss_packed* p, const rtoss_conv_desc* d) {
     rtoss_conv_desc dd = *d;
+    dd.x_channel_stride = 0;   // (of the copy)
     if (p->ksize == 1 && d->stride == 2) {
         dd.H = (d->H - 1) / 2 + 1;
         dd.W = (d->W - 1) / 2 + 1;
@@ -745,8 +748,9 @@ static rtoss_conv_desc repacked_desc(const rtoss_packed* p, const rtoss_conv_des
     }
     return dd;
 }
+static bool x_is_slice(const rtoss_packed* p, const rtoss_conv_desc* d) { return d->x_channel_stride && d->x_channel_stride != p->Cin; }
 bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) {
-    if (d->path != RTOSS_PATH_AUTO || d->residual_dev || !p->wtc || p->dtype == RTOSS_F32 || (int)d->io_dtype != (int)p->dtype) return false;
+    if (d->path != RTOSS_PATH_AUTO || d->residual_dev || x_is_slice(p, d) || !p->wtc || p->dtype == RTOSS_F32 || (int)d->io_dtype != (int)p->dtype) return false;
     if (d->layout == RTOSS_NHWC && rows_fit_tma(p)) return false;   // (native, or declined for another reason)
     if (p->ksize == 3 && p->Cin <= 4) return false;
     if (!encode_fn()) return false;

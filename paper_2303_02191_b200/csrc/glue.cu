@@ -16,6 +16,7 @@ struct GlueArgs {
     int k, stride, pad;
     int layout, act;
     int y_c_off, y_c_stride;
+    int x_c_stride;   // (up-sampling)
 };
 
 __device__ __forceinline__ size_t idx_of(int layout, int n, int c, int h, int w, int C, int H, int W) {
@@ -78,7 +79,7 @@ __global__ void upsample2x_kernel(const GlueArgs a) {
             n = (int)(r / a.Ho);
         }
         y[idx_of(a.layout, n, a.y_c_off + c, oh, ow, a.y_c_stride, a.Ho, a.Wo)] =
-            x[idx_of(a.layout, n, c, oh >> 1, ow >> 1, a.C, a.H, a.W)];
+            x[idx_of(a.layout, n, c, oh >> 1, ow >> 1, a.x_c_stride, a.H, a.W)];
     }
 }
 
@@ -140,6 +141,45 @@ __global__ void maxpool_vec8_kernel(const GlueArgs a) {
     }
 }
 
+// Three chained k x k maxima of stride 1 in one launch (the pools of an SPPF block and the concatenation of their results):
+// a block takes eight channels of one image into shared memory, and each pool is a maximum along the rows, then along the
+// columns (a maximum selects one of its inputs, in any order the same bits).  Pools and copies one by one were bound by 25
+// reads of every pixel and by their launches: 20 x 20 x 256, 16 images, seven launches 57 us.
+constexpr int kPyramidPx = 6400;   // two maps of 16 bytes a pixel in 200 KB
+
+template <typename T>
+__global__ void pool_pyramid_kernel(const GlueArgs a) {
+    rtoss_dev::pdl_enter();
+    extern __shared__ uint4 pyramid_smem[];
+    const int C8 = a.C >> 3, n = (int)(blockIdx.x / (unsigned)C8), c8 = (int)(blockIdx.x - (unsigned)n * (unsigned)C8);
+    const int px = a.H * a.W, reach = a.pad;
+    uint4* map = pyramid_smem;
+    uint4* rows = pyramid_smem + px;
+    T* y = reinterpret_cast<T*>(a.y) + (size_t)n * px * a.y_c_stride + a.y_c_off + c8 * 8;
+    for (int p = threadIdx.x; p < px; p += blockDim.x) map[p] = *reinterpret_cast<const uint4*>(y + (size_t)p * a.y_c_stride);
+    __syncthreads();
+    __align__(16) T init[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) init[j] = from_f32<T>(-INFINITY);   // padding never wins, and neither does a NaN
+    for (int pool = 1; pool <= 3; ++pool) {
+        for (int p = threadIdx.x; p < px; p += blockDim.x) {
+            const int w = p % a.W, first = p - min(w, reach), last = p + min(a.W - 1 - w, reach);
+            uint4 m = *reinterpret_cast<const uint4*>(init);
+            for (int q = first; q <= last; ++q) m = max8<T>(m, map[q]);
+            rows[p] = m;
+        }
+        __syncthreads();
+        for (int p = threadIdx.x; p < px; p += blockDim.x) {
+            const int h = p / a.W, first = p - min(h, reach) * a.W, last = p + min(a.H - 1 - h, reach) * a.W;
+            uint4 m = rows[first];
+            for (int q = first + a.W; q <= last; q += a.W) m = max8<T>(m, rows[q]);
+            map[p] = m;
+            *reinterpret_cast<uint4*>(y + (size_t)p * a.y_c_stride + (size_t)pool * a.C) = m;
+        }
+        __syncthreads();
+    }
+}
+
 template <typename T>
 __global__ void upsample2x_vec8_kernel(const GlueArgs a) {
     rtoss_dev::pdl_enter();
@@ -154,7 +194,7 @@ __global__ void upsample2x_vec8_kernel(const GlueArgs a) {
         const int oh = (int)(r % a.Ho);
         const int n = (int)(r / a.Ho);
         *reinterpret_cast<uint4*>(y + (((size_t)n * a.Ho + oh) * a.Wo + ow) * a.y_c_stride + a.y_c_off + c8 * 8) =
-            *reinterpret_cast<const uint4*>(x + (((size_t)n * a.H + (oh >> 1)) * a.W + (ow >> 1)) * a.C + c8 * 8);
+            *reinterpret_cast<const uint4*>(x + (((size_t)n * a.H + (oh >> 1)) * a.W + (ow >> 1)) * a.x_c_stride + c8 * 8);
     }
 }
 
@@ -203,7 +243,7 @@ rtoss_status rtoss_maxpool2d(const void* x_dev, void* y_dev, int N, int C, int H
     if (Ho < 1 || Wo < 1) return RTOSS_ERR_INVALID_ARG;
     const int cs = y_channel_stride ? y_channel_stride : C;
     if (y_channel_offset < 0 || cs < y_channel_offset + C) return RTOSS_ERR_INVALID_ARG;
-    GlueArgs a{x_dev, nullptr, y_dev, N, C, H, W, Ho, Wo, k, stride, pad, (int)layout, 0, y_channel_offset, cs};
+    GlueArgs a{x_dev, nullptr, y_dev, N, C, H, W, Ho, Wo, k, stride, pad, (int)layout, 0, y_channel_offset, cs, C};
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (vec8_ok(a, (int)dtype)) {
         const int g8 = grid_for((size_t)N * (C / 8) * Ho * Wo);
@@ -220,14 +260,22 @@ rtoss_status rtoss_maxpool2d(const void* x_dev, void* y_dev, int N, int C, int H
 
 rtoss_status rtoss_upsample2x(const void* x_dev, void* y_dev, int N, int C, int H, int W, rtoss_layout layout,
                               rtoss_dtype dtype, int y_channel_offset, int y_channel_stride, void* cuda_stream) {
+    return rtoss_upsample2x_slice(x_dev, 0, y_dev, N, C, H, W, layout, dtype, y_channel_offset, y_channel_stride, cuda_stream);
+}
+
+rtoss_status rtoss_upsample2x_slice(const void* x_dev, int x_channel_stride, void* y_dev, int N, int C, int H, int W,
+                                    rtoss_layout layout, rtoss_dtype dtype, int y_channel_offset, int y_channel_stride,
+                                    void* cuda_stream) {
     if (!x_dev || !y_dev || N < 1 || C < 1 || H < 1 || W < 1 || !ok_dtype(dtype) ||
         (layout != RTOSS_NCHW && layout != RTOSS_NHWC))
         return RTOSS_ERR_INVALID_ARG;
     const int cs = y_channel_stride ? y_channel_stride : C;
     if (y_channel_offset < 0 || cs < y_channel_offset + C) return RTOSS_ERR_INVALID_ARG;
-    GlueArgs a{x_dev, nullptr, y_dev, N, C, H, W, 2 * H, 2 * W, 0, 0, 0, (int)layout, 0, y_channel_offset, cs};
+    const int xs = x_channel_stride ? x_channel_stride : C;
+    if (xs < C) return RTOSS_ERR_INVALID_ARG;
+    GlueArgs a{x_dev, nullptr, y_dev, N, C, H, W, 2 * H, 2 * W, 0, 0, 0, (int)layout, 0, y_channel_offset, cs, xs};
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    if (vec8_ok(a, (int)dtype)) {
+    if (vec8_ok(a, (int)dtype) && xs % 8 == 0) {
         const int g8 = grid_for((size_t)N * (C / 8) * 4 * H * W);
         if (dtype == RTOSS_BF16) rtoss_dev::launch_pdl(upsample2x_vec8_kernel<__nv_bfloat16>, g8, 256, 0, s, a);
         else rtoss_dev::launch_pdl(upsample2x_vec8_kernel<__half>, g8, 256, 0, s, a);
@@ -237,6 +285,22 @@ rtoss_status rtoss_upsample2x(const void* x_dev, void* y_dev, int N, int C, int 
     if (dtype == RTOSS_F32) rtoss_dev::launch_pdl(upsample2x_kernel<float>, grid, 256, 0, s, a);
     else if (dtype == RTOSS_BF16) rtoss_dev::launch_pdl(upsample2x_kernel<__nv_bfloat16>, grid, 256, 0, s, a);
     else rtoss_dev::launch_pdl(upsample2x_kernel<__half>, grid, 256, 0, s, a);
+    return cudaGetLastError() == cudaSuccess ? RTOSS_OK : RTOSS_ERR_CUDA;
+}
+
+rtoss_status rtoss_pool_pyramid(void* y_dev, int N, int C, int H, int W, int k, rtoss_layout layout, rtoss_dtype dtype,
+                                int y_channel_offset, int y_channel_stride, void* cuda_stream) {
+    if (!y_dev || N < 1 || C < 1 || H < 1 || W < 1 || k < 1 || k % 2 == 0 || !ok_dtype(dtype) || (layout != RTOSS_NCHW && layout != RTOSS_NHWC) ||
+        y_channel_offset < 0 || y_channel_stride < y_channel_offset + 4 * C)
+        return RTOSS_ERR_INVALID_ARG;
+    GlueArgs a{y_dev, nullptr, y_dev, N, C, H, W, H, W, k, 1, k / 2, (int)layout, 0, y_channel_offset, y_channel_stride, y_channel_stride};
+    const long long blocks = (long long)N * (C / 8);
+    const size_t smem = (size_t)H * W * 32;
+    if (!vec8_ok(a, (int)dtype) || (long long)H * W > kPyramidPx || blocks > 0x7FFFFFFFLL) return RTOSS_ERR_UNSUPPORTED;
+    auto kernel = dtype == RTOSS_BF16 ? pool_pyramid_kernel<__nv_bfloat16> : pool_pyramid_kernel<__half>;
+    if (smem > 48 * 1024 && cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPyramidPx * 32) != cudaSuccess) return RTOSS_ERR_CUDA;
+    const int threads = H * W >= 512 ? 512 : (H * W + 31) / 32 * 32;
+    rtoss_dev::launch_pdl(kernel, (unsigned)blocks, (unsigned)threads, smem, (cudaStream_t)cuda_stream, a);
     return cudaGetLastError() == cudaSuccess ? RTOSS_OK : RTOSS_ERR_CUDA;
 }
 

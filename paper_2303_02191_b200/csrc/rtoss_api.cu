@@ -71,6 +71,10 @@ rtoss_status check_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
         set_err(ctx, "conv", "output channel slice does not fit y_channel_stride");
         return RTOSS_ERR_INVALID_ARG;
     }
+    if (d->x_channel_stride != 0 && d->x_channel_stride < p->Cin) {
+        set_err(ctx, "conv", "x_channel_stride below Cin");
+        return RTOSS_ERR_INVALID_ARG;
+    }
     if ((int64_t)d->H * d->W > (int64_t)1 << 30) {
         set_err(ctx, "conv", "H*W above 2^30");
         return RTOSS_ERR_UNSUPPORTED;
@@ -90,6 +94,11 @@ int dispatch_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
     const bool tc_ok = d->path != RTOSS_PATH_FMA && rtoss_tc_eligible(p, d, x, y);
     if (d->residual_dev && !tc_ok) {
         set_err(ctx, "conv", "a residual operand is only taken by the tensor path (see rtoss.h)");
+        *st = RTOSS_ERR_UNSUPPORTED;
+        return 0;
+    }
+    if (d->x_channel_stride && d->x_channel_stride != p->Cin && !tc_ok) {
+        set_err(ctx, "conv", "an input slice is only taken by the tensor path (see rtoss.h)");
         *st = RTOSS_ERR_UNSUPPORTED;
         return 0;
     }
@@ -557,7 +566,8 @@ void spans_of(const rtoss_conv_item& it, Span* x, Span* y, Span* r) {
     const size_t Ho = (size_t)((d.H - 1) / S + 1), Wo = (size_t)((d.W - 1) / S + 1);
     const size_t pitch = d.y_channel_stride ? (size_t)d.y_channel_stride : (size_t)p->Cout;
     x->lo = reinterpret_cast<uintptr_t>(it.x_dev);
-    x->hi = x->lo + (size_t)d.N * d.H * d.W * p->Cin * es;
+    const size_t x_pitch = d.x_channel_stride ? (size_t)d.x_channel_stride : (size_t)p->Cin;
+    x->hi = x->lo + ((size_t)d.N * d.H * d.W * x_pitch - (x_pitch - (size_t)p->Cin)) * es;
     // (a call that writes a channel slice is given the buffer's base: the span is the whole buffer)
     y->lo = reinterpret_cast<uintptr_t>(it.y_dev);
     y->hi = y->lo + (size_t)d.N * Ho * Wo * pitch * es;
@@ -739,6 +749,10 @@ rtoss_status rtoss_conv_pattern_host(rtoss_ctx* ctx, const rtoss_packed* p, cons
     if (!ctx || !p) return RTOSS_ERR_INVALID_ARG;
     rtoss_status st = check_conv(ctx, p, x_host, y_host, desc, p->ksize, false);
     if (st != RTOSS_OK) return st;
+    if (desc->x_channel_stride && desc->x_channel_stride != p->Cin) {
+        set_err(ctx, "conv", "the host-buffer entry point takes no input slice");
+        return RTOSS_ERR_UNSUPPORTED;
+    }
     if (desc->residual_dev) {
         set_err(ctx, "conv", "the host-buffer entry point takes no residual operand");
         return RTOSS_ERR_UNSUPPORTED;

@@ -10,7 +10,7 @@
 // Host-side cache of encoded TMA descriptors (encoding costs microseconds per call).
 struct rtoss_tmap_entry {
     const void* base;
-    int dims[6];  // what the descriptor was encoded for
+    int dims[7];  // what the descriptor was encoded for
     int valid;
     alignas(64) unsigned char map[128];
 };

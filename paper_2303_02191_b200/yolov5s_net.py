@@ -118,6 +118,79 @@ def fuse_shortcuts(ops):
     return out
 
 
+def fuse_pools(ops, bufs):
+    """Three chained 5x5 pools whose input and results are copied into neighbouring slices of one buffer, and read by
+    nothing else, become ('pyramid', input, buffer, offset): the pools run inside the buffer (the copy of the input stays)."""
+    reads = {}
+    for op in ops:
+        for s_ in _operands(op):
+            reads.setdefault(s_, []).append(op)
+    out = list(ops)
+    for first in [op for op in ops if op[0] == "copy"]:
+        src, cat, off = first[1:]
+        C, chain, cur = bufs[src][0], [], src
+        for i in range(1, 4):
+            pool = [op for op in reads[cur] if op[0] == "pool5" and op[3] == 0 and bufs[op[2]] == bufs[src]]
+            if len(pool) != 1 or sorted(map(repr, reads[cur])) != sorted(map(repr, [pool[0], ("copy", cur, cat, off + (i - 1) * C)])):
+                break
+            cur = pool[0][2]
+            chain += [pool[0], ("copy", cur, cat, off + i * C)]
+        if len(chain) == 6 and reads[cur] == [chain[-1]] and all(op in out for op in chain):
+            at = out.index(chain[-1])
+            out[at] = ("pyramid", src, cat, off)
+            for op in chain[:-1]:
+                out.remove(op)
+    return out
+
+
+def _operands(op):
+    return (op[2],) if op[0] == "conv" else (op[2], op[4]) if op[0] == "convres" else (op[1], op[2]) if op[0] == "add" else (op[1],)
+
+
+def _target(op):
+    return op[{"conv": 3, "convres": 5, "add": 3, "pool5": 2, "up": 2, "copy": 2, "pyramid": 2}[op[0]]]
+
+
+def share_slices(ops, bufs):
+    """Concatenation without copies: a buffer that is copied into a slice of another one and written by a convolution is
+    laid out as that slice from the start, when all its readers can read a slice (convolutions, up-sampling).  The operand
+    of a shortcut lies where the result does, so the buffers along a chain of bottlenecks share the slice: each is dead
+    when the next is written (nothing reads it but the convolution whose result the next one is computed from, and the
+    shortcut itself, element by element).  Returns (ops without those copies, {buffer: (buffer it lies in, offset)})."""
+    home = {}
+    writers, readers = {}, {}
+    for op in ops:
+        writers.setdefault(_target(op), []).append(op)
+        for s_ in _operands(op):
+            readers.setdefault(s_, []).append(op)
+
+    def chain_of(name, seen):
+        """The buffers that have to share name's place, or None."""
+        w = writers.get(name, [])
+        if len(w) != 1 or w[0][0] not in ("conv", "convres") or name in home or name in seen or (w[0][0] == "conv" and w[0][4] != 0):
+            return None
+        if w[0][0] == "conv":
+            return [name]
+        _, _, src, _, other, _ = w[0]
+        if bufs[other] != bufs[name] or any(op != w[0] and not (op[0] == "conv" and _target(op) == src) for op in readers[other]):
+            return None
+        rest = chain_of(other, seen + [name])
+        return None if rest is None else [name] + rest
+
+    out = []
+    for op in ops:
+        if op[0] == "copy":
+            _, src, cat, off = op
+            ok = all(r == op or (r[0] == "conv") or (r[0] == "up") or (r[0] == "pyramid" and r[2:] == (cat, off)) for r in readers[src])
+            group = chain_of(src, []) if ok and cat not in home and src not in OUTPUTS else None
+            if group:
+                for name in group:
+                    home[name] = (cat, off)
+                continue
+        out.append(op)
+    return out, home
+
+
 class GpuNet:
     """The program on the GPU through the C-ABI library: NHWC, bf16 (or fp16), k-entry patterns."""
 
@@ -128,10 +201,13 @@ class GpuNet:
         self.ops, self.bufs, self.layers = program(H0, W0)
         if fuse_residual:
             self.ops = fuse_shortcuts(self.ops)
+        self.copying, self.home, self.inside = self.ops, {}, {}   # (the program with its copies, should the library decline a slice)
+        self._share()
         self.unfused = set()   # layers whose fused call the library declined: convolution and add run separately
         self.rounds, self.probed, self.steps = None, False, None
         tdt = {"bf16": torch.bfloat16, "f16": torch.float16}[dtype]
-        self.t = {n: torch.zeros((N, H, W, C), dtype=tdt, device="cuda") for n, (C, H, W) in self.bufs.items()}
+        self.tdt = tdt
+        self._allocate()
         masks = rt.rtoss_pattern_preset(k, rt.PRESET_CENTRE8 if k == 4 else rt.PRESET_CONN4)
         self.packed, self.bias = [], []
         for i, L in enumerate(self.layers):
@@ -141,20 +217,56 @@ class GpuNet:
             self.bias.append(torch.from_numpy(synth.bias(seed, 2000 + i, L["cout"])).cuda())
         torch.cuda.synchronize()
 
+    def _share(self):
+        ops = fuse_pools(self.copying, self.bufs)
+        shared, home = share_slices(ops, self.bufs)
+        kept = {op[1] for op in shared if op[0] == "copy"}
+        pyramids = [op for op in ops if op[0] == "pyramid"]
+        if any(op[1] in kept or self.bufs[op[1]][1] * self.bufs[op[1]][2] > 6400 for op in pyramids):
+            shared, home = share_slices(self.copying, self.bufs)   # (the pools one by one, see rtoss_pool_pyramid)
+        self.ops, self.home = shared, home
+        self.inside = {}
+        for op in self.copying:
+            if op[0] == "copy" and op[1] in home:
+                self.inside.setdefault(op[2], []).append(op[1])
+
+    def _allocate(self):
+        torch, N = self.torch, self.N
+        old = getattr(self, "t", None)
+        self.t = {n: torch.zeros((N, H, W, C), dtype=self.tdt, device="cuda") for n, (C, H, W) in self.bufs.items() if n not in self.home}
+        if old:
+            for n in ("in",) + OUTPUTS:
+                self.t[n] = old[n]     # what the caller holds
+        for n, (cat, off) in self.home.items():
+            self.t[n] = self.t[cat][..., off:off + self.bufs[n][0]]
+
+    def _copying(self):
+        """The library declined a slice: back to dense buffers and copies."""
+        self.ops, self.home, self.inside = self.copying, {}, {}
+        self.rounds = self.steps = None
+        self._allocate()
+
     def set_input(self, x_nchw):
         self.t["in"].copy_(self.torch.from_numpy(x_nchw).permute(0, 2, 3, 1).to(self.t["in"].dtype))
 
     def _reads(self, op):
-        if op[0] == "conv":
-            return (op[2],)
-        if op[0] == "convres":
-            return (op[2], op[4])
-        if op[0] == "add":
-            return (op[1], op[2])
-        return (op[1],)
+        """A reader of a whole concatenation also reads the buffers that lie in it."""
+        names = _operands(op)
+        return names + tuple(n for s_ in names for n in self.inside.get(s_, ()))
 
     def _write(self, op):
-        return op[{"conv": 3, "convres": 5, "add": 3, "pool5": 2, "up": 2, "copy": 2}[op[0]]]
+        return _target(op)
+
+    def _x(self, name):
+        """(tensor, channels of the tensor it is a slice of; 0: dense)"""
+        return self.t[name], self.bufs[self.home[name][0]][0] if name in self.home else 0
+
+    def _y(self, name, off=0):
+        """(tensor, channel offset, channels of the tensor)"""
+        if name in self.home:
+            cat, at = self.home[name]
+            return self.t[cat], at + off, self.bufs[cat][0]
+        return self.t[name], off, self.bufs[name][0]
 
     def run(self, grouped=True, chained=False):
         """One pass.  grouped: operations are issued round by round (schedule.levels: a buffer is ready when every slice
@@ -162,9 +274,16 @@ class GpuNet:
         operation in program order."""
         self.launches = 0      # kernel launches of this pass
         if not grouped or not self.probed:
-            for op in self.ops:
-                self._run_op(op)
-            self.probed = True     # the first pass finds out which fused shortcut calls the library declines
+            try:
+                for op in self.ops:
+                    self._run_op(op)
+            except self.rt.RtossError as err:
+                if err.status != self.rt.ERR_UNSUPPORTED or not self.home:
+                    raise
+                self._copying()
+                for op in self.ops:
+                    self._run_op(op)
+            self.probed = True     # the first pass finds out which fused shortcut calls and slices the library declines
             return
         if self.rounds is None:
             # as soon as possible: the two 1x1 branches that open a C3 block then share a round (and a launch)
@@ -199,11 +318,15 @@ class GpuNet:
         L = self.layers[i]
         if op[0] == "conv":
             _, _, src, dst, off = op
-            return self.ctx.conv_item(self.packed[i], t[src], t[dst], N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i],
-                                      off, self.bufs[dst][0])
+            x, xs = self._x(src)
+            y, off, ys = self._y(dst, off)
+            return self.ctx.conv_item(self.packed[i], x, y, N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i],
+                                      off, ys, x_channel_stride=xs)
         _, _, src, tmp, other, dst = op
-        return self.ctx.conv_item(self.packed[i], t[src], t[dst], N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i],
-                                  residual=t[other], residual_after_act=True)
+        x, xs = self._x(src)
+        y, off, ys = self._y(dst)
+        return self.ctx.conv_item(self.packed[i], x, y, N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i], off, ys,
+                                  residual=self._y(other)[0], residual_after_act=True, x_channel_stride=xs)
 
     def _run_op(self, op):
         rt, N, t = self.rt, self.N, self.t
@@ -212,19 +335,22 @@ class GpuNet:
             _, i, src, dst, off = op
             L = self.layers[i]
             fn = self.ctx.rtoss_conv3x3_pattern if L["ksize"] == 3 else self.ctx.rtoss_conv1x1_pattern
-            fn(self.packed[i], t[src], t[dst], N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i],
-               off, self.bufs[dst][0])
+            x, xs = self._x(src)
+            y, off, ys = self._y(dst, off)
+            fn(self.packed[i], x, y, N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i], off, ys, x_channel_stride=xs)
         elif op[0] == "convres":   # second convolution of a bottleneck + its shortcut in one call
             _, i, src, tmp, other, dst = op
             L = self.layers[i]
             fn = self.ctx.rtoss_conv3x3_pattern if L["ksize"] == 3 else self.ctx.rtoss_conv1x1_pattern
             if i not in self.unfused:
                 try:
-                    fn(self.packed[i], t[src], t[dst], N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i],
-                       residual=t[other], residual_after_act=True)
+                    x, xs = self._x(src)
+                    y, off, ys = self._y(dst)
+                    fn(self.packed[i], x, y, N, L["H"], L["W"], L["stride"], rt.NHWC, rt.ACT_SILU, self.bias[i], off, ys,
+                       residual=self._y(other)[0], residual_after_act=True, x_channel_stride=xs)
                     return
                 except rt.RtossError as err:
-                    if err.status != rt.ERR_UNSUPPORTED:
+                    if err.status != rt.ERR_UNSUPPORTED or self.home:
                         raise
                     self.unfused.add(i)
                     self.rounds = self.steps = None
@@ -238,7 +364,11 @@ class GpuNet:
             rt.rtoss_maxpool2d(t[op[1]], t[op[2]], N, C, H, W, 5, 1, 2, rt.NHWC, op[3], self.bufs[op[2]][0])
         elif op[0] == "up":
             C, H, W = self.bufs[op[1]]
-            rt.rtoss_upsample2x(t[op[1]], t[op[2]], N, C, H, W, rt.NHWC, op[3], self.bufs[op[2]][0])
+            x, xs = self._x(op[1])
+            rt.rtoss_upsample2x_slice(x, xs, t[op[2]], N, C, H, W, rt.NHWC, op[3], self.bufs[op[2]][0])
+        elif op[0] == "pyramid":
+            C, H, W = self.bufs[op[1]]
+            rt.rtoss_pool_pyramid(t[op[2]], N, C, H, W, 5, rt.NHWC, op[3], self.bufs[op[2]][0])
         elif op[0] == "copy":
             C, H, W = self.bufs[op[1]]
             rt.rtoss_maxpool2d(t[op[1]], t[op[2]], N, C, H, W, 1, 1, 0, rt.NHWC, op[3], self.bufs[op[2]][0])
