@@ -108,7 +108,9 @@ int dispatch_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
         return 0;
     }
     if (tc_ok) return rtoss_launch_conv_tc(ctx, p, x, y, d, stream);
-    if (rtoss_tc_repack_eligible(p, d)) {
+    const bool repack = rtoss_tc_repack_eligible(p, d);
+    if (rtoss_few_eligible(p, d, x, repack)) return rtoss_launch_conv_few(p, x, y, d, stream);
+    if (repack) {
         const int e = rtoss_launch_conv_tc_repacked(ctx, p, x, y, d, stream);
         if (e >= 0) return e;   // (-1: no memory for the copy of x; the FMA path needs none)
     }
@@ -134,12 +136,16 @@ void* rtoss_ctx_pool(const rtoss_ctx* ctx) {
         props.location.id = ctx->device;
         cudaMemPool_t pool = nullptr;
         unsigned long long keep = kPoolKeep;
+        // the context's first such call may lie inside a stream capture, which making a pool is no part of
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        cudaThreadExchangeStreamCaptureMode(&mode);
         if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
             cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
             ctx->pool = pool;
         } else {
             cudaGetLastError();   // (without a pool the calls that want one run on the FMA path)
         }
+        cudaThreadExchangeStreamCaptureMode(&mode);
     }
     return ctx->pool;
 }

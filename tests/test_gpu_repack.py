@@ -107,3 +107,25 @@ def test_repacked_calls_on_two_streams_and_in_a_graph():
     assert c.rtoss_device_status() == 0
     for j in jobs:
         j[0].close()
+
+
+def test_first_repacked_call_of_a_context_inside_a_capture():
+    """The pool of the channels-last copies is made on first use, which a stream capture does not forbid."""
+    masks, k = _table(4), 4
+    w = synth.kaiming_weights(63, 0, 64, 96, 3)
+    xd = gu.to_dev(synth.activations(63, 0, 2, 96, 24, 24), "bf16")
+    y, want = (torch.zeros((2, 64, 24, 24), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    c = rt.Context(0)
+    wd = torch.from_numpy(w).cuda()
+    packed = c.rtoss_pack(wd, 3, masks, k, c.rtoss_select_patterns(wd, 3, masks, k), rt.BF16)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        c.rtoss_conv3x3_pattern(packed, xd, y, 2, 24, 24, 1, rt.NCHW, rt.ACT_SILU, None)
+    g.replay()
+    c.rtoss_conv3x3_pattern(packed, xd, want, 2, 24, 24, 1, rt.NCHW, rt.ACT_SILU, None)
+    torch.cuda.synchronize()
+    assert want.abs().max() > 0 and torch.equal(y, want)
+    packed.close()
+    del g
+    c.close()
