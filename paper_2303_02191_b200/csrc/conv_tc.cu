@@ -755,10 +755,6 @@ bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) {
     if (p->ksize == 3 && p->Cin <= 4) return false;
     if (!encode_fn()) return false;
     const rtoss_conv_desc dd = repacked_desc(p, d);
-    // Small 3x3 layers of few channels: two launches cost more than the FMA kernel's few rounds (16->32 @42x10, batch 8:
-    // 27.9 us here, 10.3 us there; 16->30 @23x20: 21 / 10; from about 2^17 outputs on the FMA kernel needs more than one
-    // wave: 16->32 @100x101, batch 2: 19 us here, 46 us there).
-    if (p->ksize == 3 && p->Cin <= 16 && (long long)dd.N * ((dd.H - 1) / dd.stride + 1) * ((dd.W - 1) / dd.stride + 1) * p->Cout <= (1 << 17)) return false;
     return plan_exists(p, &dd);
 }
 // Returns a cudaError_t, or -1 when there was no memory for the channels-last copy (nothing was launched).  The copy

@@ -125,6 +125,9 @@ int rtoss_launch_to_dense(const rtoss_packed* p, void* w_out, void* stream);
 int rtoss_launch_pid_histogram(const uint8_t* pid, int64_t n, int P, unsigned long long* counts, void* stream);
 int rtoss_launch_conv3x3(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                          const rtoss_conv_desc* d, void* stream);
+// (repack: the call may run on the tensor path behind a layout pass instead)
+bool rtoss_few_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, bool repack);
+int rtoss_launch_conv_few(const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, void* stream);
 int rtoss_launch_conv1x1(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                          const rtoss_conv_desc* d, void* stream);
 // Number of issue words of a layer (tiles of 128 filter rows x blocks of 64 channels).
