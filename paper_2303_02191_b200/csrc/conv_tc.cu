@@ -152,11 +152,14 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
     const int cap = 227 * 1024 - 64;
     double best = 0;
     bool found = false;
-    for (int nseg = 1; nseg <= 16; ++nseg) {
-        const int tw = (Wo + nseg - 1) / nseg;
+    // One row of pixels (1x1, see row_form): tiles of any multiple of 16 of them.
+    const bool one_row = ksize == 1 && S == 1 && k.N == 1 && Ho == 1;
+    for (int seg = 1; seg <= 16; ++seg) {
+        const int tw = one_row ? (16 * seg < Wo ? 16 * seg : Wo) : (Wo + seg - 1) / seg, nseg = one_row ? (Wo + tw - 1) / tw : seg;
         const int wq = tw + halo;
         if (wq > max_pitch || wq > 256) continue;
-        if (nseg > 1 && (tw < 4 || (Wo + nseg - 2) / (nseg - 1) == tw) && found) continue;   // (the same columns as with fewer segments)
+        if (one_row && 16 * (seg - 1) >= Wo) break;
+        if (!one_row && nseg > 1 && (tw < 4 || (Wo + nseg - 2) / (nseg - 1) == tw) && found) continue;   // (the same columns as with fewer segments)
         for (int th = 1; th <= Ho; ++th) {
             const int rows_staged = th + halo;
             if (th * wq > 256 || rows_staged * S > 256) break;
@@ -294,9 +297,21 @@ PlanKey plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, int sms, int d
     return k;
 }
 
+// A 1x1 convolution of stride 1 over channels-last images is one over a single row of N*H*W pixels, which can be cut into
+// tiles of exactly as many positions as a tile takes: rows of 68, 80 or 272 pixels fill 204, 240 and 136 of 256 (bf16
+// 256->1024 @50x68 x4 11.3 us instead of 11.7, the 38 such layers of the large detector at batch 4 11 us less; no layer slower).
+rtoss_conv_desc row_form(const rtoss_packed* p, const rtoss_conv_desc* d) {
+    rtoss_conv_desc dd = *d;
+    if (p->ksize == 1 && d->stride == 1 && d->layout == RTOSS_NHWC && (long long)d->N * d->H * d->W <= 1ll << 30) {
+        dd.W = d->N * d->H * d->W;
+        dd.N = dd.H = 1;
+    }
+    return dd;
+}
+
 // Can the layer be cut at all?  Its smallest tile is one row of the narrowest segment, with a weight stage per tap.
 bool plan_exists(const rtoss_packed* p, const rtoss_conv_desc* d) {
-    const int S = d->stride, Wo = (d->W - 1) / S + 1;
+    const int S = d->stride, Wo = p->ksize == 1 && S == 1 && row_form(p, d).H == 1 ? 16 : (d->W - 1) / S + 1;
     const bool f32 = p->dtype == RTOSS_F32, k3 = p->ksize == 3;
     const int wq = (Wo + 15) / 16 + (k3 ? (S == 1 ? 2 : 1) : 0);
     if (wq > (S == 1 ? 256 : 128)) return false;
@@ -564,7 +579,8 @@ static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const
         long tiles = 0;
         bool ok = true;
         for (int i = 0; i < n && ok; ++i) {
-            PlanKey key = plan_key(ps[i], ds[i], sms, ctx_dev(ctx));
+            const rtoss_conv_desc dd = row_form(ps[i], ds[i]);
+            PlanKey key = plan_key(ps[i], &dd, sms, ctx_dev(ctx));
             key.shared = n > 1 ? 1 : 2;
             key.max_px = px;
             TcPlan plan;
@@ -594,7 +610,8 @@ double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* con
 // channel blocks, and how many tiles it has.  (Shared launches never split.)
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
-    if (!plan_tc(plan_key(p, d, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    const rtoss_conv_desc dd = row_form(p, d);
+    if (!plan_tc(plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
     *us = plan.us;
     *ks = plan.KS;
     *tiles = plan.tiles;
@@ -667,8 +684,10 @@ static SharedKernel shared_kernel(const rtoss_ctx* ctx, bool f32, const TcLaunch
 }
 
 // One convolution, channels last in x.  repacked: x is the copy of rtoss_launch_conv_tc_repacked.
-static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, bool repacked,
+static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* call, bool repacked,
                          void* stream) {
+    const rtoss_conv_desc row = row_form(p, call);
+    const rtoss_conv_desc* d = &row;
     const int sms = ctx_sms(ctx);
     int e = ensure_device(ctx);
     if (e) return e;
@@ -859,7 +878,7 @@ int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* 
                 a_max = 0;
                 for (int q = 0; q < m; ++q) {
                     const int i = set[q];
-                    rtoss_conv_desc dd = *ds[i];
+                    rtoss_conv_desc dd = row_form(ps[i], ds[i]);
                     static const int dummy = 0;
                     dd.residual_dev = under ? &dummy : nullptr;   // (only the plan's memory budget looks at it here)
                     PlanKey key = plan_key(ps[i], &dd, sms, ctx_dev(ctx));
