@@ -651,8 +651,9 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
 
 // The kernel a launch of one convolution runs: a form where there is one for it, else the general one.
 static SingleKernel single_kernel(const rtoss_ctx* ctx, bool f32, bool repacked, const TcArgs& a) {
-    if (!f32 && (a.taps == 1 || a.G == 3) && (a.pxm || a.nchw || (a.y_c_stride % 8 == 0 && a.y_c_off % 8 == 0 && a.Cout % 8 == 0))) {
-        const int form = form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
+    if (!f32 && (a.taps == 1 || a.G == 3)) {
+        const bool pieces = a.pxm || a.nchw || (a.y_c_stride % 8 == 0 && a.y_c_off % 8 == 0 && a.Cout % 8 == 0);
+        const int form = (pieces ? 0 : kFormElem) | form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
         if (void* k = form_kernel(ctx, a.is_bf16, false, form)) return reinterpret_cast<SingleKernel>(k);
     }
     if (f32) return conv_tc_kernel<float, TcLaunch1>;

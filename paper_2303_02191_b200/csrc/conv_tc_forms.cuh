@@ -17,6 +17,8 @@ constexpr int kKind1 = 1, kKindPxm = 2, kKind3 = 3;
 template <int K, int A> using Plain = std::integer_sequence<int, form_of(K, A, false, 0, false), form_of(K, A, true, 0, false)>;
 template <int K, int A> using Nchw = std::integer_sequence<int, form_of(K, A, false, 0, true), form_of(K, A, true, 0, true)>;
 template <int K, int A, int R> using Resid = std::integer_sequence<int, form_of(K, A, false, R, false), form_of(K, A, true, R, false)>;
+template <int K, bool S> using Elem = std::integer_sequence<int, form_of(K, kNone, S, 0, false) | kFormElem, form_of(K, kRelu, S, 0, false) | kFormElem,
+                                                            form_of(K, kSilu, S, 0, false) | kFormElem, form_of(K, kSiluX, S, 0, false) | kFormElem>;
 using Pxm = std::integer_sequence<int, form_of(kKindPxm, kNone, false, 0, false), form_of(kKindPxm, kRelu, false, 0, false),
                                   form_of(kKindPxm, kSilu, false, 0, false), form_of(kKindPxm, kSiluX, false, 0, false),
                                   form_of(kKindPxm, kNone, false, 0, true), form_of(kKindPxm, kRelu, false, 0, true),
@@ -59,6 +61,10 @@ FormTable make_forms() {
     add_forms<T, TcLaunch1>(t.one, t.n_one, Resid<kKind1, kRelu, 1>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Resid<kKind3, kSilu, 2>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Pxm());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind1, false>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind1, true>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind3, false>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind3, true>());
     // several convolutions
     add_forms<T, TcLaunchN>(t.shared, t.n_shared, std::integer_sequence<int, form_of(kKind1, -1, false, 0, false), form_of(kKind1, kNone, false, 0, false),
                                                                        form_of(kKind1, kRelu, false, 0, false), form_of(kKind1, kSilu, false, 0, false),

@@ -901,8 +901,9 @@ __device__ __forceinline__ bool wait_deps(const G& g, unsigned dep_mask) {
 //   bit 5     cut along K
 //   bits 6-7  residual operand: 0 none, 1 in front of the activation, 2 behind it, 3 from the arguments
 //   bit 8     the output is NCHW
-// Forms are for 16-bit data; channels-last outputs leave in whole 16-byte pieces (filters in multiples of eight, aligned
-// channel slices).
+//   bit 9     element stores (no residual): filter counts of no multiple of eight, unaligned channel slices
+// Forms are for 16-bit data; but for bit 9, channels-last outputs leave in whole 16-byte pieces.
+constexpr int kFormElem = 512;
 constexpr int form_of(int kind, int act, bool split, int res, bool nchw) { return kind | (act + 1) << 2 | (split ? 32 : 0) | res << 6 | (nchw ? 256 : 0); }
 
 // kRep: the launch follows a layout pass (rtoss_launch_conv_tc_repacked): 16-bit outputs may be NCHW and SiLU takes its
@@ -916,6 +917,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
     constexpr int kKind = kForm & 3, kAct = ((kForm >> 2) & 7) - 1;   // (kAny: both from the arguments)
     constexpr bool kSplitF = (kForm & 32) != 0, kNchw = (kForm & 256) != 0;
     constexpr int kRes = (kForm >> 6) & 3;
+    constexpr bool kElem = (kForm & kFormElem) != 0;
     constexpr bool kActKnown = kAct >= 0;
     constexpr int kActC = kActKnown ? kAct : 0;
     extern __shared__ unsigned char smem_dyn[];
@@ -1434,13 +1436,13 @@ conv_tc_kernel(const __grid_constant__ G g) {
             const float bv = (a.bias && co_ok) ? __ldg(a.bias + co) : 0.f;
             const unsigned patch = s_tmem_ptr + 16 + (unsigned)(warp - 2) * kPatchBytes;  // shared address
             // (fp32 outputs leave through the element stores below: a warp's 32 filters of one position are 128 contiguous bytes)
-            const bool vec_ok = !kAny ? !kNchw && co0 + row0 < a.Cout : !kF32 && (a.y_c_stride % 8 == 0) && ((a.y_c_off + co0) % 8 == 0) && (co0 + row0 + 32 <= a.Cout);
+            const bool vec_ok = !kAny ? !kNchw && !kElem && co0 + row0 < a.Cout : !kF32 && (a.y_c_stride % 8 == 0) && ((a.y_c_off + co0) % 8 == 0) && (co0 + row0 + 32 <= a.Cout);
             T* yb = (kRep || kNchw) ? yg + (size_t)n * a.y_img + ((size_t)y0 * a.Wo + x0) * a.y_c_stride + (size_t)(a.y_c_off + co0 + row0) * a.y_co
                          : yg + (((size_t)n * a.Ho + y0) * a.Wo + x0) * a.y_c_stride + a.y_c_off + co0 + row0;
             const int n_co = a.Cout - co0 - row0;   // this quarter's filters inside the layer (at most 32 count)
             unsigned ry = (unsigned)min(a.TH, a.Ho - y0);   // rows / columns inside the image
             const unsigned rx = (unsigned)min(a.TW, a.Wo - x0);
-            if (!kAny && !kNchw && co0 + row0 + 8 * (lane & 3) >= a.Cout) ry = 0;   // this lane's eight filters are beyond the layer
+            if (!kAny && !kNchw && !kElem && co0 + row0 + 8 * (lane & 3) >= a.Cout) ry = 0;   // this lane's eight filters are beyond the layer
             const int c_first = (sub + 4 * copy) * 32, c_step = 128 * a.R;
             const T* rb = (kAny ? a.resid != nullptr : kRes != 0) ? reinterpret_cast<const T*>(a.resid) + (yb - yg) : nullptr;   // laid out like y
             const bool post = (kAny || kRes == 3) ? a.resid_post != 0 : kRes == 2;
@@ -1474,7 +1476,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 if (ok) {
                     const int row = quarter * 32 + lane;
 #define RTOSS_SHARES(ACT_) \
-        epilogue_from_shares<T, ACT_, !kAny>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post, kNchw || (kRep && a.nchw), n_co, a.y_co)
+        epilogue_from_shares<T, ACT_, !kAny && !kElem>(sA, a.KS, rank, n_lc, sub, row, a.N_px, bs, vec_ok, co_ok, patch, s_tab, pos_tab, yb, ry, rx, lane, rb, post, kNchw || (kRep && a.nchw), n_co, a.y_co)
                     if constexpr (kActKnown) RTOSS_SHARES(kActC);
                     else if (a.act == RTOSS_ACT_SILU) RTOSS_SHARES(RTOSS_ACT_SILU);
                     else if (a.act == RTOSS_ACT_RELU) RTOSS_SHARES(RTOSS_ACT_RELU);
@@ -1484,7 +1486,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 }
                 continue;
             }
-            bool stored = !kAny;
+            bool stored = !kAny && !kElem;
             if constexpr (!kF32) {
                 if (vec_ok) {
                     stored = true;
@@ -1524,8 +1526,9 @@ conv_tc_kernel(const __grid_constant__ G g) {
 #undef RTOSS_NCHW
                 }
             }
-            if (kAny && !stored) {
+            if ((kAny || kElem) && !stored) {
                 // ragged filter counts, unaligned channel slices, fp32 data: element stores, lane = filter
+                const int act = kActKnown ? kActC : a.act;
                 for (int c0 = c_first; c0 < a.N_px; c0 += c_step) {
                     unsigned r[32];
                     tmem_ld32(d_base + (unsigned)c0, r);
@@ -1536,8 +1539,8 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         const bool in_img = co_ok && (e.y >> 16) < ry && (e.y & 0xFFFFu) < rx;
                         float v = __uint_as_float(r[j]) + bv;
                         if (rb && in_img && !post) v = to_f32<T>(from_f32<T>(v)) + to_f32<T>(__ldcg(rb + e.x + lane));   // round, then add the residual
-                        if (a.act == RTOSS_ACT_RELU) v = fmaxf(v, 0.f);
-                        if (a.act == RTOSS_ACT_SILU) {
+                        if (act == RTOSS_ACT_RELU) v = fmaxf(v, 0.f);
+                        if (act == RTOSS_ACT_SILU) {
                             if (kF32) {
                                 v = silu_f32(v);
                             } else {
@@ -1546,7 +1549,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                 v = v * fmaf(0.5f, th, 0.5f);
                             }
                         }
-                        if (kRep && a.act == kActSiluX) v = silu_exp(v);
+                        if ((kRep || kElem) && act == kActSiluX) v = silu_exp(v);
                         if (rb && in_img && post) v = to_f32<T>(from_f32<T>(v)) + to_f32<T>(__ldcg(rb + e.x + lane));   // behind the activation
                         if (co_ok && (e.y >> 16) < ry && (e.y & 0xFFFFu) < rx) yb[e.x + lane] = from_f32<T>(v);
                     }
