@@ -684,6 +684,9 @@ static SharedKernel shared_kernel(const rtoss_ctx* ctx, bool f32, const TcLaunch
     return conv_tc_kernel<float, TcLaunchN>;
 }
 
+// Filter tiles of a problem (the positions on M: one covers the layer).
+static int pxm_tiles(const TcArgs& a) { return a.pxm ? 1 : a.co_tiles; }
+
 // One convolution, channels last in x.  repacked: x is the copy of rtoss_launch_conv_tc_repacked.
 static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* call, bool repacked,
                          void* stream) {
@@ -720,8 +723,6 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     a.KS = plan.KS;
     a.cb_per = plan.cb_per;
     magic_of(a.KS, a.div_ks);
-    // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM
-    const size_t smem = (size_t)(plan.smem > 116 * 1024 ? plan.smem : 116 * 1024);
     size_t n_units = (size_t)d->N * a.tiles_y * a.tiles_x * a.co_tiles * a.KS;
     if (ctx->inject_next) {
         // failure-detection hook: honoured by a launch of one CTA only (every role of that CTA then runs into its
@@ -732,6 +733,31 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     }
     g.unit_end[0] = (int)n_units;
     dim3 grid((unsigned)(n_units < (size_t)sms ? n_units : (size_t)sms));
+    int smem_need = plan.smem;
+    if (a.KS == 1) {
+        // Weights that fit beside three activation stages (or the plan's own number) stay in shared memory while a CTA walks
+        // its tiles: bf16 1x1 64->64 @160x160 x16 24.7 -> 23.7 us, 128->512 @100x136 x4 16.2 -> 15.9, 3x3 24->24 @100x100 x16
+        // (rows of 48 bytes, which weight copies take slowly) 30.2 -> 15.9; with two stages 512->256 @100x136 x4 16.4 -> 22.4.
+        const int stages = a.ncb * (a.taps / a.G), ct = pxm_tiles(a);
+        const int fixed = plan.smem - plan.NA * (int)a.a_stage - plan.NB * (int)a.b_stage;
+        const int na_room = (227 * 1024 - 64 - fixed - stages * (int)a.b_stage) / (int)a.a_stage, na = na_room < kMaxA ? na_room : kMaxA;
+        const unsigned even = grid.x - grid.x % (unsigned)ct;   // CTAs that keep their filter tile from tile to tile
+        if (stages <= kMaxB && na >= 2 && (na >= 3 || na >= plan.NA) && even > 0 && n_units > (size_t)even && (n_units + even - 1) / even == (n_units + grid.x - 1) / grid.x) {
+            a.resident = 1;
+            grid.x = even;
+            a.NA = na;
+            a.NB = stages;
+            a.sB_off = (unsigned)a.NA * a.a_stage;
+            const int rings = (int)(a.sB_off + (unsigned)a.NB * a.b_stage);
+            g.res_off = rings;
+            g.ring_bytes = rings + (d->residual_dev ? kEpiWarps * kResStage : 0);
+            g.max_na = a.NA;
+            g.max_nb = a.NB;
+            smem_need = rings + fixed;
+        }
+    }
+    // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM
+    const size_t smem = (size_t)(smem_need > 116 * 1024 ? smem_need : 116 * 1024);
     cudaError_t le;
     if (a.KS > 1) {
         // one cluster per tile; if the device cannot place the clusters the layer runs uncut

@@ -139,6 +139,8 @@ struct TcArgs {
     // CTA passes to a problem of another geometry its rings run empty first (see bar_switch in the kernel).
     int NA, NB;
     unsigned a_stage, b_stage, sB_off;
+    int resident;         // NB is a tile's number of weight stages and all tiles of a CTA have the same filters: the stages are
+                          // filled once and serve every tile (launches of one problem)
     int geo;
     int tab;              // which of the launch's position tables
     // over_res: this problem's rings reach into the launch's residual staging area (only problems without a residual
@@ -862,8 +864,8 @@ struct Ring {
     int s = 0;
     unsigned par = 0;
     __device__ __forceinline__ unsigned parity() const { return (par >> s) & 1u; }
-    __device__ __forceinline__ void advance(int n) {
-        par ^= 1u << s;
+    __device__ __forceinline__ void advance(int n, unsigned flip = 1u) {   // flip 0: the stages are filled once and stay
+        par ^= flip << s;
         if (++s == n) s = 0;
     }
 };
@@ -1122,6 +1124,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         rb.advance(a.NB);
                     }
                 }
+                if (!kMulti && a.resident) break;
             }
             if (!ok) atomicExch(g.status, 4);
         }
@@ -1148,6 +1151,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
             Ring ra, rb;
             int as = 0, n_done = 0;
             unsigned pacc = 0;                  // phase parity of the accumulator ring
+            const unsigned flip_b = !kMulti && g.prob[0].resident ? 0u : 1u;   // (see TcArgs::resident)
             unsigned peek = 0;                  // what umma_block_peek saw of the stages now current
             int since_res = 1 << 20;            // tiles issued since this CTA's last tile with a residual operand
             auto mk = [&desc_hi](unsigned lo) { return ((unsigned long long)desc_hi << 32) | lo; };
@@ -1240,7 +1244,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         ra.advance(NA);   // now at the next stages, which the instruction below looks at
-                        rb.advance(NB);
+                        rb.advance(NB, flip_b);
                         const int sa_n = ra.s, sb_n = rb.s;
                         const unsigned pa_n = ra.parity(), pb_n = rb.parity();
                         const unsigned wl0 = desc_lo0 + (sB >> 4) + (unsigned)sb * bstage16;
@@ -1264,7 +1268,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                             }
                         }
                         acc = 1;
-                        umma_commit(leader, bar_emptyB + 8 * sb);
+                        umma_commit(kMulti || flip_b ? leader : 0u, bar_emptyB + 8 * sb);
                         umma_commit(leader, bar_emptyA + 8 * sa);
                         continue;
                     }
@@ -1285,7 +1289,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                                 const unsigned wl0 = desc_lo0 + (sB >> 4) + (unsigned)sb * bstage16;
                                 const unsigned m_first = (unsigned)(bits >> (12 * s3)) & nkmask;
-                                rb.advance(NB);
+                                rb.advance(NB, flip_b);
                                 if (kAny ? !pxm : true) {
                                     // the first tap of the stage goes out together with a look at the next stages
                                     peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl0 + tap16[s3 * 3]), idesc, acc, leader ? m_first : 0u,
@@ -1301,7 +1305,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                         issue_tap(d_base, wl0 + i * wtile16, xl0 + tap16[s3 * 3 + i],
                                                   (unsigned)(bits >> (12 * s3 + 4 * i)) & nkmask, acc);
                                 }
-                                umma_commit(leader, bar_emptyB + 8 * sb);  // this weight stage may be refilled once the MMAs have read it
+                                umma_commit(kMulti || flip_b ? leader : 0u, bar_emptyB + 8 * sb);  // this weight stage may be refilled once the MMAs have read it
                             }
                         }
                     } else if constexpr (kAny) {
@@ -1321,8 +1325,8 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                 issue_tap(d_base, wl0 + i * wtile16, xl0 + off, m4, acc);
                                 if (kF32 && v < a.taps_real) issue_tap(d_base, wl0 + i * wtile16, xl0 + off + ((unsigned)a.lo_off >> 4), m4, acc);
                             }
-                            umma_commit(leader, bar_emptyB + 8 * sb);
-                            rb.advance(NB);
+                            umma_commit(kMulti || flip_b ? leader : 0u, bar_emptyB + 8 * sb);
+                            rb.advance(NB, flip_b);
                         }
                     }
                     if (ok) umma_commit(leader, bar_emptyA + 8 * sa);
