@@ -75,18 +75,23 @@ int max_clusters(int dev, int ks, int sms) {
     return have * sms / 148 < have ? have * sms / 148 : have;
 }
 
-// Expected time of a launch, in microseconds, for one way of cutting a layer.  The constants are a fit to 8 000 measured
-// (layer, tile, split) combinations of the two detectors' layers and odd shapes, batch 1 to 18, launches back to back
-// (programmatic dependent launch); typical error 10 %, and the plan it picks is within 1.5 % of the best measured one over
-// all layers.  What it knows:
-//   - an instruction takes N / 2 cycles for N positions, but never less than 79; per weight stage 0.2 us of barrier
-//     round trip, per channel block 0.1;
-//   - a CTA is fed at most 87 KB per us;
+// Expected time of a launch, in microseconds, for one way of cutting a layer.  16-bit data: the constants are a fit to 6 500
+// measured (layer, tile, split) combinations of the two detectors' layers at eleven sizes, batch 1 to 16, launches back to
+// back (programmatic dependent launch); typical error 7 %, and the plan it picks is on average 1.9 % from the best measured
+// one (4 % with the constants of the kernel before it was compiled in forms).  fp32 keeps the fit made then.  What it knows:
+//   - an instruction takes N / 2 cycles for N positions, but never less than 47; per weight stage 0.13 us of barrier
+//     round trip;
+//   - a CTA is fed at most 118 KB per us (tiles of stride 2, whose boxes overlap, count 0.56);
 //   - the epilogue's sixteen warps take the accumulator in chunks of 32 columns, four warps a chunk: up to 128 positions
-//     cost what 32 cost, 0.5 us; positions on M: filters in groups of 16 instead;
-//   - a launch costs 1.9 us whatever it does, 0.6 more when it leaves no SM for the next one to start on, and 0.5 us until
+//     cost what 32 cost, 0.57 us; positions on M: filters in groups of 16 instead;
+//   - a launch costs 1.9 us whatever it does, 0.9 more when it leaves no SM for the next one to start on, and 0.5 us until
 //     its first operands are there;
-//   - sharing a tile's channel blocks: 0.13 us + 0.34 per CTA of the cluster + 0.33 per chunk exchanged.
+//   - sharing a tile's channel blocks: 0.39 us + 0.27 per CTA of the cluster + 0.37 per chunk exchanged.
+struct PlanFit {
+    double cycles, stage, block, feed, lone, epi_pxm, epi_split, epi, launch, busy, first, tail, split, split_cta, split_chunk, strided;
+};
+constexpr PlanFit kFit16 = {46.7, 0.13, 0.027, 118, 1.05, 0.473, 0.116, 0.573, 1.93, 0.905, 0.50, 0.297, 0.39, 0.273, 0.369, 0.563};
+constexpr PlanFit kFit32 = {79.0, 0.205, 0.09, 87, 0.0, 0.46, 0.26, 0.52, 1.92, 0.59, 0.51, 0.61, 0.13, 0.34, 0.33, 1.0};
 struct PlanCost {
     double us, tile_us, epi_us;
 };
@@ -97,18 +102,20 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
     const int slab_ch = f32 ? 8 : 16, cb_ch = row_bytes / (f32 ? 4 : 2);
     const double slabs = (double)(k.Cin < cb_ch ? k.Cin : cb_ch) / slab_ch * (f32 ? 3 : 1);
     const int wstages = f32 ? 2 * taps / G : taps / G;
-    const double instr = (pxm ? 79.0 * halves : n_px > 158 ? n_px / 2.0 : 79.0) / 1900.0;
-    const double mma = taps * slabs * instr + 0.205 * wstages + 0.09;
+    const PlanFit& f = f32 ? kFit32 : kFit16;
+    const double instr = (pxm ? f.cycles * halves : n_px / 2.0 > f.cycles ? n_px / 2.0 : f.cycles) / 1900.0;
+    const double mma = taps * slabs * instr + f.stage * wstages + f.block;
     const double kb_b = (double)taps * w_rows * row_bytes * (f32 ? 2 : 1) / 1024.0, kb_a = a_bytes / 1024.0;
-    double blk = mma > (kb_a + kb_b) / 87.0 ? mma : (kb_a + kb_b) / 87.0;
+    const double kb_fed = kb_a * (k.S == 2 ? f.strided : 1.0);
+    double blk = mma > (kb_fed + kb_b) / f.feed ? mma : (kb_fed + kb_b) / f.feed;
     // one activation stage: loads and instructions take turns (fp32: and one warp's split of the block between them)
-    if (na == 1) blk = mma + (f32 ? 0.045 * kb_a : 0.35 * kb_a / 87.0);
+    if (na == 1) blk = mma + (f32 ? 0.045 * kb_a : f.lone * kb_fed / 87.0);
     if (f32 && G == 3) blk += 2.0;   // (then only two weight stages fit: the ring's round trip shows)
     const int chunks = (n_px + 31) / 32;
     double epi;
-    if (pxm) epi = 0.92 * 0.5 * ((halves * ((k.Cout + 15) / 16) + 3) / 4);
-    else if (KS > 1) epi = 0.52 * 0.5 * ((2 * ((chunks + KS - 1) / KS) + 3) / 4);
-    else epi = 0.52 * ((chunks + 4 * R - 1) / (4 * R));
+    if (pxm) epi = f.epi_pxm * ((halves * ((k.Cout + 15) / 16) + 3) / 4);
+    else if (KS > 1) epi = f.epi_split * ((2 * ((chunks + KS - 1) / KS) + 3) / 4);
+    else epi = f.epi * ((chunks + 4 * R - 1) / (4 * R));
     if (f32) epi *= 12.9;   // element stores
     const double first_kb = kb_a + kb_b / taps * G;
     PlanCost c;
@@ -116,9 +123,9 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
     c.epi_us = epi;
     const long ctas = tiles * KS < k.sms ? tiles * KS : k.sms;
     const long waves = (tiles * KS + k.sms - 1) / k.sms;
-    double us = 1.92 + (ctas > k.sms / 2 ? 0.59 * (ctas - k.sms / 2) / (k.sms / 2.0) : 0.0) + 0.51 + first_kb / 87.0 + c.tile_us + epi;
-    if (waves > 1) us += (waves - 1) * (c.tile_us > epi ? c.tile_us : epi) + 0.61 * tiles / k.sms;
-    if (KS > 1) us += 0.13 + 0.34 * KS + 0.33 * chunks;
+    double us = f.launch + (ctas > k.sms / 2 ? f.busy * (ctas - k.sms / 2) / (k.sms / 2.0) : 0.0) + f.first + first_kb / f.feed + c.tile_us + epi;
+    if (waves > 1) us += (waves - 1) * (c.tile_us > epi ? c.tile_us : epi) + f.tail * tiles / k.sms;
+    if (KS > 1) us += f.split + f.split_cta * KS + f.split_chunk * chunks;
     c.us = us;
     return c;
 }
