@@ -350,10 +350,12 @@ rtoss_status rtoss_pack(rtoss_ctx* ctx, const void* w_dev, rtoss_dtype w_dtype, 
     if (e == cudaSuccess)  // also writes the handle's own copy of the ids and the tensor path's dense-expanded weights
         le = rtoss_launch_pack_values(w_dev, w_dtype, p->n_kernels, make_table(masks_host, P), pid_dev, k, p->val,
                                       compute_dtype, p->pid, p->wtc, ksize, Cout, Cin, cuda_stream);
-    // the ordering pass also gathers which (tap, channel slab) pairs of every filter tile hold kept weights; its words start at zero
+    // The ordering pass reads the handle's copy of the ids, which pack_values has just written: it loads words of four and sixteen
+    // ids, and the caller's array may start at any byte.
+    // It also gathers which (tap, channel slab) pairs of every filter tile hold kept weights; its words start at zero.
     if (e == cudaSuccess && !le && p->issue) e = cudaMemsetAsync(p->issue, 0, sizeof(unsigned long long) * (size_t)p->issue_n, s);
     if (e == cudaSuccess && !le && ksize == 3)
-        le = rtoss_launch_pack_order(pid_dev, Cout, Cin, P, p->perm, p->bucket_off, p->masks_dev, p->issue,
+        le = rtoss_launch_pack_order(p->pid, Cout, Cin, P, p->perm, p->bucket_off, p->masks_dev, p->issue,
                                      rtoss_issue_cb_log2(compute_dtype), cuda_stream);
     if (e != cudaSuccess || le) {
         rtoss_status r = cuda_fail(ctx, "pack launch", e != cudaSuccess ? (int)e : le);
