@@ -438,6 +438,8 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
 
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc) return (int)cudaErrorNotSupported;
+    // The driver encodes for the thread's current context, and a thread that has made no runtime call yet has none.
+    auto bind_context = [&] { return (int)cudaSetDevice(ctx->device); };
     const CUtensorMapDataType dt = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : a.is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
     // activations: descriptor cached per (pointer, shape, box)
     const int key[7] = {d->N, d->H, d->W, p->Cin, plan.rows_staged * 8 + S, plan.Wq * 4 + (int)p->dtype, d->x_channel_stride};   // (row size: a function of Cin and dtype)
@@ -455,6 +457,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
         cuuint32_t box[4] = {(cuuint32_t)a.cb_ch, (cuuint32_t)(plan.Wq * S), (cuuint32_t)(plan.rows_staged * S), 1};
         cuuint32_t es[4] = {1, (cuuint32_t)S, (cuuint32_t)S, 1};
         ea->valid = 0;
+        if (const int e = bind_context()) return e;
         CUresult r = enc(reinterpret_cast<CUtensorMap*>(ea->map), dt, 4, const_cast<void*>(x), dims, strides, box, es,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -471,6 +474,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
         cuuint32_t box[3] = {(cuuint32_t)a.cb_ch, (cuuint32_t)w_rows, (cuuint32_t)plan.G};  // a weight stage is one copy
         cuuint32_t es[3] = {1, 1, 1};
         eb->valid = 0;
+        if (const int e = bind_context()) return e;
         CUresult r = enc(reinterpret_cast<CUtensorMap*>(eb->map), dt, 3, p->wtc, dims, strides, box, es,
                          CU_TENSOR_MAP_INTERLEAVE_NONE, row_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
