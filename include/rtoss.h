@@ -20,6 +20,10 @@
  *     Calls only enqueue work on it and never synchronise, unless stated.
  *   - Every call returns an rtoss_status; argument errors are detected on the
  *     host before anything is launched.  Nothing throws or aborts.
+ *   - Several host threads may convolve on one context, and on one handle, at the
+ *     same time, each on a stream of its own (rtoss_conv_pattern_host and
+ *     rtoss_conv_chain say what else they ask for).  The text of
+ *     rtoss_last_error is the context's: the last failing call of any thread.
  *   - There is no CPU fallback: without a CUDA device rtoss_create fails.
  */
 #ifndef RTOSS_H

@@ -5,6 +5,7 @@
 
 #include <atomic>
 #include <cstring>
+#include <mutex>
 #include <utility>
 
 #include "conv_tc_kernel.cuh"
@@ -12,18 +13,20 @@
 namespace {
 
 PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const PFN_cuTensorMapEncodeTiled_v12000 fn = []() -> PFN_cuTensorMapEncodeTiled_v12000 {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+            return nullptr;
+        return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
+    }();
     return fn;
 }
+
+// Held while a tensor map is looked up, encoded or copied out.  The maps lie in the context (activations) and in the handle
+// (weights), and both may be in use by several threads at once, a handle by several contexts too: one lock for all.  (An
+// uncontended lock costs some 20 ns of a call's 3 us of host time.)
+std::mutex g_maps;
 
 inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
@@ -441,6 +444,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     // The driver encodes for the thread's current context, and a thread that has made no runtime call yet has none.
     auto bind_context = [&] { return (int)cudaSetDevice(ctx->device); };
     const CUtensorMapDataType dt = f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : a.is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    std::lock_guard<std::mutex> hold(g_maps);
     // activations: descriptor cached per (pointer, shape, box)
     const int key[7] = {d->N, d->H, d->W, p->Cin, plan.rows_staged * 8 + S, plan.Wq * 4 + (int)p->dtype, d->x_channel_stride};   // (row size: a function of Cin and dtype)
     rtoss_tmap_entry* ea = nullptr;
