@@ -5,9 +5,9 @@
 // Here the input channels of a tile are dealt to the eight warps of a CTA (warp w takes channels w, w + 8, ...), every
 // lane keeps four neighbouring output pixels of four filters, its windows come straight from global memory (one channel
 // ahead), and the eight partial sums of an output are added up in shared memory at the end: no barrier inside the loop,
-// four times as many CTAs, a chain of two or three latencies in all.  The weights of eight of the warp's channels are
-// expanded by the warp itself, a lane per (channel, filter); a handle's arrays may be read ahead of the wait for earlier
-// kernels (conv_common.cuh), so the first expansion overlaps the kernel in front.
+// four times as many CTAs, a chain of two or three latencies in all.  The weights of eight channels per warp are expanded at a
+// time, a thread per (channel, filter); a handle's arrays may be read ahead of the wait for earlier kernels (conv_common.cuh),
+// so the first expansion overlaps the kernel in front.
 // Sums are fp32; an output's order of summation is fixed (channels of a warp ascending, then warps ascending).
 #include "conv_common.cuh"
 
@@ -25,7 +25,7 @@ struct FewArgs {
     const uint16_t* masks;
     const float* bias;
     int val_dtype;
-    int N, Cin, Cout, H, W, Ho, Wo, k, act;
+    int N, Cin, Cout, H, W, Ho, Wo, k, P, act;
     int LX, LY, tiles_x, tiles_y;
     long long runs;                       // 1x1: full runs of nine
     long long x_img, x_ch, x_row, x_px;   // element strides of x
@@ -39,7 +39,8 @@ template <typename T, int KS, int S, bool kVec>
 __global__ void __launch_bounds__(kFewWarps * 32, 2) conv_few_kernel(const FewArgs a) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     constexpr int WH = KS, WW = (kFewPx - 1) * S + KS, kSlots = KS == 3 ? 12 : 1;
-    __shared__ __align__(16) float sW[kFewWarps][kFewCh][kFewCo][kSlots];
+    __shared__ __align__(16) float sW[kFewWarps][kFewCh * kFewCo * kSlots + 4];   // (+4: neighbouring channels on different banks)
+    __shared__ uint16_t sM[256];
     __shared__ float sR[kFewWarps][kFewCo * kFewPx][33];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, co0 = blockIdx.y * kFewCo;
     int tile = blockIdx.x;
@@ -51,10 +52,58 @@ __global__ void __launch_bounds__(kFewWarps * 32, 2) conv_few_kernel(const FewAr
     constexpr int kPad = KS / 2;
     const int ix = ox * S - kPad, iy = oy * S - kPad;
 
-    // A lane expands the kernel of channel warp + 8 (i0 + lane / 4), filter co0 + lane % 4.
+    // A 3x3 kernel's dense weights: mask m, kept values v.
+    auto put3 = [&](float* to, unsigned m, const float (&v)[9]) {
+        float4* z = reinterpret_cast<float4*>(to);
+        z[0] = z[1] = z[2] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 9; ++j)
+            if (m) {   // value j belongs to the j-th kept tap
+                to[__ffs(m) - 1] = v[j];
+                m &= m - 1;
+            }
+    };
+    // The first kFewCh channels of every warp, ahead of the wait: the block's threads take (channel, filter) pairs whose ids and
+    // values are neighbours, so that a CTA asks L2 for every line once, and the masks come in once a CTA.  The reads have to come
+    // from L2: nothing orders this SM's L1 behind the kernel that wrote the handle (conv_common.cuh).  fp32 and 16-bit calls of
+    // 10 to 3000 CTAs, 260 of them, launches back to back, against each warp reading its own channels through L1: as fast on
+    // average, 3x3 7->7 @11x106 x12 4.0 -> 4.6 us, fp32 1x1 calls of 200 to 450 CTAs up to 1.27 times slower (fewer registers
+    // let four CTAs on an SM instead of three, which share the SMs out less evenly).  Each warp's own channels from L2: 3 to 6 %
+    // slower, 5.2 us; with an acquire fence, which empties the L1 under the CTAs already running: 3 %, 1x1 46->323 @19x9 x2
+    // 5.8 -> 8.7 us; behind the wait: 6 to 9 %.
+    {
+        const int ci = threadIdx.x % (kFewWarps * kFewCh), f = threadIdx.x / (kFewWarps * kFewCh), co = co0 + f;
+        const bool real = ci < a.Cin && co < a.Cout;
+        float* to = sW[ci % kFewWarps] + (ci / kFewWarps * kFewCo + f) * kSlots;
+        unsigned p = 0;
+        sM[threadIdx.x] = (int)threadIdx.x < a.P ? __ldcg(a.masks + threadIdx.x) : (uint16_t)0;   // (an id outside the table keeps nothing)
+        if constexpr (KS == 3) {
+            float v[9];
+            const size_t kid = (size_t)co * a.Cin + ci;
+            if (real) p = __ldcg(a.pid + kid);
+            if (real) load_vals_cg(a.val, kid, a.k, a.val_dtype, v);
+            __syncthreads();
+            put3(to, real ? sM[p] : 0u, v);
+        } else {
+            const long long e = (long long)co * a.Cin + ci, g = e / 9;
+            const int t = (int)(e - 9 * g);
+            const bool kept = real && g < a.runs;
+            if (kept) p = __ldcg(a.pid + g);
+            __syncthreads();
+            float w = 0.f;
+            if (kept) {
+                const unsigned m = sM[p];
+                if (m & (1u << t)) w = load_val_cg(a.val, (size_t)(g * a.k + __popc(m & ((1u << t) - 1u))), a.val_dtype);
+            }
+            to[0] = w;
+        }
+        __syncthreads();
+    }
+    // The next ones, behind the wait, by the warp itself: a lane expands the kernel of channel warp + 8 (i0 + lane / 4), filter
+    // co0 + lane % 4.
     auto expand = [&](int i0) {
         const int q = lane / kFewCo, f = lane % kFewCo, ci = warp + kFewWarps * (i0 + q), co = co0 + f;
-        float* to = sW[warp][q][f];
+        float* to = sW[warp] + lane * kSlots;
         const bool real = ci < a.Cin && co < a.Cout;
         if constexpr (KS == 3) {
             float v[9];
@@ -64,23 +113,16 @@ __global__ void __launch_bounds__(kFewWarps * 32, 2) conv_few_kernel(const FewAr
                 const unsigned p = __ldg(a.pid + kid);
 #pragma unroll
                 for (int j = 0; j < 9; ++j) v[j] = j < a.k ? load_val(a.val, kid * a.k + j, a.val_dtype) : 0.f;
-                m = __ldg(a.masks + p);
+                m = sM[p];
             }
-            float4* z = reinterpret_cast<float4*>(to);
-            z[0] = z[1] = z[2] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < 9; ++j)
-                if (m) {   // value j belongs to the j-th kept tap
-                    to[__ffs(m) - 1] = v[j];
-                    m &= m - 1;
-                }
+            put3(to, m, v);
         } else {
             float w = 0.f;
             if (real) {
                 const long long e = (long long)co * a.Cin + ci, g = e / 9;
                 const int t = (int)(e - 9 * g);
                 if (g < a.runs) {
-                    const unsigned m = __ldg(a.masks + __ldg(a.pid + g));
+                    const unsigned m = sM[__ldg(a.pid + g)];
                     if (m & (1u << t)) w = load_val(a.val, (size_t)(g * a.k + __popc(m & ((1u << t) - 1u))), a.val_dtype);
                 }
             }
@@ -89,7 +131,6 @@ __global__ void __launch_bounds__(kFewWarps * 32, 2) conv_few_kernel(const FewAr
         __syncwarp();
     };
     const int mine = a.Cin > warp ? (a.Cin - warp + kFewWarps - 1) / kFewWarps : 0;   // this warp's channels
-    expand(0);
     // which values of the window lie inside the image
     unsigned inside = 0;
 #pragma unroll
@@ -173,7 +214,7 @@ __global__ void __launch_bounds__(kFewWarps * 32, 2) conv_few_kernel(const FewAr
         }
 #pragma unroll
         for (int f = 0; f < kFewCo; ++f) {
-            const float* w = sW[warp][i % kFewCh][f];
+            const float* w = sW[warp] + (i % kFewCh * kFewCo + f) * kSlots;
             float wv[kSlots];
             if constexpr (KS == 3) {
 #pragma unroll
@@ -272,6 +313,7 @@ int rtoss_launch_conv_few(const rtoss_packed* p, const void* x, void* y, const r
     a.Ho = (d->H - 1) / d->stride + 1;
     a.Wo = (d->W - 1) / d->stride + 1;
     a.k = p->k;
+    a.P = p->P;
     a.act = (int)d->act;
     a.runs = p->n_kernels;
     const long long cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;

@@ -945,7 +945,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles = g.unit_end[g.n_prob - 1];  // units of work over all problems: (tile, share of the channel blocks)
     // Programmatic dependent launch: the next kernel of the stream may start its own prologue now (on SMs this
-    // grid leaves free); it reads or writes nothing before its own griddepcontrol.wait.
+    // grid leaves free); before its own griddepcontrol.wait it reads nothing but handles (see conv_common.cuh).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
     if (threadIdx.x == 0) {
@@ -1224,7 +1224,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 // which (tap, slab) pairs of this filter tile hold kept weights: one word per channel block, the next
                 // block's word asked for while this block's instructions go out
                 const unsigned long long* iss = a.issue ? a.issue + (size_t)ti.cot * a.ncb : nullptr;
-                unsigned long long bits = iss ? __ldg(iss + ks * a.cb_per) : ~0ull;
+                unsigned long long bits = iss ? __ldcg(iss + ks * a.cb_per) : ~0ull;
                 ok = mbar_wait(bar_accEmpty + 8 * as, pacc ^ 1, g.wait_cycles);  // epilogue has drained this stage
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1272,7 +1272,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         umma_commit(leader, bar_emptyA + 8 * sa);
                         continue;
                     }
-                    const unsigned long long bits_n = (iss && cb + 1 < cb_end) ? __ldg(iss + cb + 1) : ~0ull;
+                    const unsigned long long bits_n = (iss && cb + 1 < cb_end) ? __ldcg(iss + cb + 1) : ~0ull;
                     if (!(peek & 1u)) ok = mbar_wait(bar_rdyA + 8 * sa, ra.parity(), g.wait_cycles);   // (peek stays 0 on the paths that do not look ahead)
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");

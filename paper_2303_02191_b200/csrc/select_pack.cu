@@ -26,6 +26,11 @@ template <> __device__ __forceinline__ float narrow<float>(float v) { return v; 
 template <> __device__ __forceinline__ __nv_bfloat16 narrow<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 template <> __device__ __forceinline__ __half narrow<__half>(float v) { return __float2half_rn(v); }
 
+// (__ldcg takes no 16-bit floating types here)
+__device__ __forceinline__ float ld_cg(const float* p) { return __ldcg(p); }
+__device__ __forceinline__ __nv_bfloat16 ld_cg(const __nv_bfloat16* p) { return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p))); }
+__device__ __forceinline__ __half ld_cg(const __half* p) { return __ushort_as_half(__ldcg(reinterpret_cast<const unsigned short*>(p))); }
+
 // Copy the 9*count weights of `count` consecutive kernels starting at kernel
 // `first` into shared memory, coalesced, 16 bytes per thread where the chunk is
 // whole.  The base pointer is 16-byte aligned and a full chunk is a multiple
@@ -199,7 +204,7 @@ __global__ void __launch_bounds__(kSharedMaxFB) select_shared_kernel(const T* __
 // before this one: a model's layers are expanded one call after the other, and all but the stores of a call then overlaps
 // the call before it.  (Sixty-eight layers in a row: 3.4 us a
 // layer with a gather per element behind the wait, 1.2 now.)
-// Loads go to L2 (ld.cg): the L1 of this SM may hold lines from before the handle was written.
+// All of these loads go to L2 (see conv_common.cuh).
 template <typename V>
 __global__ void __launch_bounds__(kSelThreads) to_dense_kernel(const V* __restrict__ val, const uint8_t* __restrict__ pid,
                                                                const uint16_t* __restrict__ masks, int k, int64_t n_kernels, int64_t n_dense,
@@ -220,7 +225,7 @@ __global__ void __launch_bounds__(kSelThreads) to_dense_kernel(const V* __restri
             const V* src = val + first * k;
             const int n = count * k, nv = n * (int)sizeof(V) / 16;
             for (int i = tid; i < nv; i += kSelThreads) reinterpret_cast<uint4*>(sv)[i] = __ldcg(reinterpret_cast<const uint4*>(src) + i);
-            for (int i = nv * 16 / (int)sizeof(V) + tid; i < n; i += kSelThreads) sv[i] = src[i];
+            for (int i = nv * 16 / (int)sizeof(V) + tid; i < n; i += kSelThreads) sv[i] = ld_cg(src + i);
         }
         __syncthreads();
         if (tid < count) {
