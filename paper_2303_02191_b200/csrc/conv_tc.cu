@@ -258,7 +258,8 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
 // The plan of a call.  The split is decided as if the call had a residual operand, whether it has one or not: a call with
 // a residual then adds up its products in the order of the same call without one (same bits).
 // Searching takes tens of microseconds of host time, more than a launch: every thread remembers the plans of its last
-// few hundred kinds of call.  A plan is a function of sizes alone, so it does not matter which thread or context asks.
+// few hundred kinds of call.  A plan is a function of its key and of the device's cluster limits, which whoever plans for a
+// device has had asked first (ensure_device): it does not matter which thread or context asks.
 bool plan_tc(const PlanKey& k, TcPlan* out) {
     struct Memo {
         PlanKey key;
@@ -618,6 +619,7 @@ static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const
     return best;
 }
 double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds) {
+    if (ensure_device(ctx)) return 1e30;   // (the launch that follows reports the error)
     return shared_cost(ctx, n, ps, ds, nullptr);
 }
 
@@ -626,7 +628,7 @@ double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* con
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
     const rtoss_conv_desc dd = row_form(p, d);
-    if (!plan_tc(plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    if (ensure_device(ctx) || !plan_tc(plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
     *us = plan.us;
     *ks = plan.KS;
     *tiles = plan.tiles;
