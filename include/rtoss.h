@@ -425,8 +425,23 @@ rtoss_status rtoss_inject_lost_copy(rtoss_ctx* ctx);
 rtoss_status rtoss_conv_pattern_host(rtoss_ctx* ctx, const rtoss_packed* p, const void* x_host, void* y_host,
                                      const rtoss_conv_desc* desc);
 
-/* How the FMA path would tile a 3x3 call (host arithmetic only, nothing is launched; for Cin <= 4 only small_cin is
- * set: that kernel has no staging plan).  staging: 0 = plain loads, 1 = NCHW rows as aligned vectors of vector_bytes
+/* Which kernels a single convolution call runs on (host arithmetic only; nothing is launched, no device is touched).
+ * desc as in the call; its pointers are not dereferenced, x, y and a residual operand count as 16-byte aligned.  Returns
+ * what the call would return for an argument it does not take (RTOSS_ERR_INVALID_ARG, RTOSS_ERR_UNSUPPORTED).  A call
+ * on RTOSS_ROUTE_TENSOR_REPACKED for which there is no memory runs as RTOSS_ROUTE_STAGED.  Not part of the paper's method. */
+typedef enum {
+    RTOSS_ROUTE_TENSOR = 0,          /* tensor path, x where it lies */
+    RTOSS_ROUTE_TENSOR_REPACKED = 1, /* tensor path behind the pass that writes x channels last */
+    RTOSS_ROUTE_STEM = 2,            /* FMA path, 3x3 of at most four input channels (three 16-bit ones: matrix instructions) */
+    RTOSS_ROUTE_FEW = 3,             /* FMA path, few outputs: channels over the warps, nothing staged */
+    RTOSS_ROUTE_STAGED = 4           /* FMA path, tiles staged in shared memory (rtoss_fma_plan3x3 for 3x3) */
+} rtoss_route;
+rtoss_status rtoss_conv_route_of(const rtoss_conv_desc* desc, int ksize, int Cin, int Cout, rtoss_dtype packed_dtype,
+                                 rtoss_route* out);
+
+/* How the staged kernels of the FMA path tile a 3x3 call (host arithmetic only, nothing is launched; for Cin <= 4 only
+ * small_cin is set: that kernel has no staging plan).  Calls of few outputs run on another kernel, which stages nothing:
+ * rtoss_conv_route_of says which.  staging: 0 = plain loads, 1 = NCHW rows as aligned vectors of vector_bytes
  * through cp.async, 2 = NHWC pixels as 16-byte vectors through cp.async.  With staging 1 the address of every vector,
  *   ((n*Cin + ci)*H*W + iy*W + tx*lanes_x*pixels_per_lane*stride - vector_bytes/es + j*vector_bytes/es) * es
  * (es = bytes per activation, tx = tile column, j = vector inside the staged row), is a multiple of vector_bytes for a

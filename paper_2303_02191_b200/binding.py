@@ -20,6 +20,7 @@ NCHW, NHWC = 0, 1
 ACT_NONE, ACT_RELU, ACT_SILU = 0, 1, 2
 PRESET_ALL, PRESET_CONN4, PRESET_CENTRE8, PRESET_DENSE = 0, 1, 2, 3
 PATH_AUTO, PATH_FMA, PATH_TENSOR = 0, 1, 2
+ROUTE_TENSOR, ROUTE_TENSOR_REPACKED, ROUTE_STEM, ROUTE_FEW, ROUTE_STAGED = 0, 1, 2, 3, 4
 DTYPE_NAMES = {"f32": F32, "bf16": BF16, "f16": F16}
 ACT_NAMES = {"none": ACT_NONE, "relu": ACT_RELU, "silu": ACT_SILU}
 
@@ -28,7 +29,7 @@ SYMBOLS = [
     "rtoss_pattern_table_validate", "rtoss_group_layers", "rtoss_select_patterns", "rtoss_pack",
     "rtoss_packed_info_get", "rtoss_packed_export", "rtoss_packed_to_dense", "rtoss_packed_destroy",
     "rtoss_conv3x3_pattern", "rtoss_conv1x1_pattern", "rtoss_conv_pattern_host", "rtoss_device_status", "rtoss_prune_dense_static", "rtoss_maxpool2d", "rtoss_upsample2x", "rtoss_add_act", "rtoss_pattern_usage",
-    "rtoss_upsample2x_slice", "rtoss_pool_pyramid",
+    "rtoss_upsample2x_slice", "rtoss_pool_pyramid", "rtoss_conv_route_of",
     "rtoss_pattern_rank", "rtoss_pattern_table_derive",
     "rtoss_batch_create", "rtoss_batch_select_pack", "rtoss_batch_destroy",
     "rtoss_select_patterns_shared", "rtoss_conv_group", "rtoss_set_wait_limit", "rtoss_inject_lost_copy",
@@ -121,6 +122,7 @@ def _load():
     lib.rtoss_chain_deps_spans.argtypes = [ctypes.POINTER(ctypes.c_uint64), ci, ctypes.POINTER(ctypes.c_uint32)]
     lib.rtoss_set_wait_limit.argtypes = [vp, ctypes.c_longlong]
     lib.rtoss_inject_lost_copy.argtypes = [vp]
+    lib.rtoss_conv_route_of.argtypes = [ctypes.POINTER(ConvDesc), ci, ci, ci, ci, ctypes.POINTER(ci)]
     lib.rtoss_fma_plan3x3.argtypes = [ctypes.POINTER(ConvDesc), ci, ci, ci, ci, ctypes.POINTER(FmaPlan)]
     lib.rtoss_select_patterns_shared.argtypes = [vp, vp, ci, ci, ci, ci, ci, vp, ci, ci, vp, vp]
     lib.rtoss_prune_dense_static.argtypes = [vp, ci, ci, ci, ci, vp, ci, ci, vp, vp]
@@ -233,6 +235,17 @@ def rtoss_pool_pyramid(y, N, C, H, W, k, layout=NHWC, y_channel_offset=0, y_chan
 def rtoss_add_act(a, b, y, act=ACT_NONE):
     _glue_check(lib.rtoss_add_act(a.data_ptr(), b.data_ptr(), y.data_ptr(), a.numel(), _torch_dtype_code(a), act, _stream()))
     return y
+
+
+def rtoss_conv_route_of(N, H, W, stride, ksize, layout, io_dtype, Cin, Cout, path=PATH_AUTO, packed_dtype=None, residual=False):
+    """Which kernels a single call runs on (ROUTE_*; host arithmetic, nothing is launched)."""
+    d = ConvDesc(int(N), int(H), int(W), int(stride), int(layout), int(io_dtype), ACT_NONE, None, 0, 0, int(path), 16 if residual else None, 0, 0)
+    route = ctypes.c_int(-1)
+    st = lib.rtoss_conv_route_of(ctypes.byref(d), int(ksize), int(Cin), int(Cout), int(io_dtype if packed_dtype is None else packed_dtype),
+                                 ctypes.byref(route))
+    if st != OK:
+        raise RtossError(st, status_string(st))
+    return route.value
 
 
 def rtoss_fma_plan3x3(N, H, W, stride, layout, io_dtype, Cin, Cout, k, packed_dtype=None):

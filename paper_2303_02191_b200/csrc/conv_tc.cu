@@ -567,16 +567,18 @@ bool rtoss_tc_weights_eligible(const rtoss_packed* p) { return p->dtype != RTOSS
 // Layers whose channels-last activations TMA can read where they lie.
 static bool rows_fit_tma(const rtoss_packed* p) { return p->Cin % (p->dtype == RTOSS_F32 ? 4 : 8) == 0; }
 
-// Can this call run on the tensor path?
-bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y) {
+// Can this call run on the tensor path?  (rtoss_tc_takes: by its sizes, types and alignment; no device is asked.)
+bool rtoss_tc_takes(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y) {
     if (!p->wtc || !rows_fit_tma(p)) return false;
     if (d->layout != RTOSS_NHWC || (int)d->io_dtype != (int)p->dtype) return false;
     if ((reinterpret_cast<uintptr_t>(x) & 15) || (reinterpret_cast<uintptr_t>(y) & 15)) return false;
     if (d->x_channel_stride % (p->dtype == RTOSS_F32 ? 4 : 8) != 0) return false;   // a slice: the pitch as TMA wants it
-    if (!encode_fn()) return false;
     // a residual operand: 16-byte aligned, and not for the positions-as-M form (narrow 1x1 layers)
     if (d->residual_dev && (use_pxm(p) || (reinterpret_cast<uintptr_t>(d->residual_dev) & 15))) return false;
     return plan_exists(p, d);
+}
+bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y) {
+    return rtoss_tc_takes(p, d, x, y) && encode_fn();
 }
 
 // May this call be one of several in a launch?  (Tensor path with the filters on M.)
@@ -812,14 +814,14 @@ static rtoss_conv_desc repacked_desc(const rtoss_packed* p, const rtoss_conv_des
     return dd;
 }
 static bool x_is_slice(const rtoss_packed* p, const rtoss_conv_desc* d) { return d->x_channel_stride && d->x_channel_stride != p->Cin; }
-bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) {
+bool rtoss_tc_takes_repacked(const rtoss_packed* p, const rtoss_conv_desc* d) {
     if (d->path != RTOSS_PATH_AUTO || d->residual_dev || x_is_slice(p, d) || !p->wtc || p->dtype == RTOSS_F32 || (int)d->io_dtype != (int)p->dtype) return false;
     if (d->layout == RTOSS_NHWC && rows_fit_tma(p)) return false;   // (native, or declined for another reason)
     if (p->ksize == 3 && p->Cin <= 4) return false;
-    if (!encode_fn()) return false;
     const rtoss_conv_desc dd = repacked_desc(p, d);
     return plan_exists(p, &dd);
 }
+bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) { return rtoss_tc_takes_repacked(p, d) && encode_fn(); }
 // Returns a cudaError_t, or -1 when there was no memory for the channels-last copy (nothing was launched).  The copy
 // lives from here to the end of the convolution in the stream's order, in the context's pool: any number of streams and
 // threads may be in such a call, and inside a stream capture the copy belongs to the graph.

@@ -86,6 +86,14 @@ rtoss_status check_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     return RTOSS_OK;
 }
 
+// Which kernels run a call, given whether the tensor path takes it as it is or behind a layout pass.
+rtoss_route route_of(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, bool tc, bool repack) {
+    if (tc) return RTOSS_ROUTE_TENSOR;
+    if (p->ksize == 3 && p->Cin <= 4) return RTOSS_ROUTE_STEM;
+    if (rtoss_few_eligible(p, d, x, repack)) return RTOSS_ROUTE_FEW;
+    return repack ? RTOSS_ROUTE_TENSOR_REPACKED : RTOSS_ROUTE_STAGED;
+}
+
 // Pick the kernel family for one convolution call and launch it.  Returns the CUDA error code of
 // the launch; *st is set when the requested path cannot take the call.
 int dispatch_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, void* stream,
@@ -108,9 +116,9 @@ int dispatch_conv(rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
         return 0;
     }
     if (tc_ok) return rtoss_launch_conv_tc(ctx, p, x, y, d, stream);
-    const bool repack = rtoss_tc_repack_eligible(p, d);
-    if (rtoss_few_eligible(p, d, x, repack)) return rtoss_launch_conv_few(p, x, y, d, stream);
-    if (repack) {
+    const rtoss_route route = route_of(p, d, x, false, rtoss_tc_repack_eligible(p, d));
+    if (route == RTOSS_ROUTE_FEW) return rtoss_launch_conv_few(p, x, y, d, stream);
+    if (route == RTOSS_ROUTE_TENSOR_REPACKED) {
         const int e = rtoss_launch_conv_tc_repacked(ctx, p, x, y, d, stream);
         if (e >= 0) return e;   // (-1: no memory for the copy of x; the FMA path needs none)
     }
@@ -498,6 +506,25 @@ rtoss_status rtoss_conv1x1_pattern(rtoss_ctx* ctx, const rtoss_packed* p, const 
     int e = dispatch_conv(ctx, p, x_dev, y_dev, desc, cuda_stream, &st);
     if (st != RTOSS_OK) return st;
     return e ? cuda_fail(ctx, "conv1x1 launch", e) : RTOSS_OK;
+}
+
+rtoss_status rtoss_conv_route_of(const rtoss_conv_desc* d, int ksize, int Cin, int Cout, rtoss_dtype packed_dtype, rtoss_route* out) {
+    if (!d || !out || (ksize != 1 && ksize != 3) || Cin < 1 || Cout < 1 || !dtype_ok(packed_dtype)) return RTOSS_ERR_INVALID_ARG;
+    rtoss_ctx ctx;
+    rtoss_packed p;
+    memset(&ctx, 0, sizeof(ctx));
+    memset(&p, 0, sizeof(p));
+    p.Cin = Cin, p.Cout = Cout, p.ksize = ksize, p.dtype = packed_dtype;
+    alignas(16) static char aligned[16];   // stands for every array of the call (never dereferenced)
+    if (rtoss_tc_weights_eligible(&p)) p.wtc = aligned;
+    rtoss_conv_desc dd = *d;
+    if (dd.residual_dev) dd.residual_dev = aligned;
+    rtoss_status st = check_conv(&ctx, &p, aligned, aligned, &dd, ksize, true);
+    if (st != RTOSS_OK) return st;
+    const bool tc = d->path != RTOSS_PATH_FMA && rtoss_tc_takes(&p, &dd, aligned, aligned);
+    if (!tc && (dd.residual_dev || (d->x_channel_stride && d->x_channel_stride != Cin) || d->path == RTOSS_PATH_TENSOR)) return RTOSS_ERR_UNSUPPORTED;
+    *out = route_of(&p, &dd, aligned, tc, rtoss_tc_takes_repacked(&p, &dd));
+    return RTOSS_OK;
 }
 
 rtoss_status rtoss_conv_group(rtoss_ctx* ctx, const rtoss_conv_item* items, int n, int* launches, void* cuda_stream) {

@@ -139,10 +139,12 @@ static inline int rtoss_issue_words(int Cout, int Cin, int ksize, rtoss_dtype d)
 
 // tensor path (conv_tc.cu)
 bool rtoss_tc_weights_eligible(const rtoss_packed* p);
+bool rtoss_tc_takes(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y);   // (the device aside)
 bool rtoss_tc_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y);
 int rtoss_launch_conv_tc(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                          const rtoss_conv_desc* d, void* stream);
 // 16-bit calls the tensor path takes after a pass that writes x channels last (repack.cu); -1: no memory for the copy
+bool rtoss_tc_takes_repacked(const rtoss_packed* p, const rtoss_conv_desc* d);   // (the device aside)
 bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d);
 int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                                   const rtoss_conv_desc* d, void* stream);
