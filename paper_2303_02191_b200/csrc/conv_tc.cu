@@ -819,6 +819,8 @@ bool rtoss_tc_takes_repacked(const rtoss_packed* p, const rtoss_conv_desc* d) {
     if (d->layout == RTOSS_NHWC && rows_fit_tma(p)) return false;   // (native, or declined for another reason)
     if (p->ksize == 3 && p->Cin <= 4) return false;
     const rtoss_conv_desc dd = repacked_desc(p, d);
+    // (the pass counts its pieces, and its blocks, with 31 bits: copies of up to 32 GiB)
+    if ((long long)dd.N * dd.H * dd.W > 0x7FFFFFFFLL / (rtoss_cin_pitch(p->Cin, p->dtype) / 8)) return false;
     return plan_exists(p, &dd);
 }
 bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) { return rtoss_tc_takes_repacked(p, d) && encode_fn(); }

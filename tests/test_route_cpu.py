@@ -15,6 +15,9 @@ CALLS = [
     ((1, 32, 32, 1, 3, rt.NHWC, BF16, 32, 32, rt.PATH_FMA, BF16), rt.ROUTE_FEW),
     ((8, 80, 80, 1, 3, rt.NHWC, BF16, 128, 128, rt.PATH_FMA, BF16), rt.ROUTE_STAGED),
     ((8, 80, 80, 1, 3, rt.NHWC, BF16, 128, 128, rt.PATH_AUTO, F32), rt.ROUTE_STAGED),     # (the handle's type is not the data's)
+    ((100, 1024, 1024, 1, 3, rt.NHWC, BF16, 150, 8, rt.PATH_AUTO, BF16), rt.ROUTE_TENSOR_REPACKED),
+    ((200, 1024, 1024, 1, 3, rt.NHWC, BF16, 150, 8, rt.PATH_AUTO, BF16), rt.ROUTE_STAGED),   # (a copy of more than 2^31 pieces of 16 bytes)
+    ((200, 1024, 1024, 1, 3, rt.NCHW, BF16, 150, 8, rt.PATH_AUTO, BF16), rt.ROUTE_STAGED),
     ((32, 80, 80, 1, 1, rt.NCHW, F32, 256, 256, rt.PATH_AUTO, F32), rt.ROUTE_STAGED),
 ]
 
