@@ -826,21 +826,17 @@ bool rtoss_tc_takes_repacked(const rtoss_packed* p, const rtoss_conv_desc* d) {
 bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d) { return rtoss_tc_takes_repacked(p, d) && encode_fn(); }
 // Returns a cudaError_t, or -1 when there was no memory for the channels-last copy (nothing was launched).  The copy
 // lives from here to the end of the convolution in the stream's order, in the context's pool: any number of streams and
-// threads may be in such a call, and inside a stream capture the copy belongs to the graph.
+// threads may be in such a call.  Inside a stream capture the copy belongs to the graph (rtoss_copy_get).
 int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d,
                                   void* stream) {
     const rtoss_conv_desc dd = repacked_desc(p, d);
     const int cp = rtoss_cin_pitch(p->Cin, p->dtype), S = dd.stride == d->stride ? 1 : 2;
-    void* ws = nullptr;
-    const size_t bytes = (size_t)dd.N * dd.H * dd.W * cp * 2;
-    void* pool = rtoss_ctx_pool(ctx);
-    if (!pool || cudaMallocFromPoolAsync(&ws, bytes, (cudaMemPool_t)pool, (cudaStream_t)stream) != cudaSuccess) {
-        cudaGetLastError();
-        return -1;
-    }
+    bool of_graph = false;
+    void* ws = rtoss_copy_get(ctx, (size_t)dd.N * dd.H * dd.W * cp * 2, stream, &of_graph);
+    if (!ws) return -1;
     int e = rtoss_launch_repack16(x, ws, dd.N, p->Cin, cp, d->H, d->W, S, d->layout, stream);
     if (!e) e = launch_single(ctx, p, ws, y, &dd, true, stream);
-    const cudaError_t fe = cudaFreeAsync(ws, (cudaStream_t)stream);
+    const cudaError_t fe = of_graph ? cudaSuccess : cudaFreeAsync(ws, (cudaStream_t)stream);
     return e ? e : (int)fe;
 }
 

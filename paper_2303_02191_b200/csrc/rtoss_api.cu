@@ -134,7 +134,56 @@ rtoss_device_guard::~rtoss_device_guard() {
     if (switched) cudaSetDevice(prev);
 }
 
-void* rtoss_ctx_pool(const rtoss_ctx* ctx) {
+// ---- memory of the channels-last copies --------------------------------------------------------------------------
+// A call on a stream takes its copy from the context's pool in stream order and gives it back the same way.  A call inside a
+// stream capture must not do that: allocation nodes would come into the caller's graph, which could then be instantiated
+// once only and be neither cloned nor a child of another graph.  Its copy is allocated at once and owned by the graph, through
+// a user object that the graph, its executables and its clones hold references to; when the last of them is gone and its
+// launches have finished, the copy joins a list, from which the next call that looks (a user object's destructor may not call
+// CUDA itself) gives it back to the pool.
+namespace {
+
+struct GraphCopy {
+    void* mem;
+    int device;
+    GraphCopy* next;
+};
+std::mutex g_dead_lock;
+GraphCopy* g_dead = nullptr;
+
+void CUDART_CB graph_copy_dead(void* holder) {
+    GraphCopy* c = static_cast<GraphCopy*>(holder);
+    std::lock_guard<std::mutex> hold(g_dead_lock);
+    c->next = g_dead;
+    g_dead = c;
+}
+
+// Frees the copies on this context's device that no graph holds any more.
+void collect_dead(const rtoss_ctx* ctx) {
+    GraphCopy* mine = nullptr;
+    {
+        std::lock_guard<std::mutex> hold(g_dead_lock);
+        for (GraphCopy** at = &g_dead; *at;) {
+            GraphCopy* c = *at;
+            if (c->device != ctx->device) {
+                at = &c->next;
+                continue;
+            }
+            *at = c->next;
+            c->next = mine;
+            mine = c;
+        }
+    }
+    while (mine) {   // (not under the lock: freeing waits for the device, and a destructor may want the lock)
+        GraphCopy* c = mine;
+        mine = c->next;
+        cudaFree(c->mem);
+        delete c;
+    }
+}
+
+// The context's pool; null: not to be had.
+cudaMemPool_t copy_pool(const rtoss_ctx* ctx) {
     static std::mutex making;   // (two threads may make their first such call on one context at once)
     std::lock_guard<std::mutex> hold(making);
     if (!ctx->pool) {
@@ -144,7 +193,7 @@ void* rtoss_ctx_pool(const rtoss_ctx* ctx) {
         props.location.id = ctx->device;
         cudaMemPool_t pool = nullptr;
         unsigned long long keep = kPoolKeep;
-        // the context's first such call may lie inside a stream capture, which making a pool is no part of
+        // (another thread's stream capture may be under way, which making a pool is no part of)
         cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
         cudaThreadExchangeStreamCaptureMode(&mode);
         if (cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
@@ -155,7 +204,48 @@ void* rtoss_ctx_pool(const rtoss_ctx* ctx) {
         }
         cudaThreadExchangeStreamCaptureMode(&mode);
     }
-    return ctx->pool;
+    return (cudaMemPool_t)ctx->pool;
+}
+
+void* graph_copy(const rtoss_ctx* ctx, size_t bytes, cudaGraph_t graph) {
+    collect_dead(ctx);
+    void* mem = nullptr;
+    if (cudaMalloc(&mem, bytes) != cudaSuccess) return nullptr;
+    GraphCopy* c = new (std::nothrow) GraphCopy{mem, ctx->device, nullptr};
+    cudaUserObject_t owner = nullptr;
+    if (!c || cudaUserObjectCreate(&owner, c, graph_copy_dead, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+        delete c;
+        cudaFree(mem);
+        return nullptr;
+    }
+    if (cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+        cudaUserObjectRelease(owner, 1);   // (its destructor hands the memory to the list)
+        return nullptr;
+    }
+    return mem;
+}
+
+}  // namespace
+
+void* rtoss_copy_get(const rtoss_ctx* ctx, size_t bytes, void* stream, bool* of_graph) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    void* mem = nullptr;
+    *of_graph = false;
+    if (cudaStreamGetCaptureInfo((cudaStream_t)stream, &status, nullptr, &graph) == cudaSuccess) {
+        if (status == cudaStreamCaptureStatusNone) {
+            cudaMemPool_t pool = copy_pool(ctx);
+            if (pool && cudaMallocFromPoolAsync(&mem, bytes, pool, (cudaStream_t)stream) != cudaSuccess) mem = nullptr;
+        } else if (status == cudaStreamCaptureStatusActive) {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (what happens here is no part of the capture)
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            mem = graph_copy(ctx, bytes, graph);
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            *of_graph = mem != nullptr;
+        }
+    }
+    if (!mem) cudaGetLastError();
+    return mem;
 }
 
 extern "C" {
@@ -215,6 +305,7 @@ void rtoss_destroy(rtoss_ctx* ctx) {
     if (ctx->ws_y) cudaFree(ctx->ws_y);
     if (ctx->dev_status) cudaFree(ctx->dev_status);
     if (ctx->chain_done) cudaFree(ctx->chain_done);
+    collect_dead(ctx);
     if (ctx->pool) cudaMemPoolDestroy((cudaMemPool_t)ctx->pool);   // (memory still in use by the stream is released when its free is reached)
     cudaSetDevice(prev);
     delete ctx;

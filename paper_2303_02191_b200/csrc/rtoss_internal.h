@@ -43,7 +43,7 @@ struct rtoss_ctx {
     mutable int inject_next;   // failure-detection test hook: the next tensor-path launch withholds its first weight copy
     mutable rtoss_tmap_entry tmap_cache[32];  // activation descriptors of the tensor path, round robin
     mutable int tmap_next;
-    mutable void* pool;        // cudaMemPool_t, made at first use (rtoss_ctx_pool), of the channels-last copies some calls need (stream-ordered; keeps at most kPoolKeep bytes)
+    mutable void* pool;        // cudaMemPool_t of the channels-last copies some calls need, made at first use (rtoss_copy_get; keeps at most kPoolKeep bytes)
     unsigned* chain_done;      // device: RTOSS_CHAIN_SLOTS x RTOSS_CHAIN_SLOT_WORDS completion counters, all zero at rest
     mutable int chain_next;    // the block the next launch with dependent convolutions takes
 };
@@ -148,7 +148,8 @@ bool rtoss_tc_takes_repacked(const rtoss_packed* p, const rtoss_conv_desc* d);  
 bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d);
 int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                                   const rtoss_conv_desc* d, void* stream);
-void* rtoss_ctx_pool(const rtoss_ctx* ctx);   // null: none to be had
+// memory for such a copy, freed by the caller in stream order or (of_graph) with the graph being captured; null: none to be had
+void* rtoss_copy_get(const rtoss_ctx* ctx, size_t bytes, void* stream, bool* of_graph);
 int rtoss_launch_repack16(const void* x, void* out, int N, int Cin, int cp, int H, int W, int S, rtoss_layout layout, void* stream);
 bool rtoss_tc_groupable(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y);
 // several independent convolutions in one launch: 0 = launched, -1 = the set cannot share a launch (nothing launched)
