@@ -274,26 +274,35 @@ static bool few_vec(const rtoss_conv_desc* d, const void* x) {
 }
 
 // Is this a call for the kernel above?  Its time grows with its CTAs (tiles of 128 pixels x 4 filters) from the first on, that
-// of the staged kernels in steps of a full device, so there is a number of CTAs up to which this one is faster.
-// fp32, default layout, this kernel / the staged one, us:
-//   3x3  32->32 @32x32 (64 CTAs) 3.6 / 15.7      512->512 @10x10 (256; no vectors) 66 / 196   256->256 @40x40 (960) 97 / 226
-//        64->64 @80x80 x4 (3200) 96 / 120        256->256 @40x40 x4 (3840) 352 / 467          64->64 @80x80 x8 (6400) 191 / 129
-//        without vectors: 64->64 @80x80 x2 (1600) 67 / 67, x4 (3200) 130 / 118
-//   1x1  32->32 @32x32 (64 CTAs) 2.9 / 24.8      512->512 @20x20 x4 (2560) 106 / 370          256->256 @40x40 x4 (3840) 86 / 148
-//        64->64 @80x80 x8 (6400) 56 / 47         without vectors: 256->256 @40x40 x4 124 / 148
+// of the staged kernels in steps of a full device, so there is a number of CTAs up to which this one is faster.  420 calls of
+// 300 to 9000 CTAs, both layouts, all types, 1 to 512 channels, this kernel's time / the staged one's:
+//   3x3  at most 8 channels (one a warp: expansion and sum are all a CTA does)  315 CTAs 0.87, 560 0.99, 636 1.18, 660 0.73, 732 1.23,
+//                  768 0.59, 900 1.11, 1000 1.37, 1050 2.07, 3528 1.95
+//        9 to 16        664 0.44, 1020 0.57, 1092 0.88, 1290 1.04, 1590 1.25, 1848 1.63, 3871 1.71
+//        more, default layout with whole vectors   1080 0.89, 3200 0.80 (64->64 @80x80 x4), 3840 0.75, 6400 1.48, 7020 1.40
+//        more, other    1200 0.86, 1600 1.00, 3200 1.10, 5040 1.64; 16 bits channels last 1020 0.93, 1428 1.12, 1440 1.28
+//        channels last in multiples of 8, which the staged kernel fetches as whole vectors   120 CTAs 0.64, 150 0.73, 240 0.98, 300 1.23,
+//                  480 1.95, 640 1.33, 1260 2.88 (96->77 @23x104 x3 98 / 282 us)
+//   1x1  at most 16 channels   3060 0.79, 3864 0.86, 4725 1.15, 5640 1.24
+//        more           2560 0.29, 3570 0.64, 5220 0.86, 6400 1.19; without vectors 3840 0.84
 // 16-bit calls that the tensor cores would take behind a layout pass (two launches, 5 us and more): only where a warp's
-// share of the channels is short.  bf16, this kernel / the tensor cores:
-//   3x3, default layout  32->32 @32x32 5.5 / 8.5, 48->48 @40x40 8.8 / 8.9, 64->64 @40x40 11.2 / 8.0; channels last 30->32 @32x32 8.5 / 6.7
-//   1x1                  42->139 @30x9 x3 5.4 / 6.4, 64->64 @40x40 5.8 / 6.0, 16->32 @100x101 x2 10.3 / 7.0
+// share of the channels is short.  160 calls, by CTAs x channels per warp, this kernel / the tensor cores:
+//   3x3, default layout, up to 48 channels   280 0.52, 480 0.69, 594 0.89, 600 1.12, 702 1.08, 1024 1.73; channels last, up to 16  504 0.85, 1056 2.08
+//   1x1  at most 8 channels   360 0.64, 666 0.73, 750 1.07, 1302 1.56; up to 64, default layout   675 0.46, 1122 0.63, 1450 0.58, 1815 0.70, 1848 1.14;
+//        channels last  600 0.90, 936 1.20, 1188 0.95, 1440 1.19
 bool rtoss_few_eligible(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, bool repack) {
     if (p->ksize == 3 && p->Cin <= 4) return false;   // (stems have their own kernel)
     int lx, ly;
     const long long ctas = (long long)d->N * few_lanes((d->H - 1) / d->stride + 1, (d->W - 1) / d->stride + 1, &lx, &ly) * ((p->Cout + kFewCo - 1) / kFewCo);
     if (repack) {
         const long long steps = ctas * ((p->Cin + kFewWarps - 1) / kFewWarps);
-        return p->ksize == 3 ? p->Cin <= (d->layout == RTOSS_NCHW ? 48 : 16) && steps <= 1100 : p->Cin <= 64 && steps <= 2000;
+        return p->ksize == 3 ? p->Cin <= (d->layout == RTOSS_NCHW ? 48 : 16) && steps <= 600 : p->Cin <= 64 && steps <= (p->Cin <= 8 ? 700 : d->layout == RTOSS_NCHW ? 1800 : 1200);
     }
-    return ctas <= (p->ksize == 3 ? (few_vec(d, x) ? 4000 : 1600) : (few_vec(d, x) ? 5000 : 4000));
+    const bool vec = few_vec(d, x);
+    if (p->ksize == 1) return ctas <= (vec && p->Cin > 16 ? 5000 : 4200);
+    if (d->layout == RTOSS_NHWC && p->Cin % 8 == 0) return ctas <= 150;
+    if (p->Cin <= 16) return ctas <= (p->Cin <= 8 ? 800 : 1200);
+    return ctas <= (vec ? 4000 : d->layout == RTOSS_NHWC && d->io_dtype != RTOSS_F32 ? 1400 : 1600);
 }
 
 int rtoss_launch_conv_few(const rtoss_packed* p, const void* x, void* y, const rtoss_conv_desc* d, void* stream) {

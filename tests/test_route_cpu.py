@@ -18,6 +18,13 @@ CALLS = [
     ((100, 1024, 1024, 1, 3, rt.NHWC, BF16, 150, 8, rt.PATH_AUTO, BF16), rt.ROUTE_TENSOR_REPACKED),
     ((200, 1024, 1024, 1, 3, rt.NHWC, BF16, 150, 8, rt.PATH_AUTO, BF16), rt.ROUTE_STAGED),   # (a copy of more than 2^31 pieces of 16 bytes)
     ((200, 1024, 1024, 1, 3, rt.NCHW, BF16, 150, 8, rt.PATH_AUTO, BF16), rt.ROUTE_STAGED),
+    # where the few-outputs kernel was measured to be the slower one: one channel a warp, two a warp, pixels of whole vectors
+    ((2, 31, 72, 1, 3, rt.NCHW, F16, 5, 215, rt.PATH_FMA, F16), rt.ROUTE_STAGED),
+    ((2, 31, 72, 1, 3, rt.NCHW, F16, 17, 215, rt.PATH_FMA, F16), rt.ROUTE_FEW),
+    ((1, 120, 100, 1, 3, rt.NHWC, F32, 13, 100, rt.PATH_FMA, F32), rt.ROUTE_STAGED),
+    ((3, 23, 104, 1, 3, rt.NHWC, BF16, 96, 77, rt.PATH_FMA, BF16), rt.ROUTE_STAGED),
+    ((3, 23, 104, 1, 3, rt.NHWC, BF16, 97, 77, rt.PATH_FMA, BF16), rt.ROUTE_FEW),
+    ((14, 8, 28, 1, 3, rt.NCHW, F16, 6, 127, rt.PATH_AUTO, F16), rt.ROUTE_TENSOR_REPACKED),
     ((32, 80, 80, 1, 1, rt.NCHW, F32, 256, 256, rt.PATH_AUTO, F32), rt.ROUTE_STAGED),
 ]
 
