@@ -395,9 +395,10 @@ rtoss_status rtoss_chain_deps_spans(const uint64_t* spans, int n, uint32_t* afte
  * of 8): x is first written once as channels last, into stream-ordered memory of the context (at most 1 GiB of it is kept
  * between calls; rtoss_destroy gives it back; a call for which there is no memory runs on the FMA path), and y is written
  * in the layout asked for.  A call inside a stream capture allocates its copy at once, and the copy belongs to the graph:
- * the graph, its executables and its clones share it, it holds no allocation node, and the memory is freed when the
- * last of them is gone, by the next captured call of that kind or rtoss_destroy.  Such calls take no residual operand; RTOSS_PATH_TENSOR refuses them, RTOSS_PATH_FMA does
- * without the copy.
+ * the graph, its executables and its clones share it (so do calls that follow one another in the capture), it holds no
+ * allocation node, and the memory is freed when the last of them is gone, by the next captured call of that kind or
+ * rtoss_destroy.  Such calls take no residual operand; RTOSS_PATH_TENSOR refuses them, RTOSS_PATH_FMA does without
+ * the copy.
  *
  * Device-side waits of that path are bounded.  If one runs out, the kernel records a non-zero code in
  * the context and returns; rtoss_device_status synchronises the device, reports the code

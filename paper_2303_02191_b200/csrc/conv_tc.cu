@@ -832,11 +832,16 @@ int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, c
     const rtoss_conv_desc dd = repacked_desc(p, d);
     const int cp = rtoss_cin_pitch(p->Cin, p->dtype), S = dd.stride == d->stride ? 1 : 2;
     bool of_graph = false;
-    void* ws = rtoss_copy_get(ctx, (size_t)dd.N * dd.H * dd.W * cp * 2, stream, &of_graph);
+    size_t bytes = (size_t)dd.N * dd.H * dd.W * cp * 2;
+    void* ws = rtoss_copy_get(ctx, &bytes, stream, &of_graph);
     if (!ws) return -1;
     int e = rtoss_launch_repack16(x, ws, dd.N, p->Cin, cp, d->H, d->W, S, d->layout, stream);
     if (!e) e = launch_single(ctx, p, ws, y, &dd, true, stream);
-    const cudaError_t fe = of_graph ? cudaSuccess : cudaFreeAsync(ws, (cudaStream_t)stream);
+    if (of_graph) {
+        if (!e) rtoss_copy_read(ws, bytes, stream);
+        return e;
+    }
+    const cudaError_t fe = cudaFreeAsync(ws, (cudaStream_t)stream);
     return e ? e : (int)fe;
 }
 

@@ -139,8 +139,9 @@ rtoss_device_guard::~rtoss_device_guard() {
 // stream capture must not do that: allocation nodes would come into the caller's graph, which could then be instantiated
 // once only and be neither cloned nor a child of another graph.  Its copy is allocated at once and owned by the graph, through
 // a user object that the graph, its executables and its clones hold references to; when the last of them is gone and its
-// launches have finished, the copy joins a list, from which the next call that looks (a user object's destructor may not call
-// CUDA itself) gives it back to the pool.
+// launches have finished, the copy joins a list (a user object's destructor may not call CUDA itself), which the next captured
+// call or rtoss_destroy frees.  Calls that follow one another inside a capture share one copy's memory, as they do outside: a
+// network's graph holds as much as its largest layer needs, not the sum.
 namespace {
 
 struct GraphCopy {
@@ -207,6 +208,55 @@ cudaMemPool_t copy_pool(const rtoss_ctx* ctx) {
     return (cudaMemPool_t)ctx->pool;
 }
 
+// The copies last used inside captures: memory, its size, and the node of the convolution that read it.
+struct LastCopy {
+    unsigned long long capture;
+    cudaGraphNode_t reader;
+    void* mem;
+    size_t bytes;
+};
+std::mutex g_last_lock;
+LastCopy g_last[8];
+int g_last_next = 0;
+
+// Is `node` among `from` or the nodes in front of them?  (At most kLook nodes are looked at; beyond that: no.)
+bool behind(cudaGraphNode_t node, const cudaGraphNode_t* from, size_t n) {
+    constexpr size_t kLook = 64, kDeps = 8;
+    cudaGraphNode_t seen[kLook];
+    size_t n_seen = 0;
+    auto add = [&](cudaGraphNode_t v) {
+        for (size_t i = 0; i < n_seen; ++i)
+            if (seen[i] == v) return;
+        if (n_seen < kLook) seen[n_seen++] = v;
+    };
+    for (size_t i = 0; i < n; ++i) add(from[i]);
+    for (size_t i = 0; i < n_seen; ++i) {
+        if (seen[i] == node) return true;
+        cudaGraphNode_t deps[kDeps];
+        cudaGraphEdgeData edges[kDeps];
+        size_t n_deps = kDeps;
+        if (cudaGraphNodeGetDependencies_v2(seen[i], deps, edges, &n_deps) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        for (size_t j = 0; j < n_deps && j < kDeps; ++j) add(deps[j]);
+    }
+    return false;
+}
+
+// Memory of at least `*bytes` that an earlier call of this capture has done with: what is captured next comes behind its reader.
+void* done_with(unsigned long long capture, size_t* bytes, const cudaGraphNode_t* deps, size_t n_deps) {
+    std::lock_guard<std::mutex> hold(g_last_lock);
+    for (LastCopy& l : g_last)
+        if (l.mem && l.capture == capture && l.bytes >= *bytes && behind(l.reader, deps, n_deps)) {
+            void* mem = l.mem;
+            *bytes = l.bytes;
+            l.mem = nullptr;   // (until its new reader is known)
+            return mem;
+        }
+    return nullptr;
+}
+
 void* graph_copy(const rtoss_ctx* ctx, size_t bytes, cudaGraph_t graph) {
     collect_dead(ctx);
     void* mem = nullptr;
@@ -227,25 +277,47 @@ void* graph_copy(const rtoss_ctx* ctx, size_t bytes, cudaGraph_t graph) {
 
 }  // namespace
 
-void* rtoss_copy_get(const rtoss_ctx* ctx, size_t bytes, void* stream, bool* of_graph) {
+void* rtoss_copy_get(const rtoss_ctx* ctx, size_t* bytes, void* stream, bool* of_graph) {
     cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
     cudaGraph_t graph = nullptr;
     void* mem = nullptr;
     *of_graph = false;
-    if (cudaStreamGetCaptureInfo((cudaStream_t)stream, &status, nullptr, &graph) == cudaSuccess) {
+    unsigned long long capture = 0;
+    const cudaGraphNode_t* deps = nullptr;
+    const cudaGraphEdgeData* edges = nullptr;
+    size_t n_deps = 0;
+    if (cudaStreamGetCaptureInfo_v3((cudaStream_t)stream, &status, &capture, &graph, &deps, &edges, &n_deps) == cudaSuccess) {
         if (status == cudaStreamCaptureStatusNone) {
             cudaMemPool_t pool = copy_pool(ctx);
-            if (pool && cudaMallocFromPoolAsync(&mem, bytes, pool, (cudaStream_t)stream) != cudaSuccess) mem = nullptr;
+            if (pool && cudaMallocFromPoolAsync(&mem, *bytes, pool, (cudaStream_t)stream) != cudaSuccess) mem = nullptr;
         } else if (status == cudaStreamCaptureStatusActive) {
             cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (what happens here is no part of the capture)
             cudaThreadExchangeStreamCaptureMode(&mode);
-            mem = graph_copy(ctx, bytes, graph);
+            mem = done_with(capture, bytes, deps, n_deps);
+            if (!mem) mem = graph_copy(ctx, *bytes, graph);
             cudaThreadExchangeStreamCaptureMode(&mode);
             *of_graph = mem != nullptr;
         }
     }
     if (!mem) cudaGetLastError();
     return mem;
+}
+
+void rtoss_copy_read(void* mem, size_t bytes, void* stream) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    LastCopy l = {0, nullptr, mem, bytes};
+    const cudaGraphNode_t* deps = nullptr;
+    const cudaGraphEdgeData* edges = nullptr;
+    size_t n_deps = 0;
+    if (cudaStreamGetCaptureInfo_v3((cudaStream_t)stream, &status, &l.capture, nullptr, &deps, &edges, &n_deps) != cudaSuccess ||
+        status != cudaStreamCaptureStatusActive || n_deps != 1) {
+        cudaGetLastError();
+        return;
+    }
+    l.reader = deps[0];   // (what the next node of the stream comes behind: the convolution)
+    std::lock_guard<std::mutex> hold(g_last_lock);
+    g_last[g_last_next] = l;
+    g_last_next = (g_last_next + 1) % 8;
 }
 
 extern "C" {

@@ -149,7 +149,9 @@ bool rtoss_tc_repack_eligible(const rtoss_packed* p, const rtoss_conv_desc* d);
 int rtoss_launch_conv_tc_repacked(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                                   const rtoss_conv_desc* d, void* stream);
 // memory for such a copy, freed by the caller in stream order or (of_graph) with the graph being captured; null: none to be had
-void* rtoss_copy_get(const rtoss_ctx* ctx, size_t bytes, void* stream, bool* of_graph);
+// (*bytes: its size on return, for rtoss_copy_read)
+void* rtoss_copy_get(const rtoss_ctx* ctx, size_t* bytes, void* stream, bool* of_graph);
+void rtoss_copy_read(void* mem, size_t bytes, void* stream);   // of_graph: the kernel that reads the copy is what was captured last
 int rtoss_launch_repack16(const void* x, void* out, int N, int Cin, int cp, int H, int W, int S, rtoss_layout layout, void* stream);
 bool rtoss_tc_groupable(const rtoss_packed* p, const rtoss_conv_desc* d, const void* x, const void* y);
 // several independent convolutions in one launch: 0 = launched, -1 = the set cannot share a launch (nothing launched)

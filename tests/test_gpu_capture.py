@@ -70,6 +70,47 @@ def test_a_captured_call_leaves_the_graph_free():
     packed.close()
 
 
+def test_calls_of_a_capture_share_memory_only_in_order():
+    """Calls one behind the other (growing, shrinking, a foreign kernel between them) and calls on a second stream of the same
+    capture, which must not use the first one's copy while it is read: the results of calls one by one."""
+    c, N = gu.ctx(), 4
+    jobs = []
+    for i, (C, H, W) in enumerate([(64, 60, 62), (96, 120, 90), (64, 60, 62), (80, 100, 90), (96, 120, 90), (64, 60, 62)]):
+        packed = _layer(C, 72, 3)
+        x = torch.randn((N, C, H, W), device="cuda").to(torch.bfloat16)
+        y, want = (torch.zeros((N, 72, H, W), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        c.rtoss_conv3x3_pattern(packed, x, want, N, H, W)
+        jobs.append((packed, x, y, want, H, W))
+    other = torch.cuda.Stream()
+    z = torch.zeros(1 << 20, device="cuda")
+
+    def calls():
+        here = torch.cuda.current_stream()
+        for i, (packed, x, y, _, H, W) in enumerate(jobs):
+            if i % 3 == 2:
+                other.wait_stream(here)
+                with torch.cuda.stream(other):
+                    c.rtoss_conv3x3_pattern(packed, x, y, N, H, W)
+            else:
+                c.rtoss_conv3x3_pattern(packed, x, y, N, H, W)
+                z.add_(1)
+        here.wait_stream(other)
+
+    e = _instantiate(_capture(calls))
+    for _ in range(10):
+        for j in jobs:
+            j[2].zero_()
+        torch.cuda.synchronize()
+        _ok(cr.cudaGraphLaunch(e, torch.cuda.current_stream().cuda_stream))
+        torch.cuda.synchronize()
+        for j in jobs:
+            assert torch.equal(j[2], j[3])
+    _ok(cr.cudaGraphExecDestroy(e))
+    assert c.rtoss_device_status() == 0
+    for j in jobs:
+        j[0].close()
+
+
 def test_the_copies_come_back():
     c, N, C, H, W = rt.Context(0), 8, 64, 512, 512      # 256 MiB a copy
     packed = _layer(C, 16, 1)
@@ -87,5 +128,8 @@ def test_the_copies_come_back():
         torch.cuda.synchronize()
         _ok(cr.cudaGraphExecDestroy(e))
     assert free0 - torch.cuda.mem_get_info()[0] < 3 << 29       # (twelve copies are 3 GiB)
+    graph = _capture(lambda: [c.rtoss_conv1x1_pattern(packed, x, y, N, H, W) for _ in range(12)])
+    assert free0 - torch.cuda.mem_get_info()[0] < 3 << 29       # one behind the other: one copy
+    _ok(cr.cudaGraphDestroy(graph))
     packed.close()
     c.close()
