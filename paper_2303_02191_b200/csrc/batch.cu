@@ -2,12 +2,12 @@
 // of a model in two launches instead of three per layer.  The per-kernel arithmetic is the one of the single-layer
 // calls (select_core.cuh), so the results are the same bits.
 //
-//   batch_select_pack_kernel : two kernels / runs of nine per thread, 512 per block step; a block step ("chunk")
+//   batch_select_pack_kernel : two kernels / runs of nine per thread, 512 or 128 per block step; a block step ("chunk")
 //                              belongs to one layer and is described by a table built at plan time.
 //                              Writes the pattern id (caller's array and the handle's), the k kept values and the
 //                              tensor path's dense-expanded weights.
 //   batch_order_kernel       : per (3x3 layer, input channel) the stable order of filters by pattern id, sixteen
-//                              channels to a block, through a task -> layer table.
+//                              channels to a block or one to a warp, through a task -> layer table.
 //
 // A layer that inherits its parent's patterns (Section IV.A: children of a group share the parent's kernel
 // patterns) evaluates the selection on the PARENT's weights and packs its own with the result; it reads no other
@@ -28,8 +28,12 @@
 
 namespace {
 
-constexpr int kBatchThreads = 256;
-constexpr int kChunk = kBatchThreads * rtoss_dev::kPair;   // kernels per block step
+// Threads of a block, kPair kernels to a thread; a block step ("chunk") is that many kernels.  Models of at most two blocks of
+// 256 threads an SM are cut into blocks of 64: more SMs take part in the stores, and registers are left for four patterns in
+// flight.  Whole pass, blocks of 256 / of 64: 32x16 3x3 in fp32 13.2 / 7.8 us, 64x64 3x3 with 49 patterns 12.9 / 8.8, 512x256 1x1
+// 4.2 / 3.4, 256x256 3x3 with 49 patterns 16.5 / 14.3, 20 layers of 64x64 in fp32 (160 blocks of 256) 11.6 / 10.2.
+constexpr int kBatchThreads = 256, kSmallThreads = 64;
+__host__ __device__ constexpr int chunk_of(int threads) { return threads * rtoss_dev::kPair; }
 
 struct alignas(16) BatchLayer {
     const void* w;      // weights to pack
@@ -50,6 +54,7 @@ struct alignas(16) BatchLayer {
     int w_dtype, sel_dtype, v_dtype;
     unsigned chunk0;  // first chunk of this layer
     unsigned task0;   // first ordering task (3x3 layers)
+    int sixteens;     // how its channels are ordered (order_in_sixteens)
     uint16_t masks[256];
 };
 
@@ -61,21 +66,22 @@ struct BatchChunk {
 
 // 9*count weights of `count` consecutive kernels starting at kernel `first`, as raw bytes, coalesced; 16 bytes per
 // thread where the chunk is whole (a whole chunk is a multiple of 16 bytes and the base is 16-byte aligned).
+template <int T>
 __device__ __forceinline__ void stage_raw(const void* w, long long first, int count, int esize, unsigned char* smem) {
     const unsigned char* src = reinterpret_cast<const unsigned char*>(w) + (size_t)first * 9 * esize;
     const int bytes = count * 9 * esize;
-    if (count == kChunk) {
+    if (count == chunk_of(T)) {
         const uint4* s4 = reinterpret_cast<const uint4*>(src);
         uint4* d4 = reinterpret_cast<uint4*>(smem);
-        for (int i = threadIdx.x; i < bytes / 16; i += kBatchThreads) d4[i] = __ldg(s4 + i);
+        for (int i = threadIdx.x; i < bytes / 16; i += T) d4[i] = __ldg(s4 + i);
     } else if (esize == 4) {
         const uint32_t* s1 = reinterpret_cast<const uint32_t*>(src);
         uint32_t* d1 = reinterpret_cast<uint32_t*>(smem);
-        for (int i = threadIdx.x; i < bytes / 4; i += kBatchThreads) d1[i] = s1[i];
+        for (int i = threadIdx.x; i < bytes / 4; i += T) d1[i] = s1[i];
     } else {
         const uint16_t* s1 = reinterpret_cast<const uint16_t*>(src);
         uint16_t* d1 = reinterpret_cast<uint16_t*>(smem);
-        for (int i = threadIdx.x; i < bytes / 2; i += kBatchThreads) d1[i] = s1[i];
+        for (int i = threadIdx.x; i < bytes / 2; i += T) d1[i] = s1[i];
     }
 }
 
@@ -85,13 +91,14 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* g) {
 
 // Starts fetching a chunk: the layer's record (unless it is there already) and the weights its selection reads.  A ragged chunk's last bytes are plain
 // loads (16-bit weights: 2-byte pieces).
+template <int T>
 __device__ __forceinline__ void fetch_chunk(const BatchLayer* layers, const BatchChunk& c, BatchLayer* s_layer, unsigned char* raw) {
     const unsigned char* rec = reinterpret_cast<const unsigned char*>(layers + c.layer);
     if (s_layer)
-        for (int o = (int)threadIdx.x * 16; o < (int)sizeof(BatchLayer); o += kBatchThreads * 16) 
+        for (int o = (int)threadIdx.x * 16; o < (int)sizeof(BatchLayer); o += T * 16) 
             cp_async16(reinterpret_cast<unsigned char*>(s_layer) + o, rec + o);
     const int whole = (int)(c.bytes & ~15u);
-    for (int o = (int)threadIdx.x * 16; o < whole; o += kBatchThreads * 16) cp_async16(raw + o, c.src + o);
+    for (int o = (int)threadIdx.x * 16; o < whole; o += T * 16) cp_async16(raw + o, c.src + o);
     const int o = whole + (int)threadIdx.x * 2;
     if (o < (int)c.bytes) *reinterpret_cast<uint16_t*>(raw + o) = *reinterpret_cast<const uint16_t*>(c.src + o);
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -108,7 +115,7 @@ template <typename T> __device__ __forceinline__ float raw_at(const unsigned cha
     else return rtoss_dev::to_f32<T>(reinterpret_cast<const T*>(raw)[e]);
 }
 
-template <typename T>
+template <int kUnroll, typename T>
 __device__ __forceinline__ void select_chunk(const BatchLayer& L, long long first, int count, const unsigned char* raw, const rtoss_dev::PatternFactors* factors,
                                              uint8_t* s_pid, uint16_t* s_mask) {
     using namespace rtoss_dev;
@@ -117,7 +124,7 @@ __device__ __forceinline__ void select_chunk(const BatchLayer& L, long long firs
     f32x2 q[9];
     int best[kPair];
     load_pair<T>(raw, (int)threadIdx.x, q);
-    select_best2(q, L.masks, factors, L.P, best);
+    select_best2<kUnroll>(q, L.masks, factors, L.P, best);
     const long long i = first + base;
     const unsigned ids = (unsigned)best[0] | (unsigned)best[1] << 8;
     *reinterpret_cast<uint16_t*>(s_pid + base) = (uint16_t)ids;
@@ -165,14 +172,14 @@ template <typename V> __device__ __forceinline__ void put_one(V* at, int64_t lo_
     }
 }
 
-template <typename T, typename V>
+template <int kThreads, typename T, typename V>
 __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first, int count, const unsigned char* raw, const uint8_t* s_pid,
                                            const uint16_t* s_mask, const unsigned long long* s_taps) {
     using namespace rtoss_dev;
     V* val = reinterpret_cast<V*>(L.val) + first * L.k;   // (a chunk's first value is at a multiple of 512 k)
     if (sizeof(V) == 2 && L.k == 4) {
         // the usual case: a kernel's four values are one aligned 8-byte word
-        for (int g = (int)threadIdx.x; g < count; g += kBatchThreads) {
+        for (int g = (int)threadIdx.x; g < count; g += kThreads) {
             const unsigned taps = (unsigned)s_taps[s_pid[g]];
             const unsigned char* w = raw + (size_t)g * 9 * sizeof(T);
             uint2 u;
@@ -188,7 +195,7 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
             const int tap = (int)(s_taps[s_pid[g]] >> (4 * (o - g * k))) & 15;
             return raw_at<T>(raw, g * 9 + tap);
         };
-        for (int o = 2 * (int)threadIdx.x; o < n; o += 2 * kBatchThreads) {
+        for (int o = 2 * (int)threadIdx.x; o < n; o += 2 * kThreads) {
             const float a = value(o);
             if (o + 1 < n) {
                 const float b = value(o + 1);
@@ -270,9 +277,9 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
         // the flat matrix: four positions to a thread (a multiple of four: at most two kernels, one aligned word)
         const int n = count * 9;
         const bool words = cin_p == Cin && (tap_step & 3) == 0;   // (rows as long as the layer's; fp32 remainders aligned alike)
-        for (int e = 4 * (int)threadIdx.x; e < n; e += 4 * kBatchThreads) {
+        for (int e = 4 * (int)threadIdx.x; e < n; e += 4 * kThreads) {
             const int g = (int)(((unsigned)e * 7282u) >> 16);   // e / 9 (e is below 2^13)
-            const unsigned mm = ((unsigned)s_mask[g] | (unsigned)s_mask[min(g + 1, kChunk - 1)] << 9) >> (e - 9 * g);   // bit j: position e + j is kept
+            const unsigned mm = ((unsigned)s_mask[g] | (unsigned)s_mask[min(g + 1, chunk_of(kThreads) - 1)] << 9) >> (e - 9 * g);   // bit j: position e + j is kept
             const int64_t f = first * 9 + e;
             float v[4];
             if constexpr (sizeof(T) == 4) {
@@ -306,17 +313,19 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
 // Bound by instructions (0.75 a cycle and scheduler; 35 % of the copy rate).  32 M weights, 8 patterns of four taps: 131 us
 // with one kernel per thread that held its weights in registers through all outputs, 65 us in this form; 20 us instead of
 // 31 for 7 M.  (Prefetching the next chunk with a second buffer cost occupancy and was slower: 142 us on the older form.)
-__global__ void __launch_bounds__(kBatchThreads, 6) batch_select_pack_kernel(const BatchLayer* __restrict__ layers,
+template <int T>
+__global__ void __launch_bounds__(T, T == kBatchThreads ? 6 : 8) batch_select_pack_kernel(const BatchLayer* __restrict__ layers,
                                                                           const BatchChunk* __restrict__ chunks,
                                                                           unsigned n_chunks, int order_follows) {
     // The ordering kernel behind this one waits for the end of this grid and does not let its own successors start before
     // its end, so it may be set up meanwhile; no other kernel may be (a reader of handles does not wait).
     if (order_follows) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     rtoss_dev::pdl_enter_handle_writer();
-    __shared__ __align__(16) unsigned char raw[kChunk * 9 * 4];
+    constexpr int kStep = chunk_of(T), kUnroll = T == kBatchThreads ? 2 : 4;   // (patterns in flight: few warps have only themselves to overlap)
+    __shared__ __align__(16) unsigned char raw[kStep * 9 * 4];
     __shared__ BatchLayer s_layer;
-    __shared__ __align__(16) uint16_t s_mask[kChunk];
-    __shared__ __align__(16) uint8_t s_pid[kChunk];
+    __shared__ __align__(16) uint16_t s_mask[kStep];
+    __shared__ __align__(16) uint8_t s_pid[kStep];
     __shared__ rtoss_dev::PatternFactors s_factors[rtoss_dev::kFactorPatterns];
     __shared__ unsigned long long s_taps[256];   // a pattern's taps in ascending order, four bits each
     const unsigned per = n_chunks / gridDim.x, extra = n_chunks % gridDim.x;
@@ -326,43 +335,46 @@ __global__ void __launch_bounds__(kBatchThreads, 6) batch_select_pack_kernel(con
     uint32_t have = 0xFFFFFFFFu;   // which layer s_layer is
     for (unsigned chunk = begin; chunk < end; ++chunk) {
         const bool fresh = c.layer != have;
-        fetch_chunk(layers, c, fresh ? &s_layer : nullptr, raw);
+        fetch_chunk<T>(layers, c, fresh ? &s_layer : nullptr, raw);
         have = c.layer;
         c = chunks[min(chunk + 1, end - 1)];
         asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();
         const BatchLayer& L = s_layer;
-        const long long first = (long long)(chunk - L.chunk0) * kChunk;
-        const int count = (int)(L.n_kernels - first < kChunk ? L.n_kernels - first : kChunk);
+        const long long first = (long long)(chunk - L.chunk0) * kStep;
+        const int count = (int)(L.n_kernels - first < kStep ? L.n_kernels - first : kStep);
         // the layer's first chunk clears its issue words: the ordering kernel (next launch) ORs the bits in
         if (chunk == L.chunk0 && L.issue)
-            for (int i = threadIdx.x; i < L.issue_n; i += kBatchThreads) L.issue[i] = 0ull;
-        if (fresh && (int)threadIdx.x < L.P) {
-            const unsigned m = L.masks[threadIdx.x];
+            for (int i = threadIdx.x; i < L.issue_n; i += T) L.issue[i] = 0ull;
+#pragma unroll 1
+        for (int p0 = 0; p0 < 256; p0 += T) {
+            const int p = p0 + (int)threadIdx.x;
+            if (!fresh || p >= L.P) break;
+            const unsigned m = L.masks[p];
             unsigned long long taps = 0;
             int j = 0;
 #pragma unroll
             for (int t = 0; t < 9; ++t)
                 if (m & (1u << t)) taps |= (unsigned long long)t << (4 * j++);
-            s_taps[threadIdx.x] = taps;
-            if (threadIdx.x < rtoss_dev::kFactorPatterns) {
+            s_taps[p] = taps;
+            if (p < rtoss_dev::kFactorPatterns) {
 #pragma unroll
                 for (int t = 0; t < 10; ++t) {
                     const float f = (m >> t) & 1u ? 1.f : 0.f;   // (bit 9 is never set)
-                    s_factors[threadIdx.x].f[t] = rtoss_dev::pack_f32x2(f, f);
+                    s_factors[p].f[t] = rtoss_dev::pack_f32x2(f, f);
                 }
             }
         }
         if (fresh) __syncthreads();
-        if (L.sel_dtype == RTOSS_F32) select_chunk<float>(L, first, count, raw, s_factors, s_pid, s_mask);
-        else if (L.sel_dtype == RTOSS_BF16) select_chunk<__nv_bfloat16>(L, first, count, raw, s_factors, s_pid, s_mask);
-        else select_chunk<__half>(L, first, count, raw, s_factors, s_pid, s_mask);
+        if (L.sel_dtype == RTOSS_F32) select_chunk<kUnroll, float>(L, first, count, raw, s_factors, s_pid, s_mask);
+        else if (L.sel_dtype == RTOSS_BF16) select_chunk<kUnroll, __nv_bfloat16>(L, first, count, raw, s_factors, s_pid, s_mask);
+        else select_chunk<kUnroll, __half>(L, first, count, raw, s_factors, s_pid, s_mask);
         __syncthreads();
         if (L.w_sel != L.w) {   // the patterns are inherited: this layer's own weights take the buffer
-            stage_raw(L.w, first, count, L.w_dtype == RTOSS_F32 ? 4 : 2, raw);
+            stage_raw<T>(L.w, first, count, L.w_dtype == RTOSS_F32 ? 4 : 2, raw);
             __syncthreads();
         }
-#define RTOSS_PACK(T_, V_) pack_chunk<T_, V_>(L, first, count, raw, s_pid, s_mask, s_taps)
+#define RTOSS_PACK(T_, V_) pack_chunk<T, T_, V_>(L, first, count, raw, s_pid, s_mask, s_taps)
 #define RTOSS_PACK_TO(V_)                                       \
     if (L.w_dtype == RTOSS_F32) RTOSS_PACK(float, V_);          \
     else if (L.w_dtype == RTOSS_BF16) RTOSS_PACK(__nv_bfloat16, V_); \
@@ -377,28 +389,33 @@ __global__ void __launch_bounds__(kBatchThreads, 6) batch_select_pack_kernel(con
     rtoss_dev::handle_writer_done();
 }
 
-__global__ void __launch_bounds__(rtoss_dev::kOrderThreads, 4) batch_order_kernel(const BatchLayer* __restrict__ layers,
-                                                                             const uint32_t* __restrict__ task_layer, unsigned n_tasks) {
+// kSixteens: some layer is ordered sixteen channels to a block; else all go a channel to a warp, in blocks half the size.
+template <bool kSixteens>
+__global__ void __launch_bounds__(kSixteens ? rtoss_dev::kOrderThreads : rtoss_dev::kOrderWarps * 32, kSixteens ? 4 : 1)
+    batch_order_kernel(const BatchLayer* __restrict__ layers, const uint32_t* __restrict__ task_layer, unsigned n_tasks) {
     using namespace rtoss_dev;
-    __shared__ union {
-        struct {
-            uint32_t fill[kOrderThreads / 32][256];
-            uint16_t mask[kOrderThreads / 32][256];
-        } many;
-        OrderFew few;
-    } sh;
+    struct Many {
+        uint32_t fill[kOrderWarps][256];
+        uint16_t mask[kOrderWarps][256];
+    };
+    union Shared {
+        Many many;
+        typename std::conditional<kSixteens, OrderFew, Many>::type few;
+    };
+    __shared__ Shared sh;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // the first task's record is the plan's, which no kernel writes: it comes in ahead of the wait for the pattern ids
-    if (blockIdx.x < n_tasks) asm volatile("prefetch.global.L2 [%0];" ::"l"(layers + __ldg(task_layer + blockIdx.x)));
+    uint32_t layer = blockIdx.x < n_tasks ? __ldcg(task_layer + blockIdx.x) : 0u;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(layers + layer));
     pdl_enter_handle_writer();
     for (unsigned task = blockIdx.x; task < n_tasks; task += gridDim.x) {
-        const BatchLayer& L = layers[task_layer[task]];
-        const int ci0 = (int)(task - L.task0) * kOrderChannels, cb_log2 = L.v_dtype == RTOSS_F32 ? 5 : 6;
-        if (order_few(L.Cout, L.P)) {
-            order_channels_few(L.pid, L.Cout, L.Cin, L.P, ci0, L.perm, L.bucket_off, sh.few, L.masks, L.issue, cb_log2);
-        } else {
-            for (int ci = ci0 + warp; ci < min(ci0 + kOrderChannels, L.Cin); ci += kOrderThreads / 32)
-                order_channel(L.pid, L.Cout, L.Cin, L.P, ci, L.perm, L.bucket_off, sh.many.fill[warp], sh.many.mask[warp], lane, L.masks, L.issue, cb_log2);
+        if (task != blockIdx.x) layer = task_layer[task];
+        const BatchLayer& L = layers[layer];
+        const int ci0 = (int)(task - L.task0) * order_channels_of(L.sixteens != 0), cb_log2 = L.v_dtype == RTOSS_F32 ? 5 : 6;
+        if (kSixteens && L.sixteens) {
+            if constexpr (kSixteens) order_channels_few(L.pid, L.Cout, L.Cin, L.P, ci0, L.perm, L.bucket_off, sh.few, L.masks, L.issue, cb_log2);
+        } else if (warp < kOrderWarps && ci0 + warp < L.Cin) {
+            order_channel(L.pid, L.Cout, L.Cin, L.P, ci0 + warp, L.perm, L.bucket_off, sh.many.fill[warp], sh.many.mask[warp], lane, L.masks, L.issue, cb_log2);
         }
         __syncthreads();   // the shared arrays are free
     }
@@ -419,6 +436,8 @@ struct rtoss_batch {
     BatchChunk* chunks_dev;
     uint32_t* task_layer_dev;
     unsigned n_chunks, n_tasks;
+    int threads;     // of a block of the first kernel
+    bool sixteens;   // some layer's channels are ordered sixteen to a block
 };
 
 extern "C" {
@@ -433,6 +452,15 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
     std::vector<BatchLayer> layers((size_t)L);
     std::vector<BatchChunk> chunks;
     std::vector<uint32_t> task_layer;
+    long long kernels = 0, steps = 0;   // 3x3 kernels, which the ordering kernel sees; block steps of the first kernel, in large ones
+    bool sixteens = false;
+    for (int i = 0; i < L; ++i) {
+        const long long n = (long long)items[i].Cout * items[i].Cin / (items[i].ksize == 3 ? 1 : 9);   // (checked below)
+        kernels += items[i].ksize == 3 ? n : 0;
+        steps += (n + chunk_of(kBatchThreads) - 1) / chunk_of(kBatchThreads);
+    }
+    const int threads = steps <= 2 * ctx->sm_count ? kSmallThreads : kBatchThreads;
+    const long long chunk = chunk_of(threads);
     for (int i = 0; i < L; ++i) {
         const rtoss_batch_item& it = items[i];
         rtoss_packed* p = it.packed;
@@ -501,19 +529,22 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
         B.v_dtype = (int)p->dtype;
         memcpy(B.masks, it.masks_host, sizeof(uint16_t) * (size_t)it.P);
         B.chunk0 = (unsigned)chunks.size();
-        const long long nc = (p->n_kernels + kChunk - 1) / kChunk;
+        const long long nc = (p->n_kernels + chunk - 1) / chunk;
         if ((long long)chunks.size() + nc > 0x7FFFFFFFLL) {
             set_err(ctx, "model too large for one batch");
             return RTOSS_ERR_UNSUPPORTED;
         }
         const size_t kernel_bytes = 9 * (B.sel_dtype == RTOSS_F32 ? 4 : 2);
         for (long long c = 0; c < nc; ++c) {
-            const long long left = p->n_kernels - c * kChunk;
-            chunks.push_back(BatchChunk{static_cast<const unsigned char*>(B.w_sel) + (size_t)c * kChunk * kernel_bytes,
-                                        (unsigned)((left < kChunk ? left : kChunk) * (long long)kernel_bytes), (unsigned)i});
+            const long long left = p->n_kernels - c * chunk;
+            chunks.push_back(BatchChunk{static_cast<const unsigned char*>(B.w_sel) + (size_t)c * chunk * kernel_bytes,
+                                        (unsigned)((left < chunk ? left : chunk) * (long long)kernel_bytes), (unsigned)i});
         }
+        B.sixteens = rtoss_dev::order_in_sixteens(it.Cout, it.P, kernels) ? 1 : 0;
+        const int per = rtoss_dev::order_channels_of(B.sixteens != 0);
+        sixteens = sixteens || (it.ksize == 3 && B.sixteens);
         B.task0 = (unsigned)task_layer.size();
-        if (it.ksize == 3) task_layer.insert(task_layer.end(), (size_t)((it.Cin + rtoss_dev::kOrderChannels - 1) / rtoss_dev::kOrderChannels), (uint32_t)i);
+        if (it.ksize == 3) task_layer.insert(task_layer.end(), (size_t)((it.Cin + per - 1) / per), (uint32_t)i);
     }
     rtoss_batch* b = new (std::nothrow) rtoss_batch();
     if (!b) return RTOSS_ERR_ALLOC;
@@ -522,9 +553,15 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
     b->L = L;
     b->n_chunks = (unsigned)chunks.size();
     b->n_tasks = (unsigned)task_layer.size();
+    b->sixteens = sixteens;
+    b->threads = threads;
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(ctx->device);
+    rtoss_dev::rtoss_writers_carveout(batch_select_pack_kernel<kSmallThreads>);
+    rtoss_dev::rtoss_writers_carveout(batch_select_pack_kernel<kBatchThreads>);
+    rtoss_dev::rtoss_writers_carveout(batch_order_kernel<false>);
+    rtoss_dev::rtoss_writers_carveout(batch_order_kernel<true>);
     cudaError_t e = cudaMalloc((void**)&b->layers_dev, sizeof(BatchLayer) * (size_t)L);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->chunks_dev, sizeof(BatchChunk) * (chunks.size() + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->task_layer_dev, sizeof(uint32_t) * (task_layer.size() + 1));
@@ -563,16 +600,21 @@ rtoss_status rtoss_batch_select_pack(rtoss_ctx* ctx, const rtoss_batch* b, void*
     cudaStream_t s = (cudaStream_t)cuda_stream;
     cudaError_t e = cudaSuccess;
     const unsigned cap = (unsigned)ctx->sm_count * 8u;
-    if (b->n_chunks) {
+    if (b->n_chunks && b->threads == kSmallThreads) {
+        e = rtoss_dev::launch_pdl(batch_select_pack_kernel<kSmallThreads>, b->n_chunks, kSmallThreads, 0, s, (const BatchLayer*)b->layers_dev,
+                                  (const BatchChunk*)b->chunks_dev, b->n_chunks, (int)(b->n_tasks != 0));
+    } else if (b->n_chunks) {
         const unsigned resident = (unsigned)ctx->sm_count * 6u;   // (what the kernel's launch bounds allow)
         const unsigned grid = b->n_chunks < resident ? b->n_chunks : resident;
-        e = rtoss_dev::launch_pdl(batch_select_pack_kernel, grid, kBatchThreads, 0, s, (const BatchLayer*)b->layers_dev,
+        e = rtoss_dev::launch_pdl(batch_select_pack_kernel<kBatchThreads>, grid, kBatchThreads, 0, s, (const BatchLayer*)b->layers_dev,
                                   (const BatchChunk*)b->chunks_dev, b->n_chunks, (int)(b->n_tasks != 0));
     }
     if (e == cudaSuccess && b->n_tasks) {
         const unsigned grid = b->n_tasks < cap ? b->n_tasks : cap;
-        e = rtoss_dev::launch_pdl(batch_order_kernel, grid, rtoss_dev::kOrderThreads, 0, s, (const BatchLayer*)b->layers_dev,
-                                  (const uint32_t*)b->task_layer_dev, b->n_tasks);
+        e = b->sixteens ? rtoss_dev::launch_pdl(batch_order_kernel<true>, grid, rtoss_dev::kOrderThreads, 0, s, (const BatchLayer*)b->layers_dev,
+                                                (const uint32_t*)b->task_layer_dev, b->n_tasks)
+                        : rtoss_dev::launch_pdl(batch_order_kernel<false>, grid, rtoss_dev::kOrderWarps * 32, 0, s, (const BatchLayer*)b->layers_dev,
+                                                (const uint32_t*)b->task_layer_dev, b->n_tasks);
     }
     if (e != cudaSuccess) {
         cudaGetLastError();

@@ -88,7 +88,19 @@ __device__ __forceinline__ void pdl_enter() {
 }
 
 __device__ __forceinline__ void pdl_enter_handle_writer() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void handle_writer_done() { __threadfence(); }
+// (All threads of the block: the barrier hands their writes to the thread whose fence then covers them all.)
+__device__ __forceinline__ void handle_writer_done() {
+    __syncthreads();
+    if (threadIdx.x == 0) asm volatile("fence.acq_rel.gpu;" ::: "memory");
+}
+
+// The kernels that write handles follow one another in pairs whose shared memory differs (6 to 46 KB a block).  An SM that has
+// to move the line between its shared memory and its L1 first runs empty, which cost 5 us between two of them: all of them
+// ask for the same line (a hint; set per device, before the first launch).
+template <typename... KArgs>
+inline void rtoss_writers_carveout(void (*kern)(KArgs...)) {
+    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+}
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

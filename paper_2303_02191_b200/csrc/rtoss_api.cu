@@ -520,11 +520,10 @@ rtoss_status rtoss_pack(rtoss_ctx* ctx, const void* w_dev, rtoss_dtype w_dtype, 
     if (masks_changed) e = cudaMemcpyAsync(p->masks_dev, p->masks, sizeof(uint16_t) * 256, cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess)  // also writes the handle's own copy of the ids and the tensor path's dense-expanded weights
         le = rtoss_launch_pack_values(w_dev, w_dtype, p->n_kernels, make_table(masks_host, P), pid_dev, k, p->val,
-                                      compute_dtype, p->pid, p->wtc, ksize, Cout, Cin, cuda_stream);
+                                      compute_dtype, p->pid, p->wtc, ksize, Cout, Cin, p->issue, p->issue_n, cuda_stream);
     // The ordering pass reads the handle's copy of the ids, which pack_values has just written: it loads words of four and sixteen
     // ids, and the caller's array may start at any byte.
-    // It also gathers which (tap, channel slab) pairs of every filter tile hold kept weights; its words start at zero.
-    if (e == cudaSuccess && !le && p->issue) e = cudaMemsetAsync(p->issue, 0, sizeof(unsigned long long) * (size_t)p->issue_n, s);
+    // It also gathers which (tap, channel slab) pairs of every filter tile hold kept weights (pack_values cleared the words).
     if (e == cudaSuccess && !le && ksize == 3)
         le = rtoss_launch_pack_order(p->pid, Cout, Cin, P, p->perm, p->bucket_off, p->masks_dev, p->issue,
                                      rtoss_issue_cb_log2(compute_dtype), cuda_stream);

@@ -116,6 +116,7 @@ int rtoss_launch_select(const void* w, rtoss_dtype wdt, int64_t n_kernels, const
                         void* stream);
 int rtoss_launch_pack_values(const void* w, rtoss_dtype wdt, int64_t n_kernels, const MaskTable& t, const uint8_t* pid,
                              int k, void* val, rtoss_dtype vdt, uint8_t* pid_copy, void* wtc, int ksize, int Cout, int Cin,
+                             unsigned long long* issue, int issue_n,
                              void* stream);
 int rtoss_launch_pack_order(const uint8_t* pid, int Cout, int Cin, int P, uint32_t* perm, uint32_t* bucket_off,
                             const uint16_t* masks_dev, unsigned long long* issue, int cb_log2, void* stream);

@@ -175,7 +175,7 @@ struct __align__(16) PatternFactors {
 // A sum is nine fused multiply-adds with the pattern's factors: fma(1, q, s) is q + s rounded once and fma(0, q, s) is s,
 // as long as no square is infinite or not a number -- such a pair takes the loop of predicated additions, and so do
 // tables of more than kFactorPatterns patterns.  (Testing nine mask bits per pattern took 47 instructions per pattern and pair.)
-template <typename Tab>
+template <int kUnroll, typename Tab>
 __device__ __forceinline__ void select_best2(f32x2 (&q)[9], const Tab& tab, const PatternFactors* factors, int P, int (&best)[kPair]) {
     float best_s[kPair] = {-1.f, -1.f};
     best[0] = best[1] = 0;
@@ -188,7 +188,7 @@ __device__ __forceinline__ void select_best2(f32x2 (&q)[9], const Tab& tab, cons
     unpack_f32x2(all, a, b);
     const float inf = __int_as_float(0x7F800000);
     if (P <= kFactorPatterns && a < inf && b < inf) {
-#pragma unroll 2
+#pragma unroll kUnroll
         for (int p = 0; p < P; ++p) {
             const ulonglong2* f = reinterpret_cast<const ulonglong2*>(factors[p].f);
             f32x2 s = 0;
@@ -345,7 +345,18 @@ struct OrderFew {
     uint16_t list[kOrderChannels][kFewFilters + 2];
     uint16_t masks[kFewPatterns];
 };
-__device__ __forceinline__ bool order_few(int Cout, int P) { return Cout <= kFewFilters && P <= kFewPatterns; }
+// Which form: kernels = how many the launch orders in all.  Barriers and walks of the form of sixteens take 7 us however little
+// there is to sort (ordering kernel alone; a warp for each channel 4.5 us at 64 filters, 18 at 600): it is for layers of more
+// than 128 filters and for launches whose instructions count.  Whole pass, sixteens / warps: 50 layers of 16x32 (25 600 kernels) 8.8 / 7.3 us,
+// 5 of 40x300 (60 000) 10.3 / 9.4, 20 of 64x64 (81 920) 8.9 / 9.0, 12 of 100x200 (240 000) 11.5 / 15.3.  Layers that fit neither limit: a warp each
+// (600x64: 28.7 us with two channels to each of eight warps of a block, 14.6 with one to each of four).
+constexpr int kManyKernels = 80000;
+inline __host__ __device__ bool order_in_sixteens(int Cout, int P, long long kernels) {
+    return Cout <= kFewFilters && P <= kFewPatterns && (Cout > 128 || kernels > kManyKernels);
+}
+// Channels to a block: sixteen, or one to each of four warps.
+constexpr int kOrderWarps = 4;
+inline __host__ __device__ int order_channels_of(bool sixteens) { return sixteens ? kOrderChannels : kOrderWarps; }
 
 // All threads of the block; `masks` as the device sees the table (global or shared).
 __device__ __forceinline__ void order_channels_few(const uint8_t* __restrict__ pid, int Cout, int Cin, int P, int ci0,

@@ -82,8 +82,10 @@ __global__ void __launch_bounds__(kSelThreads) pack_values_kernel(const T* __res
                                                                   MaskTable table, const uint8_t* pid, int k,
                                                                   V* __restrict__ val, uint8_t* pid_copy,
                                                                   V* __restrict__ wtc, int ksize, int Cin,
-                                                                  rtoss_wtc_layout lay) {
+                                                                  rtoss_wtc_layout lay, unsigned long long* __restrict__ issue, int issue_n) {
     rtoss_dev::pdl_enter_handle_writer();
+    // the ordering pass (next launch) ORs its bits into the issue words (a memset in front cost a launch, 1.9 us of a call's 10.4)
+    for (int i = blockIdx.x * kSelThreads + threadIdx.x; i < issue_n; i += gridDim.x * kSelThreads) issue[i] = 0ull;
     __shared__ __align__(16) T sw[kSelThreads * 9];
     const int64_t n_chunks = (n_kernels + kSelThreads - 1) / kSelThreads;
     for (int64_t chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
@@ -105,28 +107,22 @@ __global__ void __launch_bounds__(kSelThreads) pack_values_kernel(const T* __res
     rtoss_dev::handle_writer_done();
 }
 
-// Per input channel: stable counting sort of the filters by pattern id, kOrderChannels per block.
-__global__ void __launch_bounds__(rtoss_dev::kOrderThreads, 4) pack_order_kernel(const uint8_t* __restrict__ pid, int Cout, int Cin,
-                                                                            int P, uint32_t* __restrict__ perm,
-                                                                            uint32_t* __restrict__ bucket_off,
-                                                                            const uint16_t* __restrict__ masks,
-                                                                            unsigned long long* __restrict__ issue, int cb_log2) {
+// Per input channel: stable counting sort of the filters by pattern id, in one of two forms (order_in_sixteens).
+template <bool kSixteens>
+__global__ void __launch_bounds__(kSixteens ? rtoss_dev::kOrderThreads : rtoss_dev::kOrderWarps * 32, kSixteens ? 4 : 1)
+    pack_order_kernel(const uint8_t* __restrict__ pid, int Cout, int Cin, int P, uint32_t* __restrict__ perm, uint32_t* __restrict__ bucket_off,
+                      const uint16_t* __restrict__ masks, unsigned long long* __restrict__ issue, int cb_log2) {
     using namespace rtoss_dev;
     pdl_enter_handle_writer();
-    __shared__ union {
-        struct {
-            uint32_t fill[kOrderThreads / 32][256];
-            uint16_t mask[kOrderThreads / 32][256];
-        } many;
-        OrderFew few;
-    } sh;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int ci0 = blockIdx.x * kOrderChannels;
-    if (order_few(Cout, P)) {
-        order_channels_few(pid, Cout, Cin, P, ci0, perm, bucket_off, sh.few, masks, issue, cb_log2);
+    const int ci0 = blockIdx.x * order_channels_of(kSixteens);
+    if constexpr (kSixteens) {
+        __shared__ OrderFew few;
+        order_channels_few(pid, Cout, Cin, P, ci0, perm, bucket_off, few, masks, issue, cb_log2);
     } else {
-        for (int ci = ci0 + warp; ci < min(ci0 + kOrderChannels, Cin); ci += kOrderThreads / 32)
-            order_channel(pid, Cout, Cin, P, ci, perm, bucket_off, sh.many.fill[warp], sh.many.mask[warp], lane, masks, issue, cb_log2);
+        __shared__ uint32_t fill[kOrderWarps][256];
+        __shared__ uint16_t mask[kOrderWarps][256];
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        if (ci0 + warp < Cin) order_channel(pid, Cout, Cin, P, ci0 + warp, perm, bucket_off, fill[warp], mask[warp], lane, masks, issue, cb_log2);
     }
     handle_writer_done();
 }
@@ -271,40 +267,66 @@ int rtoss_launch_select(const void* w, rtoss_dtype wdt, int64_t n_kernels, const
     return (int)cudaGetLastError();
 }
 
+// Once per device (see rtoss_writers_carveout).
+template <typename T>
+static void prepare_pack_of() {
+    rtoss_dev::rtoss_writers_carveout(pack_values_kernel<T, float>);
+    rtoss_dev::rtoss_writers_carveout(pack_values_kernel<T, __nv_bfloat16>);
+    rtoss_dev::rtoss_writers_carveout(pack_values_kernel<T, __half>);
+}
+static void prepare_pack() {
+    static std::atomic<bool> done[64];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev].load(std::memory_order_acquire)) return;
+    prepare_pack_of<float>();
+    prepare_pack_of<__nv_bfloat16>();
+    prepare_pack_of<__half>();
+    rtoss_dev::rtoss_writers_carveout(pack_order_kernel<false>);
+    rtoss_dev::rtoss_writers_carveout(pack_order_kernel<true>);
+    done[dev].store(true, std::memory_order_release);
+}
+
 template <typename T>
 static int launch_pack_values_t(const T* w, int64_t n, const MaskTable& t, const uint8_t* pid, int k, void* val,
-                                rtoss_dtype vdt, uint8_t* pid_copy, void* wtc, int ksize, int Cin, rtoss_wtc_layout lay, cudaStream_t s) {
+                                rtoss_dtype vdt, uint8_t* pid_copy, void* wtc, int ksize, int Cin, rtoss_wtc_layout lay, unsigned long long* issue, int issue_n,
+                                cudaStream_t s) {
     const int grid = grid_for((n + kSelThreads - 1) / kSelThreads);
     switch (vdt) {
-        case RTOSS_F32: rtoss_dev::launch_pdl(pack_values_kernel<T, float>, grid, kSelThreads, 0, s, w, n, t, pid, k, (float*)val, pid_copy, (float*)wtc, ksize, Cin, lay); break;
+        case RTOSS_F32: rtoss_dev::launch_pdl(pack_values_kernel<T, float>, grid, kSelThreads, 0, s, w, n, t, pid, k, (float*)val, pid_copy, (float*)wtc, ksize, Cin, lay, issue, issue_n); break;
         case RTOSS_BF16:
-            rtoss_dev::launch_pdl(pack_values_kernel<T, __nv_bfloat16>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__nv_bfloat16*)val, pid_copy, (__nv_bfloat16*)wtc, ksize, Cin, lay);
+            rtoss_dev::launch_pdl(pack_values_kernel<T, __nv_bfloat16>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__nv_bfloat16*)val, pid_copy, (__nv_bfloat16*)wtc, ksize, Cin, lay, issue, issue_n);
             break;
-        case RTOSS_F16: rtoss_dev::launch_pdl(pack_values_kernel<T, __half>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__half*)val, pid_copy, (__half*)wtc, ksize, Cin, lay); break;
+        case RTOSS_F16: rtoss_dev::launch_pdl(pack_values_kernel<T, __half>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__half*)val, pid_copy, (__half*)wtc, ksize, Cin, lay, issue, issue_n); break;
     }
     return (int)cudaGetLastError();
 }
 
 int rtoss_launch_pack_values(const void* w, rtoss_dtype wdt, int64_t n_kernels, const MaskTable& t, const uint8_t* pid,
                              int k, void* val, rtoss_dtype vdt, uint8_t* pid_copy, void* wtc, int ksize, int Cout, int Cin,
-                             void* stream) {
+                             unsigned long long* issue, int issue_n, void* stream) {
     const rtoss_wtc_layout lay = rtoss_wtc_layout_of(Cout, Cin, ksize, vdt);
     if (n_kernels <= 0) return 0;
+    prepare_pack();
     cudaStream_t s = (cudaStream_t)stream;
     switch (wdt) {
-        case RTOSS_F32: return launch_pack_values_t<float>((const float*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, s);
+        case RTOSS_F32: return launch_pack_values_t<float>((const float*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, issue, issue_n, s);
         case RTOSS_BF16:
-            return launch_pack_values_t<__nv_bfloat16>((const __nv_bfloat16*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, s);
-        case RTOSS_F16: return launch_pack_values_t<__half>((const __half*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, s);
+            return launch_pack_values_t<__nv_bfloat16>((const __nv_bfloat16*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, issue, issue_n, s);
+        case RTOSS_F16: return launch_pack_values_t<__half>((const __half*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, issue, issue_n, s);
     }
     return (int)cudaErrorInvalidValue;
 }
 
 int rtoss_launch_pack_order(const uint8_t* pid, int Cout, int Cin, int P, uint32_t* perm, uint32_t* bucket_off,
                             const uint16_t* masks_dev, unsigned long long* issue, int cb_log2, void* stream) {
-    const int grid = (Cin + rtoss_dev::kOrderChannels - 1) / rtoss_dev::kOrderChannels;
-    rtoss_dev::launch_pdl(pack_order_kernel, grid, rtoss_dev::kOrderThreads, 0, (cudaStream_t)stream, pid, Cout, Cin, P, perm, bucket_off,
-                          masks_dev, issue, cb_log2);
+    const bool sixteens = rtoss_dev::order_in_sixteens(Cout, P, (long long)Cout * Cin);
+    const int per = rtoss_dev::order_channels_of(sixteens), grid = (Cin + per - 1) / per;
+    if (sixteens)
+        rtoss_dev::launch_pdl(pack_order_kernel<true>, grid, rtoss_dev::kOrderThreads, 0, (cudaStream_t)stream, pid, Cout, Cin, P, perm, bucket_off, masks_dev,
+                              issue, cb_log2);
+    else
+        rtoss_dev::launch_pdl(pack_order_kernel<false>, grid, rtoss_dev::kOrderWarps * 32, 0, (cudaStream_t)stream, pid, Cout, Cin, P, perm, bucket_off,
+                              masks_dev, issue, cb_log2);
     return (int)cudaGetLastError();
 }
 
