@@ -465,7 +465,8 @@ rtoss_status rtoss_fma_plan3x3(const rtoss_conv_desc* desc, int Cin, int Cout, i
 /* The tensor path's tiling of a call, host arithmetic only (nothing is launched, no device is touched): what the
  * launcher of a single call would choose for a layer of this shape on a device of sm_count SMs (0: 148).  desc gives N,
  * H, W, stride, layout and whether there is a residual operand (any non-null residual_dev; it is not dereferenced).
- * (1x1 calls of stride 1 on channels-last images run as ONE image of one row of N*H*W pixels: ask for that to see them cut.)
+ * 1x1 calls of stride 1 are cut as one image of one row of N*H*W pixels.  Where all weights of a tile stay in shared memory
+ * while a CTA walks its tiles, weight_stages is their number of stages (it may be 1).
  * eligible = 0 when the tensor path does not take the shape (then the rest is zero).  Lets the CPU tests check the
  * planner's invariants -- shared memory within an SM's, at most 256 positions and 256 box elements per dimension,
  * stage sizes multiples of the swizzle atom -- and shows how a layer is cut.  Not part of the paper's method.

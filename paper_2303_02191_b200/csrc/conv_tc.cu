@@ -637,6 +637,19 @@ bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rto
     return true;
 }
 
+// Weights that fit beside three activation stages (or the plan's own number) stay in shared memory while a CTA walks its tiles:
+// bf16 1x1 64->64 @160x160 x16 24.7 -> 23.7 us, 128->512 @100x136 x4 16.2 -> 15.9, 3x3 24->24 @100x100 x16 (rows of 48 bytes, which
+// weight copies take slowly) 30.2 -> 15.9; with two stages 512->256 @100x136 x4 16.4 -> 22.4.
+// stages: weight stages of a tile; ct: filter tiles.  Gives the activation stages and the CTAs (a multiple of ct: each keeps its
+// filter tile from tile to tile).
+static bool resident_rings(const TcPlan& plan, int a_stage, int b_stage, int stages, int ct, size_t units, int sms, int* na, unsigned* ctas) {
+    const int fixed = plan.smem - plan.NA * a_stage - plan.NB * b_stage, room = (227 * 1024 - 64 - fixed - stages * b_stage) / a_stage;
+    const unsigned grid = (unsigned)(units < (size_t)sms ? units : (size_t)sms), even = grid - grid % (unsigned)ct;
+    *na = room < kMaxA ? room : kMaxA;
+    *ctas = even;
+    return stages <= kMaxB && *na >= 2 && (*na >= 3 || *na >= plan.NA) && even > 0 && units > (size_t)even && (units + even - 1) / even == (units + grid - 1) / grid;
+}
+
 extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize, int Cin, int Cout, rtoss_dtype dtype, int sm_count,
                                             rtoss_tensor_plan* out) {
     if (!d || !out || (ksize != 1 && ksize != 3) || Cin < 1 || Cout < 1 || (int)dtype < 0 || (int)dtype > 2 || d->N < 1 || d->H < 1 ||
@@ -653,7 +666,8 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     const int w_rows = pxm ? round_up(Cout, 16) : kMTile;
     const int row_bytes = row_bytes_of(p);
     TcPlan plan;
-    if (!plan_tc(plan_key(p, d, sms, -1), &plan)) return RTOSS_OK;
+    const rtoss_conv_desc row = row_form(p, d);
+    if (!plan_tc(plan_key(p, &row, sms, -1), &plan)) return RTOSS_OK;
     out->eligible = 1;
     out->rows_per_tile = plan.TH, out->cols_per_tile = plan.TW, out->pitch = plan.Wq, out->positions = plan.N_px;
     out->act_stages = plan.NA, out->weight_stages = plan.NB, out->taps_per_weight_stage = plan.G;
@@ -665,6 +679,15 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     out->positions_on_m = pxm ? 1 : 0;
     out->tiles = (int)(plan.tiles > 0x7FFFFFFF ? 0x7FFFFFFF : plan.tiles);
     out->split_k = plan.KS;
+    if (plan.KS == 1) {
+        const int stages = ncb_of(p) * ((ksize == 3 ? 9 : 1) * (f32 ? 2 : 1) / plan.G);
+        int na;
+        unsigned ctas;
+        if (resident_rings(plan, out->act_stage_bytes, out->weight_stage_bytes, stages, pxm ? 1 : (Cout + kMTile - 1) / kMTile, (size_t)plan.tiles, sms, &na, &ctas)) {
+            out->shared_bytes += (na - plan.NA) * out->act_stage_bytes + (stages - plan.NB) * out->weight_stage_bytes;
+            out->act_stages = na, out->weight_stages = stages;
+        }
+    }
     return RTOSS_OK;
 }
 
@@ -754,16 +777,13 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     dim3 grid((unsigned)(n_units < (size_t)sms ? n_units : (size_t)sms));
     int smem_need = plan.smem;
     if (a.KS == 1) {
-        // Weights that fit beside three activation stages (or the plan's own number) stay in shared memory while a CTA walks
-        // its tiles: bf16 1x1 64->64 @160x160 x16 24.7 -> 23.7 us, 128->512 @100x136 x4 16.2 -> 15.9, 3x3 24->24 @100x100 x16
-        // (rows of 48 bytes, which weight copies take slowly) 30.2 -> 15.9; with two stages 512->256 @100x136 x4 16.4 -> 22.4.
-        const int stages = a.ncb * (a.taps / a.G), ct = pxm_tiles(a);
-        const int fixed = plan.smem - plan.NA * (int)a.a_stage - plan.NB * (int)a.b_stage;
-        const int na_room = (227 * 1024 - 64 - fixed - stages * (int)a.b_stage) / (int)a.a_stage, na = na_room < kMaxA ? na_room : kMaxA;
-        const unsigned even = grid.x - grid.x % (unsigned)ct;   // CTAs that keep their filter tile from tile to tile
-        if (stages <= kMaxB && na >= 2 && (na >= 3 || na >= plan.NA) && even > 0 && n_units > (size_t)even && (n_units + even - 1) / even == (n_units + grid.x - 1) / grid.x) {
+        const int stages = a.ncb * (a.taps / a.G);
+        int na;
+        unsigned even;
+        if (resident_rings(plan, (int)a.a_stage, (int)a.b_stage, stages, pxm_tiles(a), n_units, sms, &na, &even)) {
             a.resident = 1;
             grid.x = even;
+            smem_need = plan.smem + (na - plan.NA) * (int)a.a_stage + (stages - plan.NB) * (int)a.b_stage;
             a.NA = na;
             a.NB = stages;
             a.sB_off = (unsigned)a.NA * a.a_stage;
@@ -772,7 +792,6 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
             g.ring_bytes = rings + (d->residual_dev ? kEpiWarps * kResStage : 0);
             g.max_na = a.NA;
             g.max_nb = a.NB;
-            smem_need = rings + fixed;
         }
     }
     // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM

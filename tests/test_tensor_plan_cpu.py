@@ -18,6 +18,8 @@ def check(N, H, W, S, ks, Cin, Cout, dt, residual=False):
     if not p.eligible:
         return p
     Ho, Wo = synth.out_hw(H, W, S)
+    if ks == 1 and S == 1:      # cut as one row of all pixels
+        N, Ho, Wo = 1, 1, N * H * W
     halo = (2 if S == 1 else 1) if ks == 3 else 0
     assert p.shared_bytes <= CAP
     assert 16 <= p.positions <= 256 and p.positions % 16 == 0
@@ -29,7 +31,10 @@ def check(N, H, W, S, ks, Cin, Cout, dt, residual=False):
     # stage sizes are multiples of the swizzle atom (8 rows), so every stage starts on an atom boundary
     assert p.act_stage_bytes % (8 * p.row_bytes) == 0 and p.weight_stage_bytes % (8 * p.row_bytes) == 0
     assert p.sub_tiles == (4 if (ks == 3 and S == 2) else 1)
-    assert 1 <= p.act_stages <= 4 and 2 <= p.weight_stages <= 8
+    assert 1 <= p.act_stages <= 4 and 1 <= p.weight_stages <= 8
+    if p.weight_stages < 2:     # all weights of a tile stay in shared memory: its one stage, and more tiles than CTAs
+        ncb_ = -(-Cin // (p.row_bytes // es))
+        assert ncb_ * (ks * ks * (2 if dt == F32 else 1) // p.taps_per_weight_stage) == 1 and p.tiles > 148 - 148 % (1 if p.positions_on_m else -(-Cout // 128))
     assert p.taps_per_weight_stage in ((1, 3) if ks == 3 else (1,))
     assert p.act_stages * p.act_stage_bytes + p.weight_stages * p.weight_stage_bytes < p.shared_bytes
     # the tiles cover the output
@@ -70,6 +75,24 @@ def test_ineligible_shapes_and_bad_arguments():
     for bad in ((0, 8, 8, 1, 3, 64, 64), (1, 8, 8, 3, 3, 64, 64), (1, 8, 8, 1, 2, 64, 64), (1, 8, 8, 1, 3, 0, 64)):
         with pytest.raises(rt.RtossError):
             rt.rtoss_tensor_plan_of(*bad, BF16)
+
+
+@pytest.mark.parametrize("N,H,W", [(1, 1, 1), (1, 20, 20), (4, 50, 68), (3, 7, 300), (16, 160, 160), (2, 5, 700)])
+@pytest.mark.parametrize("Cin,Cout", [(64, 64), (256, 1024), (72, 200), (2048, 512)])
+def test_rows_of_all_pixels(N, H, W, Cin, Cout):
+    """1x1 layers of stride 1: the plan of the images is the plan of one row of their pixels, tiles of one row, as many positions
+    as they have pixels (rounded up to 16)."""
+    p = check(N, H, W, 1, 1, Cin, Cout, BF16)
+    q = check(1, 1, N * H * W, 1, 1, Cin, Cout, BF16)
+    assert p.eligible and all(getattr(p, f) == getattr(q, f) for f, _ in p._fields_)
+    assert p.rows_per_tile == 1 and p.positions == -(-p.cols_per_tile // 16) * 16
+
+
+def test_weights_that_stay():
+    p = check(16, 160, 160, 1, 1, 64, 64, BF16)       # one stage of weights, thousands of tiles
+    assert p.weight_stages == 1 and p.act_stages >= 3
+    q = check(4, 100, 136, 1, 1, 512, 256, BF16)      # eight stages do not fit beside three activation stages
+    assert q.act_stages * q.act_stage_bytes + q.weight_stages * q.weight_stage_bytes <= q.shared_bytes
 
 
 def test_narrow_layers_stage_half_rows_and_keep_a_deeper_ring():
