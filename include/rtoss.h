@@ -506,7 +506,9 @@ rtoss_status rtoss_upsample2x_slice(const void* x_dev, int x_channel_stride, voi
                                     void* cuda_stream);
 /* Three chained k x k max-pools of stride 1 (k odd, padding k/2) inside one tensor: channels [offset, offset + C) are
  * the input, the pooled maps go to the three C-channel slices behind it (what rtoss_maxpool2d gives, three times).
- * 16-bit NHWC, C, offset and stride multiples of 8, y_dev 16-byte aligned, H*W <= 6400; else RTOSS_ERR_UNSUPPORTED. */
+ * 16-bit NHWC, C, offset and stride multiples of 8, y_dev 16-byte aligned, H*W <= RTOSS_POOL_PYRAMID_PX; else
+ * RTOSS_ERR_UNSUPPORTED. */
+#define RTOSS_POOL_PYRAMID_PX 6400
 rtoss_status rtoss_pool_pyramid(void* y_dev, int N, int C, int H, int W, int k, rtoss_layout layout, rtoss_dtype dtype,
                                 int y_channel_offset, int y_channel_stride, void* cuda_stream);
 /* y = act(a + b) over n_elements contiguous elements (residual connections); the sum is formed in fp32 and

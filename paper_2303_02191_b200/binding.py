@@ -20,6 +20,7 @@ NCHW, NHWC = 0, 1
 ACT_NONE, ACT_RELU, ACT_SILU = 0, 1, 2
 PRESET_ALL, PRESET_CONN4, PRESET_CENTRE8, PRESET_DENSE = 0, 1, 2, 3
 PATH_AUTO, PATH_FMA, PATH_TENSOR = 0, 1, 2
+POOL_PYRAMID_PX = 6400
 ROUTE_TENSOR, ROUTE_TENSOR_REPACKED, ROUTE_STEM, ROUTE_FEW, ROUTE_STAGED = 0, 1, 2, 3, 4
 DTYPE_NAMES = {"f32": F32, "bf16": BF16, "f16": F16}
 ACT_NAMES = {"none": ACT_NONE, "relu": ACT_RELU, "silu": ACT_SILU}

@@ -145,7 +145,7 @@ __global__ void maxpool_vec8_kernel(const GlueArgs a) {
 // a block takes eight channels of one image into shared memory, and each pool is a maximum along the rows, then along the
 // columns (a maximum selects one of its inputs, in any order the same bits).  Pools and copies one by one were bound by 25
 // reads of every pixel and by their launches: 20 x 20 x 256, 16 images, 53 us in seven launches, 10.2 here (one image 28.5 / 4.6).
-constexpr int kPyramidPx = 6400;   // two maps of 16 bytes a pixel in 200 KB
+constexpr int kPyramidPx = RTOSS_POOL_PYRAMID_PX;   // two maps of 16 bytes a pixel in 200 KB
 
 template <typename T>
 __global__ void pool_pyramid_kernel(const GlueArgs a) {

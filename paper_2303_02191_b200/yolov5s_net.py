@@ -192,9 +192,15 @@ def share_slices(ops, bufs):
 
 
 class GpuNet:
-    """The program on the GPU through the C-ABI library: NHWC, bf16 (or fp16), k-entry patterns."""
+    """The program on the GPU through the C-ABI library: NHWC, bf16 (or fp16), k-entry patterns.
 
-    def __init__(self, ctx, N, H0=640, W0=640, k=4, seed=0, dtype="bf16", fuse_residual=True):
+    t holds the program's buffers by name.  After a pass t["in"], t[name] of OUTPUTS and the concatenations hold their values.
+    Of the others only those that `whole` names do: with share_slices a buffer that goes into a concatenation is a view of it
+    (not contiguous), and the buffers along a chain of bottlenecks share one place, which ends up with the last one's values; and
+    a convolution that takes its shortcut along (fuse_residual) never writes its result in front of it.  A program that reads
+    buffers in between passes share_slices=False (dense buffers and copies, as many launches more)."""
+
+    def __init__(self, ctx, N, H0=640, W0=640, k=4, seed=0, dtype="bf16", fuse_residual=True, share_slices=True):
         import torch
         from . import binding as rt
         self.rt, self.ctx, self.N, self.torch = rt, ctx, N, torch
@@ -202,7 +208,8 @@ class GpuNet:
         if fuse_residual:
             self.ops = fuse_shortcuts(self.ops)
         self.copying, self.home, self.inside = self.ops, {}, {}   # (the program with its copies, should the library decline a slice)
-        self._share()
+        if share_slices:
+            self._share()
         self.unfused = set()   # layers whose fused call the library declined: convolution and add run separately
         self.rounds, self.probed, self.steps = None, False, None
         tdt = {"bf16": torch.bfloat16, "f16": torch.float16}[dtype]
@@ -222,7 +229,7 @@ class GpuNet:
         shared, home = share_slices(ops, self.bufs)
         kept = {op[1] for op in shared if op[0] == "copy"}
         pyramids = [op for op in ops if op[0] == "pyramid"]
-        if any(op[1] in kept or self.bufs[op[1]][1] * self.bufs[op[1]][2] > 6400 for op in pyramids):
+        if any(op[1] in kept or self.bufs[op[1]][1] * self.bufs[op[1]][2] > self.rt.POOL_PYRAMID_PX for op in pyramids):
             shared, home = share_slices(self.copying, self.bufs)   # (the pools one by one, see rtoss_pool_pyramid)
         self.ops, self.home = shared, home
         self.inside = {}
@@ -239,6 +246,16 @@ class GpuNet:
                 self.t[n] = old[n]     # what the caller holds
         for n, (cat, off) in self.home.items():
             self.t[n] = self.t[cat][..., off:off + self.bufs[n][0]]
+
+    @property
+    def whole(self):
+        """Names of the buffers that hold their own values after a pass."""
+        place, last = {}, {}
+        for op in self.ops:
+            n = _target(op)
+            place[n] = self.home.get(n, (n, None))
+            last[place[n]] = n
+        return {"in"} | {n for n in place if last[place[n]] == n}
 
     def _copying(self):
         """The library declined a slice: back to dense buffers and copies."""

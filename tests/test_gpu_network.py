@@ -128,3 +128,23 @@ def test_chained_retinanet_shaped_network_small_input():
         assert np.array_equal(sep[name], one_by_one[name]), name
     plain.close()
     net.close()
+
+
+def test_buffers_that_hold_their_values_after_a_pass():
+    """GpuNet.whole against a network that shares nothing: every buffer it names holds the same bits, the outputs and the
+    concatenations are among them; without sharing all but those that fused shortcuts skip are."""
+    from paper_2303_02191_b200 import yolov5s_net as yn
+    ctx = gu.ctx()
+    x = synth.activations(25, 1, 1, 3, 96, 128)
+    nets = [yn.GpuNet(ctx, 1, 96, 128, share_slices=share) for share in (True, False)]
+    for net in nets:
+        net.set_input(x)
+        net.run()
+    torch.cuda.synchronize()
+    shared, dense = nets
+    assert not dense.home and shared.home
+    fused = {op[3] for op in dense.ops if op[0] == "convres"}
+    assert dense.whole == set(dense.bufs) - fused
+    assert set(yn.OUTPUTS) | {"in"} | {cat for cat, _ in shared.home.values()} <= shared.whole < dense.whole | fused
+    for name in shared.whole:
+        assert torch.equal(shared.t[name], dense.t[name]), name
