@@ -217,7 +217,9 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
                     if (k.shared == 1) {
                         // One of several problems that run side by side and together fill the SMs: what counts is the work
                         // a tile does for the time it keeps a CTA (3x3 stride 1: bound by its instructions, N / 2 cycles but
-                        // never less than 76; other tiles by what surrounds the instructions: as many positions as fit).
+                        // never less than 76; other tiles by what surrounds the instructions: as many positions as fit).  The 76
+                        // and the factors below are of the kernel whose issuing thread was alone in its warp; the single
+                        // launches' model has 47 since (kFit16), these tiles have not been measured again.
                         const bool by_cycles = ksize == 3 && S == 1 && n_px / 2.0 < 128.0;
                         const double cyc = by_cycles ? (n_px / 2.0 > 76.0 ? n_px / 2.0 : 76.0) : 128.0;
                         const double eff = (double)(th * tw) / (2.0 * cyc) * Ho / (double)(ty * th) * Wo / (double)(tw * nseg);

@@ -1,12 +1,12 @@
-// Tensor-core path of the pattern convolutions (bf16 / fp16, NHWC, stride 1 or 2).
+// Tensor-core path of the pattern convolutions (bf16 / fp16 / fp32, NHWC, stride 1 or 2).
 //
 // Per-kernel patterns cannot be compacted into a dense contraction (every
 // filter keeps different (channel, tap) positions), so this path evaluates the
 // convolution of Section II.B of arXiv 2303.02191 as a masked dense implicit
 // GEMM on the 5th-generation tensor cores: the pruned taps are multiplied as
 // zeros.  It performs 9/k times the non-zero FLOPs and is still several times
-// faster than the FMA-pipe gather for 16-bit data; the FMA path stays the one
-// for fp32 and for shapes this kernel does not take.
+// faster than the FMA pipes; the FMA path stays the one for shapes and layouts
+// this kernel does not take.
 //
 // GEMM view:  D[co, position] = sum over taps t and channels ci of
 //                               Wt[t][co][ci] * X[position shifted by t, ci]
@@ -22,10 +22,9 @@
 //     dropped.
 //   * Operand roles: the weights are the M operand (128 filters = the 128 TMEM
 //     lanes), the positions are the N operand (up to 256 per instruction), K =
-//     16 channels per instruction.  One instruction costs about 140 cycles
-//     whatever N is, and with M = 64 as with M = 128 (measured), so N
-//     must be wide: 128 x 256 x 16 per instruction runs near the tensor peak,
-//     128 x 128 x 16 at half of it (measured on this kernel with both roles).
+//     16 channels per instruction.  One instruction takes N / 2 cycles, but
+//     never less than about 47, and with M = 64 as long as with M = 128
+//     (measured), so N must be wide.
 //   * Weights are the dense-expanded form Wt[t][co][ci] that rtoss_pack builds
 //     next to the packed arrays; one TMA box per (kernel row of three taps,
 //     channel block); filters
