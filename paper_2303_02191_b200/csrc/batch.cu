@@ -558,10 +558,10 @@ rtoss_status rtoss_batch_create(rtoss_ctx* ctx, const rtoss_batch_item* items, i
     int prev = 0;
     cudaGetDevice(&prev);
     cudaSetDevice(ctx->device);
-    rtoss_dev::rtoss_writers_carveout(batch_select_pack_kernel<kSmallThreads>);
-    rtoss_dev::rtoss_writers_carveout(batch_select_pack_kernel<kBatchThreads>);
-    rtoss_dev::rtoss_writers_carveout(batch_order_kernel<false>);
-    rtoss_dev::rtoss_writers_carveout(batch_order_kernel<true>);
+    if (threads == kSmallThreads) rtoss_dev::writers_carveout<batch_select_pack_kernel<kSmallThreads>>();
+    else rtoss_dev::writers_carveout<batch_select_pack_kernel<kBatchThreads>>();
+    if (sixteens) rtoss_dev::writers_carveout<batch_order_kernel<true>>();
+    else rtoss_dev::writers_carveout<batch_order_kernel<false>>();
     cudaError_t e = cudaMalloc((void**)&b->layers_dev, sizeof(BatchLayer) * (size_t)L);
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->chunks_dev, sizeof(BatchChunk) * (chunks.size() + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&b->task_layer_dev, sizeof(uint32_t) * (task_layer.size() + 1));

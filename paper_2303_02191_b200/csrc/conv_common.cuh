@@ -6,6 +6,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "rtoss_internal.h"
 
 namespace rtoss_dev {
@@ -96,10 +98,14 @@ __device__ __forceinline__ void handle_writer_done() {
 
 // The kernels that write handles follow one another in pairs whose shared memory differs (6 to 46 KB a block).  An SM that has
 // to move the line between its shared memory and its L1 first runs empty, which cost 5 us between two of them: all of them
-// ask for the same line (a hint; set per device, before the first launch).
-template <typename... KArgs>
-inline void rtoss_writers_carveout(void (*kern)(KArgs...)) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+// ask for the same line (a hint; set once per device, before a kernel's first launch).
+template <auto kKernel>
+inline void writers_carveout() {
+    static std::atomic<bool> done[64];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev].load(std::memory_order_relaxed)) return;
+    if (cudaFuncSetAttribute(kKernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) != cudaSuccess) cudaGetLastError();
+    done[dev].store(true, std::memory_order_relaxed);
 }
 
 template <typename... KArgs, typename... Args>

@@ -267,36 +267,22 @@ int rtoss_launch_select(const void* w, rtoss_dtype wdt, int64_t n_kernels, const
     return (int)cudaGetLastError();
 }
 
-// Once per device (see rtoss_writers_carveout).
-template <typename T>
-static void prepare_pack_of() {
-    rtoss_dev::rtoss_writers_carveout(pack_values_kernel<T, float>);
-    rtoss_dev::rtoss_writers_carveout(pack_values_kernel<T, __nv_bfloat16>);
-    rtoss_dev::rtoss_writers_carveout(pack_values_kernel<T, __half>);
-}
-static void prepare_pack() {
-    static std::atomic<bool> done[64];
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || done[dev].load(std::memory_order_acquire)) return;
-    prepare_pack_of<float>();
-    prepare_pack_of<__nv_bfloat16>();
-    prepare_pack_of<__half>();
-    rtoss_dev::rtoss_writers_carveout(pack_order_kernel<false>);
-    rtoss_dev::rtoss_writers_carveout(pack_order_kernel<true>);
-    done[dev].store(true, std::memory_order_release);
-}
-
 template <typename T>
 static int launch_pack_values_t(const T* w, int64_t n, const MaskTable& t, const uint8_t* pid, int k, void* val,
                                 rtoss_dtype vdt, uint8_t* pid_copy, void* wtc, int ksize, int Cin, rtoss_wtc_layout lay, unsigned long long* issue, int issue_n,
                                 cudaStream_t s) {
     const int grid = grid_for((n + kSelThreads - 1) / kSelThreads);
     switch (vdt) {
-        case RTOSS_F32: rtoss_dev::launch_pdl(pack_values_kernel<T, float>, grid, kSelThreads, 0, s, w, n, t, pid, k, (float*)val, pid_copy, (float*)wtc, ksize, Cin, lay, issue, issue_n); break;
+        case RTOSS_F32:
+            rtoss_dev::writers_carveout<pack_values_kernel<T, float>>();
+            rtoss_dev::launch_pdl(pack_values_kernel<T, float>, grid, kSelThreads, 0, s, w, n, t, pid, k, (float*)val, pid_copy, (float*)wtc, ksize, Cin, lay, issue, issue_n); break;
         case RTOSS_BF16:
+            rtoss_dev::writers_carveout<pack_values_kernel<T, __nv_bfloat16>>();
             rtoss_dev::launch_pdl(pack_values_kernel<T, __nv_bfloat16>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__nv_bfloat16*)val, pid_copy, (__nv_bfloat16*)wtc, ksize, Cin, lay, issue, issue_n);
             break;
-        case RTOSS_F16: rtoss_dev::launch_pdl(pack_values_kernel<T, __half>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__half*)val, pid_copy, (__half*)wtc, ksize, Cin, lay, issue, issue_n); break;
+        case RTOSS_F16:
+            rtoss_dev::writers_carveout<pack_values_kernel<T, __half>>();
+            rtoss_dev::launch_pdl(pack_values_kernel<T, __half>, grid, kSelThreads, 0, s, w, n, t, pid, k, (__half*)val, pid_copy, (__half*)wtc, ksize, Cin, lay, issue, issue_n); break;
     }
     return (int)cudaGetLastError();
 }
@@ -306,7 +292,6 @@ int rtoss_launch_pack_values(const void* w, rtoss_dtype wdt, int64_t n_kernels, 
                              unsigned long long* issue, int issue_n, void* stream) {
     const rtoss_wtc_layout lay = rtoss_wtc_layout_of(Cout, Cin, ksize, vdt);
     if (n_kernels <= 0) return 0;
-    prepare_pack();
     cudaStream_t s = (cudaStream_t)stream;
     switch (wdt) {
         case RTOSS_F32: return launch_pack_values_t<float>((const float*)w, n_kernels, t, pid, k, val, vdt, pid_copy, wtc, ksize, Cin, lay, issue, issue_n, s);
@@ -321,12 +306,15 @@ int rtoss_launch_pack_order(const uint8_t* pid, int Cout, int Cin, int P, uint32
                             const uint16_t* masks_dev, unsigned long long* issue, int cb_log2, void* stream) {
     const bool sixteens = rtoss_dev::order_in_sixteens(Cout, P, (long long)Cout * Cin);
     const int per = rtoss_dev::order_channels_of(sixteens), grid = (Cin + per - 1) / per;
-    if (sixteens)
+    if (sixteens) {
+        rtoss_dev::writers_carveout<pack_order_kernel<true>>();
         rtoss_dev::launch_pdl(pack_order_kernel<true>, grid, rtoss_dev::kOrderThreads, 0, (cudaStream_t)stream, pid, Cout, Cin, P, perm, bucket_off, masks_dev,
                               issue, cb_log2);
-    else
+    } else {
+        rtoss_dev::writers_carveout<pack_order_kernel<false>>();
         rtoss_dev::launch_pdl(pack_order_kernel<false>, grid, rtoss_dev::kOrderWarps * 32, 0, (cudaStream_t)stream, pid, Cout, Cin, P, perm, bucket_off,
                               masks_dev, issue, cb_log2);
+    }
     return (int)cudaGetLastError();
 }
 
