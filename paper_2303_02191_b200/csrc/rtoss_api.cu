@@ -282,19 +282,21 @@ void* rtoss_copy_get(const rtoss_ctx* ctx, size_t* bytes, void* stream, bool* of
     cudaGraph_t graph = nullptr;
     void* mem = nullptr;
     *of_graph = false;
-    unsigned long long capture = 0;
-    const cudaGraphNode_t* deps = nullptr;
-    const cudaGraphEdgeData* edges = nullptr;
-    size_t n_deps = 0;
-    if (cudaStreamGetCaptureInfo_v3((cudaStream_t)stream, &status, &capture, &graph, &deps, &edges, &n_deps) == cudaSuccess) {
+    if (cudaStreamIsCapturing((cudaStream_t)stream, &status) == cudaSuccess && status != cudaStreamCaptureStatusInvalidated) {
         if (status == cudaStreamCaptureStatusNone) {
             cudaMemPool_t pool = copy_pool(ctx);
             if (pool && cudaMallocFromPoolAsync(&mem, *bytes, pool, (cudaStream_t)stream) != cudaSuccess) mem = nullptr;
-        } else if (status == cudaStreamCaptureStatusActive) {
+        } else {
+            unsigned long long capture = 0;
+            const cudaGraphNode_t* deps = nullptr;
+            const cudaGraphEdgeData* edges = nullptr;
+            size_t n_deps = 0;
             cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;   // (what happens here is no part of the capture)
             cudaThreadExchangeStreamCaptureMode(&mode);
-            mem = done_with(capture, bytes, deps, n_deps);
-            if (!mem) mem = graph_copy(ctx, *bytes, graph);
+            if (cudaStreamGetCaptureInfo_v3((cudaStream_t)stream, &status, &capture, &graph, &deps, &edges, &n_deps) == cudaSuccess) {
+                mem = done_with(capture, bytes, deps, n_deps);
+                if (!mem) mem = graph_copy(ctx, *bytes, graph);
+            }
             cudaThreadExchangeStreamCaptureMode(&mode);
             *of_graph = mem != nullptr;
         }
