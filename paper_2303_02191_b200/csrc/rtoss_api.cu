@@ -631,7 +631,7 @@ rtoss_status rtoss_packed_export(rtoss_ctx* ctx, const rtoss_packed* p, uint8_t*
 rtoss_status rtoss_packed_to_dense(rtoss_ctx* ctx, const rtoss_packed* p, void* w_masked_dev, void* cuda_stream) {
     if (!ctx || !p || !w_masked_dev) return RTOSS_ERR_INVALID_ARG;
     rtoss_device_guard on_device(p->device);   // the caller's current device comes back when the call returns
-    int e = rtoss_launch_to_dense(p, w_masked_dev, cuda_stream);
+    int e = rtoss_launch_to_dense(p, ctx->sm_count > 0 ? ctx->sm_count : 148, w_masked_dev, cuda_stream);
     return e ? cuda_fail(ctx, "to_dense launch", e) : RTOSS_OK;
 }
 

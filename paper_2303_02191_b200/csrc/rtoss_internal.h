@@ -122,7 +122,7 @@ int rtoss_launch_pack_order(const uint8_t* pid, int Cout, int Cin, int P, uint32
                             const uint16_t* masks_dev, unsigned long long* issue, int cb_log2, void* stream);
 int rtoss_launch_select_shared(const void* w, rtoss_dtype wdt, int Cout, int Cin, int FB, int CB, const MaskTable& t, int P,
                                uint8_t* pid, void* stream);
-int rtoss_launch_to_dense(const rtoss_packed* p, void* w_out, void* stream);
+int rtoss_launch_to_dense(const rtoss_packed* p, int sms, void* w_out, void* stream);
 int rtoss_launch_pid_histogram(const uint8_t* pid, int64_t n, int P, unsigned long long* counts, void* stream);
 int rtoss_launch_conv3x3(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, void* y,
                          const rtoss_conv_desc* d, void* stream);

@@ -26,11 +26,6 @@ template <> __device__ __forceinline__ float narrow<float>(float v) { return v; 
 template <> __device__ __forceinline__ __nv_bfloat16 narrow<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 template <> __device__ __forceinline__ __half narrow<__half>(float v) { return __float2half_rn(v); }
 
-// (__ldcg takes no 16-bit floating types here)
-__device__ __forceinline__ float ld_cg(const float* p) { return __ldcg(p); }
-__device__ __forceinline__ __nv_bfloat16 ld_cg(const __nv_bfloat16* p) { return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p))); }
-__device__ __forceinline__ __half ld_cg(const __half* p) { return __ushort_as_half(__ldcg(reinterpret_cast<const unsigned short*>(p))); }
-
 // Copy the 9*count weights of `count` consecutive kernels starting at kernel
 // `first` into shared memory, coalesced, 16 bytes per thread where the chunk is
 // whole.  The base pointer is 16-byte aligned and a full chunk is a multiple
@@ -194,49 +189,69 @@ __global__ void __launch_bounds__(kSharedMaxFB) select_shared_kernel(const T* __
     }
 }
 
-// Dense masked weights from the packed form.  A block expands 256 kernels in shared memory and writes their 2304 weights as
+// Dense masked weights from the packed form.  A block expands its kernels in shared memory and writes their weights as
 // consecutive 16-byte words.  Everything it reads belongs to the handle, and the kernels that write a handle never let a
 // successor start early (pdl_enter_handle_writer), so the reading and the expansion run ahead of the wait for the kernels
 // before this one: a model's layers are expanded one call after the other, and all but the stores of a call then overlaps
-// the call before it.  (Sixty-eight layers in a row: 3.4 us a
-// layer with a gather per element behind the wait, 1.2 now.)
+// the calls before it.
+// What bounds a row of such calls is the hop from the end of one kernel to the end of the next: 0.7 us with nothing but a few
+// stores in it, more with more blocks (empty kernels: 0.55 us up to 148 blocks, 0.9 with 592, 1.57 with 1184).  Hence at most one
+// block an SM, with its whole share of the layer in shared memory and the words a thread stores in registers when the wait
+// ends, and blocks small enough (256 threads, at most 73 KB) for calls that wait to be on an SM together: fetching takes longer
+// than a hop.  57 layers of 7 M weights in a row 50.3 -> 46.3 us, 68 layers of 32 M 86 -> 77 (against a block per 256 kernels that
+// stored from shared memory; stored that way, one block an SM took 52 and 82).
 // All of these loads go to L2 (see conv_common.cuh).
+constexpr int kDenseThreads = 256;
+constexpr int kDenseHold = 5;        // 16-byte words of its output a thread holds in registers (a step of up to 1136 kernels in 16 bits)
+constexpr int kDenseBytes = 73728;   // of shared memory at most: ids, kept values and dense weights of a block's kernels
 template <typename V>
-__global__ void __launch_bounds__(kSelThreads) to_dense_kernel(const V* __restrict__ val, const uint8_t* __restrict__ pid,
-                                                               const uint16_t* __restrict__ masks, int k, int64_t n_kernels, int64_t n_dense,
-                                                               V* __restrict__ out) {
+__global__ void __launch_bounds__(kDenseThreads, 4) to_dense_kernel(const V* __restrict__ val, const uint8_t* __restrict__ pid,
+                                                                    const uint16_t* __restrict__ masks, int k, int64_t n_kernels, int64_t n_dense,
+                                                                    int step, V* __restrict__ out) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ __align__(16) V sv[kSelThreads * 9];    // kept values, k per kernel
-    __shared__ __align__(16) V sd[kSelThreads * 9];    // the chunk's dense weights
+    extern __shared__ __align__(16) unsigned char dense_smem[];
+    V* sd = reinterpret_cast<V*>(dense_smem);   // the step's dense weights
+    V* sv = sd + (size_t)step * 9;              // its kept values, k per kernel
+    uint8_t* sid = reinterpret_cast<uint8_t*>(sv + (size_t)step * k);   // and its pattern ids (a step is a multiple of sixteen kernels)
+    __shared__ __align__(16) uint16_t sm[256];
     const int tid = (int)threadIdx.x;
+    // n bytes from src (both sides 16-byte aligned) on their way to shared memory; the odd bytes at the end of the last step at once
+    auto fetch = [&](void* to, const void* src, int n) {
+        const int whole = n & ~15;
+        for (int i = tid * 16; i < whole; i += kDenseThreads * 16)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(to) + (unsigned)i), "l"(static_cast<const char*>(src) + i) : "memory");
+        if (tid < n - whole) static_cast<uint8_t*>(to)[whole + tid] = __ldcg(static_cast<const uint8_t*>(src) + whole + tid);
+    };
+    fetch(sm, masks, 512);
     bool waited = false;
-    const int64_t n_chunks = (n_kernels + kSelThreads - 1) / kSelThreads;
     const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
-    for (int64_t chunk = blockIdx.x; chunk < n_chunks; chunk += gridDim.x) {
-        const int64_t first = chunk * kSelThreads;
-        const int count = (int)(n_kernels - first < kSelThreads ? n_kernels - first : kSelThreads);
-        unsigned m = 0;
-        if (tid < count) m = __ldcg(masks + __ldcg(pid + first + tid));
-        {
-            const V* src = val + first * k;
-            const int n = count * k, nv = n * (int)sizeof(V) / 16;
-            for (int i = tid; i < nv; i += kSelThreads) reinterpret_cast<uint4*>(sv)[i] = __ldcg(reinterpret_cast<const uint4*>(src) + i);
-            for (int i = nv * 16 / (int)sizeof(V) + tid; i < n; i += kSelThreads) sv[i] = ld_cg(src + i);
-        }
+    for (int64_t first = (int64_t)blockIdx.x * step; first < n_kernels; first += (int64_t)gridDim.x * step) {
+        const int count = (int)(n_kernels - first < step ? n_kernels - first : step);
+        fetch(sid, pid + first, count);
+        fetch(sv, val + first * k, count * k * (int)sizeof(V));
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
-        if (tid < count) {
-            const V* s = sv + tid * k;
-            V* d = sd + tid * 9;
+        for (int g = tid; g < count; g += kDenseThreads) {
+            const unsigned m = sm[sid[g]];
+            const V* s = sv + g * k;
+            V* d = sd + g * 9;
 #pragma unroll
             for (int t = 0; t < 9; ++t) d[t] = (m >> t) & 1u ? *s++ : narrow<V>(0.f);
         }
         __syncthreads();
+        V* dst = out + first * 9;   // (a whole step is a multiple of 16 bytes)
+        const int n = count * 9, nv = aligned ? n * (int)sizeof(V) / 16 : 0;
+        uint4 hold[kDenseHold];   // (behind the wait there is then nothing left to do but to store)
+#pragma unroll
+        for (int j = 0; j < kDenseHold; ++j)
+            if (tid + j * kDenseThreads < nv) hold[j] = reinterpret_cast<const uint4*>(sd)[tid + j * kDenseThreads];
         if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");   // the output may still be read by an earlier kernel
         waited = true;
-        V* dst = out + first * 9;   // (a whole chunk is a multiple of 16 bytes)
-        const int n = count * 9, nv = aligned ? n * (int)sizeof(V) / 16 : 0;
-        for (int i = tid; i < nv; i += kSelThreads) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(sd)[i];
-        for (int i = nv * 16 / (int)sizeof(V) + tid; i < n; i += kSelThreads) dst[i] = sd[i];
+#pragma unroll
+        for (int j = 0; j < kDenseHold; ++j)
+            if (tid + j * kDenseThreads < nv) reinterpret_cast<uint4*>(dst)[tid + j * kDenseThreads] = hold[j];
+        for (int i = tid + kDenseHold * kDenseThreads; i < nv; i += kDenseThreads) reinterpret_cast<uint4*>(dst)[i] = reinterpret_cast<const uint4*>(sd)[i];
+        for (int i = nv * 16 / (int)sizeof(V) + tid; i < n; i += kDenseThreads) dst[i] = sd[i];
         __syncthreads();
     }
     if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -335,27 +350,38 @@ int rtoss_launch_select_shared(const void* w, rtoss_dtype wdt, int Cout, int Cin
     return (int)e;
 }
 
-int rtoss_launch_to_dense(const rtoss_packed* p, void* w_out, void* stream) {
+template <typename V>
+static int launch_to_dense_t(const rtoss_packed* p, int64_t n_dense, int sms, void* w_out, cudaStream_t s) {
+    // kernels of a block: an SM's share of the layer, but no fewer than a small block's worth and no more than fit
+    const int per_kernel = (9 + p->k) * (int)sizeof(V) + 1;
+    const int64_t most = kDenseBytes / per_kernel / 16 * 16;
+    int64_t step = ((p->n_kernels + sms - 1) / sms + 15) / 16 * 16;
+    if (step < 256) step = 256;
+    if (step > most) step = most;
+    int64_t grid = (p->n_kernels + step - 1) / step;
+    if (grid < 1) grid = 1;
+    if (grid > 8 * (int64_t)sms) grid = 8 * (int64_t)sms;
+    static std::atomic<bool> done[64];   // the function may take that much shared memory (once per device)
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || !done[dev].load(std::memory_order_acquire)) {
+        const cudaError_t e = cudaFuncSetAttribute(to_dense_kernel<V>, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseBytes);
+        if (e != cudaSuccess) return (int)e;
+        rtoss_dev::writers_carveout<to_dense_kernel<V>>();
+        if (dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
+    }
+    return (int)rtoss_dev::launch_pdl(to_dense_kernel<V>, (unsigned)grid, kDenseThreads, (size_t)(step * per_kernel), s, (const V*)p->val, (const uint8_t*)p->pid,
+                                      (const uint16_t*)p->masks_dev, p->k, p->n_kernels, n_dense, (int)step, (V*)w_out);
+}
+
+int rtoss_launch_to_dense(const rtoss_packed* p, int sms, void* w_out, void* stream) {
     const int64_t n_dense = p->ksize == 3 ? p->n_kernels * 9 : (int64_t)p->Cout * p->Cin;
     if (n_dense <= 0) return 0;
-    cudaStream_t s = (cudaStream_t)stream;
-    const int threads = kSelThreads;
-    const int grid = grid_for((p->n_kernels + threads - 1) / threads);
     switch (p->dtype) {
-        case RTOSS_F32:
-            rtoss_dev::launch_pdl(to_dense_kernel<float>, grid, threads, 0, s, (const float*)p->val, p->pid, p->masks_dev, p->k, p->n_kernels,
-                                                            n_dense, (float*)w_out);
-            break;
-        case RTOSS_BF16:
-            rtoss_dev::launch_pdl(to_dense_kernel<__nv_bfloat16>, grid, threads, 0, s, (const __nv_bfloat16*)p->val, p->pid, p->masks_dev,
-                                                                    p->k, p->n_kernels, n_dense, (__nv_bfloat16*)w_out);
-            break;
-        case RTOSS_F16:
-            rtoss_dev::launch_pdl(to_dense_kernel<__half>, grid, threads, 0, s, (const __half*)p->val, p->pid, p->masks_dev, p->k,
-                                                             p->n_kernels, n_dense, (__half*)w_out);
-            break;
+        case RTOSS_F32: return launch_to_dense_t<float>(p, n_dense, sms, w_out, (cudaStream_t)stream);
+        case RTOSS_BF16: return launch_to_dense_t<__nv_bfloat16>(p, n_dense, sms, w_out, (cudaStream_t)stream);
+        case RTOSS_F16: return launch_to_dense_t<__half>(p, n_dense, sms, w_out, (cudaStream_t)stream);
     }
-    return (int)cudaGetLastError();
+    return (int)cudaErrorInvalidValue;
 }
 
 // ---------------------------------------------------------------------------------------------
