@@ -152,19 +152,34 @@ template <typename V> __device__ __forceinline__ unsigned round2(float a, float 
         return *reinterpret_cast<const unsigned*>(&u);
     }
 }
-// Two neighbouring positions as one aligned word; fp32: tf32 heads, and the remainders lo_at further on (see expand_one).
-template <typename V> __device__ __forceinline__ void put_pair(V* at, int64_t lo_at, float a, float b) {
+// Two neighbouring positions (f, f even) as one aligned word; fp32: tf32 heads, and what corrects them lo_at further on (see
+// expand_one).
+template <typename V> __device__ __forceinline__ void put_pair(V* wtc, int64_t f, int64_t lo_at, bool corr16, float a, float b) {
     using namespace rtoss_dev;
+    V* at = wtc + f;
     if constexpr (sizeof(V) == 4) {
+        if (corr16) {
+            const float ha = tf32_near(a), hb = tf32_near(b);
+            *reinterpret_cast<float2*>(at) = make_float2(ha, hb);
+            put_corr16_two(wtc + lo_at, f, a, b, __fsub_rn(a, ha), __fsub_rn(b, hb));
+            return;
+        }
         *reinterpret_cast<float2*>(at) = make_float2(tf32_head(a), tf32_head(b));
         *reinterpret_cast<float2*>(at + lo_at) = make_float2(__fsub_rn(a, tf32_head(a)), __fsub_rn(b, tf32_head(b)));
     } else {
         *reinterpret_cast<unsigned*>(at) = round2<V>(a, b);
     }
 }
-template <typename V> __device__ __forceinline__ void put_one(V* at, int64_t lo_at, float a) {
+template <typename V> __device__ __forceinline__ void put_one(V* wtc, int64_t f, int64_t lo_at, bool corr16, float a) {
     using namespace rtoss_dev;
+    V* at = wtc + f;
     if constexpr (sizeof(V) == 4) {
+        if (corr16) {
+            const float h = tf32_near(a);
+            *at = h;
+            put_corr16_one(wtc + lo_at, f, a, __fsub_rn(a, h));
+            return;
+        }
         *at = tf32_head(a);
         at[lo_at] = __fsub_rn(a, tf32_head(a));
     } else {
@@ -225,12 +240,13 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
         const bool word = two && p1 == p0 + 1 && (p0 & 1) == 0 && (tap_step & 1) == 0 && (copy_step & 1) == 0;
         V* at = wtc + p0;
         const int64_t d1 = p1 - p0;
+        const bool corr16 = sizeof(V) == 4 && rtoss_f32_corr16(Cin, 3);
         if (word && L.lay.copies == 1) {
 #pragma unroll
             for (int t = 0; t < 9; ++t, at += tap_step) {
                 const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
                 const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
-                put_pair<V>(at, lo_at, a, b);
+                put_pair<V>(wtc, at - wtc, lo_at, corr16, a, b);
             }
             return;
         }
@@ -265,10 +281,10 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
                     const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
                     const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
                     if (word) {
-                        put_pair<V>(to, lo_at, a, b);
+                        put_pair<V>(wtc, to - wtc, lo_at, corr16, a, b);
                     } else {
-                        put_one<V>(to, lo_at, a);
-                        if (two) put_one<V>(to + d1, lo_at, b);
+                        put_one<V>(wtc, to - wtc, lo_at, corr16, a);
+                        if (two) put_one<V>(wtc, to - wtc + d1, lo_at, corr16, b);
                     }
                 }
             }
@@ -304,7 +320,7 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
             } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (e + j < n) put_one<V>(wtc + f + j + (cin_p != Cin ? (int64_t)((unsigned)(f + j) / (unsigned)Cin) * (cin_p - Cin) : 0), tap_step, v[j]);
+                    if (e + j < n) put_one<V>(wtc, f + j + (cin_p != Cin ? (int64_t)((unsigned)(f + j) / (unsigned)Cin) * (cin_p - Cin) : 0), tap_step, false, v[j]);
             }
         }
     }

@@ -103,17 +103,25 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
     const bool f32 = k.dtype == RTOSS_F32;
     const int taps = k.ksize == 3 ? 9 : 1;
     const int slab_ch = f32 ? 8 : 16, cb_ch = row_bytes / (f32 ? 4 : 2);
-    const double slabs = (double)(k.Cin < cb_ch ? k.Cin : cb_ch) / slab_ch * (f32 ? 3 : 1);
+    const bool corr16 = f32 && rtoss_f32_corr16(k.Cin, k.ksize);
+    const double slabs = (double)(k.Cin < cb_ch ? k.Cin : cb_ch) / slab_ch * (corr16 ? 2 : f32 ? 3 : 1);
     const int wstages = f32 ? 2 * taps / G : taps / G;
     const PlanFit& f = f32 ? kFit32 : kFit16;
     const double instr = (pxm ? f.cycles * halves : n_px / 2.0 > f.cycles ? n_px / 2.0 : f.cycles) / 1900.0;
-    const double mma = taps * slabs * instr + f.stage * wstages + f.block;
+    double mma = taps * slabs * instr + f.stage * wstages + f.block;
+    if (corr16) {
+        // fp32 3x3 layers whose small products are bf16 ones, 256->256 @80x80 x32 cut in eight ways, 96 to 240 positions a tile: a
+        // weight stage of one tap takes its four instructions + 0.1 us, at least 0.28; one of three taps its twelve + 0.27
+        const double s = G * 4 * (n_px / 2.0 > 47.0 ? n_px / 2.0 : 47.0) / 1900.0 + (G == 3 ? 0.27 : 0.10);
+        mma = wstages * (s > 0.28 ? s : 0.28) + f.block;
+    }
     const double kb_b = (double)taps * w_rows * row_bytes * (f32 ? 2 : 1) / 1024.0, kb_a = a_bytes / 1024.0;
     const double kb_fed = kb_a * (k.S == 2 ? f.strided : 1.0);
-    double blk = mma > (kb_fed + kb_b) / f.feed ? mma : (kb_fed + kb_b) / f.feed;
+    const double feed = (kb_fed + kb_b) / (corr16 ? 110 : f.feed);
+    double blk = mma > feed ? mma : feed;
     // one activation stage: loads and instructions take turns (fp32: and one warp's split of the block between them)
     if (na == 1) blk = mma + (f32 ? 0.045 * kb_a : f.lone * kb_fed / 87.0);
-    if (f32 && G == 3) blk += 2.0;   // (then only two weight stages fit: the ring's round trip shows)
+    if (f32 && !corr16 && G == 3) blk += 2.0;   // (then only two weight stages fit: the ring's round trip shows)
     const int chunks = (n_px + 31) / 32;
     double epi;
     if (pxm) epi = f.epi_pxm * ((halves * ((k.Cout + 15) / 16) + 3) / 4);
@@ -428,6 +436,8 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     // N/8 and M/16
     const unsigned fmt = f32 ? 2u : a.is_bf16 ? 1u : 0u;
     a.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((unsigned)(plan.N_px >> 3) << 17) | ((unsigned)(kMTile >> 4) << 24);
+    a.corr16 = f32 && rtoss_f32_corr16(p->Cin, p->ksize) ? 1 : 0;
+    a.idesc16 = (a.idesc & ~((7u << 7) | (7u << 10))) | (1u << 7) | (1u << 10);   // (bf16)
     a.pxm = pxm ? 1 : 0;
     a.MH = plan.N_px > 128 ? 2 : 1;
     a.n_cols = round_up(p->Cout, 16);
@@ -516,6 +526,8 @@ int ensure_device(const rtoss_ctx* ctx) {
             e = cudaFuncSetAttribute(conv_tc_kernel<__half, TcLaunchN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(conv_tc_kernel<float, TcLaunch1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(conv_tc_kernel<float, TcLaunch1, false, kFormCorr>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(conv_tc_kernel<float, TcLaunchN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e == cudaSuccess)
@@ -693,6 +705,8 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     return RTOSS_OK;
 }
 
+static int threads_of(bool f32) { return f32 ? kThreadsOf<float> : kThreadsOf<__half>; }
+
 // The kernel a launch of one convolution runs: a form where there is one for it, else the general one.
 static SingleKernel single_kernel(const rtoss_ctx* ctx, bool f32, bool repacked, const TcArgs& a) {
     if (!f32 && (a.taps == 1 || a.G == 3)) {
@@ -700,7 +714,7 @@ static SingleKernel single_kernel(const rtoss_ctx* ctx, bool f32, bool repacked,
         const int form = (pieces ? 0 : kFormElem) | form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
         if (void* k = form_kernel(ctx, a.is_bf16, false, form)) return reinterpret_cast<SingleKernel>(k);
     }
-    if (f32) return conv_tc_kernel<float, TcLaunch1>;
+    if (f32) return a.corr16 ? conv_tc_kernel<float, TcLaunch1, false, kFormCorr> : conv_tc_kernel<float, TcLaunch1>;
     if (repacked) return a.is_bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1, true> : conv_tc_kernel<__half, TcLaunch1, true>;
     return a.is_bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1> : conv_tc_kernel<__half, TcLaunch1>;
 }
@@ -801,7 +815,7 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     cudaError_t le;
     if (a.KS > 1) {
         // one cluster per tile; if the device cannot place the clusters the layer runs uncut
-        le = rtoss_dev::launch_pdl(single_kernel(ctx, f32, repacked, a), grid, kTcThreads, smem, (cudaStream_t)stream, a.KS, g);
+        le = rtoss_dev::launch_pdl(single_kernel(ctx, f32, repacked, a), grid, threads_of(f32), smem, (cudaStream_t)stream, a.KS, g);
         if (le == cudaSuccess) return 0;
         cudaGetLastError();
         a.KS = 1;
@@ -811,7 +825,7 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
         g.unit_end[0] = (int)n_units;
         grid = dim3((unsigned)(n_units < (size_t)sms ? n_units : (size_t)sms));
     }
-    le = rtoss_dev::launch_pdl(single_kernel(ctx, f32, repacked, a), grid, kTcThreads, smem, (cudaStream_t)stream, 1, g);
+    le = rtoss_dev::launch_pdl(single_kernel(ctx, f32, repacked, a), grid, threads_of(f32), smem, (cudaStream_t)stream, 1, g);
     return (int)le;
 }
 
@@ -1075,7 +1089,7 @@ int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* 
     if (smem_need > (size_t)cap) return -1;
     const size_t smem = smem_need > 116 * 1024 ? smem_need : 116 * 1024;
     dim3 grid((unsigned)grid_n);
-    const cudaError_t le = rtoss_dev::launch_pdl(shared_kernel(ctx, ps[0]->dtype == RTOSS_F32, g), grid, kTcThreads, smem, (cudaStream_t)stream, 1, g);
+    const cudaError_t le = rtoss_dev::launch_pdl(shared_kernel(ctx, ps[0]->dtype == RTOSS_F32, g), grid, threads_of(ps[0]->dtype == RTOSS_F32), smem, (cudaStream_t)stream, 1, g);
     return (int)le;
 }
 

@@ -54,8 +54,17 @@
 //   * fp32 data runs on the same pipeline with kind::tf32 instructions and three products per tap in place of one:
 //     every value is split into a tf32 head (19 leading bits) and the remainder, x = xh + xl, w = wh + wl, and
 //     wh*xh + wh*xl + wl*xh is accumulated in fp32 (the dropped wl*xl is below 2^-21 of the product).  The weights are
-//     split when they are packed; an activation block is split in shared memory by the warp that fetched it (head in
-//     place, remainder into the second half of the stage) before the MMA thread may read it.
+//     split when they are packed; an activation block is split in shared memory by four warps (head in place, remainder
+//     into the second half of the stage) before the MMA thread may read it.  (One warp, the one that fetches, took 48 clocks
+//     a row, 14 000 for 288 rows, and the copy of the next block waited for it.)
+//     3x3 layers of whole blocks of 32 channels form the two small products from bf16 numbers, at twice the tf32 rate and
+//     in two instructions of 16 channels instead of four of eight: bf16(w) * bf16(xl) + bf16(wl) * bf16(x), heads rounded to
+//     nearest.  Eight instructions a tap and block instead of twelve; bf16 has fp32's range.  Rounding the factors of a
+//     product that is 2^-12 of the sum costs 7e-7 of it, but what decides is the tensor core's own accumulation, which cuts
+//     off and loses in proportion to the instructions issued: relative error against 64-bit sums 2.7e-6 -> 1.8e-6 for 32 to
+//     256 channels, 4.5e-6 -> 3.0e-6 for 512.  (1x1 layers, with a ninth of the instructions, err by 7e-7 in all with three
+//     tf32 products, and keep them.)  256->256 @80x80 x32 962 -> 650 us; the four units of tensor time it takes instead of six
+//     are 585 us at the bf16 peak.
 //   * One launch may carry several independent convolutions ("problems": the pyramid levels of a detection tower,
 //     the two branches of a block): the tile list runs over all of them, every role looks its tile's problem up.
 //     Small problems then fill the tail of the large ones' waves instead of paying a launch each.
@@ -67,6 +76,7 @@
 #include <cuda.h>
 
 #include "conv_common.cuh"
+#include "select_core.cuh"
 
 
 namespace {
@@ -75,7 +85,9 @@ using namespace rtoss_dev;
 
 constexpr int kEpiWarps = 16;
 constexpr int kTcThreads = (3 + kEpiWarps) * 32;  // activation TMA warp, MMA warp, sixteen epilogue warps, weight TMA warp
-constexpr int kWeightWarp = 2 + kEpiWarps;        // the last warp loads the weights
+constexpr int kWeightWarp = 2 + kEpiWarps;        // this warp loads the weights; it is the last one but for fp32 data
+constexpr int kSplitWarps = 4;                    // fp32: behind it, the warps that split the activation blocks
+template <typename T> constexpr int kThreadsOf = kTcThreads + (sizeof(T) == 4 ? kSplitWarps * 32 : 0);
 constexpr int kPatchRows = 16;       // positions an epilogue warp turns at a time
 constexpr int kMaxA = 4, kMaxB = 8;  // most activation stages / weight slots
 constexpr int kMTile = 128;          // filters per tile = TMEM lanes
@@ -132,7 +144,9 @@ struct TcArgs {
     int row_bytes;
     unsigned desc_hi;
     int taps_real;        // 9 or 1; `taps` counts weight tiles per channel block: twice that for fp32 (heads, then remainders)
-    int lo_off;           // fp32: byte offset of the remainders inside an activation stage
+    int lo_off;           // fp32: byte offset of the second half of an activation stage (remainders, or what corr16 says)
+    int corr16;           // fp32: the two small products of a tap are bf16 ones (see the head of the file)
+    unsigned idesc16;     // and their instruction descriptor
     // The operand rings this problem runs with: NA activation stages of a_stage bytes from the start of the ring area, NB
     // weight stages of b_stage bytes from sB_off.  Problems of one launch with the same `geo` share all five; where a
     // CTA passes to a problem of another geometry its rings run empty first (see bar_switch in the kernel).
@@ -892,6 +906,53 @@ __device__ __forceinline__ bool wait_deps(const G& g, unsigned dep_mask) {
     return true;
 }
 
+// fp32 activation blocks in shared memory (see the head of the file): n16 pieces of 16 bytes at src, split by kSplitWarps warps.
+// Heads in place, fp32 remainders at dst.
+__device__ __forceinline__ void split_block32(unsigned src, unsigned dst, int n16, int first) {
+#pragma unroll 4
+    for (int i = first; i < n16; i += kSplitWarps * 32) {
+        const uint4 u = lds128(src + 16u * i);
+        const float v[4] = {__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w)};
+        float h[4], l[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) h[e] = tf32_head(v[e]), l[e] = __fsub_rn(v[e], h[e]);
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(src + 16u * i), "f"(h[0]), "f"(h[1]), "f"(h[2]), "f"(h[3]) : "memory");
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(dst + 16u * i), "f"(l[0]), "f"(l[1]), "f"(l[2]), "f"(l[3]) : "memory");
+    }
+}
+// Heads (nearest) in place; at dst per pixel 32 channels in bf16, then their 32 remainders, in the swizzle TMA would have used
+// (16-byte piece j of row r lies at j ^ (r mod 8)).  A lane takes two neighbouring pieces of a row, eight channels; lanes of odd
+// rows store the two results the other way round, which keeps eight lanes on 32 different banks.
+__device__ __forceinline__ void split_block16(unsigned src, unsigned dst, int n16, int first) {
+#pragma unroll 2
+    for (int i = first; i < n16 >> 1; i += kSplitWarps * 32) {
+        const unsigned r = (unsigned)i >> 2, m = (unsigned)i & 3u, x7 = r & 7u;
+        const unsigned row = src + (r << 7), p0 = row + (((2 * m) ^ x7) << 4), p1 = row + (((2 * m + 1) ^ x7) << 4);
+        const uint4 u0 = lds128(p0), u1 = lds128(p1);
+        const float v[8] = {__uint_as_float(u0.x), __uint_as_float(u0.y), __uint_as_float(u0.z), __uint_as_float(u0.w),
+                            __uint_as_float(u1.x), __uint_as_float(u1.y), __uint_as_float(u1.z), __uint_as_float(u1.w)};
+        float h[8];
+        unsigned w16[4], l16[4];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) h[e] = tf32_near(v[e]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            w16[e] = bf16x2_sat(v[2 * e], v[2 * e + 1]);
+            l16[e] = bf16x2_sat(__fsub_rn(v[2 * e], h[2 * e]), __fsub_rn(v[2 * e + 1], h[2 * e + 1]));
+        }
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(p0), "f"(h[0]), "f"(h[1]), "f"(h[2]), "f"(h[3]) : "memory");
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(p1), "f"(h[4]), "f"(h[5]), "f"(h[6]), "f"(h[7]) : "memory");
+        const unsigned at = dst + (r << 7) + ((m ^ x7) << 4);   // (the remainders: the same with bit 6 flipped)
+        const bool odd = (r & 1u) != 0;
+        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(odd ? at ^ 64u : at), "r"(odd ? l16[0] : w16[0]),
+                     "r"(odd ? l16[1] : w16[1]), "r"(odd ? l16[2] : w16[2]), "r"(odd ? l16[3] : w16[3])
+                     : "memory");
+        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(odd ? at : at ^ 64u), "r"(odd ? w16[0] : l16[0]),
+                     "r"(odd ? w16[1] : l16[1]), "r"(odd ? w16[2] : l16[2]), "r"(odd ? w16[3] : l16[3])
+                     : "memory");
+    }
+}
+
 // What a launch is known to be when its kernel is compiled (0: anything).  Every launch starts on cold instruction caches,
 // and a layer of the small networks is over after three microseconds: the general kernel is 220 KB of code of which a
 // launch runs a tenth, in pieces all over it.  A form has nothing in it but what its launches run (25 to 50 KB).  Measured,
@@ -904,17 +965,19 @@ __device__ __forceinline__ bool wait_deps(const G& g, unsigned dep_mask) {
 //   bit 8     the output is NCHW
 //   bit 9     element stores (no residual): filter counts of no multiple of eight, unaligned channel slices
 // Forms are for 16-bit data; but for bit 9, channels-last outputs leave in whole 16-byte pieces.
-constexpr int kFormElem = 512;
+//   bit 10    fp32 with bf16 corrections (the only form of fp32 data; as a run-time branch it cost narrow layers without them 4 %)
+constexpr int kFormElem = 512, kFormCorr = 1024;
 constexpr int form_of(int kind, int act, bool split, int res, bool nchw) { return kind | (act + 1) << 2 | (split ? 32 : 0) | res << 6 | (nchw ? 256 : 0); }
 
 // kRep: the launch follows a layout pass (rtoss_launch_conv_tc_repacked): 16-bit outputs may be NCHW and SiLU takes its
 // exponential form.  An instantiation of its own: carried as run-time branches the two cost every other launch 0.5-1 %.
 template <typename T, typename G, bool kRep = false, int kForm = 0>
-__global__ void __launch_bounds__(kTcThreads, 1)
+__global__ void __launch_bounds__(kThreadsOf<T>, 1)
 conv_tc_kernel(const __grid_constant__ G g) {
     constexpr bool kMulti = sizeof(G) > sizeof(TcLaunch1);
     constexpr bool kF32 = sizeof(T) == 4;   // fp32 data: tf32 instructions, three products per tap (see the head of the file)
-    constexpr bool kAny = kForm == 0;
+    constexpr bool kAny = (kForm & ~kFormCorr) == 0;
+    constexpr bool kCorr1 = (kForm & kFormCorr) != 0;   // (fp32, one convolution: whether a.corr16; several: as it says)
     constexpr int kKind = kForm & 3, kAct = ((kForm >> 2) & 7) - 1;   // (kAny: both from the arguments)
     constexpr bool kSplitF = (kForm & 32) != 0, kNchw = (kForm & 256) != 0;
     constexpr int kRes = (kForm >> 6) & 3;
@@ -951,7 +1014,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
         for (int i = 0; i < g.max_na; ++i) {
             mbar_init(bar_fullA + 8 * i, 1);
             mbar_init(bar_emptyA + 8 * i, 1);
-            mbar_init(bar_loFull + 8 * i, 1);
+            mbar_init(bar_loFull + 8 * i, kSplitWarps);
         }
         for (int i = 0; i < g.max_nb; ++i) {
             mbar_init(bar_fullB + 8 * i, 1);
@@ -971,7 +1034,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
     // Where position p of a tile's list lies: the same for every tile (the tile's origin and the image's edges
     // come in per tile), so the epilogue looks it up instead of dividing.  {element offset from the tile's first
     // output, row << 16 | column}; positions that are no output (pitch padding, the list's tail) get 0xFFFFFFFF.
-    for (int q = threadIdx.x; q < g.n_tabs * kMaxPx; q += kTcThreads) {
+    for (int q = threadIdx.x; q < g.n_tabs * kMaxPx; q += kThreadsOf<T>) {
         int owner = 0;   // (any problem that uses the table describes it)
         while (owner + 1 < g.n_prob && g.prob[owner].tab != q / kMaxPx) ++owner;
         const TcArgs& a = g.prob[owner];
@@ -1006,8 +1069,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
         // hundred cycles whatever the size, so the activations and the weights have a producer thread each, and a
         // weight stage (G taps) is ONE copy.
         asm volatile("griddepcontrol.wait;" ::: "memory");   // the activations come from the kernels before this one
-        if (kF32 || lane == 0) {
-            // (fp32: all 32 lanes walk the loop; lane 0 issues the copies, then the warp splits the block that arrived)
+        if (lane == 0) {
             bool ok = true;
             Ring ra;
             int pi = 0, cur_pi = -1;
@@ -1020,10 +1082,8 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     // another problem: if its rings are laid out differently, the old ones must have run empty; if it
                     // depends on problems of this launch, they must be complete
                     const bool regeo = cur_pi >= 0 && a.geo != g.prob[cur_pi].geo;
-                    if (lane == 0) {
-                        if (regeo) ok = mbar_wait(bar_switch, n_sw & 1u, g.wait_cycles);
-                        if (ok && a.dep_mask) ok = wait_deps(g, a.dep_mask);
-                    }
+                    if (regeo) ok = mbar_wait(bar_switch, n_sw & 1u, g.wait_cycles);
+                    if (ok && a.dep_mask) ok = wait_deps(g, a.dep_mask);
                     if (regeo) {
                         ++n_sw;
                         ra.s = 0;
@@ -1036,52 +1096,17 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 const int cb_end = min(a.ncb, (ks + 1) * a.cb_per);
                 for (int cb = ks * a.cb_per; cb < cb_end; ++cb) {
                     const int sa = ra.s;
-                    const unsigned pa = ra.parity();
-                    if (lane == 0) {
-                        ok = ok && mbar_wait(bar_emptyA + 8 * sa, pa ^ 1, g.wait_cycles);
-                        if (ok) {
-                            const int n_sub = (kKind == 1 || kKind == 2) ? 1 : a.n_sub;
-                            mbar_expect_tx(bar_fullA + 8 * sa, a.a_tx_bytes * n_sub);
-                            for (int sub = 0; sub < n_sub; ++sub)
-                                tma_load_4d(sA + sa * a.a_stage + sub * a.sub_bytes, &g.tmA[pi], cb * a.cb_ch, x0 * a.S + a.x_add[sub],
-                                            y0 * a.S + a.y_add[sub], n, bar_fullA + 8 * sa);
-                        }
-                    }
-                    if (kF32) {
-                        // Split the block: x = head + remainder, head = the 19 leading bits (what a tf32 operand holds), in
-                        // place; the remainder (exact in fp32) goes to the second half of the stage.  Plain loads and stores
-                        // of this warp; the fence hands them to the proxy the tensor core reads through; then the stage is
-                        // announced to the MMA thread.  Any word may be split: rows the copy did not write are never outputs.
-                        ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
-                        if (ok) {
-                            if (lane == 0) ok = mbar_wait(bar_fullA + 8 * sa, pa, g.wait_cycles);
-                            ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
-                        }
-                        if (ok) {
-                            const unsigned src = sA + sa * a.a_stage, dst = src + (unsigned)a.lo_off;
-                            const int n16 = (a.n_sub * a.sub_bytes) >> 4;
-#pragma unroll 4
-                            for (int i = lane; i < n16; i += 32) {
-                                unsigned v[4], h[4], l[4];
-                                asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(src + 16u * i));
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    h[e] = v[e] & 0xFFFFE000u;
-                                    l[e] = __float_as_uint(__fsub_rn(__uint_as_float(v[e]), __uint_as_float(h[e])));
-                                }
-                                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(src + 16u * i), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
-                                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst + 16u * i), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
-                            }
-                            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                            __syncwarp();
-                            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_loFull + 8 * sa) : "memory");
-                        }
-                    }
+                    ok = ok && mbar_wait(bar_emptyA + 8 * sa, ra.parity() ^ 1, g.wait_cycles);
                     if (!ok) break;
+                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : a.n_sub;
+                    mbar_expect_tx(bar_fullA + 8 * sa, a.a_tx_bytes * n_sub);
+                    for (int sub = 0; sub < n_sub; ++sub)
+                        tma_load_4d(sA + sa * a.a_stage + sub * a.sub_bytes, &g.tmA[pi], cb * a.cb_ch, x0 * a.S + a.x_add[sub],
+                                    y0 * a.S + a.y_add[sub], n, bar_fullA + 8 * sa);
                     ra.advance(a.NA);
                 }
             }
-            if (!ok && lane == 0) atomicExch(g.status, 1);
+            if (!ok) atomicExch(g.status, 1);
         }
         __syncwarp();  // lanes 1..31 wait here for lane 0: the warp reaches the final barrier as one
     } else if (warp == kWeightWarp) {
@@ -1314,15 +1339,36 @@ conv_tc_kernel(const __grid_constant__ G g) {
                             if (!ok) break;
                             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                             const unsigned wl0 = desc_lo0 + (sB >> 4) + (unsigned)sb * bstage16;
-                            for (int i = 0; i < a.G; ++i) {
-                                // weight tile v of the block: tap v (16-bit data); fp32: the heads of tap v, then (v >= 9
-                                // resp. 1) the remainders of tap v - 9.  Heads meet the activations' heads and remainders,
-                                // remainders the heads only.
-                                const int v = t0 + i, t = v >= a.taps_real ? v - a.taps_real : v;
-                                const unsigned off = (unsigned)(a.tap_sub[t] * a.sub_bytes + a.tap_shift[t] * a.row_bytes) >> 4;
-                                const unsigned m4 = (unsigned)(bits >> (4 * t)) & nkmask;
-                                issue_tap(d_base, wl0 + i * wtile16, xl0 + off, m4, acc);
-                                if (kF32 && v < a.taps_real) issue_tap(d_base, wl0 + i * wtile16, xl0 + off + ((unsigned)a.lo_off >> 4), m4, acc);
+                            // weight tile v of the block: tap v (16-bit data); fp32: the heads of tap v, then (v >= 9 resp. 1) what
+                            // corrects tap v - 9.  Heads meet the activations' heads and remainders, remainders the heads
+                            // only; with bf16 corrections heads meet heads, and the rest is in the second arrays.
+                            if (kF32 && (kMulti ? a.corr16 != 0 : kCorr1)) {
+                                const unsigned xr0 = xl0 + ((unsigned)a.lo_off >> 4);
+                                for (int i = 0; i < a.G; ++i) {
+                                    const int v = t0 + i, t = v >= 9 ? v - 9 : v;
+                                    const unsigned off = (unsigned)(a.tap_sub[t] * a.sub_bytes + a.tap_shift[t] * a.row_bytes) >> 4;
+                                    const unsigned m4 = (unsigned)(bits >> (4 * t)) & nkmask;
+                                    if (v < 9) {
+                                        issue_tap(d_base, wl0 + i * wtile16, xl0 + off, m4, acc);
+                                        continue;
+                                    }
+                                    const unsigned wr = wl0 + i * wtile16, xr = xr0 + off;
+#pragma unroll
+                                    for (int h = 0; h < 2; ++h) {   // sixteen channels (a tap's heads came first: the accumulator holds something)
+                                        if ((m4 >> (2 * h)) & 3u) {
+                                            umma_f16<false>(leader, d_base, mk(wr + 2 * h), mk(xr + 4 + 2 * h), a.idesc16, 1u);
+                                            umma_f16<false>(leader, d_base, mk(wr + 4 + 2 * h), mk(xr + 2 * h), a.idesc16, 1u);
+                                        }
+                                    }
+                                }
+                            } else {
+                                for (int i = 0; i < a.G; ++i) {
+                                    const int v = t0 + i, t = v >= a.taps_real ? v - a.taps_real : v;
+                                    const unsigned off = (unsigned)(a.tap_sub[t] * a.sub_bytes + a.tap_shift[t] * a.row_bytes) >> 4;
+                                    const unsigned m4 = (unsigned)(bits >> (4 * t)) & nkmask;
+                                    issue_tap(d_base, wl0 + i * wtile16, xl0 + off, m4, acc);
+                                    if (kF32 && v < a.taps_real) issue_tap(d_base, wl0 + i * wtile16, xl0 + off + ((unsigned)a.lo_off >> 4), m4, acc);
+                                }
                             }
                             umma_commit(kMulti || flip_b ? leader : 0u, bar_emptyB + 8 * sb);
                             rb.advance(NB, flip_b);
@@ -1349,6 +1395,38 @@ conv_tc_kernel(const __grid_constant__ G g) {
             }
             if (!ok && leader) atomicExch(g.status, 2);
         }
+        __syncwarp();
+    } else if (kF32 && warp > kWeightWarp) {
+        // ---------------- fp32: the warps that split the activation blocks.  x = head + remainder; the head takes the value's
+        // place, the second half of the stage receives what the small products need.  Plain loads and stores; the fence hands
+        // them to the proxy the tensor core reads through; then the stage is announced to the MMA thread.  Any word may be
+        // split: rows the copy did not write are never outputs.
+        bool ok = true;
+        Ring ra;
+        int pi = 0, cur_pi = -1;
+        for (int unit = blockIdx.x; unit < n_tiles && ok; unit += gridDim.x) {
+            int local;
+            pi = find_problem<kMulti>(g, unit, local, pi);
+            const TcArgs& a = g.prob[pi];
+            if (kMulti && pi != cur_pi) {
+                if (cur_pi >= 0 && a.geo != g.prob[cur_pi].geo) ra.s = 0;   // (a new layout's first stage is full only behind the switch)
+                cur_pi = pi;
+            }
+            const int ks = tile_of(a, local).ks, cb_end = min(a.ncb, (ks + 1) * a.cb_per);
+            for (int cb = ks * a.cb_per; cb < cb_end; ++cb, ra.advance(a.NA)) {
+                if (lane == 0) ok = mbar_wait(bar_fullA + 8 * ra.s, ra.parity(), g.wait_cycles);
+                ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
+                if (!ok) break;
+                const unsigned src = sA + ra.s * a.a_stage, dst = src + (unsigned)a.lo_off;
+                const int n16 = (a.n_sub * a.sub_bytes) >> 4, first = (warp - kWeightWarp - 1) * 32 + lane;
+                if (kMulti ? a.corr16 != 0 : kCorr1) split_block16(src, dst, n16, first);
+                else split_block32(src, dst, n16, first);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar_loFull + 8 * ra.s) : "memory");
+            }
+        }
+        if (!ok && lane == 0) atomicExch(g.status, 1);
         __syncwarp();
     } else {
         // ---------------- epilogue: TMEM -> registers -> bias / activation -> NHWC global

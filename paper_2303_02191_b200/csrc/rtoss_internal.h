@@ -96,6 +96,13 @@ struct rtoss_wtc_layout {
     int cin_p;   // channels per row as stored: rows of 16-bit weights are padded with zeros to a multiple of 16 bytes (TMA strides)
 };
 static inline int rtoss_cin_pitch(int Cin, rtoss_dtype d) { return d == RTOSS_F32 ? Cin : (Cin + 7) / 8 * 8; }
+// fp32 3x3 layers of whole blocks of 32 channels: the second array of the dense-expanded weights holds, per block of 32 channels
+// (128 bytes), 32 weights rounded to bf16 and then their 32 remainders behind the tf32 heads, rounded to bf16; other fp32
+// layers hold the remainders in fp32 there.  (conv_tc_kernel.cuh says what they are multiplied with, and why only these.)
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+static inline bool rtoss_f32_corr16(int Cin, int ksize) { return ksize == 3 && Cin % 32 == 0; }
 static inline rtoss_wtc_layout rtoss_wtc_layout_of(int Cout, int Cin, int ksize, rtoss_dtype d) {
     rtoss_wtc_layout l;
     l.cin_p = rtoss_cin_pitch(Cin, d);

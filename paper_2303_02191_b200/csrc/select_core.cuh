@@ -38,6 +38,37 @@ __device__ __forceinline__ int select_best(const float (&w)[9], const Tab& tab, 
     return best;
 }
 
+// An fp32 value's tf32 head: the 19 leading bits; or the nearest value of 19 bits (a value that would round to infinity is cut
+// off instead), whose remainder is half as large.
+__device__ __forceinline__ float tf32_head(float f) { return __uint_as_float(__float_as_uint(f) & 0xFFFFE000u); }
+__device__ __forceinline__ float tf32_near(float f) {
+    const unsigned u = __float_as_uint(f), r = (u + 0x1000u) & 0xFFFFE000u;
+    return __uint_as_float((r & 0x7F800000u) == 0x7F800000u ? u & 0xFFFFE000u : r);
+}
+// Two floats rounded to bf16, a in the low half; finite values stay finite.
+__device__ __forceinline__ unsigned bf16x2_sat(float a, float b) {
+    unsigned d;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+    return d;
+}
+// The second array of rtoss_f32_corr16 layers: weight and remainder of flat position f (rows are whole blocks of 32 channels)
+// into its block; two neighbouring positions, f even.
+__device__ __forceinline__ uint16_t* corr16_at(float* lo, int64_t f) { return reinterpret_cast<uint16_t*>(lo) + 2 * (f & ~(int64_t)31) + (f & 31); }
+__device__ __forceinline__ void put_corr16_one(float* lo, int64_t f, float w, float rest) {
+    const unsigned u = bf16x2_sat(w, rest);
+    uint16_t* at = corr16_at(lo, f);
+    at[0] = (uint16_t)u;
+    at[32] = (uint16_t)(u >> 16);
+}
+__device__ __forceinline__ void put_corr16_two(float* lo, int64_t f, float w0, float w1, float rest0, float rest1) {
+    uint16_t* at = corr16_at(lo, f);
+    *reinterpret_cast<unsigned*>(at) = bf16x2_sat(w0, w1);
+    *reinterpret_cast<unsigned*>(at + 32) = bf16x2_sat(rest0, rest1);
+}
+__device__ __forceinline__ float to_float(float v) { return v; }
+__device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
+__device__ __forceinline__ float to_float(__half v) { return __half2float(v); }
+
 template <typename V> __device__ __forceinline__ V narrow_to(float v);
 template <> __device__ __forceinline__ float narrow_to<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 narrow_to<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
@@ -49,8 +80,9 @@ __device__ __forceinline__ void expand_one(const float* w, unsigned m, int64_t i
                                            int rep_rows, int copies, int cin_p) {
     // (layers hold fewer than 2^31 kernels: 32-bit division, several times cheaper than the 64-bit one)
     const int64_t co = (int64_t)((unsigned)i / (unsigned)Cin), ci = i - co * Cin;
-    // fp32: the tensor path multiplies tf32 operands, so every weight is stored as its tf32 head (the 19 leading bits)
-    // and, in a second copy of the array behind the first, the remainder (exact in fp32)
+    // fp32: the tensor path multiplies tf32 operands, so every weight is stored as its tf32 head and, in a second copy of
+    // the array behind the first, what corrects it: the remainder (exact in fp32), or two bf16 numbers (rtoss_f32_corr16)
+    const bool corr16 = rtoss_f32_corr16(Cin, ksize);
     const int64_t lo_at = (int64_t)(ksize == 3 ? 9 : 1) * rows * cin_p;
 #pragma unroll
     for (int t = 0; t < 9; ++t) {
@@ -58,7 +90,7 @@ __device__ __forceinline__ void expand_one(const float* w, unsigned m, int64_t i
         V lo = v;
         if (sizeof(V) == 4) {
             const float f = (m & (1u << t)) ? w[t] : 0.f;
-            const float head = __uint_as_float(__float_as_uint(f) & 0xFFFFE000u);
+            const float head = corr16 ? tf32_near(f) : tf32_head(f);
             v = narrow_to<V>(head);
             lo = narrow_to<V>(__fsub_rn(f, head));
         }
@@ -66,7 +98,11 @@ __device__ __forceinline__ void expand_one(const float* w, unsigned m, int64_t i
             const int64_t at = ((int64_t)t * rows + co) * cin_p + ci;   // copy 0; copy c lies c * rep_rows rows further down
             for (int c = 0; c < copies; ++c) {
                 wtc[at + (int64_t)c * rep_rows * cin_p] = v;
-                if (sizeof(V) == 4) wtc[lo_at + at + (int64_t)c * rep_rows * cin_p] = lo;
+                if (sizeof(V) == 4) {
+                    const int64_t f = at + (int64_t)c * rep_rows * cin_p;
+                    if (corr16) put_corr16_one(reinterpret_cast<float*>(wtc) + lo_at, f, to_float(v) + to_float(lo), to_float(lo));
+                    else wtc[lo_at + f] = lo;
+                }
             }
         } else {
             int64_t at = i * 9 + t;   // flat position; rows are cin_p apart where they are padded
@@ -81,7 +117,7 @@ __device__ __forceinline__ void expand_one(const float* w, unsigned m, int64_t i
 // val[i*k ...]; and, where the handle carries dense-expanded weights for the tensor path (wtc != nullptr), all nine
 // taps, pruned ones as +0:  3x3 -> wtc[t][row][ci] with `rows` rows of cin_p channels per tap, filter co = i / Cin at rows
 // c*rep_rows + co for c < copies (one copy at row co in the plain layout);  1x1 -> position 9*i + t of the flat matrix.  fp32 handles hold
-// two such arrays back to back: tf32 heads, then remainders.
+// two such arrays back to back: tf32 heads, then what corrects them (expand_one).
 template <typename V>
 __device__ __forceinline__ void pack_one(const float (&w)[9], unsigned m, int64_t i, int k, V* __restrict__ val,
                                          V* __restrict__ wtc, int ksize, int Cin, int rows, int rep_rows, int copies, int cin_p) {
@@ -216,8 +252,6 @@ __device__ __forceinline__ void select_best2(f32x2 (&q)[9], const Tab& tab, cons
         }
     }
 }
-
-__device__ __forceinline__ float tf32_head(float f) { return __uint_as_float(__float_as_uint(f) & 0xFFFFE000u); }
 
 // Stable counting sort of the Cout filters of input channel ci by pattern id, by one warp: perm[ci*Cout + j] lists
 // the filters by ascending id (ties by ascending filter), bucket_off[ci*(P+1) + p] is where pattern p starts.
