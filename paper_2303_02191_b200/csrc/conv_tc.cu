@@ -63,6 +63,8 @@ struct PlanKey {
                      // do per cycle; 2: with nothing beside it
     int max_px;      // most positions per tile
     int force_G, n_tabs;
+    int three;       // fp32: the cost of three tf32 products, whatever the layer's kernel forms (see plan_tc)
+    int most_cb;     // most channel blocks one CTA adds up (0: any number)
 };
 
 // Most thread-block clusters of `ks` CTAs (one CTA per SM) a device holds at once.  Clusters live inside a GPC and the
@@ -103,7 +105,7 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
     const bool f32 = k.dtype == RTOSS_F32;
     const int taps = k.ksize == 3 ? 9 : 1;
     const int slab_ch = f32 ? 8 : 16, cb_ch = row_bytes / (f32 ? 4 : 2);
-    const bool corr16 = f32 && rtoss_f32_corr16(k.Cin, k.ksize);
+    const bool corr16 = f32 && rtoss_f32_corr16(k.Cin, k.ksize) && !k.three;
     const double slabs = (double)(k.Cin < cb_ch ? k.Cin : cb_ch) / slab_ch * (corr16 ? 2 : f32 ? 3 : 1);
     const int wstages = f32 ? 2 * taps / G : taps / G;
     const PlanFit& f = f32 ? kFit32 : kFit16;
@@ -211,11 +213,13 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
                 for (int ks = 1; ks <= 8; ++ks) {
                     if (only_ks && ks != only_ks) continue;
                     int cb_per = ncb;
+                    if (ks == 1 && !only_ks && k.most_cb && ncb > k.most_cb) continue;
                     if (ks > 1) {
                         if (k.shared || pxm || R != 1 || tiles * ks > k.sms || ks > ncb) break;
                         if (tiles > max_clusters(k.dev, ks, k.sms)) continue;
                         cb_per = (ncb + ks - 1) / ks;
                         if ((ncb + cb_per - 1) / cb_per != ks) continue;   // (a share would be empty)
+                        if (k.most_cb && cb_per > k.most_cb) continue;
                         // the owners' buffers for the partial sums lie in the rings
                         const int n_lc = ((n_px + 31) / 32 + ks - 1) / ks;
                         if (ks * n_lc > 16 || ks * n_lc * 16384 > rings) continue;
@@ -289,7 +293,16 @@ bool plan_tc(const PlanKey& k, TcPlan* out) {
             m.ok = plan_search(k, k.resid != 0, 1, &m.plan);
         } else {
             int ks = 1;
-            if (plan_search(k, true, 0, &m.plan)) ks = m.plan.KS;
+            PlanKey q = k;
+            if (k.dtype == RTOSS_F32 && rtoss_f32_corr16(k.Cin, k.ksize)) {
+                // The tensor core cuts off at every accumulation: a sum may have no more of them than it had when a tap was twelve
+                // instructions instead of eight, so a layer that was cut along K then is not left in longer pieces now that
+                // its instructions are cheaper (128->128 @60x60 s2 x2 in two shares instead of four: 3.0e-6 instead of 2.7e-6).
+                q.three = 1;
+                if (plan_search(q, true, 0, &m.plan) && m.plan.KS > 1) q.most_cb = m.plan.cb_per * 3 / 2;
+                q.three = 0;
+            }
+            if (plan_search(q, true, 0, &m.plan)) ks = m.plan.KS;
             m.ok = plan_search(k, k.resid != 0, ks, &m.plan);
         }
         m.key = k;
