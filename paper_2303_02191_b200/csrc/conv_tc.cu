@@ -63,6 +63,7 @@ struct PlanKey {
                      // do per cycle; 2: with nothing beside it
     int max_px;      // most positions per tile
     int force_G, n_tabs;
+    int half;        // 3x3 stride 2 in two activation stages a channel block (see single_plan_key)
     int three;       // fp32: the cost of three tf32 products, whatever the layer's kernel forms (see plan_tc)
     int most_cb;     // most channel blocks one CTA adds up (0: any number)
 };
@@ -118,9 +119,18 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
         mma = wstages * (s > 0.28 ? s : 0.28) + f.block;
     }
     const double kb_b = (double)taps * w_rows * row_bytes * (f32 ? 2 : 1) / 1024.0, kb_a = a_bytes / 1024.0;
-    const double kb_fed = kb_a * (k.S == 2 ? f.strided : 1.0);
+    const bool half = k.half != 0;
+    const double kb_fed = kb_a * (k.S == 2 ? f.strided : 1.0) * (half ? 2 : 1);
     const double feed = (kb_fed + kb_b) / (corr16 ? 110 : f.feed);
     double blk = mma > feed ? mma : feed;
+    if (half) {
+        // a stage is asked for when the one NA before it has been read: what of its way the instructions in between do not cover
+        const double way = 0.5 + 0.5 * kb_fed / f.feed, one = mma / 3, two = 2 * mma / 3;
+        const double first = way - (na == 2 ? two : na == 3 ? mma : mma + one), second = way - (na == 2 ? one : na == 3 ? mma : mma + two);
+        const double late = mma + (first > 0 ? first : 0) + (second > 0 ? second : 0);
+        blk = late > blk ? late : blk;
+        na = 2;
+    }
     // one activation stage: loads and instructions take turns (fp32: and one warp's split of the block between them)
     if (na == 1) blk = mma + (f32 ? 0.045 * kb_a : f.lone * kb_fed / 87.0);
     if (f32 && !corr16 && G == 3) blk += 2.0;   // (then only two weight stages fit: the ring's round trip shows)
@@ -165,7 +175,8 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
     const int R = rtoss_wtc_layout_of(k.Cout, k.Cin, k.ksize, (rtoss_dtype)k.dtype).copies;
     const int S = k.S, Ho = k.Ho, Wo = k.Wo, ksize = k.ksize;
     const int halo = ksize == 3 ? (S == 1 ? 2 : 1) : 0;
-    const int n_sub = (ksize == 3 && S == 2) ? 4 : 1;
+    const bool half = k.half != 0;   // (then three taps a weight stage, and a_bytes is one of the block's two stages)
+    const int n_sub = half ? 2 : (ksize == 3 && S == 2) ? 4 : 1;
     const int max_pitch = S == 1 ? 256 : 128;  // TMA box: at most 256 elements traversed per dimension
     const int fixed = 1024 /*alignment slack*/ + 512 /*barriers*/ + kEpiWarps * kPatchBytes /*epilogue patches*/ +
                       k.n_tabs * kMaxPx * 8 /*position tables*/ + (resid ? kEpiWarps * kResStage : 0) /*staging of the residual operand*/;
@@ -195,17 +206,17 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
             const int sub_rows = round_up(need_rows, 8);
             const int a_bytes = n_sub * sub_rows * row_bytes * (f32 ? 2 : 1);   // (fp32: heads and remainders)
             const long tiles = (long)k.N * ty * nseg * co_tiles;
-            for (int G = (ksize == 3 ? 3 : 1); G >= 1; G -= 2) {
+            for (int G = (ksize == 3 ? 3 : 1); G >= (half ? 3 : 1); G -= 2) {
                 if (k.force_G && G != k.force_G) continue;   // (the problems of one launch share the weight ring: one G for all)
                 const int b_bytes = G * w_rows * row_bytes;
                 int na = (cap - fixed - 2 * b_bytes) / a_bytes;
-                if (na < 1) continue;
+                if (na < (half ? 2 : 1)) continue;
                 if (na > kMaxA) na = kMaxA;
                 // A channel block feeds nine taps: with several blocks per tile two stages cover the load.  A layer of
                 // one block per tile (at most 64 channels; 32 with 64-byte rows) has the next TILE's block as its next
                 // stage, and its instructions (18 or 36 of at most 128 cycles) are over before a fetch from L2 returns:
                 // it keeps as many stages as fit.
-                if (na > 2 && ksize == 3 && ncb > 1) na = 2;
+                if (na > 2 && ksize == 3 && ncb > 1 && !half) na = 2;
                 int nb = (cap - fixed - na * a_bytes) / b_bytes;
                 if (nb > kMaxB) nb = kMaxB;
                 if (nb < 2) continue;
@@ -404,6 +415,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     a.cb_ch = row_bytes / esize;
     a.tiles_x = plan.tiles_x;
     a.n_sub = plan.n_sub;
+    a.half = plan_k.half;
     a.sub_bytes = plan.sub_rows * row_bytes;
     if (p->ksize == 3 && S == 1) {
         a.x_add[0] = a.y_add[0] = -1;
@@ -416,7 +428,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
         }
         for (int t = 0; t < 9; ++t) {
             const int r = t / 3, c = t % 3;
-            a.tap_sub[t] = 2 * (r == 1 ? 0 : 1) + (c == 1 ? 0 : 1);
+            a.tap_sub[t] = (a.half ? 0 : 2 * (r == 1 ? 0 : 1)) + (c == 1 ? 0 : 1);   // (inside its stage)
             a.tap_shift[t] = (r == 0 ? 0 : 1) * plan.Wq + (c == 0 ? 0 : 1);
         }
     }
@@ -652,12 +664,29 @@ double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* con
     return shared_cost(ctx, n, ps, ds, nullptr);
 }
 
+// The plan key of a launch of one convolution.  16-bit 3x3 layers of stride 2 may have their channel blocks in two activation stages
+// (TcArgs::half): a second barrier round trip a block, which launches of a few microseconds feel (2 to 6 % where every layer took
+// it), against fetching under the instructions.  The model has to expect 7 % and half a microsecond of it, which is about its own
+// error; the layers that gain are then those of several tiles a CTA (20 % and more).  Decided as if the call had a residual operand, whether it has one or not: the taps
+// go out in another order, and a call with a residual adds up as the same call without one does.
+static PlanKey single_plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, int sms, int dev) {
+    PlanKey k = plan_key(p, d, sms, dev);
+    if (p->ksize != 3 || d->stride != 2 || p->dtype == RTOSS_F32) return k;
+    const int cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;   // (no form of it stores elements)
+    if (d->layout == RTOSS_NHWC && (p->Cout % 8 != 0 || cs % 8 != 0 || d->y_channel_offset % 8 != 0)) return k;
+    PlanKey one = k, two = k;
+    one.resid = two.resid = two.half = 1;
+    TcPlan a, b;
+    if (plan_tc(two, &b) && (!plan_tc(one, &a) || (b.us < 0.93 * a.us && b.us < a.us - 0.5))) k.half = 1;
+    return k;
+}
+
 // What a launch of its own is expected to take for this call (the planner's model), over how many CTAs it spreads a tile's
 // channel blocks, and how many tiles it has.  (Shared launches never split.)
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
     const rtoss_conv_desc dd = row_form(p, d);
-    if (ensure_device(ctx) || !plan_tc(plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    if (ensure_device(ctx) || !plan_tc(single_plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
     *us = plan.us;
     *ks = plan.KS;
     *tiles = plan.tiles;
@@ -694,14 +723,14 @@ extern "C" rtoss_status rtoss_tensor_plan_of(const rtoss_conv_desc* d, int ksize
     const int row_bytes = row_bytes_of(p);
     TcPlan plan;
     const rtoss_conv_desc row = row_form(p, d);
-    if (!plan_tc(plan_key(p, &row, sms, -1), &plan)) return RTOSS_OK;
+    if (!plan_tc(single_plan_key(p, &row, sms, -1), &plan)) return RTOSS_OK;
     out->eligible = 1;
     out->rows_per_tile = plan.TH, out->cols_per_tile = plan.TW, out->pitch = plan.Wq, out->positions = plan.N_px;
     out->act_stages = plan.NA, out->weight_stages = plan.NB, out->taps_per_weight_stage = plan.G;
     out->row_bytes = row_bytes;
     out->act_stage_bytes = plan.n_sub * plan.sub_rows * row_bytes * (f32 ? 2 : 1);
     out->weight_stage_bytes = plan.G * w_rows * row_bytes;
-    out->staged_rows = plan.rows_staged, out->sub_tiles = plan.n_sub;
+    out->staged_rows = plan.rows_staged, out->sub_tiles = ksize == 3 && d->stride == 2 ? 4 : 1;
     out->shared_bytes = plan.smem;
     out->positions_on_m = pxm ? 1 : 0;
     out->tiles = (int)(plan.tiles > 0x7FFFFFFF ? 0x7FFFFFFF : plan.tiles);
@@ -724,7 +753,7 @@ static int threads_of(bool f32) { return f32 ? kThreadsOf<float> : kThreadsOf<__
 static SingleKernel single_kernel(const rtoss_ctx* ctx, bool f32, bool repacked, const TcArgs& a) {
     if (!f32 && (a.taps == 1 || a.G == 3)) {
         const bool pieces = a.pxm || a.nchw || (a.y_c_stride % 8 == 0 && a.y_c_off % 8 == 0 && a.Cout % 8 == 0);
-        const int form = (pieces ? 0 : kFormElem) | form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
+        const int form = (pieces ? 0 : kFormElem) | (a.half ? kFormHalf : 0) | form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
         if (void* k = form_kernel(ctx, a.is_bf16, false, form)) return reinterpret_cast<SingleKernel>(k);
     }
     if (f32) return a.corr16 ? conv_tc_kernel<float, TcLaunch1, false, kFormCorr> : conv_tc_kernel<float, TcLaunch1>;
@@ -769,7 +798,7 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
     static thread_local TcLaunch1 g;   // several KB: kept off the stack
     ProbPlan pp;
     g.n_prob = 1;
-    PlanKey key = plan_key(p, d, sms, ctx_dev(ctx));
+    PlanKey key = single_plan_key(p, d, sms, ctx_dev(ctx));
     if (ctx->inject_next) key.sms = 1;   // (failure-detection hook: as few CTAs as the layer allows)
     e = build_problem(ctx, p, x, y, d, key, &g.prob[0], &pp, &g.tmA[0], &g.tmB[0]);
     if (e) return e;

@@ -24,6 +24,9 @@ using Pxm = std::integer_sequence<int, form_of(kKindPxm, kNone, false, 0, false)
                                   form_of(kKindPxm, kNone, false, 0, true), form_of(kKindPxm, kRelu, false, 0, true),
                                   form_of(kKindPxm, kSiluX, false, 0, true)>;
 
+// 3x3 of stride 2 in two activation stages a channel block
+template <int A, bool N> using Half = std::integer_sequence<int, form_of(kKind3, A, false, 0, N) | kFormHalf, form_of(kKind3, A, true, 0, N) | kFormHalf>;
+
 // A list of kernels as (form, function) pairs.
 struct FormEntry {
     int form;
@@ -35,7 +38,7 @@ void add_forms(FormEntry* list, int& n, std::integer_sequence<int, F...>) {
     for (const FormEntry& e : add) list[n++] = e;
 }
 
-constexpr int kMostForms = 64;
+constexpr int kMostForms = 80;
 struct FormTable {
     FormEntry one[kMostForms], shared[kMostForms];
     int n_one = 0, n_shared = 0;
@@ -61,6 +64,14 @@ FormTable make_forms() {
     add_forms<T, TcLaunch1>(t.one, t.n_one, Resid<kKind1, kRelu, 1>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Resid<kKind3, kSilu, 2>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Pxm());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kNone, false>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kRelu, false>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kSilu, false>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kSiluX, false>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, std::integer_sequence<int, form_of(kKind3, kSilu, false, 2, false) | kFormHalf, form_of(kKind3, kSilu, true, 2, false) | kFormHalf>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kNone, true>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kRelu, true>());
+    add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kSiluX, true>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind1, false>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind1, true>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Elem<kKind3, false>());
