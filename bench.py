@@ -608,9 +608,10 @@ def roofline_of(res, hbm_peak, tc_peak, peak_kind):
     flops = np.array([synth.layer_nnz_flops(L, N, k) for L, k in zip(res["layers"], res["ks"])])
     bytes_ = np.array([synth.layer_bytes(L, N, k, elem) for L, k in zip(res["layers"], res["ks"])], dtype=np.float64)
     # pipe peak per layer: the measured bf16 tensor peak; fp32 on the tensor path issues tf32 instructions (half the bf16
-    # rate) three times per product (head x head, head x remainder, remainder x head); else the nominal FMA peak
-    tc_eff = tc_peak if res["dtype"] != "f32" else tc_peak / 6
-    pipe = np.array([tc_eff if tc else ALU_PEAK_TFLOPS for tc in res["on_tc"]]) * 1e12
+    # rate) three times per product (head x head, head x remainder, remainder x head; in 3x3 layers of whole blocks of 32
+    # channels the last two are bf16 ones); else the nominal FMA peak
+    units_of = lambda L: 1 if res["dtype"] != "f32" else 4 if L["ksize"] == 3 and L["cin"] % 32 == 0 else 6
+    pipe = np.array([tc_peak / units_of(L) if tc else ALU_PEAK_TFLOPS for L, tc in zip(res["layers"], res["on_tc"])]) * 1e12
     t_pipe, t_hbm = flops / pipe, bytes_ / (hbm_peak * 1e9)
     t_roof = np.maximum(t_pipe, t_hbm)
     t_meas = res["conv_ms"] * 1e-3          # one entry per launch unit (a unit of several layers is one grouped call)
@@ -632,9 +633,10 @@ def roofline_of(res, hbm_peak, tc_peak, peak_kind):
     on_tc = res["on_tc"][members[0]]
     t_top = float(np.mean(t_meas[idx]))
     if t_pipe[members].sum() >= t_hbm[members].sum():
-        dom = {"bound": ("tensor (tf32 x3)" if res["dtype"] == "f32" else "tensor") if on_tc else "alu",
+        per_tap = units_of(res["layers"][members[0]])
+        dom = {"bound": {1: "tensor", 4: "tensor (tf32 + 2 bf16)", 6: "tensor (tf32 x3)"}[per_tap] if on_tc else "alu",
                "achieved": u_flops[top] / t_top / 1e12, "peak": pipe[members[0]] / 1e12, "unit": "TFLOP/s",
-               "peak_kind": ("of %s (bf16 cuBLAS, sustained)%s" % (peak_kind, " / 2 (tf32) / 3 (products per tap)" if res["dtype"] == "f32" else "")) if on_tc
+               "peak_kind": ("of %s (bf16 cuBLAS, sustained)%s" % (peak_kind, {1: "", 4: " / 4 (a tf32 product and two bf16 ones per tap)", 6: " / 2 (tf32) / 3 (products per tap)"}[per_tap])) if on_tc
                else "nominal, not measured: 148 SM x 128 FMA lanes x 2 x 1.965 GHz"}
     else:
         dom = {"bound": "hbm", "achieved": u_bytes[top] / t_top / 1e9, "peak": hbm_peak, "unit": "GB/s", "peak_kind": "of " + peak_kind}

@@ -385,8 +385,8 @@ rtoss_status rtoss_chain_deps_spans(const uint64_t* spans, int n, uint32_t* afte
 /* The tensor path (RTOSS_PATH_TENSOR, or RTOSS_PATH_AUTO when it applies) takes: NHWC, stride 1 or 2, io_dtype equal
  * to the packed dtype; bf16 / fp16 with Cin a multiple of 8, or fp32 with Cin a multiple of 4.  fp32 data is computed
  * with tf32 instructions on values split into a 19-bit head and a remainder (three products per tap, fp32
- * accumulation): results stay within the fp32 bound of 1e-4 of max(|y|, rms(y)) and cost six times the tensor time of
- * 16-bit data.  It multiplies blocks of 128 filters x 16
+ * accumulation; in 3x3 layers of whole blocks of 32 channels the two small products are bf16 ones): results stay within
+ * the fp32 bound of 1e-4 of max(|y|, rms(y)) and cost six (there four) times the tensor time of 16-bit data.  It multiplies blocks of 128 filters x 16
  * channels per tap on the tensor cores and leaves out the blocks in which every weight is pruned (none with
  * per-kernel patterns on ordinary weights; 9 - k of every 9 with rtoss_select_patterns_shared); inside a block the
  * pruned taps are multiplied as zeros.  Results agree with the FMA path to fp32 summation order.
@@ -474,7 +474,7 @@ rtoss_status rtoss_fma_plan3x3(const rtoss_conv_desc* desc, int Cin, int Cout, i
 typedef struct {
     int eligible;
     int rows_per_tile, cols_per_tile, pitch, positions;      /* output rows and columns of a tile, position pitch, the MMA's N */
-    int staged_rows, sub_tiles;                              /* input rows staged per tile; 4 parity sub-tiles for 3x3 stride 2 */
+    int staged_rows, sub_tiles;                              /* input rows staged per tile; 4 parity sub-tiles for 3x3 stride 2, in one or two stages */
     int act_stages, weight_stages, taps_per_weight_stage;    /* ring depths; taps fetched by one bulk copy */
     int row_bytes, act_stage_bytes, weight_stage_bytes;      /* 128, or 64 for 16-bit layers of at most 32 input channels */
     int shared_bytes;
