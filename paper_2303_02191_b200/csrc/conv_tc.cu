@@ -124,10 +124,11 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
     const double feed = (kb_fed + kb_b) / (corr16 ? 110 : f.feed);
     double blk = mma > feed ? mma : feed;
     if (half) {
-        // a stage is asked for when the one NA before it has been read: what of its way the instructions in between do not cover
+        // a stage is asked for when the one it takes the place of has been read (half_order): what of its way the instructions
+        // from there to its own do not cover
         const double way = 0.5 + 0.5 * kb_fed / f.feed, one = mma / 3, two = 2 * mma / 3;
-        const double first = way - (na == 2 ? two : na == 3 ? mma : mma + one), second = way - (na == 2 ? one : na == 3 ? mma : mma + two);
-        const double late = mma + (first > 0 ? first : 0) + (second > 0 ? second : 0);
+        const double odd = way - (na == 2 ? one : mma), even = way - (na == 2 ? one : na == 3 ? two : mma);
+        const double late = mma + (odd > 0 ? odd : 0) + (even > 0 ? even : 0);
         blk = late > blk ? late : blk;
         na = 2;
     }
@@ -313,6 +314,7 @@ bool plan_tc(const PlanKey& k, TcPlan* out) {
                 if (plan_search(q, true, 0, &m.plan) && m.plan.KS > 1) q.most_cb = m.plan.cb_per * 3 / 2;
                 q.three = 0;
             }
+            q.half = 0;   // (in two stages a layer is cut along K as in one: the same sums)
             if (plan_search(q, true, 0, &m.plan)) ks = m.plan.KS;
             m.ok = plan_search(k, k.resid != 0, ks, &m.plan);
         }
@@ -415,7 +417,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     a.cb_ch = row_bytes / esize;
     a.tiles_x = plan.tiles_x;
     a.n_sub = plan.n_sub;
-    a.half = plan_k.half;
+    a.half = plan_k.half ? 1 : 0;   // (the launch writes the order here)
     a.sub_bytes = plan.sub_rows * row_bytes;
     if (p->ksize == 3 && S == 1) {
         a.x_add[0] = a.y_add[0] = -1;
@@ -667,26 +669,30 @@ double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* con
 // The plan key of a launch of one convolution.  16-bit 3x3 layers of stride 2 may have their channel blocks in two activation stages
 // (TcArgs::half): a second barrier round trip a block, which launches of a few microseconds feel (2 to 6 % where every layer took
 // it), against fetching under the instructions.  The model has to expect 7 % and half a microsecond of it, which is about its own
-// error; the layers that gain are then those of several tiles a CTA (20 % and more).  Decided as if the call had a residual operand, whether it has one or not: the taps
-// go out in another order, and a call with a residual adds up as the same call without one does.
+// error; the layers that gain are then those of several tiles a CTA (20 % and more; 60 layers of 16 to 512 channels, batch 1 to
+// 32, take 0.935 of the time in one stage in the geometric mean, the slowest 1.016).
 static PlanKey single_plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, int sms, int dev) {
     PlanKey k = plan_key(p, d, sms, dev);
     if (p->ksize != 3 || d->stride != 2 || p->dtype == RTOSS_F32) return k;
     const int cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;   // (no form of it stores elements)
     if (d->layout == RTOSS_NHWC && (p->Cout % 8 != 0 || cs % 8 != 0 || d->y_channel_offset % 8 != 0)) return k;
-    PlanKey one = k, two = k;
-    one.resid = two.resid = two.half = 1;
+    PlanKey two = k;
+    two.half = 1;
     TcPlan a, b;
-    if (plan_tc(two, &b) && (!plan_tc(one, &a) || (b.us < 0.93 * a.us && b.us < a.us - 0.5))) k.half = 1;
-    return k;
+    return plan_tc(k, &a) && plan_tc(two, &b) && b.us < 0.93 * a.us && b.us < a.us - 0.5 ? two : k;
 }
+// TcArgs::half for NA stages: a block's odd rows are read until its end, its even rows for two thirds of it, and a stage is
+// filled again by whatever comes next once it is free.  With two stages the odd and the even rows change places from block
+// to block; with three the even rows keep theirs; with four a block has a pair.
+static unsigned half_order(int NA) { return NA == 2 ? 0u | 1u << 2 | 1u << 4 | 0u << 6 : NA == 3 ? 0u | 1u << 2 | 2u << 4 | 1u << 6 : 0u | 1u << 2 | 2u << 4 | 3u << 6; }
 
 // What a launch of its own is expected to take for this call (the planner's model), over how many CTAs it spreads a tile's
-// channel blocks, and how many tiles it has.  (Shared launches never split.)
+// channel blocks, and how many tiles it has.  (Shared launches never split.)  3x3 of stride 2 counts as in one activation stage: what
+// hangs on this is how calls are grouped, and with it where sums are cut.
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
     const rtoss_conv_desc dd = row_form(p, d);
-    if (ensure_device(ctx) || !plan_tc(single_plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    if (ensure_device(ctx) || !plan_tc(plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
     *us = plan.us;
     *ks = plan.KS;
     *tiles = plan.tiles;
@@ -852,6 +858,7 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
             g.max_nb = a.NB;
         }
     }
+    if (a.half) a.half = half_order(a.NA);
     // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM
     const size_t smem = (size_t)(smem_need > 116 * 1024 ? smem_need : 116 * 1024);
     cudaError_t le;

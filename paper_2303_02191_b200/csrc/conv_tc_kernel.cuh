@@ -119,11 +119,14 @@ struct TcArgs {
     // every role for every tile: the four divisors as multiply-and-shift pairs (see tile_of), set by the host.
     unsigned div_ks[2], div_co[2], div_tx[2], div_ty[2];
     int n_sub, sub_bytes;        // sub-tiles of an activation stage (3x3 stride 2: the 4 input phases, or 2 of them) and their size
-    // 16-bit 3x3 of stride 2, where the planner says so: a channel block comes as two activation stages, the even input rows (two
-    // column phases, read by the middle row of taps) and the odd ones (read by the other two); the taps go out in that
-    // order.  As one stage, of which only one fits beside the weights at 100 positions and more, fetching and multiplying
-    // take turns: 240->112 @132x66 x18 34.6 -> 25.9 us, 144->240 @134x71 x9 24.9 -> 19.5, 48->304 @110x115 x31 63.5 -> 50.9.
-    int half;
+    // 16-bit 3x3 of stride 2, where the planner says so (0: not): a channel block comes as two activation stages, the odd input
+    // rows (two column phases, read by the first and the last row of taps) and the even ones (read by the middle row).  The even
+    // rows are done with first, so the stages are taken in the order in which they come free, which this word lists: the
+    // stage of the odd and the even rows of a block, then of the next, two bits each (half_order).  The taps go out in their
+    // own order, so that a layer adds up here as it does in one stage.  As one stage, of which only one fits beside the
+    // weights at 100 positions and more, fetching and multiplying take turns: 240->112 @132x66 x18 34.5 -> 26.9 us, 144->240
+    // @134x71 x9 24.3 -> 19.5, 48->304 @110x115 x31 62.4 -> 50.6.
+    unsigned half;
     int x_add[4], y_add[4];      // TMA start coordinate of sub-tile s: x = x0*S + x_add[s], y = y0*S + y_add[s]
     int tap_sub[9], tap_shift[9];  // which sub-tile tap t reads, and from which start row
     int G;                                     // taps per weight stage (one barrier round trip per G taps)
@@ -973,8 +976,6 @@ __device__ __forceinline__ void split_block16(unsigned src, unsigned dst, int n1
 //   bit 10    fp32 with bf16 corrections (the only form of fp32 data; as a run-time branch it cost narrow layers without them 4 %)
 //   bit 11    3x3 of stride 2 in two activation stages a channel block (TcArgs::half)
 constexpr int kFormElem = 512, kFormCorr = 1024, kFormHalf = 2048;
-// The tap that is the i-th to go out (half: the middle row first).
-__device__ __forceinline__ int half_tap(bool half, int i) { return half && i < 6 ? (i < 3 ? i + 3 : i - 3) : i; }
 constexpr int form_of(int kind, int act, bool split, int res, bool nchw) { return kind | (act + 1) << 2 | (split ? 32 : 0) | res << 6 | (nchw ? 256 : 0); }
 
 // kRep: the launch follows a layout pass (rtoss_launch_conv_tc_repacked): 16-bit outputs may be NCHW and SiLU takes its
@@ -1081,6 +1082,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
         if (lane == 0) {
             bool ok = true;
             Ring ra;
+            int hq = 0;          // TcArgs::half: 0 or 2, which half of the order the coming block takes
             int pi = 0, cur_pi = -1;
             unsigned n_sw = 0;   // geometry changes so far
             for (int unit = blockIdx.x; unit < n_tiles && ok; unit += gridDim.x) {
@@ -1100,13 +1102,15 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     cur_pi = pi;
                 }
                 const TileIdx ti = tile_of(a, local);
+                const bool half = (kAny && !kF32) ? a.half != 0 : kHalf;
                 const int ks = ti.ks, n = ti.n;
                 const int y0 = ti.ty * a.TH, x0 = ti.tx * a.TW;
                 const int cb_end = min(a.ncb, (ks + 1) * a.cb_per);
                 for (int cb = ks * a.cb_per; cb < cb_end; ++cb) {
-                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : kHalf ? 2 : a.n_sub, n_all = (kAny && !kF32 && a.half) || kHalf ? 4 : n_sub;
-                    for (int sub0 = 0; sub0 < n_all; sub0 += n_sub) {   // (one stage, or the two of a half)
-                        const int sa = ra.s;
+                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : kHalf ? 2 : a.n_sub, n_stages = half ? 2 : 1;
+                    for (int part = 0; part < n_stages; ++part) {   // (half: the odd rows, sub-tiles 2 and 3, then the even ones)
+                        if (half) ra.s = (int)(a.half >> (2 * (hq + part))) & 3;
+                        const int sa = ra.s, sub0 = half ? 2 - 2 * part : 0;
                         ok = ok && mbar_wait(bar_emptyA + 8 * sa, ra.parity() ^ 1, g.wait_cycles);
                         if (!ok) break;
                         mbar_expect_tx(bar_fullA + 8 * sa, a.a_tx_bytes * n_sub);
@@ -1115,6 +1119,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                                         y0 * a.S + a.y_add[sub0 + sub], n, bar_fullA + 8 * sa);
                         ra.advance(a.NA);
                     }
+                    hq ^= 2;
                     if (!ok) break;
                 }
             }
@@ -1155,7 +1160,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                         // (failure-detection hook: the launch's very first weight copy is withheld, so the wait for it runs out)
                         if (!(g.inject == 1 && unit == (int)blockIdx.x && cb == ks * a.cb_per && t0 == 0)) {
                             mbar_expect_tx(bar_fullB + 8 * sb, a.b_tx_bytes * w_G);
-                            tma_load_3d(sB + sb * a.b_stage, &g.tmB[pi], cb * a.cb_ch, co0, half_tap((kAny && !kF32 && a.half) || kHalf, t0), bar_fullB + 8 * sb);
+                            tma_load_3d(sB + sb * a.b_stage, &g.tmB[pi], cb * a.cb_ch, co0, t0, bar_fullB + 8 * sb);
                         }
                         rb.advance(a.NB);
                     }
@@ -1185,6 +1190,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
             int cur_pi = -1, pi = 0;
             const unsigned bar_rdyA = kF32 ? bar_loFull : bar_fullA;   // the barrier that says an activation stage may be read
             Ring ra, rb;
+            int hq = 0;                         // (as the activation producer's)
             int as = 0, n_done = 0;
             unsigned pacc = 0;                  // phase parity of the accumulator ring
             const unsigned flip_b = !kMulti && g.prob[0].resident ? 0u : 1u;   // (see TcArgs::resident)
@@ -1245,10 +1251,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     NA = a.NA;
                     NB = a.NB;
 #pragma unroll
-                    for (int i = 0; i < 9; ++i) {
-                        const int t = half_tap((kAny && !kF32 && a.half) || kHalf, i);
-                        tap16[i] = (unsigned)(a.tap_sub[t] * a.sub_bytes + a.tap_shift[t] * a.row_bytes) >> 4;
-                    }
+                    for (int t = 0; t < 9; ++t) tap16[t] = (unsigned)(a.tap_sub[t] * a.sub_bytes + a.tap_shift[t] * a.row_bytes) >> 4;
                     wtile16 = (unsigned)(a.w_rows * a.row_bytes) >> 4;
                     desc_hi = a.desc_hi;
                     half16 = (unsigned)(128 * a.row_bytes) >> 4;   // the second 128 positions of a tile
@@ -1275,7 +1278,9 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     constexpr int kSlab = kF32 ? 8 : 16;
                     const int nk4 = (min(left, a.cb_ch) + kSlab - 1) / kSlab;
                     const unsigned nkmask = (1u << nk4) - 1u;
-                    int sa = ra.s;
+                    const bool half = (kAny && !kF32) ? a.half != 0 : kHalf;
+                    if (half) ra.s = (int)(a.half >> (2 * hq)) & 3;
+                    const int sa = ra.s;
                     if (kAny ? a.taps == 1 : kKind != 3) {
                         const int sb = rb.s;
                         if (!(peek & 1u)) ok = mbar_wait(bar_rdyA + 8 * sa, ra.parity(), g.wait_cycles);
@@ -1315,49 +1320,45 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     if (!(peek & 1u)) ok = mbar_wait(bar_rdyA + 8 * sa, ra.parity(), g.wait_cycles);   // (peek stays 0 on the paths that do not look ahead)
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    unsigned xl0 = desc_lo0 + (sA >> 4) + (unsigned)sa * astage16;
-                    const bool half = (kAny && !kF32) ? a.half != 0 : kHalf;
-                    auto second_half = [&]() {   // the block's first stage has been read, on to the second
-                        umma_commit(leader, bar_emptyA + 8 * sa);
-                        sa = ra.s;
-                        if (!(peek & 1u)) ok = ok && mbar_wait(bar_rdyA + 8 * sa, ra.parity(), g.wait_cycles);
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        xl0 = desc_lo0 + (sA >> 4) + (unsigned)sa * astage16;
-                        ra.advance(NA);
-                    };
+                    const unsigned xl0 = desc_lo0 + (sA >> 4) + (unsigned)sa * astage16;
                     ra.advance(NA);   // (sa stays this block's stage; ra is at the next one, which the look ahead reads)
                     if (kAny ? unrolled9 : kKind == 3) {
+                        if (half) ra.s = (int)(a.half >> (2 * hq + 2)) & 3;
+                        const int sa_e = ra.s;   // (half: the stage of the even rows)
                         int sa_n = ra.s;
                         unsigned pa_n = ra.parity();
-                        const unsigned long long ordered = half ? (bits & ~0xFFFFFFull) | (bits & 0xFFF) << 12 | ((bits >> 12) & 0xFFF) : bits;
 #pragma unroll
                         for (int s3 = 0; s3 < 3; ++s3) {
-                            if (s3 == 1 && half) {
-                                second_half();
-                                sa_n = ra.s;
+                            if (s3 == 1 && half) {   // the even rows; the look ahead is for the next block from here on
+                                if (!(peek & 1u)) ok = ok && mbar_wait(bar_rdyA + 8 * sa_e, ra.parity(), g.wait_cycles);
+                                ra.advance(NA);
+                                hq ^= 2;
+                                ra.s = sa_n = (int)(a.half >> (2 * hq)) & 3;
                                 pa_n = ra.parity();
                             }
+                            if (s3 == 2 && half && ok) umma_commit(leader, bar_emptyA + 8 * sa_e);
+                            const unsigned xl = s3 == 1 && half ? desc_lo0 + (sA >> 4) + (unsigned)sa_e * astage16 : xl0;
                             const int sb = rb.s;
                             if (!(peek & 2u)) ok = ok && mbar_wait(bar_fullB + 8 * sb, rb.parity(), g.wait_cycles);
                             if (ok) {
                                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                                 const unsigned wl0 = desc_lo0 + (sB >> 4) + (unsigned)sb * bstage16;
-                                const unsigned m_first = (unsigned)(ordered >> (12 * s3)) & nkmask;
+                                const unsigned m_first = (unsigned)(bits >> (12 * s3)) & nkmask;
                                 rb.advance(NB, flip_b);
                                 if (kAny ? !pxm : true) {
                                     // the first tap of the stage goes out together with a look at the next stages
-                                    peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl0 + tap16[s3 * 3]), idesc, acc, leader ? m_first : 0u,
+                                    peek = umma_block_peek<kF32>(d_base, mk(wl0), mk(xl + tap16[s3 * 3]), idesc, acc, leader ? m_first : 0u,
                                                            bar_rdyA + 8 * sa_n, pa_n, bar_fullB + 8 * rb.s, rb.parity());
                                     if (m_first) acc = 1;
 #pragma unroll
                                     for (int i = 1; i < 3; ++i)
-                                        issue_tap(d_base, wl0 + i * wtile16, xl0 + tap16[s3 * 3 + i],
-                                                  (unsigned)(ordered >> (12 * s3 + 4 * i)) & nkmask, acc);
+                                        issue_tap(d_base, wl0 + i * wtile16, xl + tap16[s3 * 3 + i],
+                                                  (unsigned)(bits >> (12 * s3 + 4 * i)) & nkmask, acc);
                                 } else {
 #pragma unroll
                                     for (int i = 0; i < 3; ++i)
-                                        issue_tap(d_base, wl0 + i * wtile16, xl0 + tap16[s3 * 3 + i],
-                                                  (unsigned)(ordered >> (12 * s3 + 4 * i)) & nkmask, acc);
+                                        issue_tap(d_base, wl0 + i * wtile16, xl + tap16[s3 * 3 + i],
+                                                  (unsigned)(bits >> (12 * s3 + 4 * i)) & nkmask, acc);
                                 }
                                 umma_commit(kMulti || flip_b ? leader : 0u, bar_emptyB + 8 * sb);  // this weight stage may be refilled once the MMAs have read it
                             }

@@ -1,6 +1,8 @@
-"""16-bit 3x3 layers of stride 2, whose channel blocks come in two activation stages (even and odd input rows): odd and even
-sides, one row or column, 64-byte rows (32 channels and fewer), ragged channels and filters, one and several channel blocks,
-few tiles (cut along K), many tiles a CTA, and a shared launch."""
+"""16-bit 3x3 layers of stride 2.  The first two tests: odd and even sides, one row or column, 64-byte rows (32 channels and
+fewer), ragged channels and filters, one and several channel blocks, cut along K, a shared launch; the planner takes them
+with a channel block in one activation stage.  The others: layers whose channel blocks come in two activation stages (odd and
+even input rows), which the plan is asked to confirm; a call adds up in the order of a shared launch, which has one stage, so
+uncut ones give its bits."""
 import pytest
 import torch
 
@@ -48,5 +50,111 @@ def test_shared_launch():
     torch.cuda.synchronize()
     for x, xd, yd in keep:
         assert orc.rel_err(gu.from_dev(yd, "nhwc"), gu.oracle_conv(3, x, wd, None, 2, "relu", "bf16")) <= TOL["bf16"]
+    assert c.rtoss_device_status() == 0
+    packed.close()
+
+
+def _two_stages(N, H, W, Cin, Cout, dt, residual=False):
+    """(in two stages?, stages, shares) by the plan: the bytes of an activation stage against those of its sub-tiles."""
+    p = rt.rtoss_tensor_plan_of(N, H, W, 2, 3, Cin, Cout, rt.DTYPE_NAMES[dt], residual=residual)
+    sub = (max(p.positions + p.pitch + 1, p.staged_rows * p.pitch) + 7) // 8 * 8 * p.row_bytes
+    return p.act_stage_bytes == 2 * sub, p.act_stages, p.split_k
+
+
+def _layer(N, Cin, Cout, H, W, dt, patterns, k=4):
+    c = gu.ctx()
+    masks = rt.rtoss_pattern_preset(k, rt.PRESET_CENTRE8 if k == 4 else rt.PRESET_CONN4)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(Cin + Cout + H)
+    w = torch.randn(Cout, Cin, 3, 3, device="cuda", generator=g) * (2.0 / (9 * Cin)) ** 0.5
+    pid = c.rtoss_select_patterns_shared(w, masks, k, 128, 16) if patterns == "block" else c.rtoss_select_patterns(w, 3, masks, k)
+    packed = c.rtoss_pack(w, 3, masks, k, pid, rt.DTYPE_NAMES[dt])
+    x = torch.randn(N, H, W, Cin, device="cuda", generator=g).to(gu.TORCH_DT[dt])
+    bias = torch.randn(Cout, device="cuda", generator=g) * 0.1
+    return c, packed, x, bias, g
+
+
+def _exact(packed, x, bias, act):
+    w = packed.to_dense().double().reshape(packed.info.Cout, packed.info.Cin, 3, 3)
+    y = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), w, bias.double(), stride=2, padding=1).permute(0, 2, 3, 1)
+    return {"none": lambda v: v, "relu": torch.relu, "silu": torch.nn.functional.silu}[act](y)
+
+
+def _near(y, ref, dt, act="none", roundings=1):
+    """Within a unit per rounding, and SiLU's approximation: tanh to 2^-11 of itself, times half of an input of up to 5.5
+    deviations, against the 0.6 that the result's root mean square is of a deviation."""
+    bound = roundings * TOL[dt] + (2 ** -11 * 5.5 / 2 / 0.6 if act == "silu" else 0)
+    return ((y.double() - ref).abs() / torch.maximum(ref.abs(), ref.pow(2).mean().sqrt())).max().item() <= bound
+
+
+UNCUT = [   # N, Cin, Cout, H, W, dtype, activation, stages
+    (10, 64, 16, 116, 55, "bf16", "none", 2), (11, 40, 16, 51, 130, "f16", "relu", 2), (8, 64, 16, 131, 26, "f16", "silu", 3),
+    (31, 56, 16, 33, 36, "bf16", "silu", 3), (18, 16, 16, 125, 125, "bf16", "relu", 3),                # (64-byte rows, resident weights)
+    (15, 160, 216, 79, 62, "bf16", "relu", 2), (8, 96, 128, 80, 80, "f16", "none", 3), (9, 416, 208, 71, 84, "bf16", "none", 3),
+]
+
+
+@pytest.mark.parametrize("patterns", ["kernel", "block"])
+@pytest.mark.parametrize("N,Cin,Cout,H,W,dt,act,stages", UNCUT)
+def test_two_stages_give_the_bits_of_one(N, Cin, Cout, H, W, dt, act, stages, patterns):
+    assert _two_stages(N, H, W, Cin, Cout, dt) == (True, stages, 1)
+    c, packed, x, bias, _ = _layer(N, Cin, Cout, H, W, dt, patterns)
+    y = [torch.empty(N, (H + 1) // 2, (W + 1) // 2, Cout, dtype=x.dtype, device="cuda") for _ in range(3)]
+    c.rtoss_conv3x3_pattern(packed, x, y[0], N, H, W, 2, rt.NHWC, rt.ACT_NAMES[act], bias)
+    assert c.rtoss_conv_group([c.conv_item(packed, x, t, N, H, W, 2, rt.NHWC, rt.ACT_NAMES[act], bias) for t in y[1:]]) == 1
+    assert torch.equal(y[0], y[1]) and torch.equal(y[1], y[2])
+    assert _near(y[0], _exact(packed, x, bias, act), dt, act)
+    assert c.rtoss_device_status() == 0
+    packed.close()
+
+
+@pytest.mark.parametrize("after_act", [False, True])
+@pytest.mark.parametrize("act", ["none", "relu", "silu"])
+@pytest.mark.parametrize("N,Cin,Cout,H,W,dt,stages", [(21, 64, 16, 24, 118, "bf16", 2), (19, 80, 16, 73, 36, "bf16", 2), (23, 64, 16, 117, 18, "f16", 2)])
+def test_residual(N, Cin, Cout, H, W, dt, stages, act, after_act):
+    assert _two_stages(N, H, W, Cin, Cout, dt, residual=True) == (True, stages, 1)
+    c, packed, x, bias, g = _layer(N, Cin, Cout, H, W, dt, "kernel")
+    res = torch.randn(N, (H + 1) // 2, (W + 1) // 2, Cout, device="cuda", generator=g).to(x.dtype)
+    y = [torch.empty_like(res) for _ in range(3)]
+    args = (N, H, W, 2, rt.NHWC, rt.ACT_NAMES[act], bias)
+    c.rtoss_conv3x3_pattern(packed, x, y[0], *args, residual=res, residual_after_act=after_act)
+    if after_act:   # (the call without the operand, and an addition)
+        c.rtoss_conv3x3_pattern(packed, x, y[1], *args)
+        assert torch.equal(y[0], (y[1].float() + res.float()).to(x.dtype))
+    else:
+        assert c.rtoss_conv_group([c.conv_item(packed, x, t, *args, residual=res) for t in y[1:]]) == 1
+        assert torch.equal(y[0], y[1]) and torch.equal(y[1], y[2])
+    assert c.rtoss_device_status() == 0
+    packed.close()
+
+
+@pytest.mark.parametrize("act", ["none", "relu", "silu"])
+@pytest.mark.parametrize("N,Cin,Cout,H,W,dt", [(10, 64, 16, 116, 55, "bf16"), (31, 56, 18, 33, 36, "f16"), (8, 96, 128, 80, 80, "bf16")])
+def test_behind_the_layout_pass(N, Cin, Cout, H, W, dt, act):
+    assert _two_stages(N, H, W, Cin, (Cout + 7) // 8 * 8, dt)[0]   # (planned alike: the filters are one tile)
+    c, packed, x, bias, _ = _layer(N, Cin, Cout, H, W, dt, "kernel")
+    xc, shape = x.permute(0, 3, 1, 2).contiguous(), (N, Cout, (H + 1) // 2, (W + 1) // 2)
+    y = torch.empty(shape, dtype=x.dtype, device="cuda")
+    c.rtoss_conv3x3_pattern(packed, xc, y, N, H, W, 2, rt.NCHW, rt.ACT_NAMES[act], bias)
+    assert _near(y.permute(0, 2, 3, 1), _exact(packed, x, bias, act), dt, act)
+    assert c.rtoss_device_status() == 0
+    packed.close()
+
+
+@pytest.mark.parametrize("N,Cin,Cout,H,W,dt,act,residual,stages,shares", [
+    (8, 392, 264, 11, 39, "bf16", "relu", False, 2, 4), (9, 384, 440, 13, 34, "f16", "silu", False, 2, 3), (9, 384, 440, 13, 34, "bf16", "silu", True, 2, 3),
+    (11, 272, 144, 14, 21, "bf16", "none", False, 3, 3), (15, 320, 72, 8, 88, "f16", "silu", False, 3, 3), (27, 312, 80, 21, 20, "bf16", "relu", True, 2, 3),
+    (4, 488, 448, 12, 123, "bf16", "silu", False, 3, 2), (5, 456, 288, 61, 11, "f16", "none", False, 3, 4),
+])
+def test_cut_along_k(N, Cin, Cout, H, W, dt, act, residual, stages, shares):
+    assert _two_stages(N, H, W, Cin, Cout, dt, residual) == (True, stages, shares)
+    c, packed, x, bias, g = _layer(N, Cin, Cout, H, W, dt, "kernel")
+    res = torch.randn(N, (H + 1) // 2, (W + 1) // 2, Cout, device="cuda", generator=g).to(x.dtype) if residual else None
+    y = torch.empty(N, (H + 1) // 2, (W + 1) // 2, Cout, dtype=x.dtype, device="cuda")
+    c.rtoss_conv3x3_pattern(packed, x, y, N, H, W, 2, rt.NHWC, rt.ACT_NAMES[act], bias, residual=res, residual_after_act=True)
+    ref = _exact(packed, x, bias, act)
+    if residual:
+        ref = ref.to(x.dtype).double() + res.double()
+    assert _near(y, ref, dt, act, 2 if residual else 1)   # (with a residual operand two roundings follow one another)
     assert c.rtoss_device_status() == 0
     packed.close()
