@@ -50,7 +50,8 @@ struct TcPlan {
     int TH, TW, Wq, N_px, NA, NB, G, n_sub, sub_rows, rows_staged, tiles_x, smem;
     int KS, cb_per;      // CTAs that share a tile's channel blocks (a cluster), blocks per share
     long tiles;          // tiles of the layer (not counting shares)
-    double us;           // what the model below expects of a launch of its own
+    int half;            // 3x3 stride 2: a channel block in two activation stages (TcArgs::half)
+    double us;           // what the model below expects of a launch of its own (half: of one with a channel block in one stage)
     double tile_us, epi_us;   // and of one tile: operands and instructions, epilogue
 };
 
@@ -63,7 +64,8 @@ struct PlanKey {
                      // do per cycle; 2: with nothing beside it
     int max_px;      // most positions per tile
     int force_G, n_tabs;
-    int half;        // 3x3 stride 2 in two activation stages a channel block (see single_plan_key)
+    int may_half;    // 3x3 stride 2: its channel blocks may come in two activation stages (see single_plan_key)
+    int half;        // and do (a search's, see plan_tc)
     int three;       // fp32: the cost of three tf32 products, whatever the layer's kernel forms (see plan_tc)
     int most_cb;     // most channel blocks one CTA adds up (0: any number)
 };
@@ -268,6 +270,7 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
                         out->smem = rings + fixed;
                         out->KS = ks;
                         out->cb_per = cb_per;
+                        out->half = k.half;
                         out->tiles = tiles;
                         out->us = c.us;
                         out->tile_us = c.tile_us;
@@ -284,7 +287,7 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
 // The plan of a call.  The split is decided as if the call had a residual operand, whether it has one or not: a call with
 // a residual then adds up its products in the order of the same call without one (same bits).
 // Searching takes tens of microseconds of host time, more than a launch: every thread remembers the plans of its last
-// few hundred kinds of call.  A plan is a function of its key and of the device's cluster limits, which whoever plans for a
+// few hundred kinds of call.  A call looks up one key, so that it never drives itself out of the memory.  A plan is a function of its key and of the device's cluster limits, which whoever plans for a
 // device has had asked first (ensure_device): it does not matter which thread or context asks.
 bool plan_tc(const PlanKey& k, TcPlan* out) {
     struct Memo {
@@ -314,9 +317,22 @@ bool plan_tc(const PlanKey& k, TcPlan* out) {
                 if (plan_search(q, true, 0, &m.plan) && m.plan.KS > 1) q.most_cb = m.plan.cb_per * 3 / 2;
                 q.three = 0;
             }
-            q.half = 0;   // (in two stages a layer is cut along K as in one: the same sums)
             if (plan_search(q, true, 0, &m.plan)) ks = m.plan.KS;
             m.ok = plan_search(k, k.resid != 0, ks, &m.plan);
+            if (m.ok && k.may_half) {
+                // In two activation stages, cut along K as in one (the same sums): a second barrier round trip a block, which
+                // launches of a few microseconds feel (2 to 6 % where every layer took it), against fetching under the
+                // instructions.  The model has to expect 7 % and half a microsecond of it, which is about its own error; the
+                // layers that gain are then those of several tiles a CTA (20 % and more; 60 layers of 16 to 512 channels, batch
+                // 1 to 32, take 0.935 of the time in one stage in the geometric mean, the slowest 1.016).
+                TcPlan two;
+                q = k;
+                q.half = 1;
+                if (plan_search(q, k.resid != 0, ks, &two) && two.us < 0.93 * m.plan.us && two.us < m.plan.us - 0.5) {
+                    two.us = m.plan.us;   // (by which calls are grouped, and that decides where sums are cut)
+                    m.plan = two;
+                }
+            }
         }
         m.key = k;
         m.set = true;
@@ -417,7 +433,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     a.cb_ch = row_bytes / esize;
     a.tiles_x = plan.tiles_x;
     a.n_sub = plan.n_sub;
-    a.half = plan_k.half ? 1 : 0;   // (the launch writes the order here)
+    a.half = plan.half ? 1 : 0;   // (the launch writes the order here)
     a.sub_bytes = plan.sub_rows * row_bytes;
     if (p->ksize == 3 && S == 1) {
         a.x_add[0] = a.y_add[0] = -1;
@@ -666,20 +682,14 @@ double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* con
     return shared_cost(ctx, n, ps, ds, nullptr);
 }
 
-// The plan key of a launch of one convolution.  16-bit 3x3 layers of stride 2 may have their channel blocks in two activation stages
-// (TcArgs::half): a second barrier round trip a block, which launches of a few microseconds feel (2 to 6 % where every layer took
-// it), against fetching under the instructions.  The model has to expect 7 % and half a microsecond of it, which is about its own
-// error; the layers that gain are then those of several tiles a CTA (20 % and more; 60 layers of 16 to 512 channels, batch 1 to
-// 32, take 0.935 of the time in one stage in the geometric mean, the slowest 1.016).
+// The plan key of a launch of one convolution: 16-bit 3x3 layers of stride 2 may have their channel blocks in two activation
+// stages.  (No form of that kernel stores elements.)
 static PlanKey single_plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, int sms, int dev) {
     PlanKey k = plan_key(p, d, sms, dev);
-    if (p->ksize != 3 || d->stride != 2 || p->dtype == RTOSS_F32) return k;
-    const int cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;   // (no form of it stores elements)
-    if (d->layout == RTOSS_NHWC && (p->Cout % 8 != 0 || cs % 8 != 0 || d->y_channel_offset % 8 != 0)) return k;
-    PlanKey two = k;
-    two.half = 1;
-    TcPlan a, b;
-    return plan_tc(k, &a) && plan_tc(two, &b) && b.us < 0.93 * a.us && b.us < a.us - 0.5 ? two : k;
+    const int cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;
+    const bool pieces = d->layout == RTOSS_NCHW || (p->Cout % 8 == 0 && cs % 8 == 0 && d->y_channel_offset % 8 == 0);
+    k.may_half = p->ksize == 3 && d->stride == 2 && p->dtype != RTOSS_F32 && pieces ? 1 : 0;
+    return k;
 }
 // TcArgs::half for NA stages: a block's odd rows are read until its end, its even rows for two thirds of it, and a stage is
 // filled again by whatever comes next once it is free.  With two stages the odd and the even rows change places from block
@@ -687,12 +697,11 @@ static PlanKey single_plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, 
 static unsigned half_order(int NA) { return NA == 2 ? 0u | 1u << 2 | 1u << 4 | 0u << 6 : NA == 3 ? 0u | 1u << 2 | 2u << 4 | 1u << 6 : 0u | 1u << 2 | 2u << 4 | 3u << 6; }
 
 // What a launch of its own is expected to take for this call (the planner's model), over how many CTAs it spreads a tile's
-// channel blocks, and how many tiles it has.  (Shared launches never split.)  3x3 of stride 2 counts as in one activation stage: what
-// hangs on this is how calls are grouped, and with it where sums are cut.
+// channel blocks, and how many tiles it has.  (Shared launches never split.)
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
     const rtoss_conv_desc dd = row_form(p, d);
-    if (ensure_device(ctx) || !plan_tc(plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    if (ensure_device(ctx) || !plan_tc(single_plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
     *us = plan.us;
     *ks = plan.KS;
     *tiles = plan.tiles;

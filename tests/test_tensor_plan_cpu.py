@@ -1,7 +1,10 @@
 """Host logic of the tensor path's tile planner (rtoss_tensor_plan_of: plain arithmetic through the C ABI, no GPU):
 the invariants the kernel and the TMA descriptors rely on, over the layer shapes of both model families and a sweep of
 odd ones."""
+import ctypes
 import itertools
+import random
+import time
 
 import pytest
 
@@ -100,3 +103,20 @@ def test_narrow_layers_stage_half_rows_and_keep_a_deeper_ring():
     assert p.row_bytes == 64 and p.act_stages > 2        # one channel block per tile: the next tile's block is the next stage
     q = check(16, 160, 160, 1, 3, 128, 128, BF16)
     assert q.row_bytes == 128 and q.act_stages == 2
+
+
+def test_a_repeated_call_is_not_planned_again():
+    """Planning searches for tens of microseconds; a thread remembers its plans, and a call looks up one key, so asking twice in a
+    row never searches twice.  The fastest of forty repeats of a thousand random layers of stride 2 against their median."""
+    rng = random.Random(6)
+    took = []
+    for _ in range(1000):
+        d = rt.ConvDesc(rng.randint(1, 32), rng.randint(7, 160), rng.randint(7, 160), 2, rt.NHWC, BF16, 0, None, 0, 0, 0, None, 0)
+        args = (ctypes.byref(d), 3, 8 * rng.randint(2, 64), 8 * rng.randint(2, 64), BF16, 0, ctypes.byref(rt.TensorPlan()))
+        best = 1 << 60
+        for _ in range(40):
+            t = time.perf_counter_ns()
+            rt.lib.rtoss_tensor_plan_of(*args)
+            best = min(best, time.perf_counter_ns() - t)
+        took.append(best)
+    assert max(took) <= 3 * sorted(took)[500]
