@@ -37,6 +37,9 @@ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 // price is one instruction per 128 positions instead of per 256: taken where few instructions are needed anyway.
 bool use_pxm(const rtoss_packed* p) { return p->Cout <= kPxmMaxCout && p->ksize == 1 && p->dtype != RTOSS_F32; }
 
+// fp32 layers whose small products are bf16 ones
+bool has_corr16(const rtoss_packed* p) { return p->dtype == RTOSS_F32 && rtoss_f32_corr16(p->Cin, p->ksize); }
+
 // Bytes of a staged row: 16-bit layers of at most 32 input channels stage 64-byte rows (64-byte swizzle) instead of
 // 128-byte rows half of which would be zero fill.
 int row_bytes_of(const rtoss_packed* p) { return (p->dtype != RTOSS_F32 && p->Cin <= 32) ? 64 : kRowBytes; }
@@ -66,8 +69,7 @@ struct PlanKey {
     int force_G, n_tabs;
     int may_half;    // 3x3 stride 2: its channel blocks may come in two activation stages (see single_plan_key)
     int half;        // and do (a search's, see plan_tc)
-    int three;       // fp32: the cost of three tf32 products, whatever the layer's kernel forms (see plan_tc)
-    int most_cb;     // most channel blocks one CTA adds up (0: any number)
+    int three;       // fp32: the cost of three tf32 products a tap, whatever the layer's kernel forms (see plan_tc)
 };
 
 // Most thread-block clusters of `ks` CTAs (one CTA per SM) a device holds at once.  Clusters live inside a GPC and the
@@ -227,13 +229,11 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
                 for (int ks = 1; ks <= 8; ++ks) {
                     if (only_ks && ks != only_ks) continue;
                     int cb_per = ncb;
-                    if (ks == 1 && !only_ks && k.most_cb && ncb > k.most_cb) continue;
                     if (ks > 1) {
                         if (k.shared || pxm || R != 1 || tiles * ks > k.sms || ks > ncb) break;
                         if (tiles > max_clusters(k.dev, ks, k.sms)) continue;
                         cb_per = (ncb + ks - 1) / ks;
                         if ((ncb + cb_per - 1) / cb_per != ks) continue;   // (a share would be empty)
-                        if (k.most_cb && cb_per > k.most_cb) continue;
                         // the owners' buffers for the partial sums lie in the rings
                         const int n_lc = ((n_px + 31) / 32 + ks - 1) / ks;
                         if (ks * n_lc > 16 || ks * n_lc * 16384 > rings) continue;
@@ -309,14 +309,12 @@ bool plan_tc(const PlanKey& k, TcPlan* out) {
         } else {
             int ks = 1;
             PlanKey q = k;
-            if (k.dtype == RTOSS_F32 && rtoss_f32_corr16(k.Cin, k.ksize)) {
-                // The tensor core cuts off at every accumulation: a sum may have no more of them than it had when a tap was twelve
-                // instructions instead of eight, so a layer that was cut along K then is not left in longer pieces now that
-                // its instructions are cheaper (128->128 @60x60 s2 x2 in two shares instead of four: 3.0e-6 instead of 2.7e-6).
-                q.three = 1;
-                if (plan_search(q, true, 0, &m.plan) && m.plan.KS > 1) q.most_cb = m.plan.cb_per * 3 / 2;
-                q.three = 0;
-            }
+            // The tensor core cuts off at every accumulation, so the longer a sum, the larger its error.  fp32 layers whose small
+            // products are bf16 ones are cut along K where three tf32 products would be: every sum then has two thirds of the
+            // accumulations that those take, which is what makes up for the rounded factors.  Cut by the cost of the cheaper
+            // instructions a layer is left in longer pieces: 96->360 @42x33 x3 in two shares instead of three errs by 3.6e-6
+            // instead of the 3.3e-6 of three products, 128->128 @60x60 s2 x2 in two instead of four by 3.0e-6 instead of 2.7e-6.
+            if (k.dtype == RTOSS_F32 && rtoss_f32_corr16(k.Cin, k.ksize)) q.three = 1;
             if (plan_search(q, true, 0, &m.plan)) ks = m.plan.KS;
             m.ok = plan_search(k, k.resid != 0, ks, &m.plan);
             if (m.ok && k.may_half) {
@@ -479,7 +477,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     // N/8 and M/16
     const unsigned fmt = f32 ? 2u : a.is_bf16 ? 1u : 0u;
     a.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((unsigned)(plan.N_px >> 3) << 17) | ((unsigned)(kMTile >> 4) << 24);
-    a.corr16 = f32 && rtoss_f32_corr16(p->Cin, p->ksize) ? 1 : 0;
+    a.corr16 = has_corr16(p) ? 1 : 0;
     a.idesc16 = (a.idesc & ~((7u << 7) | (7u << 10))) | (1u << 7) | (1u << 10);   // (bf16)
     a.pxm = pxm ? 1 : 0;
     a.MH = plan.N_px > 128 ? 2 : 1;
@@ -645,7 +643,7 @@ bool rtoss_tc_groupable(const rtoss_packed* p, const rtoss_conv_desc* d, const v
 
 // What one shared launch is expected to take for these independent calls, and the most positions a tile should have: many
 // small tiles where the set would leave SMs idle, 256 positions where it fills them for several rounds.
-static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds, int* px_out) {
+static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds, bool three, int* px_out) {
     static const int kPx[] = {256, 192, 128, 96, 64, 48, 32};
     const int sms = ctx_sms(ctx);
     double best = 1e30;
@@ -658,6 +656,7 @@ static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const
             PlanKey key = plan_key(ps[i], &dd, sms, ctx_dev(ctx));
             key.shared = n > 1 ? 1 : 2;
             key.max_px = px;
+            key.three = three && has_corr16(ps[i]) ? 1 : 0;
             TcPlan plan;
             ok = plan_tc(key, &plan);
             if (!ok) break;
@@ -677,9 +676,10 @@ static double shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const
     }
     return best;
 }
+// (Whether calls share a launch decides where sums are cut: fp32 by the cost of three tf32 products, see plan_tc.)
 double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* const* ps, const rtoss_conv_desc* const* ds) {
     if (ensure_device(ctx)) return 1e30;   // (the launch that follows reports the error)
-    return shared_cost(ctx, n, ps, ds, nullptr);
+    return shared_cost(ctx, n, ps, ds, true, nullptr);
 }
 
 // The plan key of a launch of one convolution: 16-bit 3x3 layers of stride 2 may have their channel blocks in two activation
@@ -701,7 +701,10 @@ static unsigned half_order(int NA) { return NA == 2 ? 0u | 1u << 2 | 1u << 4 | 0
 bool rtoss_tc_single_cost(const rtoss_ctx* ctx, const rtoss_packed* p, const rtoss_conv_desc* d, double* us, int* ks, long* tiles) {
     TcPlan plan;
     const rtoss_conv_desc dd = row_form(p, d);
-    if (ensure_device(ctx) || !plan_tc(single_plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx)), &plan)) return false;
+    if (ensure_device(ctx)) return false;
+    PlanKey k = single_plan_key(p, &dd, ctx_sms(ctx), ctx_dev(ctx));
+    k.three = has_corr16(p) ? 1 : 0;
+    if (!plan_tc(k, &plan)) return false;
     *us = plan.us;
     *ks = plan.KS;
     *tiles = plan.tiles;
@@ -1012,7 +1015,7 @@ int rtoss_launch_conv_tc_chain(const rtoss_ctx* ctx, int n, const rtoss_packed* 
                 const rtoss_packed* sp[kMaxProb];
                 const rtoss_conv_desc* sd[kMaxProb];
                 for (int q = 0; q < m; ++q) sp[q] = ps[set[q]], sd[q] = ds[set[q]];
-                shared_cost(ctx, m, sp, sd, &set_px);
+                shared_cost(ctx, m, sp, sd, false, &set_px);
             }
             for (int pass = 0; pass < 2; ++pass) {
                 bool agree = true;

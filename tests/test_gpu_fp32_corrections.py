@@ -68,3 +68,43 @@ def test_both_ways_of_packing(cin, cout):
     assert torch.equal(y0, _conv(c, packed, x, cout, 1))
     batch.close()
     packed.close()
+
+
+def _error(N, cin, cout, H, W, stride, k, patterns, relu):
+    c = gu.ctx()
+    masks = rt.rtoss_pattern_preset(k, rt.PRESET_CENTRE8 if k == 4 else rt.PRESET_CONN4)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(cin + cout + H + W)
+    w = torch.randn(cout, cin, 3, 3, device="cuda", generator=g) * math.sqrt(2.0 / (9 * cin))
+    pid = c.rtoss_select_patterns_shared(w, masks, k, 128, 16) if patterns == "block" else c.rtoss_select_patterns(w, 3, masks, k)
+    packed = c.rtoss_pack(w, 3, masks, k, pid, rt.F32)
+    x = torch.randn(N, H, W, cin, device="cuda", generator=g)
+    if relu:
+        x = torch.relu(x)
+    y = _conv(c, packed, x, cout, stride)
+    ref = torch.nn.functional.conv2d(x.double().permute(0, 3, 1, 2), packed.to_dense().double().reshape(w.shape), stride=stride, padding=1)
+    packed.close()
+    return ((y.double().permute(0, 3, 1, 2) - ref).norm() / ref.norm()).item()
+
+
+ERRORS = [   # N, channels, filters, H, W, stride, k, patterns, input after a ReLU, the error of three tf32 products
+    (3, 96, 360, 42, 33, 1, 4, "kernel", True, 3.31e-6),
+    (27, 96, 73, 11, 24, 1, 4, "kernel", False, 3.89e-6),
+    (2, 416, 78, 19, 37, 1, 3, "kernel", True, 3.42e-6),
+    (2, 480, 328, 12, 13, 2, 2, "kernel", False, 3.72e-6),
+    (1, 32, 16, 9, 11, 1, 2, "block", False, 1.02e-6),
+    (4, 32, 28, 76, 20, 2, 2, "block", True, 1.00e-6),
+    (2, 32, 70, 57, 10, 1, 2, "block", True, 0.95e-6),
+    (1, 96, 162, 16, 30, 1, 2, "block", True, 1.00e-6),
+    (2, 256, 64, 40, 40, 1, 2, "block", False, 4.30e-6),
+    (2, 256, 64, 40, 40, 1, 3, "block", True, 6.06e-6),
+    (1, 256, 256, 20, 20, 1, 3, "block", False, 1.35e-6),
+    (5, 96, 160, 20, 86, 2, 4, "block", True, 2.19e-6),
+]
+
+
+@pytest.mark.parametrize("N,cin,cout,H,W,stride,k,patterns,relu,bound", ERRORS)
+def test_error_no_larger_than_of_three_products(N, cin, cout, H, W, stride, k, patterns, relu, bound):
+    """Layers cut along K in several ways (the longer a share, the larger the error), and block patterns of few kept taps and channels,
+    where the fewest accumulations stand against the rounded factors."""
+    assert _error(N, cin, cout, H, W, stride, k, patterns, relu) <= bound
