@@ -1448,6 +1448,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 if (lane == 0) ok = mbar_wait(bar_fullA + 8 * ra.s, ra.parity(), g.wait_cycles);
                 ok = __shfl_sync(0xFFFFFFFFu, (int)ok, 0) != 0;
                 if (!ok) break;
+                __syncwarp();   // (lane 0 has seen the copy; a shuffle orders no memory, and all lanes read the block)
                 const unsigned src = sA + ra.s * a.a_stage, dst = src + (unsigned)a.lo_off;
                 const int n16 = (a.n_sub * a.sub_bytes) >> 4, first = (warp - kWeightWarp - 1) * 32 + lane;
                 if (kMulti ? a.corr16 != 0 : kCorr1) split_block16(src, dst, n16, first);
