@@ -376,12 +376,14 @@ static int launch_to_dense_t(const rtoss_packed* p, int64_t n_dense, int sms, vo
 int rtoss_launch_to_dense(const rtoss_packed* p, int sms, void* w_out, void* stream) {
     const int64_t n_dense = p->ksize == 3 ? p->n_kernels * 9 : (int64_t)p->Cout * p->Cin;
     if (n_dense <= 0) return 0;
+    int e = (int)cudaErrorInvalidValue;
     switch (p->dtype) {
-        case RTOSS_F32: return launch_to_dense_t<float>(p, n_dense, sms, w_out, (cudaStream_t)stream);
-        case RTOSS_BF16: return launch_to_dense_t<__nv_bfloat16>(p, n_dense, sms, w_out, (cudaStream_t)stream);
-        case RTOSS_F16: return launch_to_dense_t<__half>(p, n_dense, sms, w_out, (cudaStream_t)stream);
+        case RTOSS_F32: e = launch_to_dense_t<float>(p, n_dense, sms, w_out, (cudaStream_t)stream); break;
+        case RTOSS_BF16: e = launch_to_dense_t<__nv_bfloat16>(p, n_dense, sms, w_out, (cudaStream_t)stream); break;
+        case RTOSS_F16: e = launch_to_dense_t<__half>(p, n_dense, sms, w_out, (cudaStream_t)stream); break;
     }
-    return (int)cudaErrorInvalidValue;
+    if (e) cudaGetLastError();   // (reported here, and not by the next call as its own)
+    return e;
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -1,6 +1,8 @@
 """rtoss_packed_to_dense at the sizes where a block's share changes: fewer kernels than a block takes, one more, one block per SM
 with a ragged last share, shares that fill a block's registers or its shared memory, and layers of several steps.  Bit for
 bit the weights under their masks, rounded to the handle's type."""
+import ctypes
+
 import pytest
 import torch
 
@@ -37,4 +39,28 @@ def test_to_dense_is_the_masked_weights(cout, cin, ks, k, dt):
     want[:9 * n] = torch.where(keep.reshape(-1) != 0, w.reshape(-1)[:9 * n], torch.zeros((), device="cuda"))
     assert torch.equal(out[:w.numel()], want.to(TD[dt]))
     assert torch.all(out[w.numel():] == 7.0)
+    packed.close()
+
+
+def test_a_refused_launch_is_reported_once():
+    """The legacy stream takes no work while a stream that it waits for is captured: that call says so, and the next one, which is
+    in order, is not answered with its error."""
+    c = gu.ctx()
+    masks = rt.rtoss_pattern_preset(4, rt.PRESET_CENTRE8)
+    w = torch.randn(32, 16, 3, 3, device="cuda")
+    pid = c.rtoss_select_patterns(w, 3, masks, 4)
+    packed = c.rtoss_pack(w, 3, masks, 4, pid, rt.BF16)
+    out = packed.to_dense()   # (what a first call sets up is done)
+    torch.cuda.synchronize()
+    cudart = ctypes.CDLL("libcudart.so.12")
+    stream, graph = ctypes.c_void_p(), ctypes.c_void_p()
+    assert cudart.cudaStreamCreate(ctypes.byref(stream)) == 0
+    assert cudart.cudaStreamBeginCapture(stream, 0) == 0
+    refused = rt.lib.rtoss_packed_to_dense(c.h, packed.h, out.data_ptr(), None)
+    assert cudart.cudaStreamEndCapture(stream, ctypes.byref(graph)) != 0   # (the capture did not survive it)
+    cudart.cudaGetLastError()
+    cudart.cudaStreamDestroy(stream)
+    assert refused != rt.OK
+    assert torch.equal(pid, c.rtoss_select_patterns(w, 3, masks, 4))
+    torch.cuda.synchronize()
     packed.close()
