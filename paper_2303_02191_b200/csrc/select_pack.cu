@@ -195,11 +195,12 @@ __global__ void __launch_bounds__(kSharedMaxFB) select_shared_kernel(const T* __
 // before this one: a model's layers are expanded one call after the other, and all but the stores of a call then overlaps
 // the calls before it.
 // What bounds a row of such calls is the hop from the end of one kernel to the end of the next: 0.7 us with nothing but a few
-// stores in it, more with more blocks (empty kernels: 0.55 us up to 148 blocks, 0.9 with 592, 1.57 with 1184).  Hence at most one
-// block an SM, with its whole share of the layer in shared memory and the words a thread stores in registers when the wait
-// ends, and blocks small enough (256 threads, at most 73 KB) for calls that wait to be on an SM together: fetching takes longer
-// than a hop.  57 layers of 7 M weights in a row 50.3 -> 46.3 us, 68 layers of 32 M 86 -> 77 (against a block per 256 kernels that
-// stored from shared memory; stored that way, one block an SM took 52 and 82).
+// stores in it, more with more blocks (empty kernels: 0.55 us up to 148 blocks, 0.9 with 592, 1.57 with 1184).  Hence one block an SM
+// while its share of the layer fits into shared memory, with the words a thread stores in registers when the wait ends, and
+// blocks small enough (256 threads, at most 73 KB) for calls that wait to be on an SM together: fetching takes longer than a
+// hop.  Layers beyond that (148 x 1 000 to 3 200 kernels) take more blocks, up to eight an SM, and steps beyond those.  57 layers of 7 M weights in a row 50.3 -> 46.3 us, 68 layers of 32 M 86 -> 77 (against a block per 256 kernels that
+// stored from shared memory; stored that way, one block an SM took 52 and 82).  A layer by itself, cold: 2048x2048 fp32 73 -> 50 us
+// (4.5 TB/s), 1024x1024 bf16 23.6 -> 19.4, small ones as before.
 // All of these loads go to L2 (see conv_common.cuh).
 constexpr int kDenseThreads = 256;
 constexpr int kDenseHold = 5;        // 16-byte words of its output a thread holds in registers (a step of up to 1136 kernels in 16 bits)
@@ -222,7 +223,7 @@ __global__ void __launch_bounds__(kDenseThreads, 4) to_dense_kernel(const V* __r
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(to) + (unsigned)i), "l"(static_cast<const char*>(src) + i) : "memory");
         if (tid < n - whole) static_cast<uint8_t*>(to)[whole + tid] = __ldcg(static_cast<const uint8_t*>(src) + whole + tid);
     };
-    fetch(sm, masks, 512);
+    if (n_kernels > 0) fetch(sm, masks, 512);   // (the first step waits for it; a block without one ends with nothing under way)
     bool waited = false;
     const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
     for (int64_t first = (int64_t)blockIdx.x * step; first < n_kernels; first += (int64_t)gridDim.x * step) {

@@ -1,5 +1,6 @@
 """rtoss_packed_to_dense at the sizes where a block's share changes: fewer kernels than a block takes, one more, one block per SM
-with a ragged last share, shares that fill a block's registers or its shared memory, and layers of several steps.  Bit for
+with a ragged last share, shares that fill a block's registers or its shared memory, several blocks an SM, and blocks that take
+a second step.  Bit for
 bit the weights under their masks, rounded to the handle's type."""
 import ctypes
 
@@ -19,7 +20,10 @@ TD = {"f32": torch.float32, "bf16": torch.bfloat16, "f16": torch.float16}
     (1, 1, 3, 4, "bf16"), (16, 16, 3, 4, "bf16"), (257, 1, 3, 4, "f16"), (5, 13, 1, 3, "bf16"),
     (148, 256, 3, 4, "bf16"), (149, 257, 3, 2, "f16"),          # one block an SM, with and without a remainder
     (512, 331, 3, 4, "bf16"),                                    # more words a thread than it holds in registers
-    (331, 331, 3, 9, "f32"), (700, 600, 3, 5, "f32"),            # as many kernels as fit, and several steps
+    (331, 331, 3, 9, "f32"),                                     # the same in fp32
+    (700, 600, 3, 5, "f32"),                                     # as many kernels as fit, and more than one block an SM
+    (1100, 1101, 3, 9, "f32"),                                   # 1008 kernels a step: 18 of eight blocks an SM take a second one
+    (2, 3, 1, 4, "bf16"),                                        # nothing but trailing weights
     (2048, 1031, 1, 4, "bf16"),                                  # a 1x1 layer with trailing weights
 ])
 def test_to_dense_is_the_masked_weights(cout, cin, ks, k, dt):
