@@ -607,10 +607,8 @@ def roofline_of(res, hbm_peak, tc_peak, peak_kind):
     N, elem = res["N"], res["elem"]
     flops = np.array([synth.layer_nnz_flops(L, N, k) for L, k in zip(res["layers"], res["ks"])])
     bytes_ = np.array([synth.layer_bytes(L, N, k, elem) for L, k in zip(res["layers"], res["ks"])], dtype=np.float64)
-    # pipe peak per layer: the measured bf16 tensor peak; fp32 on the tensor path issues tf32 instructions (half the bf16
-    # rate) three times per product (head x head, head x remainder, remainder x head; in 3x3 layers of whole blocks of 32
-    # channels the last two are bf16 ones); else the nominal FMA peak
-    units_of = lambda L: 1 if res["dtype"] != "f32" else 4 if L["ksize"] == 3 and L["cin"] % 32 == 0 else 6
+    # pipe peak per layer: on the tensor path a share of the measured bf16 tensor peak, else the nominal FMA peak
+    units_of = lambda L: synth.tensor_units(L, res["dtype"])
     pipe = np.array([tc_peak / units_of(L) if tc else ALU_PEAK_TFLOPS for L, tc in zip(res["layers"], res["on_tc"])]) * 1e12
     t_pipe, t_hbm = flops / pipe, bytes_ / (hbm_peak * 1e9)
     t_roof = np.maximum(t_pipe, t_hbm)
@@ -634,7 +632,7 @@ def roofline_of(res, hbm_peak, tc_peak, peak_kind):
     t_top = float(np.mean(t_meas[idx]))
     if t_pipe[members].sum() >= t_hbm[members].sum():
         per_tap = units_of(res["layers"][members[0]])
-        dom = {"bound": {1: "tensor", 4: "tensor (tf32 + 2 bf16)", 6: "tensor (tf32 x3)"}[per_tap] if on_tc else "alu",
+        dom = {"bound": synth.TENSOR_BOUND[per_tap] if on_tc else "alu",
                "achieved": u_flops[top] / t_top / 1e12, "peak": pipe[members[0]] / 1e12, "unit": "TFLOP/s",
                "peak_kind": ("of %s (bf16 cuBLAS, sustained)%s" % (peak_kind, {1: "", 4: " / 4 (a tf32 product and two bf16 ones per tap)", 6: " / 2 (tf32) / 3 (products per tap)"}[per_tap])) if on_tc
                else "nominal, not measured: 148 SM x 128 FMA lanes x 2 x 1.965 GHz"}

@@ -96,14 +96,14 @@ def main():
         L = dict(ksize=3, stride=1, cin=C, cout=C, H=H, W=H)
         flops = synth.layer_nnz_flops(L, N, k)
         nbytes = synth.layer_bytes(L, N, k, 2 if dt == "bf16" else 4)
-        # tensor pipe: measured bf16 peak; fp32 runs tf32 instructions (half the rate) three times per product
-        pipe = (tc_peak if dt == "bf16" else tc_peak / 6) if path == rt.PATH_TENSOR else ALU_PEAK_TFLOPS
+        units = synth.tensor_units(L, dt)   # tensor pipe: a share of the measured bf16 peak
+        pipe = tc_peak / units if path == rt.PATH_TENSOR else ALU_PEAK_TFLOPS
         t_roof = max(nbytes / (hbm * 1e9), flops / (pipe * 1e12))
         rows.append(dict(dtype=dt, C=C, HW=H, N=N, k=k, path="tensor" if path == rt.PATH_TENSOR else "fma",
                          cold_ms=round(cold, 5), warm_ms=round(warm, 5), gbs=round(nbytes / cold / 1e6, 1),
                          nnz_gflops=round(flops / cold / 1e6, 1), roofline_us=round(t_roof * 1e6, 2),
                          bound="hbm" if nbytes / (hbm * 1e9) >= flops / (pipe * 1e12) else
-                         (("tensor" if dt == "bf16" else "tensor (tf32 x3)") if path == rt.PATH_TENSOR else "alu"),
+                         (synth.TENSOR_BOUND[units] if path == rt.PATH_TENSOR else "alu"),
                          frac=round(t_roof / (cold * 1e-3), 4)))
         packed.close()
         del x, y

@@ -250,6 +250,15 @@ def layer_nnz_flops(layer, N, k):
     return 2.0 * kept * N * Ho * Wo
 
 
+def tensor_units(L, dtype):
+    """Tensor time of a product on the tensor path, in bf16 products: 16-bit data 1; fp32 a tf32 product (half the rate) and two
+    small ones, tf32 too, or bf16 in 3x3 layers of whole blocks of 32 channels."""
+    return 1 if dtype != "f32" else 4 if L["ksize"] == 3 and L["cin"] % 32 == 0 else 6
+
+
+TENSOR_BOUND = {1: "tensor", 4: "tensor (tf32 + 2 bf16)", 6: "tensor (tf32 x3)"}
+
+
 def layer_bytes(layer, N, k, elem):
     """Algorithmic bytes of one call: x once, y once, packed values + pattern
     ids, bias."""

@@ -120,3 +120,9 @@ def test_a_repeated_call_is_not_planned_again():
             best = min(best, time.perf_counter_ns() - t)
         took.append(best)
     assert max(took) <= 3 * sorted(took)[500]
+
+
+@pytest.mark.parametrize("dtype,ksize,cin,units", [("bf16", 3, 64, 1), ("f16", 1, 36, 1), ("f32", 3, 64, 4), ("f32", 3, 36, 6), ("f32", 1, 64, 6)])
+def test_tensor_time_of_a_product(dtype, ksize, cin, units):
+    """What the rooflines of bench.py and the sweep divide the tensor peak by, and that both have a name for it."""
+    assert synth.tensor_units(dict(ksize=ksize, cin=cin), dtype) == units and units in synth.TENSOR_BOUND
