@@ -683,12 +683,12 @@ double rtoss_tc_shared_cost(const rtoss_ctx* ctx, int n, const rtoss_packed* con
 }
 
 // The plan key of a launch of one convolution: 16-bit 3x3 layers of stride 2 may have their channel blocks in two activation
-// stages.  (No form of that kernel stores elements.)
+// stages.  Only where there is a form for it: whole 16-byte pieces out, no residual operand.
 static PlanKey single_plan_key(const rtoss_packed* p, const rtoss_conv_desc* d, int sms, int dev) {
     PlanKey k = plan_key(p, d, sms, dev);
     const int cs = d->y_channel_stride ? d->y_channel_stride : p->Cout;
     const bool pieces = d->layout == RTOSS_NCHW || (p->Cout % 8 == 0 && cs % 8 == 0 && d->y_channel_offset % 8 == 0);
-    k.may_half = p->ksize == 3 && d->stride == 2 && p->dtype != RTOSS_F32 && pieces ? 1 : 0;
+    k.may_half = p->ksize == 3 && d->stride == 2 && p->dtype != RTOSS_F32 && pieces && !d->residual_dev ? 1 : 0;
     return k;
 }
 // TcArgs::half for NA stages: a block's odd rows are read until its end, its even rows for two thirds of it, and a stage is
@@ -774,6 +774,7 @@ static SingleKernel single_kernel(const rtoss_ctx* ctx, bool f32, bool repacked,
         const int form = (pieces ? 0 : kFormElem) | (a.half ? kFormHalf : 0) | form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
         if (void* k = form_kernel(ctx, a.is_bf16, false, form)) return reinterpret_cast<SingleKernel>(k);
     }
+    if (a.half) return nullptr;   // (forms only; single_plan_key asks for what they cover)
     if (f32) return a.corr16 ? conv_tc_kernel<float, TcLaunch1, false, kFormCorr> : conv_tc_kernel<float, TcLaunch1>;
     if (repacked) return a.is_bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1, true> : conv_tc_kernel<__half, TcLaunch1, true>;
     return a.is_bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1> : conv_tc_kernel<__half, TcLaunch1>;
@@ -871,12 +872,14 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
         }
     }
     if (a.half) a.half = half_order(a.NA);
+    SingleKernel kernel = single_kernel(ctx, f32, repacked, a);
+    if (!kernel) return (int)cudaErrorInvalidDeviceFunction;
     // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM
     const size_t smem = (size_t)(smem_need > 116 * 1024 ? smem_need : 116 * 1024);
     cudaError_t le;
     if (a.KS > 1) {
         // one cluster per tile; if the device cannot place the clusters the layer runs uncut
-        le = rtoss_dev::launch_pdl(single_kernel(ctx, f32, repacked, a), grid, threads_of(f32), smem, (cudaStream_t)stream, a.KS, g);
+        le = rtoss_dev::launch_pdl(kernel, grid, threads_of(f32), smem, (cudaStream_t)stream, a.KS, g);
         if (le == cudaSuccess) return 0;
         cudaGetLastError();
         a.KS = 1;
@@ -885,8 +888,10 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
         n_units = (size_t)d->N * a.tiles_y * a.tiles_x * a.co_tiles;
         g.unit_end[0] = (int)n_units;
         grid = dim3((unsigned)(n_units < (size_t)sms ? n_units : (size_t)sms));
+        kernel = single_kernel(ctx, f32, repacked, a);   // (uncut: another form)
+        if (!kernel) return (int)cudaErrorInvalidDeviceFunction;
     }
-    le = rtoss_dev::launch_pdl(single_kernel(ctx, f32, repacked, a), grid, threads_of(f32), smem, (cudaStream_t)stream, 1, g);
+    le = rtoss_dev::launch_pdl(kernel, grid, threads_of(f32), smem, (cudaStream_t)stream, 1, g);
     return (int)le;
 }
 

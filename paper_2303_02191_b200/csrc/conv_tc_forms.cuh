@@ -68,7 +68,6 @@ FormTable make_forms() {
     add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kRelu, false>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kSilu, false>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kSiluX, false>());
-    add_forms<T, TcLaunch1>(t.one, t.n_one, std::integer_sequence<int, form_of(kKind3, kSilu, false, 2, false) | kFormHalf, form_of(kKind3, kSilu, true, 2, false) | kFormHalf>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kNone, true>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kRelu, true>());
     add_forms<T, TcLaunch1>(t.one, t.n_one, Half<kSiluX, true>());

@@ -119,7 +119,7 @@ struct TcArgs {
     // every role for every tile: the four divisors as multiply-and-shift pairs (see tile_of), set by the host.
     unsigned div_ks[2], div_co[2], div_tx[2], div_ty[2];
     int n_sub, sub_bytes;        // sub-tiles of an activation stage (3x3 stride 2: the 4 input phases, or 2 of them) and their size
-    // 16-bit 3x3 of stride 2, where the planner says so (0: not): a channel block comes as two activation stages, the odd input
+    // 16-bit 3x3 of stride 2, where the planner says so and there is a form for it (0: not): a channel block comes as two activation stages, the odd input
     // rows (two column phases, read by the first and the last row of taps) and the even ones (read by the middle row).  The even
     // rows are done with first, so the stages are taken in the order in which they come free, which this word lists: the
     // stage of the odd and the even rows of a block, then of the next, two bits each (half_order).  The taps go out in their
@@ -990,7 +990,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
     constexpr int kKind = kForm & 3, kAct = ((kForm >> 2) & 7) - 1;   // (kAny: both from the arguments)
     constexpr bool kSplitF = (kForm & 32) != 0, kNchw = (kForm & 256) != 0;
     constexpr int kRes = (kForm >> 6) & 3;
-    constexpr bool kHalf = (kForm & kFormHalf) != 0;   // (kAny, 16-bit data: from the arguments)
+    constexpr bool kHalf = (kForm & kFormHalf) != 0;   // (forms only: as a run-time branch it costs the launches without it)
     constexpr bool kElem = (kForm & kFormElem) != 0;
     constexpr bool kActKnown = kAct >= 0;
     constexpr int kActC = kActKnown ? kAct : 0;
@@ -1102,15 +1102,14 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     cur_pi = pi;
                 }
                 const TileIdx ti = tile_of(a, local);
-                const bool half = (kAny && !kF32) ? a.half != 0 : kHalf;
                 const int ks = ti.ks, n = ti.n;
                 const int y0 = ti.ty * a.TH, x0 = ti.tx * a.TW;
                 const int cb_end = min(a.ncb, (ks + 1) * a.cb_per);
                 for (int cb = ks * a.cb_per; cb < cb_end; ++cb) {
-                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : kHalf ? 2 : a.n_sub, n_stages = half ? 2 : 1;
+                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : kHalf ? 2 : a.n_sub, n_stages = kHalf ? 2 : 1;
                     for (int part = 0; part < n_stages; ++part) {   // (half: the odd rows, sub-tiles 2 and 3, then the even ones)
-                        if (half) ra.s = (int)(a.half >> (2 * (hq + part))) & 3;
-                        const int sa = ra.s, sub0 = half ? 2 - 2 * part : 0;
+                        if (kHalf) ra.s = (int)(a.half >> (2 * (hq + part))) & 3;
+                        const int sa = ra.s, sub0 = kHalf ? 2 - 2 * part : 0;
                         ok = ok && mbar_wait(bar_emptyA + 8 * sa, ra.parity() ^ 1, g.wait_cycles);
                         if (!ok) break;
                         mbar_expect_tx(bar_fullA + 8 * sa, a.a_tx_bytes * n_sub);
@@ -1278,8 +1277,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     constexpr int kSlab = kF32 ? 8 : 16;
                     const int nk4 = (min(left, a.cb_ch) + kSlab - 1) / kSlab;
                     const unsigned nkmask = (1u << nk4) - 1u;
-                    const bool half = (kAny && !kF32) ? a.half != 0 : kHalf;
-                    if (half) ra.s = (int)(a.half >> (2 * hq)) & 3;
+                    if (kHalf) ra.s = (int)(a.half >> (2 * hq)) & 3;
                     const int sa = ra.s;
                     if (kAny ? a.taps == 1 : kKind != 3) {
                         const int sb = rb.s;
@@ -1323,21 +1321,21 @@ conv_tc_kernel(const __grid_constant__ G g) {
                     const unsigned xl0 = desc_lo0 + (sA >> 4) + (unsigned)sa * astage16;
                     ra.advance(NA);   // (sa stays this block's stage; ra is at the next one, which the look ahead reads)
                     if (kAny ? unrolled9 : kKind == 3) {
-                        if (half) ra.s = (int)(a.half >> (2 * hq + 2)) & 3;
+                        if (kHalf) ra.s = (int)(a.half >> (2 * hq + 2)) & 3;
                         const int sa_e = ra.s;   // (half: the stage of the even rows)
                         int sa_n = ra.s;
                         unsigned pa_n = ra.parity();
 #pragma unroll
                         for (int s3 = 0; s3 < 3; ++s3) {
-                            if (s3 == 1 && half) {   // the even rows; the look ahead is for the next block from here on
+                            if (s3 == 1 && kHalf) {   // the even rows; the look ahead is for the next block from here on
                                 if (!(peek & 1u)) ok = ok && mbar_wait(bar_rdyA + 8 * sa_e, ra.parity(), g.wait_cycles);
                                 ra.advance(NA);
                                 hq ^= 2;
                                 ra.s = sa_n = (int)(a.half >> (2 * hq)) & 3;
                                 pa_n = ra.parity();
                             }
-                            if (s3 == 2 && half && ok) umma_commit(leader, bar_emptyA + 8 * sa_e);
-                            const unsigned xl = s3 == 1 && half ? desc_lo0 + (sA >> 4) + (unsigned)sa_e * astage16 : xl0;
+                            if (s3 == 2 && kHalf && ok) umma_commit(leader, bar_emptyA + 8 * sa_e);
+                            const unsigned xl = s3 == 1 && kHalf ? desc_lo0 + (sA >> 4) + (unsigned)sa_e * astage16 : xl0;
                             const int sb = rb.s;
                             if (!(peek & 2u)) ok = ok && mbar_wait(bar_fullB + 8 * sb, rb.parity(), g.wait_cycles);
                             if (ok) {
