@@ -88,7 +88,9 @@ int max_clusters(int dev, int ks, int sms) {
 // Expected time of a launch, in microseconds, for one way of cutting a layer.  16-bit data: the constants are a fit to 6 500
 // measured (layer, tile, split) combinations of the two detectors' layers at eleven sizes, batch 1 to 16, launches back to
 // back (programmatic dependent launch); typical error 7 %, and the plan it picks is on average 1.9 % from the best measured
-// one (4 % with the constants of the kernel before it was compiled in forms).  fp32 keeps the fit made then.  What it knows:
+// one (4 % with the constants of the kernel before it was compiled in forms).  fp32 keeps the fit made then, when one warp split
+// the activation blocks: layers of three tf32 products take 0.47 to 1.35 of what it expects of them, 0.78 in the geometric mean
+// of 54 random ones.  What it knows:
 //   - an instruction takes N / 2 cycles for N positions, but never less than 47; per weight stage 0.13 us of barrier
 //     round trip;
 //   - a CTA is fed at most 118 KB per us (tiles of stride 2, whose boxes overlap, count 0.56);
@@ -118,7 +120,9 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
     double mma = taps * slabs * instr + f.stage * wstages + f.block;
     if (corr16) {
         // fp32 3x3 layers whose small products are bf16 ones, 256->256 @80x80 x32 cut in eight ways, 96 to 240 positions a tile: a
-        // weight stage of one tap takes its four instructions + 0.1 us, at least 0.28; one of three taps its twelve + 0.27
+        // weight stage of one tap takes its four instructions + 0.1 us, at least 0.28; one of three taps its twelve + 0.27.  66
+        // other layers (32 to 512 channels, both strides, 16 to 256 positions, cut and uncut) take 0.67 to 1.15 of the model's
+        // time, 0.83 in the geometric mean: too dear throughout, by about the same, so that it still orders the ways to cut one
         const double s = G * 4 * (n_px / 2.0 > 47.0 ? n_px / 2.0 : 47.0) / 1900.0 + (G == 3 ? 0.27 : 0.10);
         mma = wstages * (s > 0.28 ? s : 0.28) + f.block;
     }
@@ -136,7 +140,8 @@ PlanCost plan_cost(const PlanKey& k, bool pxm, int w_rows, int row_bytes, int R,
         blk = late > blk ? late : blk;
         na = 2;
     }
-    // one activation stage: loads and instructions take turns (fp32: and one warp's split of the block between them)
+    // one activation stage: loads and instructions take turns (fp32: and the split of the block between them, as long as one warp
+    // took for it; four warps do it now, and layers planned with one stage take 0.52 to 0.83 of the model's time, seven of them)
     if (na == 1) blk = mma + (f32 ? 0.045 * kb_a : f.lone * kb_fed / 87.0);
     if (f32 && !corr16 && G == 3) blk += 2.0;   // (then only two weight stages fit: the ring's round trip shows)
     const int chunks = (n_px + 31) / 32;

@@ -35,7 +35,8 @@
 //     (tcgen05.ld, bias, activation, rounding, a transpose through shared memory,
 //     16-byte NHWC stores), warp 18 issues the TMA copies of the weights (a stage
 //     of three taps is one copy: issuing a copy occupies its thread for hundreds
-//     of cycles whatever the size).  Activation and weight stages form rings
+//     of cycles whatever the size); fp32 data has four more, which split the
+//     activation blocks (see below).  Activation and weight stages form rings
 //     that run on across tiles; two accumulator stages in TMEM let the epilogue
 //     of a tile run under the MMAs of the next.
 //   * Layers with few tiles and long channel loops are cut along the channel
@@ -59,12 +60,15 @@
 //     a row, 14 000 for 288 rows, and the copy of the next block waited for it.)
 //     3x3 layers of whole blocks of 32 channels form the two small products from bf16 numbers, at twice the tf32 rate and
 //     in two instructions of 16 channels instead of four of eight: bf16(w) * bf16(xl) + bf16(wl) * bf16(x), heads rounded to
-//     nearest.  Eight instructions a tap and block instead of twelve; bf16 has fp32's range.  Rounding the factors of a
-//     product that is 2^-12 of the sum costs 7e-7 of it, but what decides is the tensor core's own accumulation, which cuts
-//     off and loses in proportion to the instructions issued: relative error against 64-bit sums 2.7e-6 -> 1.8e-6 for 32 to
-//     256 channels, 4.5e-6 -> 3.0e-6 for 512.  (1x1 layers, with a ninth of the instructions, err by 7e-7 in all with three
-//     tf32 products, and keep them.)  256->256 @80x80 x32 962 -> 650 us; the four units of tensor time it takes instead of six
-//     are 585 us at the bf16 peak.
+//     nearest.  Eight instructions a tap and block instead of twelve; bf16 has fp32's range.  The rounded factors cost 6.5e-7 of
+//     the sum where three tf32 products cost 3.5e-7, but what decides is the tensor core's own accumulation, which cuts off
+//     and loses in proportion to the instructions of a sum.  Relative error against 64-bit sums, three products -> now, by
+//     the blocks of 32 channels that one CTA adds up (four kept taps a kernel): one 2.7e-6 -> 1.8e-6, two 4.6 -> 3.0, four
+//     8.3 -> 5.4, eight 15.6 -> 10.4, sixteen 30 -> 20; block patterns of two taps 1.06 -> 0.80, 1.54 -> 1.00, 2.48 -> 1.50,
+//     4.3 -> 2.6, 8.0 -> 5.0.  158 random calls: 0.60 to 0.85 of the error of three products (the cut along K is theirs, see
+//     plan_tc).  1x1 layers, with a ninth of the instructions, keep three tf32 products (eight blocks 2.3e-6).
+//     256->256 @80x80 x32 1084 -> 755 us, the split by four warps and the corrections together; the four units of tensor time
+//     it takes instead of six are 593 us at the bf16 peak.
 //   * One launch may carry several independent convolutions ("problems": the pyramid levels of a detection tower,
 //     the two branches of a block): the tile list runs over all of them, every role looks its tile's problem up.
 //     Small problems then fill the tail of the large ones' waves instead of paying a launch each.
