@@ -436,7 +436,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     a.cb_ch = row_bytes / esize;
     a.tiles_x = plan.tiles_x;
     a.n_sub = plan.n_sub;
-    a.half = plan.half ? 1 : 0;   // (the launch writes the order here)
+    if (plan.half) a.half = 1;   // (the launch writes the order here)
     a.sub_bytes = plan.sub_rows * row_bytes;
     if (p->ksize == 3 && S == 1) {
         a.x_add[0] = a.y_add[0] = -1;
@@ -482,8 +482,7 @@ int build_problem(const rtoss_ctx* ctx, const rtoss_packed* p, const void* x, vo
     // N/8 and M/16
     const unsigned fmt = f32 ? 2u : a.is_bf16 ? 1u : 0u;
     a.idesc = (1u << 4) | (fmt << 7) | (fmt << 10) | ((unsigned)(plan.N_px >> 3) << 17) | ((unsigned)(kMTile >> 4) << 24);
-    a.corr16 = has_corr16(p) ? 1 : 0;
-    a.idesc16 = (a.idesc & ~((7u << 7) | (7u << 10))) | (1u << 7) | (1u << 10);   // (bf16)
+    if (has_corr16(p)) a.idesc16 = (a.idesc & ~((7u << 7) | (7u << 10))) | (1u << 7) | (1u << 10);   // (bf16)
     a.pxm = pxm ? 1 : 0;
     a.MH = plan.N_px > 128 ? 2 : 1;
     a.n_cols = round_up(p->Cout, 16);
@@ -779,8 +778,8 @@ static SingleKernel single_kernel(const rtoss_ctx* ctx, bool f32, bool repacked,
         const int form = (pieces ? 0 : kFormElem) | (a.half ? kFormHalf : 0) | form_of(a.taps == 9 ? 3 : a.pxm ? 2 : 1, a.act, a.KS > 1, a.resid ? 1 + a.resid_post : 0, a.nchw != 0);
         if (void* k = form_kernel(ctx, a.is_bf16, false, form)) return reinterpret_cast<SingleKernel>(k);
     }
-    if (a.half) return nullptr;   // (forms only; single_plan_key asks for what they cover)
-    if (f32) return a.corr16 ? conv_tc_kernel<float, TcLaunch1, false, kFormCorr> : conv_tc_kernel<float, TcLaunch1>;
+    if (!f32 && a.half) return nullptr;   // (forms only; single_plan_key asks for what they cover)
+    if (f32) return a.idesc16 ? conv_tc_kernel<float, TcLaunch1, false, kFormCorr> : conv_tc_kernel<float, TcLaunch1>;
     if (repacked) return a.is_bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1, true> : conv_tc_kernel<__half, TcLaunch1, true>;
     return a.is_bf16 ? conv_tc_kernel<__nv_bfloat16, TcLaunch1> : conv_tc_kernel<__half, TcLaunch1>;
 }
@@ -876,7 +875,7 @@ static int launch_single(const rtoss_ctx* ctx, const rtoss_packed* p, const void
             g.max_nb = a.NB;
         }
     }
-    if (a.half) a.half = half_order(a.NA);
+    if (!f32 && a.half) a.half = half_order(a.NA);
     SingleKernel kernel = single_kernel(ctx, f32, repacked, a);
     if (!kernel) return (int)cudaErrorInvalidDeviceFunction;
     // at least half an SM's shared memory, so that a second CTA (which would wait for TMEM) never shares the SM

@@ -79,6 +79,8 @@
 
 #include <cuda.h>
 
+#include <cstddef>
+
 #include "conv_common.cuh"
 #include "select_core.cuh"
 
@@ -112,6 +114,21 @@ struct TcArgs {
     void* y;
     const void* resid;   // residual operand laid out like y, or null
     int resid_post;      // 1: the residual is added behind the activation (y = act(conv) + residual), 0: in front of it
+    // (Between two pointers, where the struct had four bytes to spare.  A launch reads it cold: with the fields that follow moved by
+    // four bytes, and no other change, the 55 launches of the small detector took 2.5 us more, 244.5 -> 247.)
+    union {
+        // 16-bit 3x3 of stride 2, where the planner says so and there is a form for it (0: not): a channel block comes as two
+        // activation stages, the odd input rows (two column phases, read by the first and the last row of taps) and the even ones
+        // (read by the middle row).  The even rows are done with first, so the stages are taken in the order in which they come
+        // free, which this word lists: the stage of the odd and the even rows of a block, then of the next, two bits each
+        // (half_order).  The taps go out in their own order, so that a layer adds up here as it does in one stage.  As one stage,
+        // of which only one fits beside the weights at 100 positions and more, fetching and multiplying take turns: 240->112
+        // @132x66 x18 34.5 -> 26.9 us, 144->240 @134x71 x9 24.3 -> 19.5, 48->304 @110x115 x31 62.4 -> 50.6.
+        unsigned half;
+        // fp32: the instruction descriptor of the two small products of a tap where they are bf16 ones (0: they are not; see the
+        // head of the file)
+        unsigned idesc16;
+    };
     const float* bias;
     const unsigned long long* issue;   // 3x3: which (tap, slab) pairs of (filter tile, channel block) to multiply; null = all
     int N, Ho, Wo, Cin, Cout;    // output image size
@@ -123,14 +140,6 @@ struct TcArgs {
     // every role for every tile: the four divisors as multiply-and-shift pairs (see tile_of), set by the host.
     unsigned div_ks[2], div_co[2], div_tx[2], div_ty[2];
     int n_sub, sub_bytes;        // sub-tiles of an activation stage (3x3 stride 2: the 4 input phases, or 2 of them) and their size
-    // 16-bit 3x3 of stride 2, where the planner says so and there is a form for it (0: not): a channel block comes as two activation stages, the odd input
-    // rows (two column phases, read by the first and the last row of taps) and the even ones (read by the middle row).  The even
-    // rows are done with first, so the stages are taken in the order in which they come free, which this word lists: the
-    // stage of the odd and the even rows of a block, then of the next, two bits each (half_order).  The taps go out in their
-    // own order, so that a layer adds up here as it does in one stage.  As one stage, of which only one fits beside the
-    // weights at 100 positions and more, fetching and multiplying take turns: 240->112 @132x66 x18 34.5 -> 26.9 us, 144->240
-    // @134x71 x9 24.3 -> 19.5, 48->304 @110x115 x31 62.4 -> 50.6.
-    unsigned half;
     int x_add[4], y_add[4];      // TMA start coordinate of sub-tile s: x = x0*S + x_add[s], y = y0*S + y_add[s]
     int tap_sub[9], tap_shift[9];  // which sub-tile tap t reads, and from which start row
     int G;                                     // taps per weight stage (one barrier round trip per G taps)
@@ -156,9 +165,7 @@ struct TcArgs {
     int row_bytes;
     unsigned desc_hi;
     int taps_real;        // 9 or 1; `taps` counts weight tiles per channel block: twice that for fp32 (heads, then remainders)
-    int lo_off;           // fp32: byte offset of the second half of an activation stage (remainders, or what corr16 says)
-    int corr16;           // fp32: the two small products of a tap are bf16 ones (see the head of the file)
-    unsigned idesc16;     // and their instruction descriptor
+    int lo_off;           // fp32: byte offset of the second half of an activation stage (remainders, or what idesc16 says)
     // The operand rings this problem runs with: NA activation stages of a_stage bytes from the start of the ring area, NB
     // weight stages of b_stage bytes from sB_off.  Problems of one launch with the same `geo` share all five; where a
     // CTA passes to a problem of another geometry its rings run empty first (see bar_switch in the kernel).
@@ -176,6 +183,7 @@ struct TcArgs {
     // on this problem's counter that make it complete (epilogue warps x CTAs that hold units of it).
     unsigned dep_mask, done_target;
 };
+static_assert(offsetof(TcArgs, bias) == 3 * sizeof(void*), "half and idesc16 take the four bytes behind resid_post");
 
 // A launch: up to NP convolutions sharing the CTA's rings (stage sizes are the largest any of them needs).  The struct
 // travels as the kernel's parameter: a launch of one convolution carries the small instantiation (a large parameter
@@ -990,7 +998,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
     constexpr bool kMulti = sizeof(G) > sizeof(TcLaunch1);
     constexpr bool kF32 = sizeof(T) == 4;   // fp32 data: tf32 instructions, three products per tap (see the head of the file)
     constexpr bool kAny = (kForm & ~kFormCorr) == 0;
-    constexpr bool kCorr1 = (kForm & kFormCorr) != 0;   // (fp32, one convolution: whether a.corr16; several: as it says)
+    constexpr bool kCorr1 = (kForm & kFormCorr) != 0;   // (fp32, one convolution: whether a.idesc16; several: as it says)
     constexpr int kKind = kForm & 3, kAct = ((kForm >> 2) & 7) - 1;   // (kAny: both from the arguments)
     constexpr bool kSplitF = (kForm & 32) != 0, kNchw = (kForm & 256) != 0;
     constexpr int kRes = (kForm >> 6) & 3;
@@ -1110,19 +1118,24 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 const int y0 = ti.ty * a.TH, x0 = ti.tx * a.TW;
                 const int cb_end = min(a.ncb, (ks + 1) * a.cb_per);
                 for (int cb = ks * a.cb_per; cb < cb_end; ++cb) {
-                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : kHalf ? 2 : a.n_sub, n_stages = kHalf ? 2 : 1;
-                    for (int part = 0; part < n_stages; ++part) {   // (half: the odd rows, sub-tiles 2 and 3, then the even ones)
-                        if (kHalf) ra.s = (int)(a.half >> (2 * (hq + part))) & 3;
-                        const int sa = ra.s, sub0 = kHalf ? 2 - 2 * part : 0;
+                    const int n_sub = (kKind == 1 || kKind == 2) ? 1 : kHalf ? 2 : a.n_sub;
+                    auto fill = [&](int sub0) {   // one stage, sub-tiles sub0 and up
+                        const int sa = ra.s;
                         ok = ok && mbar_wait(bar_emptyA + 8 * sa, ra.parity() ^ 1, g.wait_cycles);
-                        if (!ok) break;
+                        if (!ok) return;
                         mbar_expect_tx(bar_fullA + 8 * sa, a.a_tx_bytes * n_sub);
                         for (int sub = 0; sub < n_sub; ++sub)
                             tma_load_4d(sA + sa * a.a_stage + sub * a.sub_bytes, &g.tmA[pi], cb * a.cb_ch, x0 * a.S + a.x_add[sub0 + sub],
                                         y0 * a.S + a.y_add[sub0 + sub], n, bar_fullA + 8 * sa);
                         ra.advance(a.NA);
+                    };
+                    if constexpr (kHalf) {   // the odd rows, then the even ones
+                        ra.s = (int)(a.half >> (2 * hq)) & 3;
+                        fill(2);
+                        ra.s = (int)(a.half >> (2 * hq + 2)) & 3;
+                        hq ^= 2;
                     }
-                    hq ^= 2;
+                    fill(0);
                     if (!ok) break;
                 }
             }
@@ -1375,7 +1388,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                             // weight tile v of the block: tap v (16-bit data); fp32: the heads of tap v, then (v >= 9 resp. 1) what
                             // corrects tap v - 9.  Heads meet the activations' heads and remainders, remainders the heads
                             // only; with bf16 corrections heads meet heads, and the rest is in the second arrays.
-                            if (kF32 && (kMulti ? a.corr16 != 0 : kCorr1)) {
+                            if (kF32 && (kMulti ? a.idesc16 != 0 : kCorr1)) {
                                 const unsigned xr0 = xl0 + ((unsigned)a.lo_off >> 4);
                                 for (int i = 0; i < a.G; ++i) {
                                     const int v = t0 + i, t = v >= 9 ? v - 9 : v;
@@ -1453,7 +1466,7 @@ conv_tc_kernel(const __grid_constant__ G g) {
                 __syncwarp();   // (lane 0 has seen the copy; a shuffle orders no memory, and all lanes read the block)
                 const unsigned src = sA + ra.s * a.a_stage, dst = src + (unsigned)a.lo_off;
                 const int n16 = (a.n_sub * a.sub_bytes) >> 4, first = (warp - kWeightWarp - 1) * 32 + lane;
-                if (kMulti ? a.corr16 != 0 : kCorr1) split_block16(src, dst, n16, first);
+                if (kMulti ? a.idesc16 != 0 : kCorr1) split_block16(src, dst, n16, first);
                 else split_block32(src, dst, n16, first);
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
