@@ -152,38 +152,31 @@ template <typename V> __device__ __forceinline__ unsigned round2(float a, float 
         return *reinterpret_cast<const unsigned*>(&u);
     }
 }
-// Two neighbouring positions (f, f even) as one aligned word; fp32: tf32 heads, and what corrects them lo_at further on (see
-// expand_one).
-template <typename V> __device__ __forceinline__ void put_pair(V* wtc, int64_t f, int64_t lo_at, bool corr16, float a, float b) {
+// Two neighbouring positions as one aligned word; fp32: tf32 heads, and at lo what corrects them (see expand_one).
+template <typename V, bool kCorr16> __device__ __forceinline__ void put_pair(V* at, V* lo, float a, float b) {
     using namespace rtoss_dev;
-    V* at = wtc + f;
-    if constexpr (sizeof(V) == 4) {
-        if (corr16) {
-            const float ha = tf32_near(a), hb = tf32_near(b);
-            *reinterpret_cast<float2*>(at) = make_float2(ha, hb);
-            put_corr16_two(wtc + lo_at, f, a, b, __fsub_rn(a, ha), __fsub_rn(b, hb));
-            return;
-        }
-        *reinterpret_cast<float2*>(at) = make_float2(tf32_head(a), tf32_head(b));
-        *reinterpret_cast<float2*>(at + lo_at) = make_float2(__fsub_rn(a, tf32_head(a)), __fsub_rn(b, tf32_head(b)));
-    } else {
+    if constexpr (sizeof(V) == 2) {
         *reinterpret_cast<unsigned*>(at) = round2<V>(a, b);
+    } else if constexpr (kCorr16) {
+        const float ha = tf32_near(a), hb = tf32_near(b);
+        *reinterpret_cast<float2*>(at) = make_float2(ha, hb);
+        put_corr16_two(reinterpret_cast<uint16_t*>(lo), a, b, __fsub_rn(a, ha), __fsub_rn(b, hb));
+    } else {
+        *reinterpret_cast<float2*>(at) = make_float2(tf32_head(a), tf32_head(b));
+        *reinterpret_cast<float2*>(lo) = make_float2(__fsub_rn(a, tf32_head(a)), __fsub_rn(b, tf32_head(b)));
     }
 }
-template <typename V> __device__ __forceinline__ void put_one(V* wtc, int64_t f, int64_t lo_at, bool corr16, float a) {
+template <typename V> __device__ __forceinline__ void put_one(V* at, V* lo, bool corr16, float a) {
     using namespace rtoss_dev;
-    V* at = wtc + f;
-    if constexpr (sizeof(V) == 4) {
-        if (corr16) {
-            const float h = tf32_near(a);
-            *at = h;
-            put_corr16_one(wtc + lo_at, f, a, __fsub_rn(a, h));
-            return;
-        }
-        *at = tf32_head(a);
-        at[lo_at] = __fsub_rn(a, tf32_head(a));
-    } else {
+    if constexpr (sizeof(V) == 2) {
         *at = narrow_to<V>(a);
+    } else if (corr16) {
+        const float h = tf32_near(a);
+        *at = h;
+        put_corr16_one(reinterpret_cast<uint16_t*>(lo), a, __fsub_rn(a, h));
+    } else {
+        *at = tf32_head(a);
+        *lo = __fsub_rn(a, tf32_head(a));
     }
 }
 
@@ -240,13 +233,32 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
         const bool word = two && p1 == p0 + 1 && (p0 & 1) == 0 && (tap_step & 1) == 0 && (copy_step & 1) == 0;
         V* at = wtc + p0;
         const int64_t d1 = p1 - p0;
+        // fp32: where what corrects position p lies; a tap or a copy further down is as far as in the first array (with bf16
+        // corrections both steps are whole blocks of 32 channels)
         const bool corr16 = sizeof(V) == 4 && rtoss_f32_corr16(Cin, 3);
+        auto lo_of = [&](int64_t p) -> V* {
+            if constexpr (sizeof(V) == 4) return corr16 ? reinterpret_cast<V*>(corr16_at(wtc + lo_at, p)) : wtc + lo_at + p;
+            else return nullptr;
+        };
+        V* lo = lo_of(p0);
         if (word && L.lay.copies == 1) {
+            if constexpr (sizeof(V) == 4) {
+                if (corr16) {
+                    const int64_t to_lo = lo - at;
+#pragma unroll
+                    for (int t = 0; t < 9; ++t, at += tap_step) {
+                        const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
+                        const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
+                        put_pair<V, true>(at, at + to_lo, a, b);
+                    }
+                    return;
+                }
+            }
 #pragma unroll
             for (int t = 0; t < 9; ++t, at += tap_step) {
                 const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
                 const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
-                put_pair<V>(wtc, at - wtc, lo_at, corr16, a, b);
+                put_pair<V, false>(at, at + lo_at, a, b);
             }
             return;
         }
@@ -273,18 +285,21 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
                 }
             }
         } else {
+            const int64_t to_lo = lo - at, to_lo1 = lo_of(p1) - at;
 #pragma unroll 1
             for (int c = 0; c < L.lay.copies; ++c, at += copy_step) {
                 V* to = at;
-#pragma unroll
+#pragma unroll 3
                 for (int t = 0; t < 9; ++t, to += tap_step) {
                     const float a = (mm >> t) & 1u ? raw_at<T>(raw, base * 9 + t) : 0.f;
                     const float b = (mm >> (16 + t)) & 1u ? raw_at<T>(raw, base * 9 + 9 + t) : 0.f;
-                    if (word) {
-                        put_pair<V>(wtc, to - wtc, lo_at, corr16, a, b);
+                    if (word && corr16) {
+                        put_pair<V, true>(to, to + to_lo, a, b);
+                    } else if (word) {
+                        put_pair<V, false>(to, to + to_lo, a, b);
                     } else {
-                        put_one<V>(wtc, to - wtc, lo_at, corr16, a);
-                        if (two) put_one<V>(wtc, to - wtc + d1, lo_at, corr16, b);
+                        put_one<V>(to, to + to_lo, corr16, a);
+                        if (two) put_one<V>(to + d1, to + to_lo1, corr16, b);
                     }
                 }
             }
@@ -320,13 +335,18 @@ __device__ __forceinline__ void pack_chunk(const BatchLayer& L, long long first,
             } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    if (e + j < n) put_one<V>(wtc, f + j + (cin_p != Cin ? (int64_t)((unsigned)(f + j) / (unsigned)Cin) * (cin_p - Cin) : 0), tap_step, false, v[j]);
+                    if (e + j < n) {
+                        V* at = wtc + f + j + (cin_p != Cin ? (int64_t)((unsigned)(f + j) / (unsigned)Cin) * (cin_p - Cin) : 0);
+                        put_one<V>(at, at + tap_step, false, v[j]);
+                    }
             }
         }
     }
 }
 
-// Bound by instructions (0.75 a cycle and scheduler; 35 % of the copy rate).  32 M weights, 8 patterns of four taps: 131 us
+// Bound by instructions (0.75 a cycle and scheduler; 35 % of the copy rate).  fp32 handles with bf16 corrections have a loop of
+// their own over the taps, which keeps two addresses: with the choice and the second address made per tap the kernel of 40
+// registers spilled, and 32 M bf16 weights took 107 us instead of 89 (7 M fp32 ones 41 instead of 33).  32 M weights, 8 patterns of four taps: 131 us
 // with one kernel per thread that held its weights in registers through all outputs, 65 us in this form; 20 us instead of
 // 31 for 7 M.  (Prefetching the next chunk with a second buffer cost occupancy and was slower: 142 us on the older form.)
 template <int T>

@@ -42,8 +42,8 @@ __device__ __forceinline__ int select_best(const float (&w)[9], const Tab& tab, 
 // off instead), whose remainder is half as large.
 __device__ __forceinline__ float tf32_head(float f) { return __uint_as_float(__float_as_uint(f) & 0xFFFFE000u); }
 __device__ __forceinline__ float tf32_near(float f) {
-    const unsigned u = __float_as_uint(f), r = (u + 0x1000u) & 0xFFFFE000u;
-    return __uint_as_float((r & 0x7F800000u) == 0x7F800000u ? u & 0xFFFFE000u : r);
+    const unsigned u = __float_as_uint(f);
+    return __uint_as_float(((u << 1) >= 0xFEFFE000u ? u : u + 0x1000u) & 0xFFFFE000u);
 }
 // Two floats rounded to bf16, a in the low half; finite values stay finite.
 __device__ __forceinline__ unsigned bf16x2_sat(float a, float b) {
@@ -52,64 +52,68 @@ __device__ __forceinline__ unsigned bf16x2_sat(float a, float b) {
     return d;
 }
 // The second array of rtoss_f32_corr16 layers: weight and remainder of flat position f (rows are whole blocks of 32 channels)
-// into its block; two neighbouring positions, f even.
+// into its block; two neighbouring positions, the first even.
 __device__ __forceinline__ uint16_t* corr16_at(float* lo, int64_t f) { return reinterpret_cast<uint16_t*>(lo) + 2 * (f & ~(int64_t)31) + (f & 31); }
-__device__ __forceinline__ void put_corr16_one(float* lo, int64_t f, float w, float rest) {
+__device__ __forceinline__ void put_corr16_one(uint16_t* at, float w, float rest) {
     const unsigned u = bf16x2_sat(w, rest);
-    uint16_t* at = corr16_at(lo, f);
     at[0] = (uint16_t)u;
     at[32] = (uint16_t)(u >> 16);
 }
-__device__ __forceinline__ void put_corr16_two(float* lo, int64_t f, float w0, float w1, float rest0, float rest1) {
-    uint16_t* at = corr16_at(lo, f);
+__device__ __forceinline__ void put_corr16_two(uint16_t* at, float w0, float w1, float rest0, float rest1) {
     *reinterpret_cast<unsigned*>(at) = bf16x2_sat(w0, w1);
     *reinterpret_cast<unsigned*>(at + 32) = bf16x2_sat(rest0, rest1);
 }
-__device__ __forceinline__ float to_float(float v) { return v; }
-__device__ __forceinline__ float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
-__device__ __forceinline__ float to_float(__half v) { return __half2float(v); }
-
 template <typename V> __device__ __forceinline__ V narrow_to(float v);
 template <> __device__ __forceinline__ float narrow_to<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 narrow_to<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 template <> __device__ __forceinline__ __half narrow_to<__half>(float v) { return __float2half_rn(v); }
 
-// The dense expansion of one kernel (see pack_one).
+// The dense expansion of one kernel (see pack_one).  fp32: the tensor path multiplies tf32 operands, so every weight is stored as its
+// tf32 head and, in a second copy of the array behind the first, what corrects it: the remainder (exact in fp32), or two bf16
+// numbers (rtoss_f32_corr16).  (A loop of its own for those: as a choice per tap it cost every fp32 layer, re-packing 64x36
+// 6.5 -> 7.2 us.)
 template <typename V>
 __device__ __forceinline__ void expand_one(const float* w, unsigned m, int64_t i, V* __restrict__ wtc, int ksize, int Cin, int rows,
                                            int rep_rows, int copies, int cin_p) {
-    // (layers hold fewer than 2^31 kernels: 32-bit division, several times cheaper than the 64-bit one)
-    const int64_t co = (int64_t)((unsigned)i / (unsigned)Cin), ci = i - co * Cin;
-    // fp32: the tensor path multiplies tf32 operands, so every weight is stored as its tf32 head and, in a second copy of
-    // the array behind the first, what corrects it: the remainder (exact in fp32), or two bf16 numbers (rtoss_f32_corr16)
-    const bool corr16 = rtoss_f32_corr16(Cin, ksize);
-    const int64_t lo_at = (int64_t)(ksize == 3 ? 9 : 1) * rows * cin_p;
-#pragma unroll
-    for (int t = 0; t < 9; ++t) {
-        V v = (m & (1u << t)) ? narrow_to<V>(w[t]) : narrow_to<V>(0.f);
-        V lo = v;
-        if (sizeof(V) == 4) {
-            const float f = (m & (1u << t)) ? w[t] : 0.f;
-            const float head = corr16 ? tf32_near(f) : tf32_head(f);
-            v = narrow_to<V>(head);
-            lo = narrow_to<V>(__fsub_rn(f, head));
-        }
-        if (ksize == 3) {
-            const int64_t at = ((int64_t)t * rows + co) * cin_p + ci;   // copy 0; copy c lies c * rep_rows rows further down
-            for (int c = 0; c < copies; ++c) {
-                wtc[at + (int64_t)c * rep_rows * cin_p] = v;
-                if (sizeof(V) == 4) {
-                    const int64_t f = at + (int64_t)c * rep_rows * cin_p;
-                    if (corr16) put_corr16_one(reinterpret_cast<float*>(wtc) + lo_at, f, to_float(v) + to_float(lo), to_float(lo));
-                    else wtc[lo_at + f] = lo;
-                }
-            }
+    const int64_t tap_step = (int64_t)rows * cin_p, copy_step = (int64_t)rep_rows * cin_p, lo_at = (ksize == 3 ? 9 : 1) * tap_step;
+    auto put = [&](int64_t at, float f) {
+        if constexpr (sizeof(V) == 4) {
+            wtc[at] = tf32_head(f);
+            wtc[lo_at + at] = __fsub_rn(f, tf32_head(f));
         } else {
+            wtc[at] = narrow_to<V>(f);
+        }
+    };
+    if (ksize != 3) {
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
             int64_t at = i * 9 + t;   // flat position; rows are cin_p apart where they are padded
             if (cin_p != Cin) at += (int64_t)((unsigned)at / (unsigned)Cin) * (cin_p - Cin);
-            wtc[at] = v;
-            if (sizeof(V) == 4) wtc[lo_at + at] = lo;
+            put(at, (m & (1u << t)) ? w[t] : 0.f);
         }
+        return;
+    }
+    // (layers hold fewer than 2^31 kernels: 32-bit division, several times cheaper than the 64-bit one)
+    const int64_t co = (int64_t)((unsigned)i / (unsigned)Cin), p = co * cin_p + (i - co * Cin);   // copy 0 of tap 0; copy c lies c * rep_rows rows further down
+    if constexpr (sizeof(V) == 4) {
+        if (rtoss_f32_corr16(Cin, 3)) {
+            V* at = wtc + p;
+            uint16_t* lo = corr16_at(wtc + lo_at, p);   // (taps and copies lie whole blocks apart)
+#pragma unroll
+            for (int t = 0; t < 9; ++t) {
+                const float f = (m & (1u << t)) ? w[t] : 0.f, h = tf32_near(f), rest = __fsub_rn(f, h);
+                for (int c = 0; c < copies; ++c) {
+                    at[t * tap_step + c * copy_step] = h;
+                    put_corr16_one(lo + 2 * (t * tap_step + c * copy_step), f, rest);
+                }
+            }
+            return;
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < 9; ++t) {
+        const float f = (m & (1u << t)) ? w[t] : 0.f;
+        for (int c = 0; c < copies; ++c) put(p + t * tap_step + c * copy_step, f);
     }
 }
 
