@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kDenseThreads, 4) to_dense_kernel(const V* __r
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(to) + (unsigned)i), "l"(static_cast<const char*>(src) + i) : "memory");
         if (tid < n - whole) static_cast<uint8_t*>(to)[whole + tid] = __ldcg(static_cast<const uint8_t*>(src) + whole + tid);
     };
-    if (n_kernels > 0) fetch(sm, masks, 512);   // (the first step waits for it; a block without one ends with nothing under way)
+    fetch(sm, masks, 512);
     bool waited = false;
     const bool aligned = (reinterpret_cast<uintptr_t>(out) & 15) == 0;
     for (int64_t first = (int64_t)blockIdx.x * step; first < n_kernels; first += (int64_t)gridDim.x * step) {
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kDenseThreads, 4) to_dense_kernel(const V* __r
         for (int i = nv * 16 / (int)sizeof(V) + tid; i < n; i += kDenseThreads) dst[i] = sd[i];
         __syncthreads();
     }
-    if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (!waited) asm volatile("cp.async.wait_all; griddepcontrol.wait;" ::: "memory");   // (a layer without kernels: the table's copy)
     // the trailing weights of a 1x1 layer (fewer than nine) belong to no run: pruned
     if (blockIdx.x == 0 && tid < n_dense - 9 * n_kernels) out[9 * n_kernels + tid] = narrow<V>(0.f);
 }
