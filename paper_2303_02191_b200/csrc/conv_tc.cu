@@ -292,22 +292,37 @@ bool plan_search(const PlanKey& k, bool resid, int only_ks, TcPlan* out) {
 // The plan of a call.  The split is decided as if the call had a residual operand, whether it has one or not: a call with
 // a residual then adds up its products in the order of the same call without one (same bits).
 // Searching takes tens of microseconds of host time, more than a launch: every thread remembers the plans of its last
-// few hundred kinds of call.  A call looks up one key, so that it never drives itself out of the memory.  A plan is a function of its key and of the device's cluster limits, which whoever plans for a
-// device has had asked first (ensure_device): it does not matter which thread or context asks.
+// few hundred kinds of call.  A single call looks up one key, a grouped one some fifty (ten convolutions at seven tile sizes):
+// eight ways a set, the least recently used one given up, so that a call does not drive out its own plans.  (With one way it
+// nearly always did: ten 3x3 layers on five levels took 13 to 60 us to issue, by the chance of the hash, 14 now; finding a plan
+// among eight ways takes such a call 1 us more than among one.)  A plan is a function of its key and of the device's cluster
+// limits, which whoever plans for a device has had asked first (ensure_device): it does not matter which thread or context asks.
 bool plan_tc(const PlanKey& k, TcPlan* out) {
     struct Memo {
         PlanKey key;
         TcPlan plan;
-        bool set, ok;
+        unsigned hash;
+        bool ok;
+        unsigned long long used;   // when it was last asked for (0: empty)
     };
-    constexpr int kMemo = 256;
-    static thread_local Memo memo[kMemo];
+    constexpr int kSets = 64, kWays = 8;   // (fifty keys over the sets: nine in one are as good as never)
+    static thread_local Memo memo[kSets][kWays];
+    static thread_local unsigned long long asked = 0;
     unsigned h = 2166136261u;
     const int* w = reinterpret_cast<const int*>(&k);
     for (size_t i = 0; i < sizeof(PlanKey) / sizeof(int); ++i) h = (h ^ (unsigned)w[i]) * 16777619u;
-    Memo& m = memo[(h ^ (h >> 15)) % kMemo];
-    if (!m.set || memcmp(&m.key, &k, sizeof(k)) != 0) {
-        m.set = false;
+    h ^= h >> 15;
+    h *= 0x9E3779B1u;   // (sizes are multiples of something: the low bits alone repeat)
+    Memo* set = memo[h >> 26];
+    static_assert(kSets == 1 << (32 - 26), "the hash's upper bits name a set");
+    int way = 0;
+    while (way < kWays && !(set[way].used && set[way].hash == h && memcmp(&set[way].key, &k, sizeof(k)) == 0)) ++way;
+    const bool known = way < kWays;
+    for (int i = way = known ? way : 0; !known && i < kWays; ++i)
+        if (set[i].used < set[way].used) way = i;
+    Memo& m = set[way];
+    if (!known) {
+        m.used = 0;
         const bool pxm = k.ksize == 1 && k.Cout <= kPxmMaxCout && k.dtype != RTOSS_F32;
         if (k.shared || pxm) {
             m.ok = plan_search(k, k.resid != 0, 1, &m.plan);
@@ -338,8 +353,9 @@ bool plan_tc(const PlanKey& k, TcPlan* out) {
             }
         }
         m.key = k;
-        m.set = true;
+        m.hash = h;
     }
+    m.used = ++asked;
     *out = m.plan;
     return m.ok;
 }

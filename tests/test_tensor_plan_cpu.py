@@ -122,6 +122,24 @@ def test_a_repeated_call_is_not_planned_again():
     assert max(took) <= 3 * sorted(took)[500]
 
 
+def test_fifty_calls_in_turn_are_not_planned_again():
+    """As many plans as a grouped call looks up: asked for one after the other, over and over, none of them is searched twice.
+    Twenty sets of fifty layers; the fastest of twenty rounds for each layer against their median."""
+    rng = random.Random(7)
+    for _ in range(20):
+        calls = []
+        for _ in range(50):
+            d = rt.ConvDesc(rng.randint(1, 32), rng.randint(7, 160), rng.randint(7, 160), 1, rt.NHWC, BF16, 0, None, 0, 0, 0, None, 0)
+            calls.append((ctypes.byref(d), 3, 8 * rng.randint(2, 64), 8 * rng.randint(2, 64), BF16, 0, ctypes.byref(rt.TensorPlan())))
+        best = [1 << 60] * len(calls)
+        for _ in range(20):
+            for i, args in enumerate(calls):
+                t = time.perf_counter_ns()
+                rt.lib.rtoss_tensor_plan_of(*args)
+                best[i] = min(best[i], time.perf_counter_ns() - t)
+        assert max(best) <= 3 * sorted(best)[25]
+
+
 @pytest.mark.parametrize("dtype,ksize,cin,units", [("bf16", 3, 64, 1), ("f16", 1, 36, 1), ("f32", 3, 64, 4), ("f32", 3, 36, 6), ("f32", 1, 64, 6)])
 def test_tensor_time_of_a_product(dtype, ksize, cin, units):
     """What the rooflines of bench.py and the sweep divide the tensor peak by, and that both have a name for it."""
