@@ -124,7 +124,7 @@ def test_a_repeated_call_is_not_planned_again():
 
 def test_fifty_calls_in_turn_are_not_planned_again():
     """As many plans as a grouped call looks up: asked for one after the other, over and over, none of them is searched twice.
-    Twenty sets of fifty layers; the fastest of twenty rounds for each layer against their median."""
+    Twenty sets of fifty layers; the fastest of twenty passes for each layer against their median."""
     rng = random.Random(7)
     for _ in range(20):
         calls = []
