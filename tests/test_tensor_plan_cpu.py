@@ -105,39 +105,51 @@ def test_narrow_layers_stage_half_rows_and_keep_a_deeper_ring():
     assert q.row_bytes == 128 and q.act_stages == 2
 
 
-def test_a_repeated_call_is_not_planned_again():
-    """Planning searches for tens of microseconds; a thread remembers its plans, and a call looks up one key, so asking twice in a
-    row never searches twice.  The fastest of forty repeats of a thousand random layers of stride 2 against their median."""
-    rng = random.Random(6)
-    took = []
-    for _ in range(1000):
-        d = rt.ConvDesc(rng.randint(1, 32), rng.randint(7, 160), rng.randint(7, 160), 2, rt.NHWC, BF16, 0, None, 0, 0, 0, None, 0)
-        args = (ctypes.byref(d), 3, 8 * rng.randint(2, 64), 8 * rng.randint(2, 64), BF16, 0, ctypes.byref(rt.TensorPlan()))
-        best = 1 << 60
-        for _ in range(40):
+def _random_call(rng, stride):
+    d = rt.ConvDesc(rng.randint(1, 32), rng.randint(7, 160), rng.randint(7, 160), stride, rt.NHWC, BF16, 0, None, 0, 0, 0, None, 0)
+    return ctypes.byref(d), 3, 8 * rng.randint(2, 64), 8 * rng.randint(2, 64), BF16, 0, ctypes.byref(rt.TensorPlan())
+
+
+def _fastest(calls, passes):
+    """Nanoseconds of each call, the fastest of its repeats; the calls take turns."""
+    best = [1 << 60] * len(calls)
+    for _ in range(passes):
+        for i, args in enumerate(calls):
             t = time.perf_counter_ns()
             rt.lib.rtoss_tensor_plan_of(*args)
-            best = min(best, time.perf_counter_ns() - t)
-        took.append(best)
-    assert max(took) <= 3 * sorted(took)[500]
+            best[i] = min(best[i], time.perf_counter_ns() - t)
+    return best
+
+
+def _again_if_slow(calls, passes, usual):
+    """The slowest call, measured again up to six times while it takes three times the usual: the machine may have been busy
+    elsewhere, while a call that is planned again is slow every time."""
+    for _ in range(6):
+        slowest = max(_fastest(calls, passes))
+        if slowest <= 3 * usual:
+            break
+        time.sleep(0.02)
+    return slowest
+
+
+def test_a_repeated_call_is_not_planned_again():
+    """Planning searches for tens of microseconds; a thread remembers its plans, and a call looks up one key, so asking twice in a
+    row never searches twice.  A thousand random layers of stride 2 against their median."""
+    rng = random.Random(6)
+    calls = [_random_call(rng, 2) for _ in range(1000)]
+    took = [_fastest([c], 40)[0] for c in calls]
+    usual = sorted(took)[500]
+    assert all(t <= 3 * usual or _again_if_slow([c], 40, usual) <= 3 * usual for c, t in zip(calls, took))
 
 
 def test_fifty_calls_in_turn_are_not_planned_again():
     """As many plans as a grouped call looks up: asked for one after the other, over and over, none of them is searched twice.
-    Twenty sets of fifty layers; the fastest of twenty passes for each layer against their median."""
+    Twenty sets of fifty layers against their median."""
     rng = random.Random(7)
     for _ in range(20):
-        calls = []
-        for _ in range(50):
-            d = rt.ConvDesc(rng.randint(1, 32), rng.randint(7, 160), rng.randint(7, 160), 1, rt.NHWC, BF16, 0, None, 0, 0, 0, None, 0)
-            calls.append((ctypes.byref(d), 3, 8 * rng.randint(2, 64), 8 * rng.randint(2, 64), BF16, 0, ctypes.byref(rt.TensorPlan())))
-        best = [1 << 60] * len(calls)
-        for _ in range(20):
-            for i, args in enumerate(calls):
-                t = time.perf_counter_ns()
-                rt.lib.rtoss_tensor_plan_of(*args)
-                best[i] = min(best[i], time.perf_counter_ns() - t)
-        assert max(best) <= 3 * sorted(best)[25]
+        calls = [_random_call(rng, 1) for _ in range(50)]
+        usual = sorted(_fastest(calls, 20))[25]
+        assert _again_if_slow(calls, 20, usual) <= 3 * usual
 
 
 @pytest.mark.parametrize("dtype,ksize,cin,units", [("bf16", 3, 64, 1), ("f16", 1, 36, 1), ("f32", 3, 64, 4), ("f32", 3, 36, 6), ("f32", 1, 64, 6)])
